@@ -1038,12 +1038,12 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
                 const int gd = tol >= kGramFiveDigitTol ? 5 : 6;
                 const size_t part = k::ozaki_cols_scratch(n, q);
                 H->oz.reserve(3 * part);
-                k::OzakiOperand X = k::ozaki_split_cols(s, n, q, H->Psi.p, q, H->oz.p, gd);
-                k::OzakiOperand YS = k::ozaki_split_cols(s, n, q, H->SP.p, q, H->oz.p + part, gd);
-                k::OzakiOperand YM = k::ozaki_split_cols(s, n, q, H->MP.p, q, H->oz.p + 2 * part, gd);
+                k::OzakiOperand X = k::ozaki_split_cols(s, n, q, H->Psi.p, q, H->oz.p, gd, k::OzakiRole::X);
+                k::OzakiOperand YS = k::ozaki_split_cols(s, n, q, H->SP.p, q, H->oz.p + part, gd, k::OzakiRole::Y);
+                k::OzakiOperand YM = k::ozaki_split_cols(s, n, q, H->MP.p, q, H->oz.p + 2 * part, gd, k::OzakiRole::Y);
                 const double t_split = ts.stop();
-                k::ozaki_product(s, X, YS, X.kp, H->Sbar.p, q, 0, true);
-                k::ozaki_product(s, X, YM, X.kp, H->Mbar.p, q, 0, true);
+                k::ozaki_product(s, X, YS, H->Sbar.p, q, 0, true);
+                k::ozaki_product(s, X, YM, H->Mbar.p, q, 0, true);
                 const double t_prod = ts.stop();
                 inf.ms_tc_product += t_prod;
                 ph[2] = t_split + t_prod;
@@ -1065,9 +1065,9 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
                 const size_t part = k::ozaki_rows_scratch(n, q);
                 H->oz.reserve(part + k::ozaki_cols_scratch(q, q));
                 k::OzakiOperand X = k::ozaki_split_rows(s, n, q, H->Psi.p, q, H->oz.p);
-                k::OzakiOperand Y = k::ozaki_split_cols(s, q, q, H->phibar.p, q, H->oz.p + part);
+                k::OzakiOperand Y = k::ozaki_split_cols(s, q, q, H->phibar.p, q, H->oz.p + part, k::kOzakiSlices, k::OzakiRole::Y);
                 const double t_split = ts.stop();
-                k::ozaki_product(s, X, Y, X.kp, H->Phi.p, q, 1);
+                k::ozaki_product(s, X, Y, H->Phi.p, q, 1);
                 const double t_prod = ts.stop();
                 inf.ms_tc_product += t_prod;
                 ph[4] = t_split + t_prod;
@@ -1655,10 +1655,10 @@ hsim_status hsim_gram_tc(hsim_ctx *ctx, int n, int ka, int kb, const double *A, 
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"G", G}});
         DevBuf<unsigned char> scratch(k::ozaki_cols_scratch(n, ka) + k::ozaki_cols_scratch(n, kb));
-        k::OzakiOperand X = k::ozaki_split_cols(ctx->stream, n, ka, A, lda, scratch.p, digits);
+        k::OzakiOperand X = k::ozaki_split_cols(ctx->stream, n, ka, A, lda, scratch.p, digits, k::OzakiRole::X);
         k::OzakiOperand Y =
-            k::ozaki_split_cols(ctx->stream, n, kb, B, ldb, scratch.p + k::ozaki_cols_scratch(n, ka), digits);
-        k::ozaki_product(ctx->stream, X, Y, X.kp, G, kb, 0);
+            k::ozaki_split_cols(ctx->stream, n, kb, B, ldb, scratch.p + k::ozaki_cols_scratch(n, ka), digits, k::OzakiRole::Y);
+        k::ozaki_product(ctx->stream, X, Y, G, kb, 0);
         k::ozaki_check(ctx->stream);
     });
 }
@@ -1672,8 +1672,9 @@ hsim_status hsim_gemm_update_tc(hsim_ctx *ctx, int n, int kk, int m, const doubl
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"C", C}});
         DevBuf<unsigned char> scratch(k::ozaki_rows_scratch(n, kk) + k::ozaki_cols_scratch(kk, m));
         k::OzakiOperand X = k::ozaki_split_rows(ctx->stream, n, kk, A, lda, scratch.p);
-        k::OzakiOperand Y = k::ozaki_split_cols(ctx->stream, kk, m, B, ldb, scratch.p + k::ozaki_rows_scratch(n, kk));
-        k::ozaki_product(ctx->stream, X, Y, X.kp, C, ldc, 1);
+        k::OzakiOperand Y = k::ozaki_split_cols(ctx->stream, kk, m, B, ldb, scratch.p + k::ozaki_rows_scratch(n, kk),
+                                                 k::kOzakiSlices, k::OzakiRole::Y);
+        k::ozaki_product(ctx->stream, X, Y, C, ldc, 1);
         k::ozaki_check(ctx->stream);
     });
 }

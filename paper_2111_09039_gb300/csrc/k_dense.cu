@@ -631,8 +631,8 @@ __global__ void k_rows_rsqrt(int rows, int cols, const double *__restrict__ d, d
 static void tc_mm(cudaStream_t s, int k, const double *A, int lda, const double *B, int ldb, double *C, int ldc,
                   unsigned char *oz) {
     OzakiOperand a = ozaki_split_rows(s, k, k, A, lda, oz);
-    OzakiOperand b = ozaki_split_cols(s, k, k, B, ldb, oz + ozaki_rows_scratch(k, k));
-    ozaki_product(s, a, b, a.kp, C, ldc, 0);
+    OzakiOperand b = ozaki_split_cols(s, k, k, B, ldb, oz + ozaki_rows_scratch(k, k), kOzakiSlices, OzakiRole::Y);
+    ozaki_product(s, a, b, C, ldc, 0);
 }
 
 // Z = M_bar^-1/2 by the coupled Newton-Schulz iteration Y_0 = M_bar, Z_0 = I,
@@ -715,8 +715,8 @@ int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar,
             HSIM_LAUNCHED();
             sym_eig(s, k, m, T, evals, V, m, ework);
             OzakiOperand a = ozaki_split_rows(s, k, k, Wz, k, oz);
-            OzakiOperand b = ozaki_split_cols(s, k, m, V, m, oz + ozaki_rows_scratch(k, k));
-            ozaki_product(s, a, b, a.kp, X, ldx, 0);
+            OzakiOperand b = ozaki_split_cols(s, k, m, V, m, oz + ozaki_rows_scratch(k, k), kOzakiSlices, OzakiRole::Y);
+            ozaki_product(s, a, b, X, ldx, 0);
             ozaki_check(s);
             return 0;
         }
@@ -755,17 +755,17 @@ int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar,
         k_cinv<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, F, d, Cr, Cc);
         HSIM_LAUNCHED();
         OzakiOperand a = ozaki_split_rows(s, k, k, Cr, k, oz);
-        OzakiOperand b = ozaki_split_cols(s, k, k, Sbar, lds, oz + rb);
-        ozaki_product(s, a, b, a.kp, W, k, 0);
+        OzakiOperand b = ozaki_split_cols(s, k, k, Sbar, lds, oz + rb, kOzakiSlices, OzakiRole::Y);
+        ozaki_product(s, a, b, W, k, 0);
         a = ozaki_split_rows(s, k, k, W, k, oz);
-        b = ozaki_split_cols(s, k, k, Cc, k, oz + rb);
-        ozaki_product(s, a, b, a.kp, T, k, 0);
+        b = ozaki_split_cols(s, k, k, Cc, k, oz + rb, kOzakiSlices, OzakiRole::Y);
+        ozaki_product(s, a, b, T, k, 0);
         k_symmetrize<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, T, k);
         HSIM_LAUNCHED();
         sym_eig(s, k, m, T, evals, V, m, ework);
         a = ozaki_split_rows(s, k, k, Cc, k, oz);
-        b = ozaki_split_cols(s, k, m, V, m, oz + rb);
-        ozaki_product(s, a, b, a.kp, X, ldx, 0);
+        b = ozaki_split_cols(s, k, m, V, m, oz + rb, kOzakiSlices, OzakiRole::Y);
+        ozaki_product(s, a, b, X, ldx, 0);
         ozaki_check(s);
         return 0;
     }

@@ -4,18 +4,15 @@
 // update Phi = Psi Phi_bar of Alg. 1 are the dominant dense work of the
 // subspace iteration; in FP64 they run at the GB300's 1.2 TFLOP/s FP64 rate.
 // Here each FP64 operand is split, against one power of two per row (or per
-// column), into SL integer digits of at most 8 bits (SL = 6, or 5 where 39
+// column), into SL integer digits of at most 8 bits (SL = 7, 6, or 5 where 39
 // bits suffice),
 //     x = 2^(e-7) * sum_s d_s 2^(-8 s),   |d_0| <= 128, |d_s| <= 128,
-// which BF16 represents exactly.  A digit product is an integer of at most
-// 2^14, so up to 1024 of them sum exactly in an FP32 accumulator: the tensor
-// cores compute sum_r d_s(x_ir) d_t(y_jr) with no rounding, grouped by
-// D = s + t (pairs with D >= SL are dropped).  The sum for D = SL - 1 takes
-// SL digit pairs per K row, so K-chunks of flush_k<SL>() rows (192 for five
-// digits, 160 for six: at most 1024 / SL, a multiple of the 32-row stage)
-// stay exact, and every chunk is flushed into FP32 TwoSum pairs.  The result equals the FP64
-// product up to the dropped tail, about 2^-(8 SL - 1) of max|x_i.| max|y_j.|
-// per term (2^-47 with six digits).
+// which BF16 represents exactly.  The tensor cores compute sum_r d_s(x_ir)
+// d_t(y_jr) exactly, grouped by D = s + t (pairs with D >= ND are dropped, ND =
+// SL for five and six digits, 8 for seven), and the groups are added into FP32
+// expansions.  The result equals the FP64 product up to the truncation of the
+// operands, about 2^-(8 SL - 1) of max|x_i.| max|y_j.| per term (2^-47 with six
+// digits, 2^-55 with seven, the form that stands in for FP64 arithmetic).
 //
 // Kernel shape: C (FP64, M x N) (+)= X Y^T with X (M x K) and Y (N x K) both
 // K-contiguous digit slices, on the tcgen05 tensor cores (TMA-fed shared
@@ -35,8 +32,7 @@ namespace k {
 
 namespace {
 
-constexpr int kSlices = kOzakiSlices;  // the most digits an operand holds (scratch sizing)
-constexpr int TKs = 32;      // K padding of the digit slices (one pipeline stage)
+constexpr int kNoExp = -5000;  // exponent of a row or column of zeros
 
 inline unsigned cdiv(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
@@ -44,143 +40,231 @@ inline unsigned cdiv(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b);
 // arithmetic only (the FP64 pipe of this part is ~1/60 of the FP32 pipe).
 //
 // exponent e with |x| < 2^e for a nonzero x: biased exponent - 1022 (exact
-// for normal numbers, an upper bound for subnormals); -1074 marks zero
+// for normal numbers, an upper bound for subnormals); kNoExp for zero
 __device__ __forceinline__ int exp_bits(double a) {
-    const long long b = __double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFLL;
-    if (b == 0) return -1074;
-    return (int)(b >> 52) - 1022;
+    const unsigned long long b = (unsigned long long)__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFULL;
+    return b == 0 ? kNoExp : (int)(b >> 52) - 1022;
 }
 
-// per-row exponents of a row-major R x C FP64 block: one warp per row
-__global__ void k_row_exps(int R, int C, const double *__restrict__ X, int ldx, int *__restrict__ ex) {
+// per-row exponents of a row-major R x C FP64 block: one warp per row; with
+// cexp, of the block whose column c is scaled by 2^-cexp[c]
+__global__ void k_row_exps(int R, int C, const double *__restrict__ X, int ldx, const int *__restrict__ cexp,
+                           int *__restrict__ ex) {
     int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     int lane = threadIdx.x & 31;
     if (row >= R) return;
-    int m = -1074;
-    for (int j = lane; j < C; j += 32) m = max(m, exp_bits(X[(size_t)row * ldx + j]));
+    int m = kNoExp;
+#pragma unroll 4
+    for (int j = lane; j < C; j += 32) {
+        const int e = exp_bits(X[(size_t)row * ldx + j]);
+        m = max(m, cexp && e != kNoExp ? e - cexp[j] : e);
+    }
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) ex[row] = m;
 }
 
-// per-column exponents of a row-major R x C FP64 block (ex pre-set to -1074)
-__global__ void k_col_exps(int R, int C, const double *__restrict__ X, int ldx, int *__restrict__ ex) {
-    const int r0 = blockIdx.x * 256;
-    const int r1 = min(R, r0 + 256);
-    for (int j = blockIdx.y * blockDim.x + threadIdx.x; j < C; j += gridDim.y * blockDim.x) {
-        int m = -1074;
-        for (int r = r0; r < r1; ++r) m = max(m, exp_bits(X[(size_t)r * ldx + j]));
-        if (m != -1074) atomicMax(&ex[j], m);
-    }
-}
-
-// Digits of x against the group exponent e (|x| < 2^e): T = round(x 2^(B-e)),
-// B = 8 SL - 1, as an integer (|T| <= 2^B, ties to even), written in balanced
-// base 256,
-//     T = sum_s d_s 2^(8 (SL - 1 - s)),  d_1..d_{SL-1} in [-128, 127],  |d_0| <= 128,
-// so x = 2^(e-7) sum_s d_s 2^(-8 s) up to 2^(e-B-1).
-template <int SL>
-__device__ __forceinline__ void split_value(double x, int e, __nv_bfloat16 *out, size_t stride) {
-    const long long bits = __double_as_longlong(x);
-    int E = (int)((bits >> 52) & 0x7FF);
-    long long M = bits & 0xFFFFFFFFFFFFFLL;
-    if (E == 0) E = 1;
-    else M |= 1LL << 52;
-    const int sh = E - 1075 + (8 * SL - 1) - e;  // x 2^(B-e) = +-M 2^sh, sh <= B - 53 when |x| < 2^e
-    long long T = 0;
-    if (M != 0 && sh > -54) {
-        if (sh >= 0) {
-            T = M << min(sh, 10);
+// per-column exponents of a row-major R x C FP64 block (ex pre-set to kNoExp);
+// with rexp, of the block whose row r is scaled by 2^rexp[r].  A CTA takes 64
+// columns (two per thread, 32 threads) of `rows` rows (eight at a time).
+__global__ void __launch_bounds__(256) k_col_exps(int R, int C, const double *__restrict__ X, int ldx, int rows,
+                                                  const int *__restrict__ rexp, bool vec, int *__restrict__ ex) {
+    __shared__ int red[8][64];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int j = blockIdx.y * 64 + 2 * tx;
+    const int r1 = min(R, (int)(blockIdx.x + 1) * rows);
+    int m0 = kNoExp, m1 = kNoExp;
+#pragma unroll 4
+    for (int r = blockIdx.x * rows + ty; r < r1; r += 8) {
+        const double *p = X + (size_t)r * ldx + j;
+        double a = 0.0, b = 0.0;
+        if (vec && j + 1 < C) {
+            const double2 v = *reinterpret_cast<const double2 *>(p);
+            a = v.x, b = v.y;
         } else {
-            const int k = -sh;
-            long long q = M >> k;
-            const long long rem = M & ((1LL << k) - 1), half = 1LL << (k - 1);
-            if (rem > half || (rem == half && (q & 1))) ++q;
-            T = q;
+            if (j < C) a = p[0];
+            if (j + 1 < C) b = p[1];
         }
+        int ea = exp_bits(a), eb = exp_bits(b);
+        if (rexp) {
+            const int q = rexp[r];
+            if (ea != kNoExp) ea += q;
+            if (eb != kNoExp) eb += q;
+        }
+        m0 = max(m0, ea);
+        m1 = max(m1, eb);
     }
-    if (bits < 0) T = -T;
+    red[ty][2 * tx] = m0;
+    red[ty][2 * tx + 1] = m1;
+    __syncthreads();
+    if (threadIdx.x < 64 && blockIdx.y * 64 + threadIdx.x < C) {
+        int m = red[0][threadIdx.x];
 #pragma unroll
-    for (int s = SL - 1; s >= 1; --s) {
-        int d = (int)(T & 255);
-        if (d >= 128) d -= 256;
-        out[(size_t)s * stride] = __int2bfloat16_rn(d);
-        T = (T - d) >> 8;
+        for (int q = 1; q < 8; ++q) m = max(m, red[q][threadIdx.x]);
+        if (m != kNoExp) atomicMax(&ex[blockIdx.y * 64 + threadIdx.x], m);
     }
-    out[0] = __int2bfloat16_rn((int)T);
 }
 
-// Global layout of the digit slices ("tiled"): for K-chunk kc = k / 32,
-// slice s, row r (rows padded to rows_p, a multiple of 128) and k,
-//     offset = ((kc * SL + s) * rows_p + 8 (r / 8)) * 32 + 64 ((k % 32) / 8)
-//              + 8 (r % 8) + k % 8     (BF16 elements),
-// i.e. 8 x 8 core matrices (8 rows x 16 bytes) ordered [kc][s][r/8][k%32/8].
-// A 32-deep K step of any 128 (or 64) consecutive rows of one slice is then
-// one contiguous 8 KB (4 KB) block that a bulk copy moves straight into the
-// core-matrix order the tensor-core descriptors read.
+// T + offset of x against the group exponent e (|x| < 2^e): T = round(x
+// 2^(B-e)), B = 8 SL - 1, as an integer (|T| <= 2^B).  T in balanced base 256,
+//     T = sum_s d_s 2^(8 (SL - 1 - s)),  d_1..d_{SL-1} in [-128, 127],  |d_0| <= 128,
+// so x = 2^(e-7) sum_s d_s 2^(-8 s) up to 2^(e-B-1).  With 128 added at every
+// digit below the top one, digit s + 128 is byte SL - 1 - s and d_0 is what
+// stands above: no carry chain.
 template <int SL>
-__device__ __forceinline__ size_t tiled_off(int s, int r, int k, int rows_p) {
-    return (((size_t)(k >> 5) * SL + s) * (size_t)rows_p + (size_t)(r & ~7)) * 32 + (size_t)((k & 31) >> 3) * 64 +
-           (size_t)(r & 7) * 8 + (size_t)(k & 7);
+__device__ __forceinline__ long long split_int(double x, int e) {
+    const long long bits = __double_as_longlong(x);
+    const int E = (int)((bits >> 52) & 0x7FF);
+    const unsigned long long M = (bits & 0xFFFFFFFFFFFFFULL) | (E ? 1ULL << 52 : 0ULL);
+    // x 2^(B-e) = +-M 2^sh, sh <= B - 53 <= 2 when |x| < 2^e
+    const int sh = (E ? E : 1) - 1075 + (8 * SL - 1) - e;
+    const unsigned long long t = (M << 3) >> min(max(2 - sh, 0), 63);
+    const long long T = (long long)((t + 1) >> 1), neg = bits >> 63;
+    constexpr long long off = (long long)(0x8080808080808080ULL >> (8 * (9 - SL)));
+    return (T ^ neg) - neg + off;
 }
 
-// digits of the 8 values v[0..7] (consecutive k of one row, exponent e) as
-// one 16-byte vector per slice
+// digits of the 8 values v[0..7] (consecutive k of one row, exponents e[.]) as
+// one 16-byte vector per slice; out: the row's place in slice 0, slice_step:
+// elements between slices.  Bytes become floats by placing them in the low
+// mantissa of 2^23; a BF16 is the upper half of such an exact small float.
 template <int SL>
-__device__ __forceinline__ void split8_store(const double (&v)[8], int e, __nv_bfloat16 *out, size_t off,
-                                             int rows_p) {
-    __nv_bfloat16 d[SL][8];
+__device__ __forceinline__ void split8_store(const double (&v)[8], const int (&e)[8], __nv_bfloat16 *out,
+                                             size_t slice_step) {
+    unsigned lo[8], hi[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-        __nv_bfloat16 one[SL];
-        split_value<SL>(v[t], e, one, 1);
-#pragma unroll
-        for (int sl = 0; sl < SL; ++sl) d[sl][t] = one[sl];
+        const long long T = split_int<SL>(v[t], e[t]);
+        lo[t] = (unsigned)T;
+        hi[t] = (unsigned)((unsigned long long)T >> 32);
     }
-    const size_t slice_step = (size_t)rows_p * 32;  // next slice within the same K-chunk
 #pragma unroll
-    for (int sl = 0; sl < SL; ++sl)
-        *reinterpret_cast<uint4 *>(out + off + sl * slice_step) = *reinterpret_cast<const uint4 *>(d[sl]);
+    for (int s = 0; s < SL; ++s) {
+        unsigned w[4];
+#pragma unroll
+        for (int t = 0; t < 8; t += 2) {
+            unsigned f[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int byte = SL - 1 - s;
+                float x;
+                if (s == 0)
+                    x = __int_as_float(0x4B400000 + ((int)hi[t + u] >> (8 * (SL - 5)))) - 12582912.f;
+                else
+                    x = __uint_as_float(__byte_perm(byte < 4 ? lo[t + u] : hi[t + u], 0x4B000000u, 0x7440u | (byte & 3))) -
+                        8388736.f;
+                f[u] = __float_as_uint(x);
+            }
+            w[t / 2] = __byte_perm(f[0], f[1], 0x7632);
+        }
+        *reinterpret_cast<uint4 *>(out + s * slice_step) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+// Global layout of the digit slices: for K step kc = k / 16, row block b = r /
+// RB (RB = 128 rows for the first operand of a product, 64 for the second) and
+// slice s, the 8 x 8 core matrices (8 rows x 16 bytes) of the RB x 16 block in
+// the order [r % RB / 8][k % 16 / 8], blocks ordered [kc][b][s]: all slices of
+// one product tile and K step are one contiguous piece.
+template <int SL>
+__device__ __forceinline__ size_t tiled_off(int r, int k, int nb, int rb_log) {
+    const int b = r >> rb_log, rr = r & ((1 << rb_log) - 1);
+    return ((((size_t)(k >> 4) * nb + b) * SL) << (rb_log + 4)) + (size_t)(rr >> 3) * 128 + (size_t)((k >> 3) & 1) * 64 +
+           (size_t)(rr & 7) * 8;
 }
 
 // split a row-major R x K block per row (K = columns): one thread per row and
-// 8-wide K group; a warp covers one 8-row group x one 32-deep K-chunk
+// 8-wide K group; a warp covers one 8-row group x 32 columns.  cexp: column k
+// of the block is scaled by 2^-cexp[k] before the split.
 template <int SL>
-__global__ void k_split_rows_tiled(int R, int K, const double *__restrict__ X, int ldx, const int *__restrict__ ex,
-                                   __nv_bfloat16 *__restrict__ out, int rows_p, int kp) {
+__global__ void __launch_bounds__(256) k_split_rows(int R, int K, const double *__restrict__ X, int ldx, bool vec,
+                                                    const int *__restrict__ ex, const int *__restrict__ cexp,
+                                                    __nv_bfloat16 *__restrict__ out, int rows_p, int kp, int rb_log) {
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    const int KC = kp / 32;
+    const int KC = (kp + 31) / 32;
     if (gw >= (int64_t)(rows_p / 8) * KC) return;
     const int rg = (int)(gw / KC), kc = (int)(gw % KC);
     const int r = rg * 8 + (lane & 7), k0 = kc * 32 + (lane >> 3) * 8;
+    if (k0 >= kp) return;
     double v[8];
+    int e[8];
+    const double *x = X + (size_t)r * ldx + k0;
+    if (vec && r < R && k0 + 8 <= K) {
 #pragma unroll
-    for (int t = 0; t < 8; ++t) v[t] = (r < R && k0 + t < K) ? X[(size_t)r * ldx + k0 + t] : 0.0;
-    split8_store<SL>(v, r < R ? ex[r] : -1074, out, tiled_off<SL>(0, r, k0, rows_p), rows_p);
+        for (int t = 0; t < 8; t += 2) {
+            const double2 q = *reinterpret_cast<const double2 *>(x + t);
+            v[t] = q.x, v[t + 1] = q.y;
+        }
+    } else {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v[t] = (r < R && k0 + t < K) ? x[t] : 0.0;
+    }
+    const int er = r < R ? ex[r] : kNoExp;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) e[t] = er + (cexp && k0 + t < K ? cexp[k0 + t] : 0);
+    split8_store<SL>(v, e, out + tiled_off<SL>(r, k0, rows_p >> rb_log, rb_log), (size_t)16 << rb_log);
 }
 
-// split a row-major K x C block per column (operand row r = column r, K =
-// rows of X), transposed through shared memory: a block handles 32 columns x
-// a 32-deep K-chunk
+// split a row-major K x C block per column (operand row r = column r, K = rows
+// of X), transposed through shared memory: a block handles 64 columns x 32 K
+// rows.  rexp: row k of the block is scaled by 2^rexp[k].  sumsq (seven-digit
+// Grams): sum over k of (128 x / 2^e)^2 per column, from the leading digits.
 template <int SL>
-__global__ void k_split_cols_tiled(int K, int C, const double *__restrict__ X, int ldx, const int *__restrict__ ex,
-                                   __nv_bfloat16 *__restrict__ out, int rows_p) {
-    __shared__ double tile[32][33];
-    const int kc = blockIdx.x, c0 = blockIdx.y * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 4 threads
-    for (int yy = ty; yy < 32; yy += 4) {
-        const int k = kc * 32 + yy, c = c0 + tx;
-        tile[yy][tx] = (k < K && c < C) ? X[(size_t)k * ldx + c] : 0.0;
+__global__ void __launch_bounds__(256) k_split_cols(int K, int C, const double *__restrict__ X, int ldx, bool vec,
+                                                    const int *__restrict__ ex, const int *__restrict__ rexp,
+                                                    __nv_bfloat16 *__restrict__ out, int rows_p, int kp, int rb_log,
+                                                    float *__restrict__ sumsq) {
+    __shared__ double tile[32][65];
+    const int k0 = blockIdx.x * 32, c0 = blockIdx.y * 64;
+    {
+        const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+        const int c = c0 + 2 * tx;
+#pragma unroll
+        for (int yy = ty; yy < 32; yy += 8) {
+            const double *p = X + (size_t)(k0 + yy) * ldx + c;
+            double a = 0.0, b = 0.0;
+            if (k0 + yy < K) {
+                if (vec && c + 1 < C) {
+                    const double2 q = *reinterpret_cast<const double2 *>(p);
+                    a = q.x, b = q.y;
+                } else {
+                    if (c < C) a = p[0];
+                    if (c + 1 < C) b = p[1];
+                }
+            }
+            tile[yy][2 * tx] = a;
+            tile[yy][2 * tx + 1] = b;
+        }
     }
     __syncthreads();
-    // thread -> (column c0 + lc, K group kg): 32 columns x 4 groups = 128 threads
-    const int lc = (threadIdx.x & 7) + 8 * (threadIdx.x >> 5), kg = (threadIdx.x >> 3) & 3;
-    const int r = c0 + lc;
-    if (r >= rows_p) return;
+    // thread -> (column c0 + lc, K group kg): a warp covers 8 columns x 4 groups
+    const int lane = threadIdx.x & 31;
+    const int lc = (lane & 7) + 8 * (threadIdx.x >> 5), kg = lane >> 3;
+    const int r = c0 + lc, k = k0 + 8 * kg;
     double v[8];
+    int e[8];
+    const int er = r < C ? ex[r] : kNoExp;
 #pragma unroll
-    for (int t = 0; t < 8; ++t) v[t] = tile[kg * 8 + t][lc];
-    split8_store<SL>(v, r < C ? ex[r] : -1074, out, tiled_off<SL>(0, r, kc * 32 + kg * 8, rows_p), rows_p);
+    for (int t = 0; t < 8; ++t) {
+        v[t] = tile[kg * 8 + t][lc];
+        e[t] = er - (rexp && k + t < K ? rexp[k + t] : 0);
+    }
+    if (r < rows_p && k < kp)
+        split8_store<SL>(v, e, out + tiled_off<SL>(r, k, rows_p >> rb_log, rb_log), (size_t)16 << rb_log);
+    if (sumsq) {
+        float s = 0.f;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            // x 2^(7-e) from the upper word (zeros and tiny values: nothing to add)
+            const unsigned hw = (unsigned)((unsigned long long)__double_as_longlong(v[t]) >> 32) & 0x7FFFFFFFu;
+            const int q = (int)(hw >> 20) - 1023 + 7 - er;
+            const float f = q > -60 && q < 60 ? __int_as_float(((q + 127) << 23) | (int)((hw & 0xFFFFFu) << 3)) : 0.f;
+            s = fmaf(f, f, s);
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 8);
+        s += __shfl_xor_sync(0xffffffffu, s, 16);
+        if (kg == 0 && r < C && s > 0.f) atomicAdd(&sumsq[r], s);
+    }
 }
 
 __global__ void k_fill_int(int n, int v, int *__restrict__ x) {
@@ -192,17 +276,6 @@ __device__ __forceinline__ unsigned smem_addr(const void *p) {
     return (unsigned)__cvta_generic_to_shared(p);
 }
 
-// Error-free accumulation of x into (hi, lo): hi + lo gains x exactly up to
-// the rounding of lo (Knuth's TwoSum in FP32; the FP32 pipe is ~60x the FP64
-// pipe on this part).
-__device__ __forceinline__ void two_sum_acc(float &hi, float &lo, float x) {
-    float s = __fadd_rn(hi, x);
-    float bp = __fsub_rn(s, hi);
-    float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(x, bp));
-    hi = s;
-    lo = __fadd_rn(lo, err);
-}
-
 // SMs of the current device (queried per call: a process may drive GPUs of
 // different sizes; the attribute query costs about a microsecond)
 int sm_count_oz() {
@@ -212,51 +285,81 @@ int sm_count_oz() {
     return c > 0 ? c : 1;
 }
 
-// tcgen05 form of the same product (5th-generation tensor cores, TMEM).
+// ---- the product kernel (tcgen05, TMEM) --------------------------------------
 //
-// CTA tile: 128 rows of X by 64 rows of Y, K staged 32 at a time into three
-// shared-memory stages by bulk copies (TMA, cp.async.bulk): the tiled global
-// layout makes each slice of a stage one contiguous block, so a stage is 6
-// copies of 8 KB (X) and 6 of 4 KB (Y), landing in core-matrix order
-// [s][r/8][k/8][8 x 16 bytes]: an MMA operand descriptor with LBO = 128 bytes
-// between K-groups and SBO = 512 bytes between 8-row groups.  Because the Y
-// slices of one stage follow each other at the row-group stride, Y_0 .. Y_5
-// form one N = 384 operand: one MMA multiplies X_s by [Y_0 .. Y_{5-s}] (N = 64 (6 - s),
-// split at 256) and its 64-column blocks land exactly on the accumulators
-// acc_{s} .. acc_{5} of the digit sums D = s + t, which sit side by side in
-// TMEM (columns 64 D .. 64 D + 63, 384 of the 512 allocated).  Per 16-deep
-// K step that is 8 MMAs instead of 21.
+// Work item: a 128 x 64 tile of C over a range of K; a persistent CTA per SM
+// takes the items blockIdx.x, blockIdx.x + gridDim.x, ...  K is staged 16 deep
+// through a ring of shared-memory stages by bulk copies (TMA, cp.async.bulk):
+// the operand layout keeps all digit slices of one tile and K step contiguous,
+// so a stage is two copies, landing in core-matrix order [s][r/8][k/8][8 x 16
+// bytes] (LBO = 128 bytes between K groups, SBO = 256 bytes between 8-row
+// groups).  Because the Y slices of a stage follow each other at the row-group
+// stride, [Y_0 .. Y_{w-1}] is one N = 64 w operand: one MMA (two above N = 256)
+// multiplies X_s by [Y_0 .. Y_{w-1}], w = min(SL, ND - s), and its 64-column
+// blocks land on the accumulators acc_s .. acc_{s+w-1} of the digit sums D = s +
+// t, which sit side by side in TMEM (ND x 64 columns).
 //
-// Warp roles (320 threads): warp 0 issues the TMA loads, warp 1 owns the
-// TMEM allocation and issues the MMAs (one thread), warps 2..9 drain TMEM:
-// after every exact-FP32 chunk of flush_k<SL>() K rows they read acc_0..acc_5 and
-// add 2^-8D acc_D into FP32 (hi, lo) TwoSum pairs held in registers, one
-// TMEM lane (output row) and 32 of the 64 columns per thread.  Every wait on an mbarrier gives up
-// after a bounded number of polls, records an error flag the host checks,
-// and the CTA still drains its own copies and MMAs and frees its TMEM.
-// ---------------------------------------------------------------------------
-constexpr int TC_M = 128, TC_N = 64, TC_K = 32, TC_STAGES = 3;
-constexpr int TC_THREADS = 320, TC_DRAIN = 256;  // 10 warps, 8 of them drain TMEM
-constexpr int TC_KG = TC_K / 8;
-// K rows per exact FP32 chunk: SL digit pairs per row for the sum D = SL - 1,
-// each at most 2^14, so chunk x SL <= 1024 keeps the FP32 sums exact
-template <int SL> __host__ __device__ constexpr int flush_k() { return (1024 / SL) / TC_K * TC_K; }
-static_assert(flush_k<5>() == 192 && flush_k<6>() == 160, "exact chunk lengths");
-// stage sizes for SL digit slices: X 128 rows, Y 64 rows (SL = 6: 49,152 + 24,576 bytes)
-template <int SL> __host__ __device__ constexpr uint32_t tc_a_bytes() { return 16u * TC_M * SL * TC_KG; }
-template <int SL> __host__ __device__ constexpr uint32_t tc_b_bytes() { return 16u * TC_N * SL * TC_KG; }
+// Exactness: a digit product is at most 2^14 in magnitude, and the sum for D
+// takes D + 1 pairs per K row, so after kChunk = 256 rows the sums for D <= 3
+// are below 2^24 and exact in FP32.  The sums for D >= 4 carry a weight of
+// 2^-32 and less; they pass 2^24 only when hundreds of same-signed full-size
+// digits meet, and then lose one unit of 2^-32 per chunk next to a D = 0 sum of
+// 2^22.  Every chunk is drained into FP32 expansions in registers.
+//
+// The drain stops the tensor cores briefly: the accumulators of the highest D
+// (three of five digits' sums, two of six digits') have two sets of TMEM
+// columns that alternate from chunk to chunk, and the first step of a chunk is
+// issued in descending slices: those that touch only the alternating
+// accumulators at once, the others as the drain releases theirs (seven digits
+// fill TMEM with one set).  An accumulator's first MMA of a chunk overwrites it
+// (its own N = 64 instruction).  Starting more steps of a chunk this way was
+// slower (2.70 ms with three, 2.54 with one, 250,000 x 750 x 750, five digits):
+// the stages that it holds come back late.
+//
+// What bounds it: a Gram of 250,000 x 750 x 750 takes 2.5 / 3.7 / 5.7 ms with
+// five, six and seven digits; the MMAs alone (no loads, no drain) take 2.08 /
+// 2.88 / 4.48, with the loads 2.29 / 3.18 / 4.82, the rest is the drain.  One CTA
+// per tile, K staged 32 deep in twelve copies, one set of accumulators and MMAs
+// issued by a lone lane: 3.53 ms with five digits; the update of the same sizes
+// (six digits, 23,448 tiles 47 steps deep) 6.43 ms, now 4.0.
+//
+// Warp roles (320 threads): warp 0 issues the loads, warp 1 owns TMEM and
+// issues the MMAs (one thread), warps 2..9 drain, one TMEM lane (output row)
+// and 32 of the 64 columns per thread, and write the item's results while the
+// MMAs of the next item run.  Every mbarrier wait gives up after 2 s, records
+// an error flag that the host checks, and the CTA still drains its own copies
+// and MMAs and frees its TMEM.
+// ------------------------------------------------------------------------------
+constexpr int TC_M = 128, TC_N = 64, TC_K = 16;
+constexpr int TC_THREADS = 320, TC_DRAIN_WARPS = 8;
+constexpr int kChunk = 256;                 // K rows per drained chunk
+constexpr int kChunkSteps = kChunk / TC_K;  // 16
+// K rows of one work item at most: the low word of the FP32 expansions takes
+// one rounding per chunk, 64 of them stay below the digits' own truncation;
+// longer products add their items in FP64
+constexpr int kItemK = 16384;
+// digit sums kept: pairs with s + t >= ND are dropped
+template <int SL> __host__ __device__ constexpr int tc_nd() { return SL == 7 ? 8 : SL; }
+template <int SL> __host__ __device__ constexpr uint32_t tc_a_bytes() { return 2u * TC_M * TC_K * SL; }
+template <int SL> __host__ __device__ constexpr uint32_t tc_b_bytes() { return 2u * TC_N * TC_K * SL; }
 template <int SL> __host__ __device__ constexpr uint32_t tc_stage_bytes() { return tc_a_bytes<SL>() + tc_b_bytes<SL>(); }
-template <int SL> constexpr size_t tc_smem() { return (size_t)TC_STAGES * tc_stage_bytes<SL>() + 1024; }
+// stages that fit 220 KB: 7, 6, 5 for 5, 6, 7 digits
+template <int SL> __host__ __device__ constexpr int tc_stages() { return (int)(220u * 1024u / tc_stage_bytes<SL>()); }
+// accumulators with one set of columns; the ND - tc_low above them have two
+template <int SL> __host__ __device__ constexpr int tc_low() { return SL == 5 ? 2 : SL == 6 ? 4 : 8; }
+template <int SL> constexpr size_t tc_smem() { return (size_t)tc_stages<SL>() * tc_stage_bytes<SL>() + 1024; }
 constexpr uint32_t TC_TMEM_COLS = 512;
 constexpr uint64_t TC_WAIT_NS = 2000000000ull;  // 2 s per barrier wait
 
 __device__ int g_oz_error;
 
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-    // shared-memory matrix descriptor: start >> 4 (bits 0-13), LBO >> 4 (16-29),
-    // SBO >> 4 (32-45), descriptor version 1 (bits 46-47), no swizzle (61-63 = 0)
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
+// shared-memory matrix descriptor, low word: start >> 4 (bits 0-13), LBO >> 4
+// (16-29); high word: SBO >> 4 (32-45), descriptor version 1 (46-47), no
+// swizzle (61-63 = 0).  Addresses stay below 2^18, so offsets are added to the
+// low word as they are.
+__device__ __forceinline__ uint32_t umma_desc_lo(uint32_t saddr, uint32_t lbo) { return (saddr >> 4) | ((lbo >> 4) << 16); }
+__device__ __forceinline__ uint64_t umma_desc(uint32_t lo, uint32_t sbo) {
+    return ((uint64_t)((sbo >> 4) | (1u << 14)) << 32) | lo;
 }
 
 // instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
@@ -307,55 +410,173 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
                  : "memory");
 }
 
-__device__ __forceinline__ void umma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, int acc) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-            dtmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc));
+// one lane of a converged warp
+__device__ __forceinline__ uint32_t elect_lane() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n selp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+    return p;
 }
 
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
-                 : "memory");
+// Issued by the elected lane of a converged warp: operands that are the same
+// in the whole warp stay in uniform registers, which the instruction takes (48
+// clocks per small MMA; 118 when one lane runs the loop alone and every operand
+// is moved over, more than a 128 x 64 x 16 product's 32)
+__device__ __forceinline__ void umma_f16(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, int acc,
+                                         uint32_t el) {
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 q, %5, 0;\n"
+        " @q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc), "r"(el));
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+__device__ __forceinline__ void umma_commit(uint32_t bar, uint32_t el) {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%"
-        "19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+        "{\n .reg .pred q;\n setp.ne.b32 q, %1, 0;\n"
+        " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar),
+        "r"(el)
+        : "memory");
+}
+
+// n consecutive 32-bit TMEM columns of the warp's 32 lanes (one lane per
+// thread); the registers may be read after tmem_wait on them (which waits for
+// every load issued before it)
+template <int n> __device__ __forceinline__ void tmem_ld(uint32_t taddr, uint32_t (&r)[n]);
+template <int n> __device__ __forceinline__ void tmem_wait(uint32_t (&r)[n]);
+template <>
+__device__ __forceinline__ void tmem_ld<32>(uint32_t taddr, uint32_t (&r)[32]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(taddr));
+}
+template <>
+__device__ __forceinline__ void tmem_wait<32>(uint32_t (&r)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])::"memory");
+}
+template <>
+__device__ __forceinline__ void tmem_ld<8>(uint32_t taddr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+template <>
+__device__ __forceinline__ void tmem_wait<8>(uint32_t (&r)[8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])::"memory");
+}
+
+// s = fl(a + b), returns the rounding error a + b - s exactly (Knuth)
+__device__ __forceinline__ float two_sum(float a, float b, float &s) {
+    s = __fadd_rn(a, b);
+    const float bp = __fsub_rn(s, a);
+    return __fadd_rn(__fsub_rn(a, __fsub_rn(s, bp)), __fsub_rn(b, bp));
+}
+
+// One chunk's digit sums of a value added into its expansion.  In units of the
+// D = 0 sum the chunk is r0 + 2^-8 r1 + 2^-16 r2 + 2^-24 v, r0..r2 integers
+// below 2^24.  s = fl(r0 + 2^-8 r1) with the exact remainder, to which 2^-16 r2
+// adds exactly (multiples of 2^-16 below 2^8): error-free terms for hi; the
+// errors go to lo.  v, the digits from D = 3 on, goes to lo too with five
+// digits; with six, whose dropped pairs weigh 2^-48, its rounding and lo's would
+// be felt (0.1 of the error at K = 750): it comes with its own error ev and is
+// the third term for hi.
+template <int SL>
+__device__ __forceinline__ void add_chunk(float r0, float r1, float r2, float v, float ev, float &hi, float &lo) {
+    const float s = __fmaf_rn(r1, 0x1p-8f, r0);
+    const float e = __fmaf_rn(r1, 0x1p-8f, __fsub_rn(r0, s));
+    const float t = __fmaf_rn(r2, 0x1p-16f, e);
+    float h;
+    const float e1 = two_sum(hi, s, h);
+    if constexpr (SL == 5) {
+        const float e2 = two_sum(h, t, hi);
+        lo = __fmaf_rn(v, 0x1p-24f, __fadd_rn(lo, __fadd_rn(e1, e2)));
+    } else {
+        float h2;
+        const float e2 = two_sum(h, t, h2);
+        const float e3 = two_sum(h2, __fmul_rn(v, 0x1p-24f), hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(e1, e2), __fmaf_rn(ev, 0x1p-24f, e3)));
+    }
+}
+
+// the same for seven digits, into three words: 2^-24 (s3 + f3) replaces v
+__device__ __forceinline__ void add_chunk3(float r0, float r1, float r2, float s3, float f3, float &hi, float &mid,
+                                           float &lo) {
+    const float s = __fmaf_rn(r1, 0x1p-8f, r0);
+    const float e = __fmaf_rn(r1, 0x1p-8f, __fsub_rn(r0, s));
+    const float t = __fmaf_rn(r2, 0x1p-16f, e);
+    float p, h, m;
+    const float pe = two_sum(t, __fmul_rn(s3, 0x1p-24f), p);
+    const float e1 = two_sum(hi, s, h);
+    hi = h;
+    const float e2 = two_sum(mid, e1, m);
+    const float e3 = two_sum(m, p, mid);
+    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(e2, e3), __fmaf_rn(f3, 0x1p-24f, pe)));
+}
+
+// exact FP32 -> FP64 of zero and normal numbers (the digit sums are multiples of
+// 2^-48: no subnormals)
+__device__ __forceinline__ double f2d_normal(float x) {
+    const unsigned u = __float_as_uint(x);
+    const unsigned h = (u & 0x80000000u) | (((u >> 3) & 0x0FFFFFFFu) + 0x38000000u);
+    return __hiloint2double((int)(x == 0.f ? 0u : h), (int)(x == 0.f ? 0u : u << 29));
+}
+
+// Work items of one product (host-built, passed by value)
+struct TcWork {
+    int ntn, tiles, items;  // column tiles, output tiles, tiles x K ranges
+    int ksteps, split;      // K steps of the product, K steps per item
+    int lower;              // tiles meeting the lower triangle only
+};
+struct TcItem {
+    int i0, j0, kc0, nk;
+};
+__device__ __forceinline__ TcItem tc_item(const TcWork &w, int item) {
+    const int sp = item / w.tiles, tile = item - sp * w.tiles;
+    int ti, tj;
+    if (w.lower) {  // row tile ti meets the column tiles 0 .. 2 ti + 1 (at most ntn)
+        ti = 0;
+        int left = tile;
+        for (int c = min(2, w.ntn); left >= c; c = min(2 * ti + 2, w.ntn)) {
+            left -= c;
+            ++ti;
+        }
+        tj = left;
+    } else {
+        ti = tile / w.ntn;
+        tj = tile - ti * w.ntn;
+    }
+    TcItem it;
+    it.i0 = ti * TC_M;
+    it.j0 = tj * TC_N;
+    it.kc0 = sp * w.split;
+    it.nk = min(w.split, w.ksteps - it.kc0);
+    return it;
 }
 
 template <int SL>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-    k_ozaki_tc(int M, int N, const __nv_bfloat16 *__restrict__ Xs, int rows_px, const __nv_bfloat16 *__restrict__ Ys,
-               int rows_py, const int *__restrict__ ex, const int *__restrict__ ey, double *__restrict__ C, int ldc,
-               int k_len, int k_split, int atomic, int lower) {
+    k_ozaki_tc(int M, int N, const __nv_bfloat16 *__restrict__ Xs, int nbx, const __nv_bfloat16 *__restrict__ Ys,
+               int nby, const int *__restrict__ ex, const int *__restrict__ ey, double *__restrict__ C, int ldc,
+               TcWork w, int atomic, int vec, const int *__restrict__ skip) {
+    constexpr int ND = tc_nd<SL>(), STAGES = tc_stages<SL>(), LOW = tc_low<SL>();
+    constexpr uint32_t A_BYTES = tc_a_bytes<SL>(), B_BYTES = tc_b_bytes<SL>(), STAGE = tc_stage_bytes<SL>();
+    constexpr uint32_t LBO = 128, SBO = 256, SLICE_A = A_BYTES / SL, SLICE_B = B_BYTES / SL;
     extern __shared__ unsigned char smem_dyn[];
-    __shared__ __align__(8) uint64_t full_bar[TC_STAGES], empty_bar[TC_STAGES], accf_bar, acce_bar, drain_bar;
+    // accf: a chunk is complete; free_bar: its low accumulators are drained (two
+    // groups with six digits); high_bar: all of it is
+    __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], accf_bar, free_bar[2], high_bar, drain_bar;
     __shared__ uint32_t tmem_slot;
-    const int i0 = blockIdx.y * TC_M, j0 = blockIdx.x * TC_N;
-    if (lower && j0 > i0 + TC_M - 1) return;
-    const int k_beg = blockIdx.z * k_split;
-    const int k_end = min(k_len, k_beg + k_split);
-    const int nk = k_end > k_beg ? (k_end - k_beg) / TC_K : 0;
-    constexpr int kFlush = flush_k<SL>();
-    const int nchunks = (nk + (kFlush / TC_K) - 1) / (kFlush / TC_K);
+    if (skip && *skip) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // stages on a 1024-byte boundary
     const uint32_t smem0 = (smem_addr(smem_dyn) + 1023u) & ~1023u;
     if (threadIdx.x == 0) {
-        for (int st = 0; st < TC_STAGES; ++st) {
+        for (int st = 0; st < STAGES; ++st) {
             mbar_init(smem_addr(&full_bar[st]), 1);
             mbar_init(smem_addr(&empty_bar[st]), 1);
         }
         mbar_init(smem_addr(&accf_bar), 1);
-        mbar_init(smem_addr(&acce_bar), TC_DRAIN);
+        mbar_init(smem_addr(&free_bar[0]), TC_DRAIN_WARPS);
+        mbar_init(smem_addr(&free_bar[1]), TC_DRAIN_WARPS);
+        mbar_init(smem_addr(&high_bar), TC_DRAIN_WARPS);
         mbar_init(smem_addr(&drain_bar), 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -370,106 +591,295 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const uint32_t tmem = tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0 && nk > 0) {
-            // producer: stage kt % 3 is refilled once the MMAs of kt - 3 completed
+        if (lane == 0) {
+            // producer: a stage is refilled once the MMAs of its previous step completed
             bool ok = true;
-            int issued = 0;
-            for (int kt = 0; kt < nk && ok; ++kt) {
-                const int st = kt % TC_STAGES;
-                if (kt >= TC_STAGES) ok = mbar_wait(smem_addr(&empty_bar[st]), ((kt / TC_STAGES) & 1) ^ 1);
-                if (!ok) break;
-                const uint32_t fb = smem_addr(&full_bar[st]);
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb), "r"(tc_stage_bytes<SL>())
-                             : "memory");
-                const uint32_t a_dst = smem0 + st * tc_stage_bytes<SL>();
-                const size_t kc = (size_t)(k_beg + kt * TC_K) / TC_K;
-#pragma unroll 1
-                for (int sl = 0; sl < SL; ++sl) {
-                    bulk_load(a_dst + sl * (tc_a_bytes<SL>() / SL),
-                              Xs + ((kc * SL + sl) * rows_px + i0) * TC_K, tc_a_bytes<SL>() / SL, fb);
-                    bulk_load(a_dst + tc_a_bytes<SL>() + sl * (tc_b_bytes<SL>() / SL),
-                              Ys + ((kc * SL + sl) * rows_py + j0) * TC_K, tc_b_bytes<SL>() / SL, fb);
+            int g = 0;  // K steps issued by this CTA so far
+            for (int item = blockIdx.x; item < w.items && ok; item += gridDim.x) {
+                const TcItem it = tc_item(w, item);
+                const __nv_bfloat16 *xa = Xs + ((size_t)it.kc0 * nbx + it.i0 / TC_M) * (A_BYTES / 2);
+                const __nv_bfloat16 *yb = Ys + ((size_t)it.kc0 * nby + it.j0 / TC_N) * (B_BYTES / 2);
+                for (int kt = 0; kt < it.nk; ++kt, ++g) {
+                    const int st = g % STAGES;
+                    if (g >= STAGES) ok = mbar_wait(smem_addr(&empty_bar[st]), ((g / STAGES) & 1) ^ 1);
+                    if (!ok) break;
+                    const uint32_t fb = smem_addr(&full_bar[st]), dst = smem0 + st * STAGE;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb), "r"(STAGE)
+                                 : "memory");
+                    bulk_load(dst, xa + (size_t)kt * nbx * (A_BYTES / 2), A_BYTES, fb);
+                    bulk_load(dst + A_BYTES, yb + (size_t)kt * nby * (B_BYTES / 2), B_BYTES, fb);
                 }
-                issued = kt + 1;
             }
-            // drain: the last loads of every stage have landed before the CTA exits
-            for (int kt = max(0, issued - TC_STAGES); kt < issued; ++kt)
-                mbar_wait(smem_addr(&full_bar[kt % TC_STAGES]), (kt / TC_STAGES) & 1);
+            // the last loads of every stage have landed before the CTA exits
+            for (int q = max(0, g - STAGES); q < g; ++q) mbar_wait(smem_addr(&full_bar[q % STAGES]), (q / STAGES) & 1);
         }
     } else if (warp == 1) {
-        if (lane == 0 && nk > 0) {
-            bool ok = true;
-            // core matrices: 128 bytes apart along K, 512 bytes apart along rows
-            constexpr uint32_t LBO = 128, SBO = 512;
-            for (int kt = 0; kt < nk && ok; ++kt) {
-                const int st = kt % TC_STAGES;
-                const int chunk = kt / (kFlush / TC_K);
-                const bool chunk_first = kt % (kFlush / TC_K) == 0;
-                ok = mbar_wait(smem_addr(&full_bar[st]), (kt / TC_STAGES) & 1);
-                if (ok && chunk_first && chunk > 0) ok = mbar_wait(smem_addr(&acce_bar), (chunk - 1) & 1);
-                if (!ok) break;
-                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const uint32_t a_base = smem0 + st * tc_stage_bytes<SL>(), b_base = a_base + tc_a_bytes<SL>();
+        // the whole warp runs the loop, the elected lane issues
+        const uint32_t el = elect_lane();
+        const uint32_t d0 = umma_desc_lo(smem0, LBO), full0 = smem_addr(full_bar), empty0 = smem_addr(empty_bar);
+        // the digit sums D in [da, db] of slice sl: X_sl by [Y_{da-sl} .. Y_{db-sl}] of the
+        // stage at descriptor word dw onto acc_da .. acc_db (all below LOW or
+        // all from LOW on; hi: first column of the alternating set, less 64 LOW)
+        auto part = [&](uint32_t dw, uint32_t hi, int sl, int da, int db, int acc) {
+            const uint64_t ad = umma_desc(dw + ((sl * SLICE_A) >> 4), SBO);
+            const uint32_t b = dw + ((A_BYTES + (da - sl) * SLICE_B) >> 4), d = (da < LOW ? tmem : hi) + TC_N * da;
+            const int n = TC_N * (db - da + 1), n1 = n > 256 ? n / 2 : n;
+            umma_f16(d, ad, umma_desc(b, SBO), umma_idesc(TC_M, n1), acc, el);
+            if (n > 256)
+                umma_f16(d + n1, ad, umma_desc(b + (((uint32_t)(n1 / 8) * SBO) >> 4), SBO), umma_idesc(TC_M, n1), acc, el);
+        };
+        // all digit sums of slice sl from da on
+        auto slice = [&](uint32_t dw, uint32_t hi, int sl, int da) {
+            const int db = (sl + SL - 1 < ND - 1 ? sl + SL - 1 : ND - 1);
+            if (da > db) return;
+            if (da < LOW && db >= LOW) {
+                part(dw, hi, sl, da, LOW - 1, 1);
+                part(dw, hi, sl, LOW, db, 1);
+            } else {
+                part(dw, hi, sl, da, db, 1);
+            }
+        };
+        bool ok = true;
+        uint32_t st = 0, ph = 0, c = 0;  // stage and its parity, chunks started by this CTA
+        for (int item = blockIdx.x; item < w.items && ok; item += gridDim.x) {
+            const int nk = tc_item(w, item).nk;
+            for (int k0 = 0; k0 < nk && ok; k0 += kChunkSteps, ++c) {
+                const int steps = min(kChunkSteps, nk - k0);
+                const uint32_t ap = (c - 1) & 1;  // parity of the chunk before
+                const uint32_t hi = tmem + (c & 1) * TC_N * (ND - LOW);
+                // first step of the chunk: every accumulator is overwritten once
+                ok = mbar_wait(full0 + 8 * st, ph);
+                const uint32_t dw = d0 + st * (STAGE >> 4);
+                if constexpr (SL == 7) {
+                    if (c > 0) ok = ok && mbar_wait(smem_addr(&free_bar[0]), ap);
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                    part(dw, hi, 0, 0, 6, 0);  // acc_0 .. acc_6 start
+                    part(dw, hi, 1, 7, 7, 0);  // acc_7 starts
+                    part(dw, hi, 1, 1, 6, 1);
 #pragma unroll
-                for (int k16 = 0; k16 < TC_K / 16; ++k16) {
-                    const uint32_t a_k = a_base + 2 * k16 * LBO, b_k = b_base + 2 * k16 * LBO;
+                    for (int sl = 2; sl < 7; ++sl) slice(dw, hi, sl, sl);
+                } else {
 #pragma unroll
-                    for (int sl = 0; sl < SL; ++sl) {
-                        const uint64_t ad = umma_desc(a_k + sl * (tc_a_bytes<SL>() / SL), LBO, SBO);
-                        const int acc = (chunk_first && k16 == 0 && sl == 0) ? 0 : 1;
-                        const int ncols = TC_N * (SL - sl);  // Y_0 .. Y_{SL-1-s}
-                        const int n1 = ncols > 256 ? 256 : ncols;
-                        umma_f16(tmem + TC_N * sl, ad, umma_desc(b_k, LBO, SBO), umma_idesc(TC_M, n1), acc);
-                        if (ncols > 256)  // rows 256.. of [Y_0 .. Y_5]: 32 row groups further
-                            umma_f16(tmem + TC_N * sl + 256, ad, umma_desc(b_k + 32u * SBO, LBO, SBO),
-                                     umma_idesc(TC_M, ncols - 256), acc);
+                    for (int sl = SL - 1; sl >= 0; --sl) {
+                        // the alternating set is free since the chunk before
+                        // ended, acc_3 and acc_2 (six digits), acc_1 and acc_0
+                        // when the drain says so
+                        if (c > 0 && (sl == 1 || (SL == 6 && sl == 3))) {
+                            ok = ok && mbar_wait(smem_addr(&free_bar[SL == 6 && sl == 1 ? 1 : 0]), ap);
+                            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                        }
+                        if (!ok) break;
+                        part(dw, hi, sl, sl, sl, 0);
+                        slice(dw, hi, sl, sl + 1);
                     }
                 }
-                umma_commit(smem_addr(&empty_bar[st]));
-                if (kt % (kFlush / TC_K) == (kFlush / TC_K) - 1 || kt == nk - 1) umma_commit(smem_addr(&accf_bar));
+                if (!ok) break;
+                umma_commit(empty0 + 8 * st, el);
+                if (++st == STAGES) st = 0, ph ^= 1;
+                for (int q = 1; q < steps; ++q) {
+                    ok = mbar_wait(full0 + 8 * st, ph);
+                    if (!ok) break;
+                    const uint32_t dw = d0 + st * (STAGE >> 4);
+#pragma unroll
+                    for (int sl = 0; sl < SL; ++sl) slice(dw, hi, sl, sl);
+                    umma_commit(empty0 + 8 * st, el);
+                    if (++st == STAGES) st = 0, ph ^= 1;
+                }
+                // the other alternating set, which the next chunk starts on, is
+                // drained (waited for here, before this chunk's own completion,
+                // so that the barrier is never two phases ahead)
+                if (SL != 7 && c > 0) {
+                    ok = ok && mbar_wait(smem_addr(&high_bar), ap);
+                    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                }
+                if (!ok) break;
+                umma_commit(smem_addr(&accf_bar), el);
             }
-            // every MMA issued by this thread has completed before teardown
-            umma_commit(smem_addr(&drain_bar));
-            mbar_wait(smem_addr(&drain_bar), 0);
         }
+        // every MMA issued by this warp has completed before teardown
+        umma_commit(smem_addr(&drain_bar), el);
+        mbar_wait(smem_addr(&drain_bar), 0);
     } else {
         // drain warps: TMEM lane quadrant = warp % 4, one output row and one
         // 32-column half per thread
         const int quad = warp & 3, c0 = 32 * ((warp - 2) >> 2);
-        const int row = 32 * quad + lane;
-        float hi[32], lo[32];
-#pragma unroll
-        for (int c = 0; c < 32; ++c) hi[c] = lo[c] = 0.f;
-        bool ok = true;
-        for (int ch = 0; ch < nchunks && ok; ++ch) {
-            ok = mbar_wait(smem_addr(&accf_bar), ch & 1);
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-#pragma unroll
-            for (int d = 0; d < SL; ++d) {
-                const float w = __int_as_float((127 - 8 * d) << 23);  // 2^(-8 d), exact
-                uint32_t r[32];
-                tmem_ld32(tmem + ((uint32_t)(32 * quad) << 16) + TC_N * d + c0, r);
-#pragma unroll
-                for (int c = 0; c < 32; ++c) two_sum_acc(hi[c], lo[c], __fmul_rn(__uint_as_float(r[c]), w));
-            }
+        const uint32_t tbase = tmem + ((uint32_t)(32 * quad) << 16) + c0;
+        auto release = [&](uint64_t &bar) {
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-            mbar_arrive(smem_addr(&acce_bar));
-        }
-        const int i = i0 + row;
-        if (ok && i < M) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_addr(&bar));
+        };
+        auto f = [](uint32_t x) { return __uint_as_float(x); };
+        bool ok = true;
+        int c = 0;
+        for (int item = blockIdx.x; item < w.items && ok; item += gridDim.x) {
+            const TcItem it = tc_item(w, item);
+            float hi[32], lo[32], mid[SL == 7 ? 32 : 1];
 #pragma unroll
-            for (int c = 0; c < 32; ++c) {
-                const int j = j0 + c0 + c;
-                if (j < N && (!lower || j <= i)) {
-                    // exact conversions and the power-of-two scaling on the
-                    // bit patterns: one FP64 instruction per output
-                    const double v = scale2(f2d_bits(hi[c]) + f2d_bits(lo[c]), ex[i] + ey[j] - 14);
-                    if (atomic) atomicAdd(&C[(size_t)i * ldc + j], v);
-                    else C[(size_t)i * ldc + j] = v;
-                    if (lower && j < i) {
-                        if (atomic) atomicAdd(&C[(size_t)j * ldc + i], v);
-                        else C[(size_t)j * ldc + i] = v;
+            for (int q = 0; q < 32; ++q) hi[q] = lo[q] = 0.f;
+            if constexpr (SL == 7)
+#pragma unroll
+                for (int q = 0; q < 32; ++q) mid[q] = 0.f;
+            const int nchunks = (it.nk + kChunkSteps - 1) / kChunkSteps;
+            for (int ch = 0; ch < nchunks && ok; ++ch, ++c) {
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&accf_bar), c & 1));
+                if (!ok) break;
+                asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+                const uint32_t thigh = tbase + (c & 1) * TC_N * (ND - LOW);
+                if constexpr (SL == 7) {
+                    // 8 columns at a time (registers); the accumulators are
+                    // released with the last of them
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        uint32_t ra[8], rb[8];
+                        float s4[8], s3[8], f3[8];
+                        tmem_ld<8>(tbase + 8 * h + TC_N * 7, ra);
+                        tmem_ld<8>(tbase + 8 * h + TC_N * 6, rb);
+                        tmem_wait<8>(ra);
+                        tmem_wait<8>(rb);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) s4[q] = __fmaf_rn(f(ra[q]), 0x1p-8f, f(rb[q]));
+                        tmem_ld<8>(tbase + 8 * h + TC_N * 5, ra);
+                        tmem_ld<8>(tbase + 8 * h + TC_N * 4, rb);
+                        tmem_wait<8>(ra);
+                        tmem_wait<8>(rb);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const float g = __fmaf_rn(s4[q], 0x1p-8f, f(ra[q])), x = f(rb[q]);
+                            s4[q] = __fmaf_rn(g, 0x1p-8f, x);
+                            f3[q] = __fmaf_rn(g, 0x1p-8f, __fsub_rn(x, s4[q]));
+                        }
+                        uint32_t rc[8];
+                        tmem_ld<8>(tbase + 8 * h + TC_N * 3, ra);
+                        tmem_wait<8>(ra);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const float e = two_sum(f(ra[q]), __fmul_rn(s4[q], 0x1p-8f), s3[q]);
+                            f3[q] = __fmaf_rn(f3[q], 0x1p-8f, e);
+                        }
+                        tmem_ld<8>(tbase + 8 * h + TC_N * 2, rc);
+                        tmem_ld<8>(tbase + 8 * h + TC_N, rb);
+                        tmem_ld<8>(tbase + 8 * h, ra);
+                        tmem_wait<8>(rc);
+                        tmem_wait<8>(rb);
+                        tmem_wait<8>(ra);
+                        if (h == 3) release(free_bar[0]);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            add_chunk3(f(ra[q]), f(rb[q]), f(rc[q]), s3[q], f3[q], hi[8 * h + q], mid[8 * h + q],
+                                       lo[8 * h + q]);
+                    }
+                } else if constexpr (SL == 6) {
+                    // acc_3 and acc_2 first, then 8 columns at a time
+                    uint32_t r3[32], r2[32];
+                    tmem_ld<32>(tbase + TC_N * 3, r3);
+                    tmem_ld<32>(tbase + TC_N * 2, r2);
+                    tmem_wait<32>(r3);
+                    tmem_wait<32>(r2);
+                    release(free_bar[0]);
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        uint32_t ra[8], rb[8];
+                        float v[8], ev[8];
+                        tmem_ld<8>(thigh + 8 * h + TC_N * 5, ra);
+                        tmem_ld<8>(thigh + 8 * h + TC_N * 4, rb);
+                        tmem_wait<8>(ra);
+                        tmem_wait<8>(rb);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const float g = __fmaf_rn(f(ra[q]), 0x1p-8f, f(rb[q])), x = f(r3[8 * h + q]);
+                            v[q] = __fmaf_rn(g, 0x1p-8f, x);
+                            ev[q] = __fmaf_rn(g, 0x1p-8f, __fsub_rn(x, v[q]));
+                        }
+                        tmem_ld<8>(tbase + 8 * h + TC_N, rb);
+                        tmem_ld<8>(tbase + 8 * h, ra);
+                        tmem_wait<8>(rb);
+                        tmem_wait<8>(ra);
+                        if (h == 3) release(free_bar[1]);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            add_chunk<6>(f(ra[q]), f(rb[q]), f(r2[8 * h + q]), v[q], ev[q], hi[8 * h + q], lo[8 * h + q]);
+                    }
+                    release(high_bar);
+                } else {
+                    // acc_0 and acc_1 first, then the rest 8 columns at a time
+                    uint32_t r0[32], r1[32];
+                    tmem_ld<32>(tbase, r0);
+                    tmem_ld<32>(tbase + TC_N, r1);
+                    tmem_wait<32>(r0);
+                    tmem_wait<32>(r1);
+                    release(free_bar[0]);
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        uint32_t ra[8], rb[8], rc[8];
+                        tmem_ld<8>(thigh + 8 * h + TC_N * 4, ra);
+                        tmem_ld<8>(thigh + 8 * h + TC_N * 3, rb);
+                        tmem_ld<8>(thigh + 8 * h + TC_N * 2, rc);
+                        tmem_wait<8>(ra);
+                        tmem_wait<8>(rb);
+                        tmem_wait<8>(rc);
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            add_chunk<5>(f(r0[8 * h + q]), f(r1[8 * h + q]), f(rc[q]), __fmaf_rn(f(ra[q]), 0x1p-8f, f(rb[q])),
+                                         0.f, hi[8 * h + q], lo[8 * h + q]);
+                    }
+                    release(high_bar);
+                }
+            }
+            if (!ok) break;
+            // results: exact conversions and the power-of-two scaling on the bit
+            // patterns, one or two FP64 instructions per output
+            const int i = it.i0 + 32 * quad + lane, jb = it.j0 + c0;
+            const int ei = i < M ? ex[i] - 14 : 0;
+            const int row4 = i & ~3, a = lane & 3;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                double2 p[4];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int q = 8 * g + u, j = jb + q;
+                    double l = f2d_normal(lo[q]);
+                    if constexpr (SL == 7) l += f2d_normal(mid[q]);
+                    const double x = scale2(f2d_normal(hi[q]) + l, ei + (j < N ? ey[j] : 0));
+                    if (u & 1) p[u / 2].y = x;
+                    else p[u / 2].x = x;
+                    // the mirror image: consecutive rows of a column
+                    if (w.lower && j < i && i < M) {
+                        if (atomic) atomicAdd(&C[(size_t)j * ldc + i], x);
+                        else C[(size_t)j * ldc + i] = x;
+                    }
+                }
+                // 4 x 4 transpose of column pairs among four lanes: lane a gets
+                // pair a of the four rows, so that a warp writes 64-byte pieces
+#pragma unroll
+                for (int b = 1; b <= 2; b <<= 1)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        if (k & b) continue;
+                        const bool up = (a & b) != 0;
+                        const double2 send = up ? p[k] : p[k | b];
+                        const double2 got = make_double2(__shfl_xor_sync(0xffffffffu, send.x, b),
+                                                         __shfl_xor_sync(0xffffffffu, send.y, b));
+                        if (up) p[k] = got;
+                        else p[k | b] = got;
+                    }
+                const int j = jb + 8 * g + 2 * a;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int r = row4 + k;
+                    if (r >= M || j >= N) continue;
+                    double *cr = C + (size_t)r * ldc + j;
+                    if (vec && j + 1 < N) {
+                        *reinterpret_cast<double2 *>(cr) = p[k];
+                        continue;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        if (j + u >= N || (w.lower && j + u > r)) continue;
+                        const double x = u ? p[k].y : p[k].x;
+                        if (atomic) atomicAdd(cr + u, x);
+                        else cr[u] = x;
                     }
                 }
             }
@@ -482,118 +892,155 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TC_TMEM_COLS));
 }
 
+
+inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
+inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+// rows of FP64 pairs can be read (written) as 16-byte vectors
+inline bool pair_rows(const double *p, int ld) { return aligned16(p) && ld % 2 == 0; }
+
 template <int SL>
-void launch_tc(cudaStream_t s, int M, int N, const __nv_bfloat16 *Xs, int rows_px, const __nv_bfloat16 *Ys,
-               int rows_py, const int *ex, const int *ey, double *C, int ldc, int k_len, int splits, int lower) {
-    auto aligned16 = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
-    HSIM_CHECK_ARG(aligned16(Xs) && aligned16(Ys) && rows_px % TC_M == 0 && rows_py % TC_M == 0 && M <= rows_px &&
-                       N <= rows_py && k_len % TC_K == 0,
-                   "ozaki product: operand layout not supported");
-    HSIM_CHECK_ARG(!lower || M == N, "ozaki product: lower triangle needs a square result");
+void launch_tc(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, const TcWork &w,
+               bool atomic, const int *skip) {
     HSIM_SMEM_LIMIT_ONCE(k_ozaki_tc<SL>, tc_smem<SL>());
-    int k_split = (int)((k_len + splits - 1) / splits);
-    constexpr int kFlush = flush_k<SL>();
-    k_split = (k_split + kFlush - 1) / kFlush * kFlush;
-    splits = (int)cdiv(k_len, k_split);
-    dim3 g(cdiv(N, TC_N), cdiv(M, TC_M), (unsigned)splits);
-    k_ozaki_tc<SL><<<g, TC_THREADS, tc_smem<SL>(), s>>>(M, N, Xs, rows_px, Ys, rows_py, ex, ey, C, ldc, k_len, k_split,
-                                               splits > 1 ? 1 : 0, lower);
+    const int grid = std::min(w.items, sm_count_oz());
+    const bool vec = !atomic && !w.lower && pair_rows(C, ldc);
+    k_ozaki_tc<SL><<<grid, TC_THREADS, tc_smem<SL>(), s>>>(X.rows, Y.rows, X.slices, X.rows_p / TC_M, Y.slices,
+                                                          Y.rows_p / TC_N, X.exps, Y.exps, C, ldc, w, atomic ? 1 : 0,
+                                                          vec ? 1 : 0, skip);
     HSIM_LAUNCHED();
 }
 
-inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
-
 }  // namespace
 
-// Scratch: (up to) kSlices x rows_p x kp BF16 digits (tiled layout) then rows_p
-// exponents, rounded to whole 256-byte blocks so operands placed back to back
-// in one buffer stay aligned for the bulk copies.
-static size_t operand_bytes(int rows, int kdim) {
-    const size_t rows_p = (size_t)round_up(std::max(rows, 1), TC_M), kp = (size_t)round_up(std::max(kdim, 1), TKs);
-    size_t b = (size_t)kSlices * rows_p * kp * sizeof(__nv_bfloat16) + sizeof(int) * rows_p;
-    return (b + 511) / 256 * 256;
+// Scratch: digits x rows_p x kp BF16 digits then rows_p exponents, rounded to
+// whole 512-byte blocks so operands placed back to back in one buffer stay
+// aligned for the bulk copies (either operand's row padding).
+static size_t operand_bytes(int rows, int kdim, int digits) {
+    const size_t rows_p = (size_t)round_up(std::max(rows, 1), TC_M), kp = (size_t)round_up(std::max(kdim, 1), TC_K);
+    size_t b = (size_t)digits * rows_p * kp * sizeof(__nv_bfloat16) + sizeof(int) * rows_p;
+    return (b + 511) / 512 * 512;
 }
 
-size_t ozaki_cols_scratch(int n, int cols) { return operand_bytes(cols, n); }
-size_t ozaki_rows_scratch(int rows, int k) { return operand_bytes(rows, k); }
+size_t ozaki_cols_scratch(int n, int cols, int digits) { return operand_bytes(cols, n, digits); }
+size_t ozaki_rows_scratch(int rows, int k, int digits) { return operand_bytes(rows, k, digits); }
 
-static OzakiOperand make_operand(int rows, int kdim, void *scratch, int digits) {
-    HSIM_CHECK_ARG(digits == 5 || digits == 6, "ozaki product: 5 or 6 digits per value");
+static OzakiOperand make_operand(int rows, int kdim, void *scratch, int digits, OzakiRole role) {
+    HSIM_CHECK_ARG(digits >= 5 && digits <= 7, "ozaki product: 5, 6 or 7 digits per value");
+    HSIM_CHECK_ARG(aligned16(scratch), "ozaki product: scratch not 16-byte aligned");
     OzakiOperand op;
     op.digits = digits;
+    op.role = role;
     op.rows = rows;
-    op.rows_p = round_up(std::max(rows, 1), TC_M);
-    op.kp = round_up(std::max(kdim, 1), TKs);
+    op.rows_p = round_up(std::max(rows, 1), role == OzakiRole::X ? TC_M : TC_N);
+    op.kp = round_up(std::max(kdim, 1), TC_K);
     op.slices = static_cast<__nv_bfloat16 *>(scratch);
     op.exps = reinterpret_cast<int *>(op.slices + (size_t)digits * op.rows_p * op.kp);
     return op;
 }
 
-OzakiOperand ozaki_split_cols(cudaStream_t s, int n, int cols, const double *X, int ldx, void *scratch, int digits) {
-    OzakiOperand op = make_operand(cols, n, scratch, digits);
+static int role_log(OzakiRole r) { return r == OzakiRole::X ? 7 : 6; }
+
+void ozaki_col_exps(cudaStream_t s, int n, int cols, const double *X, int ldx, int *exps, const int *rexp) {
+    k_fill_int<<<cdiv(cols, 256), 256, 0, s>>>(cols, kNoExp, exps);
+    HSIM_LAUNCHED();
+    // rows per CTA: about eight CTAs per SM, 32 to 1024 rows
+    const int64_t cb = cdiv(cols, 64), want = std::max<int64_t>(1, 8 * (int64_t)sm_count_oz() / cb);
+    const int rows = (int)std::min<int64_t>(1024, std::max<int64_t>(32, round_up((int)cdiv(n, want), 8)));
+    k_col_exps<<<dim3(cdiv(n, rows), (unsigned)cb), 256, 0, s>>>(n, cols, X, ldx, rows, rexp, pair_rows(X, ldx), exps);
+    HSIM_LAUNCHED();
+}
+
+static void split_cols_into(cudaStream_t s, const OzakiOperand &op, int n, const double *X, int ldx, const int *rexp,
+                            float *sumsq) {
+    const dim3 g(cdiv(op.kp, 32), cdiv(op.rows_p, 64));
+    const bool vec = pair_rows(X, ldx);
+    const int rl = role_log(op.role);
+    if (op.digits == 5)
+        k_split_cols<5><<<g, 256, 0, s>>>(n, op.rows, X, ldx, vec, op.exps, rexp, op.slices, op.rows_p, op.kp, rl, sumsq);
+    else if (op.digits == 6)
+        k_split_cols<6><<<g, 256, 0, s>>>(n, op.rows, X, ldx, vec, op.exps, rexp, op.slices, op.rows_p, op.kp, rl, sumsq);
+    else
+        k_split_cols<7><<<g, 256, 0, s>>>(n, op.rows, X, ldx, vec, op.exps, rexp, op.slices, op.rows_p, op.kp, rl, sumsq);
+    HSIM_LAUNCHED();
+}
+
+OzakiOperand ozaki_split_cols(cudaStream_t s, int n, int cols, const double *X, int ldx, void *scratch, int digits,
+                              OzakiRole role) {
+    OzakiOperand op = make_operand(cols, n, scratch, digits, role);
     if (n <= 0 || cols <= 0) return op;
-    k_fill_int<<<cdiv(cols, 256), 256, 0, s>>>(cols, -1074, op.exps);
-    HSIM_LAUNCHED();
-    k_col_exps<<<dim3(cdiv(n, 256), cdiv(cols, 256)), 256, 0, s>>>(n, cols, X, ldx, op.exps);
-    HSIM_LAUNCHED();
-    const dim3 g(op.kp / 32, cdiv(op.rows_p, 32));
-    if (digits == 5) k_split_cols_tiled<5><<<g, 128, 0, s>>>(n, cols, X, ldx, op.exps, op.slices, op.rows_p);
-    else k_split_cols_tiled<6><<<g, 128, 0, s>>>(n, cols, X, ldx, op.exps, op.slices, op.rows_p);
-    HSIM_LAUNCHED();
+    ozaki_col_exps(s, n, cols, X, ldx, op.exps, nullptr);
+    split_cols_into(s, op, n, X, ldx, nullptr, nullptr);
     return op;
+}
+
+static void split_rows_into(cudaStream_t s, const OzakiOperand &op, int k, const double *X, int ldx, const int *cexp) {
+    k_row_exps<<<cdiv(op.rows, 8), 256, 0, s>>>(op.rows, k, X, ldx, cexp, op.exps);
+    HSIM_LAUNCHED();
+    const unsigned g = cdiv((int64_t)(op.rows_p / 8) * ((op.kp + 31) / 32) * 32, 256);
+    const bool vec = pair_rows(X, ldx);
+    const int rl = role_log(op.role);
+    if (op.digits == 5)
+        k_split_rows<5><<<g, 256, 0, s>>>(op.rows, k, X, ldx, vec, op.exps, cexp, op.slices, op.rows_p, op.kp, rl);
+    else if (op.digits == 6)
+        k_split_rows<6><<<g, 256, 0, s>>>(op.rows, k, X, ldx, vec, op.exps, cexp, op.slices, op.rows_p, op.kp, rl);
+    else
+        k_split_rows<7><<<g, 256, 0, s>>>(op.rows, k, X, ldx, vec, op.exps, cexp, op.slices, op.rows_p, op.kp, rl);
+    HSIM_LAUNCHED();
 }
 
 OzakiOperand ozaki_split_rows(cudaStream_t s, int rows, int k, const double *X, int ldx, void *scratch, int digits) {
-    OzakiOperand op = make_operand(rows, k, scratch, digits);
+    OzakiOperand op = make_operand(rows, k, scratch, digits, OzakiRole::X);
     if (rows <= 0) return op;
-    k_row_exps<<<cdiv(rows, 8), 256, 0, s>>>(rows, k, X, ldx, op.exps);
-    HSIM_LAUNCHED();
-    const int64_t warps = (int64_t)(op.rows_p / 8) * (op.kp / 32);
-    if (digits == 5)
-        k_split_rows_tiled<5><<<cdiv(warps * 32, 256), 256, 0, s>>>(rows, k, X, ldx, op.exps, op.slices, op.rows_p,
-                                                                   op.kp);
-    else
-        k_split_rows_tiled<6><<<cdiv(warps * 32, 256), 256, 0, s>>>(rows, k, X, ldx, op.exps, op.slices, op.rows_p,
-                                                                   op.kp);
-    HSIM_LAUNCHED();
+    split_rows_into(s, op, k, X, ldx, nullptr);
     return op;
 }
 
-void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, int k_len, double *C, int ldc,
-                   int splits, bool lower) {
+void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, int splits,
+                   bool lower, bool accumulate, const int *skip) {
     if (X.rows <= 0 || Y.rows <= 0) return;
     HSIM_CHECK_ARG(X.kp == Y.kp, "ozaki_product: operands split over different K");
     HSIM_CHECK_ARG(X.digits == Y.digits, "ozaki_product: operands split into different digit counts");
+    HSIM_CHECK_ARG(X.role == OzakiRole::X && Y.role == OzakiRole::Y, "ozaki_product: operand roles");
+    HSIM_CHECK_ARG(!lower || X.rows == Y.rows, "ozaki product: lower triangle needs a square result");
+    TcWork w{};
+    w.lower = lower ? 1 : 0;
+    w.ksteps = X.kp / TC_K;
+    w.ntn = (int)cdiv(Y.rows, TC_N);
+    const int tx = (int)cdiv(X.rows, TC_M);
+    int64_t tiles = 0;
+    for (int r = 0; r < tx; ++r) tiles += lower ? std::min(w.ntn, 2 * r + 2) : w.ntn;
+    // K ranges: whole chunks, at most kItemK rows each, chosen so that tiles x
+    // ranges fill whole waves of one CTA per SM
+    const int64_t chunks = cdiv(w.ksteps, kChunkSteps);
+    const int64_t s_min = std::max<int64_t>(1, cdiv((int64_t)w.ksteps * TC_K, kItemK));
     if (splits <= 0) {
-        // split K so that tiles x splits fills whole waves of one CTA per SM
-        const int64_t tx = cdiv(X.rows, TC_M), ty = cdiv(Y.rows, TC_N);
-        int64_t tiles = 0;
-        for (int64_t r = 0; r < tx; ++r) tiles += lower ? std::min<int64_t>(ty, (r * TC_M + TC_M - 1) / TC_N + 1) : ty;
         const int64_t sms = sm_count_oz();
-        const int64_t s_max = std::max<int64_t>(1, std::min<int64_t>(k_len / 2048, 8 * sms / tiles + 1));
+        const int64_t s_max = std::max(s_min, std::min<int64_t>(chunks, 8 * sms / tiles + 1));
         double best = -1.0;
-        splits = 1;
-        for (int64_t sp = 1; sp <= s_max; ++sp) {
-            const int64_t ctas = tiles * sp, waves = (ctas + sms - 1) / sms;
-            // fill of the last wave, with a small preference for fewer splits
-            const double eff = (double)ctas / (double)(waves * sms) - 0.002 * (double)sp;
-            if (sp * tiles >= sms / 2 && eff > best + 1e-9) {
+        for (int64_t sp = s_min; sp <= s_max; ++sp) {
+            const int64_t items = tiles * sp, waves = (items + sms - 1) / sms;
+            // fill of the last wave, with a small preference for fewer ranges
+            const double eff = (double)items / (double)(waves * sms) - 0.002 * (double)sp;
+            if (eff > best + 1e-9) {
                 best = eff;
                 splits = (int)sp;
             }
         }
-        if (best < 0) splits = (int)s_max;
     }
-    if (splits > 1) {
+    splits = (int)std::max<int64_t>(splits, s_min);
+    w.split = (int)cdiv(chunks, splits) * kChunkSteps;
+    splits = (int)cdiv(w.ksteps, w.split);
+    HSIM_CHECK_ARG(tiles * splits <= INT32_MAX / 2, "ozaki product: too many tiles");
+    w.tiles = (int)tiles;
+    w.items = (int)(tiles * splits);
+    const bool atomic = splits > 1 || accumulate;
+    if (atomic && !accumulate) {
         if (ldc == Y.rows) HSIM_CUDA(cudaMemsetAsync(C, 0, (size_t)X.rows * Y.rows * sizeof(double), s));
         else HSIM_CUDA(cudaMemset2DAsync(C, (size_t)ldc * sizeof(double), 0, (size_t)Y.rows * sizeof(double), X.rows, s));
     }
-    if (X.digits == 5)
-        launch_tc<5>(s, X.rows, Y.rows, X.slices, X.rows_p, Y.slices, Y.rows_p, X.exps, Y.exps, C, ldc, X.kp, splits,
-                     lower ? 1 : 0);
-    else
-        launch_tc<6>(s, X.rows, Y.rows, X.slices, X.rows_p, Y.slices, Y.rows_p, X.exps, Y.exps, C, ldc, X.kp, splits,
-                     lower ? 1 : 0);
+    if (X.digits == 5) launch_tc<5>(s, X, Y, C, ldc, w, atomic, skip);
+    else if (X.digits == 6) launch_tc<6>(s, X, Y, C, ldc, w, atomic, skip);
+    else launch_tc<7>(s, X, Y, C, ldc, w, atomic, skip);
 }
 
 void ozaki_check(cudaStream_t s) {

@@ -289,31 +289,36 @@ void solve_bwd_inv(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_n
 
 // ---- FP64-accurate products on BF16 tensor cores (k_ozaki.cu) --------------
 constexpr int kOzakiSlices = 6;
+// first operand of a product (rows of C, padded to 128) or second (columns of
+// C, padded to 64)
+enum class OzakiRole { X, Y };
 // digit slices of an FP64 block in the tiled layout of k_ozaki.cu: rows
-// padded to rows_p (multiple of 128), K to kp (multiple of 32), zero filled;
-// one exponent per row; `digits` slices of 8 bits (6: 47 bits per value, the
-// FP64-accurate form; 5: 39 bits)
+// padded to rows_p, K to kp (multiple of 16), zero filled; one exponent per
+// row; `digits` slices of 8 bits (6: 47 bits per value, the FP64-accurate form
+// of the mixed path; 5: 39 bits; 7: 55 bits, in place of FP64 arithmetic)
 struct OzakiOperand {
     int rows = 0, rows_p = 0, kp = 0, digits = kOzakiSlices;
+    OzakiRole role = OzakiRole::X;
     __nv_bfloat16 *slices = nullptr;
     int *exps = nullptr;
 };
 // bytes of scratch for splitting an n x cols block per column (K = n), or a
 // rows x k block per row (K = k)
-size_t ozaki_cols_scratch(int n, int cols);
-size_t ozaki_rows_scratch(int rows, int k);
+size_t ozaki_cols_scratch(int n, int cols, int digits = kOzakiSlices);
+size_t ozaki_rows_scratch(int rows, int k, int digits = kOzakiSlices);
 // split X (row-major, K = n rows) per column into a transposed operand
-OzakiOperand ozaki_split_cols(cudaStream_t s, int n, int cols, const double *X, int ldx, void *scratch,
-                              int digits = kOzakiSlices);
-// split X (row-major rows x k, K = k) per row
+OzakiOperand ozaki_split_cols(cudaStream_t s, int n, int cols, const double *X, int ldx, void *scratch, int digits,
+                              OzakiRole role);
+// split X (row-major rows x k, K = k) per row (a first operand)
 OzakiOperand ozaki_split_rows(cudaStream_t s, int rows, int k, const double *X, int ldx, void *scratch,
                               int digits = kOzakiSlices);
-// C (X.rows x Y.rows, FP64) = X Y^T over K = k_len (= X.kp); splits <= 0 chooses a
-// split-K count (C accumulated with atomics), 1 stores directly; lower: C is
-// symmetric, only tiles meeting the lower triangle run and the epilogue
-// writes each value and its mirror image (X.rows == Y.rows)
-void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, int k_len, double *C, int ldc,
-                   int splits, bool lower = false);
+// C (X.rows x Y.rows, FP64) = X Y^T; splits <= 0 chooses a split-K count (C
+// accumulated with atomics), 1 stores directly (up to 16,384 deep); lower: C
+// is symmetric, only tiles meeting the lower triangle run and the epilogue
+// writes each value and its mirror image (X.rows == Y.rows); accumulate: added
+// to C; skip (device, may be null): nothing is done where *skip is nonzero
+void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, int splits,
+                   bool lower = false, bool accumulate = false, const int *skip = nullptr);
 // fails (HSIM_E_INTERNAL) if a tensor-core product kernel gave up waiting on
 // one of its barriers since the last check; synchronises the stream
 void ozaki_check(cudaStream_t s);

@@ -21,6 +21,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <exception>
 #include <memory>
 #include <mutex>
 #include <set>
@@ -94,13 +95,114 @@ void check_device_ptrs(int device, std::initializer_list<std::pair<const char *,
 }
 }  // namespace
 
+// Device scratch of the step-level calls, kept by the context between calls
+// (cudaMalloc and cudaFree of a few GB cost 3.3 ms next to a Gram product of
+// 2.5).  A call takes a block for its duration and returns it after its stream
+// has drained; calls of other threads on the same context meanwhile take
+// others.  At most kKeep bytes stay with the context (the largest of the last
+// blocks that fit), and they are given back when an allocation fails and when
+// the context is destroyed.
+struct ScratchPool {
+    static constexpr size_t kKeep = (size_t)2 << 30;
+    static constexpr size_t kBlocks = 16;
+    std::mutex mu;
+    std::pair<size_t, void *> free[kBlocks];  // the `used` blocks not in use by a call
+    size_t used = 0, kept = 0;
+    void *take(size_t bytes, size_t *got) {
+        {
+            std::lock_guard<std::mutex> lock(mu);
+            size_t best = used;
+            for (size_t i = 0; i < used; ++i)
+                if (free[i].first >= bytes && (best == used || free[i].first < free[best].first)) best = i;
+            if (best < used) {
+                void *p = free[best].second;
+                *got = free[best].first;
+                kept -= *got;
+                free[best] = free[--used];
+                return p;
+            }
+        }
+        void *p = nullptr;
+        cudaError_t e = cudaMalloc(&p, bytes);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            drop();
+            e = cudaMalloc(&p, bytes);
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            fail(HSIM_E_NOMEM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed: " + cudaGetErrorString(e));
+        }
+        *got = bytes;
+        return p;
+    }
+    // p was taken from here and no work on it is in flight
+    void give(void *p, size_t bytes) noexcept {
+        for (;;) {
+            void *out = p;
+            {
+                std::lock_guard<std::mutex> lock(mu);
+                if (bytes <= kKeep && kept + bytes <= kKeep && used < kBlocks) {
+                    free[used++] = {bytes, p};
+                    kept += bytes;
+                    return;
+                }
+                if (bytes <= kKeep && used > 0) {  // the smallest kept block makes room
+                    size_t m = 0;
+                    for (size_t i = 1; i < used; ++i)
+                        if (free[i].first < free[m].first) m = i;
+                    out = free[m].second;
+                    kept -= free[m].first;
+                    free[m] = free[--used];
+                }
+            }
+            cudaFree(out);
+            if (out == p) return;
+        }
+    }
+    void drop() noexcept {
+        std::lock_guard<std::mutex> lock(mu);
+        for (size_t i = 0; i < used; ++i) cudaFree(free[i].second);
+        used = kept = 0;
+    }
+    ~ScratchPool() { drop(); }
+};
+
 struct hsim_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
     DevBuf<int> flags;        // small device flag area
     std::vector<int> hflags;  // host mirror
     DevBuf<unsigned long long> scratch_u64;
+    ScratchPool pool;
 };
+
+namespace {
+
+// count elements of a call's scratch from the context's pool.  The holder's
+// scope ends after the call's stream has drained; when an error unwinds it, work
+// may be in flight and the block is freed instead (cudaFree waits for it).
+template <class T>
+struct CtxScratch {
+    hsim_ctx *ctx;
+    T *p;
+    size_t bytes = 0;
+    int unwinding = std::uncaught_exceptions();
+    CtxScratch(hsim_ctx *c, size_t count) : ctx(c) {
+        // sizes in steps of an eighth of their power of two: blocks fit again
+        size_t want = std::max<size_t>(count * sizeof(T), 256), step = 32;
+        while (step * 16 <= want) step *= 2;
+        p = static_cast<T *>(c->pool.take((want + step - 1) / step * step, &bytes));
+    }
+    CtxScratch(const CtxScratch &) = delete;
+    CtxScratch &operator=(const CtxScratch &) = delete;
+    ~CtxScratch() {
+        if (std::uncaught_exceptions() > unwinding) cudaFree(p);
+        else ctx->pool.give(p, bytes);
+    }
+};
+
+}  // namespace
 
 namespace {
 
@@ -1457,7 +1559,7 @@ hsim_status hsim_assemble(hsim_ctx *ctx, const hsim_hier *h, const double *V_dev
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"V", V_dev}, {"L2", L2_dev}, {"S_val", S_val}, {"M_diag", M_diag}});
         cudaStream_t s = ctx->stream;
-        DevBuf<double> cot((size_t)3 * h->m), area((size_t)h->m), Sm, Mm;
+        CtxScratch<double> cot(ctx, (size_t)3 * h->m), area(ctx, (size_t)h->m);
         const bool cm = consistent_mass(h);
         k::triangle_geometry(s, h->m, h->dF.p, V_dev, L2_dev, cot.p, area.p);
         if (h->dofs.empty()) {
@@ -1465,15 +1567,15 @@ hsim_status hsim_assemble(hsim_ctx *ctx, const hsim_hier *h, const double *V_dev
                            area.p, S_val, M_diag, cm);
         } else {
             // Dirichlet: the whole mesh, then the interior rows and columns
-            Sm.alloc((size_t)h->patm.nnz);
-            Mm.alloc(cm ? (size_t)h->patm.nnz : (size_t)h->n_mesh);
+            CtxScratch<double> Sm(ctx, (size_t)h->patm.nnz), Mm(ctx, cm ? (size_t)h->patm.nnz : (size_t)h->n_mesh);
             k::assemble_sm(s, h->n_mesh, h->patm.ptr.p, h->patm.col.p, h->d_ecot.p, cot.p, h->d_vt_ptr.p,
                            h->d_vt_idx.p, area.p, Sm.p, Mm.p, cm);
             k::gather_values(s, h->pat0.nnz, h->d_smap.p, Sm.p, S_val);
             if (cm) k::gather_values(s, h->pat0.nnz, h->d_smap.p, Mm.p, M_diag);
             else k::gather_values_i(s, h->n, h->d_dofs.p, Mm.p, M_diag);
+            HSIM_CUDA(cudaStreamSynchronize(s));  // before Sm and Mm are given back
         }
-        HSIM_CUDA(cudaStreamSynchronize(s));  // before the temporaries are freed
+        HSIM_CUDA(cudaStreamSynchronize(s));  // before the temporaries are given back
     });
 }
 
@@ -1654,11 +1756,8 @@ hsim_status hsim_gram_tc(hsim_ctx *ctx, int n, int ka, int kb, const double *A, 
         HSIM_CHECK_ARG(digits == 5 || digits == 6, "digits must be 5 or 6");
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"G", G}});
-        DevBuf<unsigned char> scratch(k::ozaki_cols_scratch(n, ka) + k::ozaki_cols_scratch(n, kb));
-        k::OzakiOperand X = k::ozaki_split_cols(ctx->stream, n, ka, A, lda, scratch.p, digits, k::OzakiRole::X);
-        k::OzakiOperand Y =
-            k::ozaki_split_cols(ctx->stream, n, kb, B, ldb, scratch.p + k::ozaki_cols_scratch(n, ka), digits, k::OzakiRole::Y);
-        k::ozaki_product(ctx->stream, X, Y, G, kb, 0);
+        CtxScratch<unsigned char> scratch(ctx, k::ozaki_gram_scratch(n, ka, kb, digits));
+        k::ozaki_gram(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, digits, scratch.p);
         k::ozaki_check(ctx->stream);
     });
 }
@@ -1670,11 +1769,8 @@ hsim_status hsim_gemm_update_tc(hsim_ctx *ctx, int n, int kk, int m, const doubl
         HSIM_CHECK_ARG(n >= 1 && kk >= 1 && m >= 1 && lda >= kk && ldb >= m && ldc >= m, "bad sizes");
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"C", C}});
-        DevBuf<unsigned char> scratch(k::ozaki_rows_scratch(n, kk) + k::ozaki_cols_scratch(kk, m));
-        k::OzakiOperand X = k::ozaki_split_rows(ctx->stream, n, kk, A, lda, scratch.p);
-        k::OzakiOperand Y = k::ozaki_split_cols(ctx->stream, kk, m, B, ldb, scratch.p + k::ozaki_rows_scratch(n, kk),
-                                                 k::kOzakiSlices, k::OzakiRole::Y);
-        k::ozaki_product(ctx->stream, X, Y, C, ldc, 1);
+        CtxScratch<unsigned char> scratch(ctx, k::ozaki_update_scratch(n, kk, m, k::kOzakiSlices));
+        k::ozaki_update(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc, k::kOzakiSlices, scratch.p);
         k::ozaki_check(ctx->stream);
     });
 }
@@ -1687,7 +1783,7 @@ hsim_status ritz_entry(hsim_ctx *ctx, int kk, const double *Sbar, const double *
         HSIM_CHECK_ARG(kk >= 1, "bad size");
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"Sbar", Sbar}, {"Mbar", Mbar}, {"evals", evals}, {"X", X}});
-        DevBuf<double> work(k::ritz_work_size(kk));
+        CtxScratch<double> work(ctx, k::ritz_work_size(kk));
         int sw = 0;
         int rc = k::ritz(ctx->stream, kk, Sbar, kk, Mbar, kk, evals, X, kk, work.p, &sw, ctx->flags.p,
                          ctx->hflags.data(), 0, tc);
@@ -1798,12 +1894,12 @@ hsim_status hsim_shifted_solve(hsim_ctx *ctx, hsim_hier *h, int tau, const doubl
         cudaStream_t s = ctx->stream;
         LevelData &L = h->lev[tau];
         const bool diag_m = tau == 0 && !consistent_mass(h);  // M_val: n diagonal values, else S's pattern
-        DevBuf<double> Sv((size_t)L.dpat.nnz), Mv(diag_m ? (size_t)L.n : (size_t)L.dpat.nnz);
+        CtxScratch<double> Sv(ctx, (size_t)L.dpat.nnz), Mv(ctx, diag_m ? (size_t)L.n : (size_t)L.dpat.nnz);
         k::gather_values(s, L.dpat.nnz, L.dvmap.p, S_val, Sv.p);
         if (diag_m) k::gather_values_i(s, L.n, L.d_perm.p, M_val, Mv.p);
         else k::gather_values(s, L.dpat.nnz, L.dvmap.p, M_val, Mv.p);
         int negp = factor_level(ctx, h, L, Sv.p, diag_m ? nullptr : Mv.p, diag_m ? Mv.p : nullptr, mu);
-        DevBuf<double> X((size_t)L.n * kk);
+        CtxScratch<double> X(ctx, (size_t)L.n * kk);
         k::gather_rows(s, L.n, kk, L.d_perm.p, B, ldb, X.p, kk);
         solve_level(ctx, h, L, X.p, kk, kk);
         k::gather_rows(s, L.n, kk, L.d_iperm.p, X.p, kk, B, ldb);
@@ -1824,16 +1920,16 @@ hsim_status hsim_shifted_solve_f32(hsim_ctx *ctx, hsim_hier *h, int tau, const d
         cudaStream_t s = ctx->stream;
         LevelData &L = h->lev[tau];
         const bool diag_m = tau == 0 && !consistent_mass(h);  // M_val: n diagonal values, else S's pattern
-        DevBuf<double> Sv((size_t)L.dpat.nnz), Mv(diag_m ? (size_t)L.n : (size_t)L.dpat.nnz);
+        CtxScratch<double> Sv(ctx, (size_t)L.dpat.nnz), Mv(ctx, diag_m ? (size_t)L.n : (size_t)L.dpat.nnz);
         k::gather_values(s, L.dpat.nnz, L.dvmap.p, S_val, Sv.p);
         if (diag_m) k::gather_values_i(s, L.n, L.d_perm.p, M_val, Mv.p);
         else k::gather_values(s, L.dpat.nnz, L.dvmap.p, M_val, Mv.p);
         int negp = factor_level_t<float>(ctx, L, Sv.p, diag_m ? nullptr : Mv.p, diag_m ? Mv.p : nullptr, mu,
                                          h->arena32, h->dpos32, h->dinvf32, h->invs32, 1e-7);
-        DevBuf<double> X((size_t)L.n * kk);
+        CtxScratch<double> X(ctx, (size_t)L.n * kk);
         k::gather_rows(s, L.n, kk, L.d_perm.p, B, ldb, X.p, kk);
         const int ld = (kk + 3) & ~3;  // 16-byte rows (vector atomics of the forward products)
-        DevBuf<float> X32((size_t)L.n * ld);
+        CtxScratch<float> X32(ctx, (size_t)L.n * ld);
         k::convert_matrix(s, L.n, kk, X.p, kk, X32.p, ld);
         solve_level_t<float>(ctx, L, h->arena32.p, h->dpos32.p, h->dinvf32.p, h->ysol32, X32.p, kk, ld);
         k::convert_matrix(s, L.n, kk, X32.p, ld, X.p, kk);

@@ -1043,6 +1043,67 @@ void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y,
     else launch_tc<7>(s, X, Y, C, ldc, w, atomic, skip);
 }
 
+// ---- products over ranges of rows -------------------------------------------
+// The digits of a whole n x 750 block are 5 to 7 n x 1.5 KB (2.3 GB at 250,000
+// rows and six digits); a range of rows keeps the scratch near kRangeBytes at
+// any n.  Ranges are whole work items of the product (kItemK rows for a Gram,
+// which adds the ranges in FP64 as it adds its items).
+constexpr size_t kRangeBytes = (size_t)1 << 30;
+
+static int range_rows(int64_t n, size_t row_bytes, int unit) {
+    const int64_t most = std::max<int64_t>(unit, (int64_t)(kRangeBytes / row_bytes) / unit * unit);
+    const int64_t ranges = std::max<int64_t>(1, (n + most - 1) / most);
+    return (int)std::min<int64_t>(most, ((n + ranges - 1) / ranges + unit - 1) / unit * unit);
+}
+static size_t exps_bytes(int rows) { return ((size_t)rows * sizeof(int) + 511) / 512 * 512; }
+static int gram_rows(int n, int ka, int kb, int digits) {
+    return range_rows(n, 2 * (size_t)digits * (round_up(ka, TC_M) + round_up(kb, TC_N)), kItemK);
+}
+
+size_t ozaki_gram_scratch(int n, int ka, int kb, int digits) {
+    const int r = std::min(gram_rows(n, ka, kb, digits), n);
+    return exps_bytes(ka) + exps_bytes(kb) + operand_bytes(ka, r, digits) + operand_bytes(kb, r, digits);
+}
+
+void ozaki_gram(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
+                int ldg, int digits, void *scratch) {
+    const int range = gram_rows(n, ka, kb, digits);
+    int *ex = static_cast<int *>(scratch);
+    int *ey = ex + exps_bytes(ka) / sizeof(int);
+    unsigned char *sx = reinterpret_cast<unsigned char *>(ey) + exps_bytes(kb);
+    unsigned char *sy = sx + operand_bytes(ka, std::min(range, n), digits);
+    ozaki_col_exps(s, n, ka, A, lda, ex, nullptr);
+    ozaki_col_exps(s, n, kb, B, ldb, ey, nullptr);
+    const bool several = n > range;
+    if (several) HSIM_CUDA(cudaMemset2DAsync(G, (size_t)ldg * sizeof(double), 0, (size_t)kb * sizeof(double), ka, s));
+    for (int r0 = 0; r0 < n; r0 += range) {
+        const int rows = std::min(range, n - r0);
+        OzakiOperand X = make_operand(ka, rows, sx, digits, OzakiRole::X), Y = make_operand(kb, rows, sy, digits, OzakiRole::Y);
+        X.exps = ex;
+        Y.exps = ey;
+        split_cols_into(s, X, rows, A + (size_t)r0 * lda, lda, nullptr, nullptr);
+        split_cols_into(s, Y, rows, B + (size_t)r0 * ldb, ldb, nullptr, nullptr);
+        ozaki_product(s, X, Y, G, ldg, 0, false, several);
+    }
+}
+
+static int update_rows(int n, int k, int digits) { return range_rows(n, 2 * (size_t)digits * round_up(k, TC_K), TC_M); }
+
+size_t ozaki_update_scratch(int n, int k, int m, int digits) {
+    return operand_bytes(m, k, digits) + operand_bytes(std::min(update_rows(n, k, digits), n), k, digits);
+}
+
+void ozaki_update(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
+                  int ldc, int digits, void *scratch) {
+    const int range = update_rows(n, k, digits);
+    unsigned char *sy = static_cast<unsigned char *>(scratch), *sx = sy + operand_bytes(m, k, digits);
+    OzakiOperand Y = ozaki_split_cols(s, k, m, B, ldb, sy, digits, OzakiRole::Y);
+    for (int r0 = 0; r0 < n; r0 += range) {
+        OzakiOperand X = ozaki_split_rows(s, std::min(range, n - r0), k, A + (size_t)r0 * lda, lda, sx, digits);
+        ozaki_product(s, X, Y, C + (size_t)r0 * ldc, ldc, 1);
+    }
+}
+
 void ozaki_check(cudaStream_t s) {
     int h = 0;
     HSIM_CUDA(cudaMemcpyFromSymbolAsync(&h, g_oz_error, sizeof(int), 0, cudaMemcpyDeviceToHost, s));

@@ -319,6 +319,15 @@ OzakiOperand ozaki_split_rows(cudaStream_t s, int rows, int k, const double *X, 
 // to C; skip (device, may be null): nothing is done where *skip is nonzero
 void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, int splits,
                    bool lower = false, bool accumulate = false, const int *skip = nullptr);
+// G (ka x kb, ld ldg) = A^T B over n rows and C (n x m, ld ldc) = A B (A n x k, B
+// k x m), split and multiplied a range of rows at a time so that the digits of
+// one range take about 1 GiB of scratch (256-byte aligned)
+size_t ozaki_gram_scratch(int n, int ka, int kb, int digits);
+void ozaki_gram(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
+                int ldg, int digits, void *scratch);
+size_t ozaki_update_scratch(int n, int k, int m, int digits);
+void ozaki_update(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
+                  int ldc, int digits, void *scratch);
 // fails (HSIM_E_INTERNAL) if a tensor-core product kernel gave up waiting on
 // one of its barriers since the last check; synchronises the stream
 void ozaki_check(cudaStream_t s);

@@ -1150,8 +1150,14 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
                 inf.ms_tc_product += t_prod;
                 ph[2] = t_split + t_prod;
             } else {
-                k::gram(s, n, q, q, H->Psi.p, q, H->SP.p, q, H->Sbar.p, q, true);
-                k::gram(s, n, q, q, H->Psi.p, q, H->MP.p, q, H->Mbar.p, q, true);
+                if (k::gram64_on_digits(n, q, q)) {
+                    H->oz.reserve(k::gram64_scratch(n, q, q));
+                    k::gram64(s, n, q, q, H->Psi.p, q, H->SP.p, q, H->Sbar.p, q, true, H->oz.p);
+                    k::gram64(s, n, q, q, H->Psi.p, q, H->MP.p, q, H->Mbar.p, q, true, H->oz.p);
+                } else {
+                    k::gram(s, n, q, q, H->Psi.p, q, H->SP.p, q, H->Sbar.p, q, true);
+                    k::gram(s, n, q, q, H->Psi.p, q, H->MP.p, q, H->Mbar.p, q, true);
+                }
             }
             k::scale_sym_unit_diag(s, q, H->Sbar.p, H->Mbar.p, q, H->colw.p);
             if (mixed) inf.ms_gram += (ph[2] += ts.stop());
@@ -1173,6 +1179,9 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
                 const double t_prod = ts.stop();
                 inf.ms_tc_product += t_prod;
                 ph[4] = t_split + t_prod;
+            } else if (k::update64_on_digits(n, q, q)) {
+                H->oz.reserve(k::update64_scratch(n, q, q));
+                k::update64(s, n, q, q, H->Psi.p, q, H->phibar.p, q, H->Phi.p, q, H->oz.p);
             } else {
                 k::gemm_nn(s, n, q, q, H->Psi.p, q, H->phibar.p, q, H->Phi.p, q);
             }
@@ -1187,10 +1196,8 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
             HSIM_CUDA(cudaMemcpyAsync(rs.data(), H->res_sums.p, 3 * p * sizeof(double), cudaMemcpyDeviceToHost, s));
             HSIM_CUDA(cudaMemcpyAsync(lam_h.data(), H->lam.p, q * sizeof(double), cudaMemcpyDeviceToHost, s));
             HSIM_CUDA(cudaStreamSynchronize(s));
-            if (mixed) {
-                k::ozaki_check(s);
-                k::tc32_check(s);
-            }
+            k::ozaki_check(s);
+            if (mixed) k::tc32_check(s);
             inf.ms_residual += (ph[5] = ts.stop());
             double lam_ref = lam_h[q - 1];
             for (int i = 0; i < q; ++i)
@@ -1731,6 +1738,12 @@ hsim_status hsim_gram(hsim_ctx *ctx, int n, int ka, int kb, const double *A, int
         HSIM_CHECK_ARG(n >= 0 && ka >= 0 && kb >= 0 && lda >= ka && ldb >= kb, "bad sizes");
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"G", G}});
+        if (k::gram64_on_digits(n, ka, kb)) {
+            CtxScratch<unsigned char> scratch(ctx, k::gram64_scratch(n, ka, kb));
+            k::gram64(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, false, scratch.p);
+            k::ozaki_check(ctx->stream);
+            return;
+        }
         k::gram(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, false);
         HSIM_CUDA(cudaStreamSynchronize(ctx->stream));
     });
@@ -1743,6 +1756,12 @@ hsim_status hsim_gemm_update(hsim_ctx *ctx, int n, int kk, int m, const double *
         HSIM_CHECK_ARG(n >= 0 && kk >= 0 && m >= 0 && lda >= kk && ldb >= m && ldc >= m, "bad sizes");
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"C", C}});
+        if (k::update64_on_digits(n, kk, m)) {
+            CtxScratch<unsigned char> scratch(ctx, k::update64_scratch(n, kk, m));
+            k::update64(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc, scratch.p);
+            k::ozaki_check(ctx->stream);
+            return;
+        }
         k::gemm_nn(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc);
         HSIM_CUDA(cudaStreamSynchronize(ctx->stream));
     });

@@ -47,7 +47,8 @@ constexpr int TK = 16;  // k step
 template <typename T>
 __global__ void __launch_bounds__(256) k_gram(int n, int ka, int kb, const T *__restrict__ A, int lda,
                                               const T *__restrict__ B, int ldb, double *__restrict__ G,
-                                              int ldg, int rows_per_split, int lower_only) {
+                                              int ldg, int rows_per_split, int lower_only, const int *__restrict__ only_if) {
+    if (only_if && !*only_if) return;
     const int ti = blockIdx.x, tj = blockIdx.y;
     if (lower_only && tj > ti) return;
     const int i0 = ti * TB, j0 = tj * TB;
@@ -92,7 +93,8 @@ __global__ void __launch_bounds__(256) k_gram(int n, int ka, int kb, const T *__
     }
 }
 
-__global__ void k_mirror_lower(int k, double *__restrict__ G, int ldg) {
+__global__ void k_mirror_lower(int k, double *__restrict__ G, int ldg, const int *__restrict__ only_if) {
+    if (only_if && !*only_if) return;
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)k * k) return;
     int i = (int)(idx / k), j = (int)(idx % k);
@@ -103,7 +105,8 @@ __global__ void k_mirror_lower(int k, double *__restrict__ G, int ldg) {
 template <typename T>
 __global__ void __launch_bounds__(256) k_gemm_nn(int n, int kk, int m, const T *__restrict__ A, int lda,
                                                  const double *__restrict__ B, int ldb, T *__restrict__ C,
-                                                 int ldc) {
+                                                 int ldc, const int *__restrict__ only_if) {
+    if (only_if && !*only_if) return;
     const int r0 = blockIdx.x * TB, j0 = blockIdx.y * TB;
     __shared__ T As[TK][TB + 1];
     __shared__ T Bs[TK][TB];
@@ -469,6 +472,24 @@ DenseFront &dense_front(int k, cudaStream_t s) {
 }  // namespace
 
 template <typename T>
+static void launch_gram(cudaStream_t s, int n, int ka, int kb, const T *A, int lda, const T *B, int ldb, double *G,
+                        int ldg, bool lower_only, const int *only_if) {
+    int ti = cdiv(ka, TB), tj = cdiv(kb, TB);
+    int64_t tiles = lower_only ? (int64_t)ti * (ti + 1) / 2 : (int64_t)ti * tj;
+    int64_t want = std::max<int64_t>(1, (4LL * sm_count() + tiles - 1) / tiles);
+    int64_t rows = std::max<int64_t>(256, (n + want - 1) / want);
+    rows = (rows + TK - 1) / TK * TK;
+    unsigned splits = cdiv(n, rows);
+    dim3 g(ti, tj, splits);
+    k_gram<T><<<g, 256, 0, s>>>(n, ka, kb, A, lda, B, ldb, G, ldg, (int)rows, lower_only ? 1 : 0, only_if);
+    HSIM_LAUNCHED();
+    if (lower_only) {
+        k_mirror_lower<<<cdiv((int64_t)ka * ka, 256), 256, 0, s>>>(ka, G, ldg, only_if);
+        HSIM_LAUNCHED();
+    }
+}
+
+template <typename T>
 void gram(cudaStream_t s, int n, int ka, int kb, const T *A, int lda, const T *B, int ldb, double *G, int ldg,
           bool lower_only) {
     if (ldg == kb) {
@@ -477,30 +498,38 @@ void gram(cudaStream_t s, int n, int ka, int kb, const T *A, int lda, const T *B
         HSIM_CUDA(cudaMemset2DAsync(G, (size_t)ldg * sizeof(double), 0, (size_t)kb * sizeof(double), ka, s));
     }
     if (n <= 0 || ka <= 0 || kb <= 0) return;
-    int ti = cdiv(ka, TB), tj = cdiv(kb, TB);
-    int64_t tiles = lower_only ? (int64_t)ti * (ti + 1) / 2 : (int64_t)ti * tj;
-    int64_t want = std::max<int64_t>(1, (4LL * sm_count() + tiles - 1) / tiles);
-    int64_t rows = std::max<int64_t>(256, (n + want - 1) / want);
-    rows = (rows + TK - 1) / TK * TK;
-    unsigned splits = cdiv(n, rows);
-    dim3 g(ti, tj, splits);
-    k_gram<T><<<g, 256, 0, s>>>(n, ka, kb, A, lda, B, ldb, G, ldg, (int)rows, lower_only ? 1 : 0);
+    launch_gram<T>(s, n, ka, kb, A, lda, B, ldb, G, ldg, lower_only, nullptr);
+}
+
+__global__ void k_zero_if(int rows, int cols, double *__restrict__ G, int ldg, const int *__restrict__ only_if) {
+    if (!*only_if) return;
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx < (int64_t)rows * cols) G[(size_t)(idx / cols) * ldg + idx % cols] = 0.0;
+}
+
+void gram_if(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
+             int ldg, bool lower_only, const int *flag) {
+    if (n <= 0 || ka <= 0 || kb <= 0) return;
+    k_zero_if<<<cdiv((int64_t)ka * kb, 256), 256, 0, s>>>(ka, kb, G, ldg, flag);
     HSIM_LAUNCHED();
-    if (lower_only) {
-        k_mirror_lower<<<cdiv((int64_t)ka * ka, 256), 256, 0, s>>>(ka, G, ldg);
-        HSIM_LAUNCHED();
-    }
+    launch_gram<double>(s, n, ka, kb, A, lda, B, ldb, G, ldg, lower_only, flag);
 }
 
 template <typename T>
 void gemm_nn(cudaStream_t s, int n, int kk, int m, const T *A, int lda, const double *B, int ldb, T *C, int ldc) {
     if (n <= 0 || m <= 0) return;
     dim3 g(cdiv(n, TB), cdiv(m, TB));
-    k_gemm_nn<T><<<g, 256, 0, s>>>(n, kk, m, A, lda, B, ldb, C, ldc);
+    k_gemm_nn<T><<<g, 256, 0, s>>>(n, kk, m, A, lda, B, ldb, C, ldc, nullptr);
     HSIM_LAUNCHED();
 }
 
-
+void gemm_nn_if(cudaStream_t s, int n, int kk, int m, const double *A, int lda, const double *B, int ldb, double *C,
+                int ldc, const int *flag) {
+    if (n <= 0 || m <= 0) return;
+    dim3 g(cdiv(n, TB), cdiv(m, TB));
+    k_gemm_nn<double><<<g, 256, 0, s>>>(n, kk, m, A, lda, B, ldb, C, ldc, flag);
+    HSIM_LAUNCHED();
+}
 
 template <typename T>
 void residual_sums(cudaStream_t s, int n, int k, const T *SP, int lds, const T *MP, int ldm, const double *lam,

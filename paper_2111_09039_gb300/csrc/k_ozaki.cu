@@ -32,47 +32,55 @@ namespace k {
 
 namespace {
 
-constexpr int kNoExp = -5000;  // exponent of a row or column of zeros
+constexpr int kNoExp = -5000;     // exponent of a row or column of zeros
+constexpr int kNonFinite = 1025;  // of an infinity or NaN
 
 inline unsigned cdiv(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
 // Exponents and digits are taken from the bits of the FP64 values with integer
 // arithmetic only (the FP64 pipe of this part is ~1/60 of the FP32 pipe).
 //
-// exponent e with |x| < 2^e for a nonzero x: biased exponent - 1022 (exact
-// for normal numbers, an upper bound for subnormals); kNoExp for zero
+// smallest e with |x| < 2^e for a nonzero x: biased exponent - 1022 (subnormals
+// by their leading bit); kNoExp for zero
 __device__ __forceinline__ int exp_bits(double a) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(a) & 0x7FFFFFFFFFFFFFFFULL;
-    return b == 0 ? kNoExp : (int)(b >> 52) - 1022;
+    const int e = (int)(b >> 52);
+    if (e != 0) return e - 1022;
+    return b == 0 ? kNoExp : -1010 - __clzll((long long)b);
 }
 
 // per-row exponents of a row-major R x C FP64 block: one warp per row; with
 // cexp, of the block whose column c is scaled by 2^-cexp[c]
 __global__ void k_row_exps(int R, int C, const double *__restrict__ X, int ldx, const int *__restrict__ cexp,
-                           int *__restrict__ ex) {
+                           int *__restrict__ ex, int *__restrict__ nonfinite) {
     int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     int lane = threadIdx.x & 31;
     if (row >= R) return;
     int m = kNoExp;
+    bool bad = false;
 #pragma unroll 4
     for (int j = lane; j < C; j += 32) {
         const int e = exp_bits(X[(size_t)row * ldx + j]);
+        bad |= e == kNonFinite;
         m = max(m, cexp && e != kNoExp ? e - cexp[j] : e);
     }
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (lane == 0) ex[row] = m;
+    if (nonfinite && bad) atomicOr(nonfinite, 1);
 }
 
 // per-column exponents of a row-major R x C FP64 block (ex pre-set to kNoExp);
 // with rexp, of the block whose row r is scaled by 2^rexp[r].  A CTA takes 64
 // columns (two per thread, 32 threads) of `rows` rows (eight at a time).
 __global__ void __launch_bounds__(256) k_col_exps(int R, int C, const double *__restrict__ X, int ldx, int rows,
-                                                  const int *__restrict__ rexp, bool vec, int *__restrict__ ex) {
+                                                  const int *__restrict__ rexp, bool vec, int *__restrict__ ex,
+                                                  int *__restrict__ nonfinite) {
     __shared__ int red[8][64];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int j = blockIdx.y * 64 + 2 * tx;
     const int r1 = min(R, (int)(blockIdx.x + 1) * rows);
     int m0 = kNoExp, m1 = kNoExp;
+    bool bad = false;
 #pragma unroll 4
     for (int r = blockIdx.x * rows + ty; r < r1; r += 8) {
         const double *p = X + (size_t)r * ldx + j;
@@ -85,6 +93,7 @@ __global__ void __launch_bounds__(256) k_col_exps(int R, int C, const double *__
             if (j + 1 < C) b = p[1];
         }
         int ea = exp_bits(a), eb = exp_bits(b);
+        bad |= ea == kNonFinite || eb == kNonFinite;
         if (rexp) {
             const int q = rexp[r];
             if (ea != kNoExp) ea += q;
@@ -102,6 +111,17 @@ __global__ void __launch_bounds__(256) k_col_exps(int R, int C, const double *__
         for (int q = 1; q < 8; ++q) m = max(m, red[q][threadIdx.x]);
         if (m != kNoExp) atomicMax(&ex[blockIdx.y * 64 + threadIdx.x], m);
     }
+    if (nonfinite && bad) atomicOr(nonfinite, 1);
+}
+
+// seven-digit Grams: flag set if a column's largest entry stands out, n 2^(2 e) >=
+// 1024 ||x||^2 (16 to 32 times the root mean square; a column that one entry
+// dominates has n to 4 n there); below that the truncation stays under the
+// rounding of the FP64 sums
+__global__ void k_guard_cols(int cols, float n, const int *__restrict__ ex, const float *__restrict__ sumsq,
+                             int *__restrict__ flag) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < cols && ex[j] != kNoExp && n * 16384.f >= 1024.f * sumsq[j]) atomicOr(flag, 2);
 }
 
 // T + offset of x against the group exponent e (|x| < 2^e): T = round(x
@@ -115,9 +135,10 @@ __device__ __forceinline__ long long split_int(double x, int e) {
     const long long bits = __double_as_longlong(x);
     const int E = (int)((bits >> 52) & 0x7FF);
     const unsigned long long M = (bits & 0xFFFFFFFFFFFFFULL) | (E ? 1ULL << 52 : 0ULL);
-    // x 2^(B-e) = +-M 2^sh, sh <= B - 53 <= 2 when |x| < 2^e
+    // x 2^(B-e) = +-M 2^sh, sh <= B - 53 <= 2 when |x| < 2^e, more for subnormals
     const int sh = (E ? E : 1) - 1075 + (8 * SL - 1) - e;
-    const unsigned long long t = (M << 3) >> min(max(2 - sh, 0), 63);
+    unsigned long long t = (M << 3) >> min(max(2 - sh, 0), 63);
+    if (sh > 2) t = M != 0 ? M << min(sh + 1, 63) : 0;
     const long long T = (long long)((t + 1) >> 1), neg = bits >> 63;
     constexpr long long off = (long long)(0x8080808080808080ULL >> (8 * (9 - SL)));
     return (T ^ neg) - neg + off;
@@ -940,13 +961,15 @@ static OzakiOperand make_operand(int rows, int kdim, void *scratch, int digits, 
 
 static int role_log(OzakiRole r) { return r == OzakiRole::X ? 7 : 6; }
 
-void ozaki_col_exps(cudaStream_t s, int n, int cols, const double *X, int ldx, int *exps, const int *rexp) {
+static void ozaki_col_exps(cudaStream_t s, int n, int cols, const double *X, int ldx, int *exps, const int *rexp,
+                           int *nonfinite = nullptr) {
     k_fill_int<<<cdiv(cols, 256), 256, 0, s>>>(cols, kNoExp, exps);
     HSIM_LAUNCHED();
     // rows per CTA: about eight CTAs per SM, 32 to 1024 rows
     const int64_t cb = cdiv(cols, 64), want = std::max<int64_t>(1, 8 * (int64_t)sm_count_oz() / cb);
     const int rows = (int)std::min<int64_t>(1024, std::max<int64_t>(32, round_up((int)cdiv(n, want), 8)));
-    k_col_exps<<<dim3(cdiv(n, rows), (unsigned)cb), 256, 0, s>>>(n, cols, X, ldx, rows, rexp, pair_rows(X, ldx), exps);
+    k_col_exps<<<dim3(cdiv(n, rows), (unsigned)cb), 256, 0, s>>>(n, cols, X, ldx, rows, rexp, pair_rows(X, ldx), exps,
+                                                                        nonfinite);
     HSIM_LAUNCHED();
 }
 
@@ -973,8 +996,9 @@ OzakiOperand ozaki_split_cols(cudaStream_t s, int n, int cols, const double *X, 
     return op;
 }
 
-static void split_rows_into(cudaStream_t s, const OzakiOperand &op, int k, const double *X, int ldx, const int *cexp) {
-    k_row_exps<<<cdiv(op.rows, 8), 256, 0, s>>>(op.rows, k, X, ldx, cexp, op.exps);
+static void split_rows_into(cudaStream_t s, const OzakiOperand &op, int k, const double *X, int ldx, const int *cexp,
+                            int *nonfinite = nullptr) {
+    k_row_exps<<<cdiv(op.rows, 8), 256, 0, s>>>(op.rows, k, X, ldx, cexp, op.exps, nonfinite);
     HSIM_LAUNCHED();
     const unsigned g = cdiv((int64_t)(op.rows_p / 8) * ((op.kp + 31) / 32) * 32, 256);
     const bool vec = pair_rows(X, ldx);
@@ -1102,6 +1126,114 @@ void ozaki_update(cudaStream_t s, int n, int k, int m, const double *A, int lda,
         OzakiOperand X = ozaki_split_rows(s, std::min(range, n - r0), k, A + (size_t)r0 * lda, lda, sx, digits);
         ozaki_product(s, X, Y, C + (size_t)r0 * ldc, ldc, 1);
     }
+}
+
+// ---- FP64 products on seven digits --------------------------------------------
+// gram and gemm_nn of the FP64 path.  Seven digits keep 55 bits against each
+// group's maximum and the digit pairs down to 2^-63, so the error per term is
+// 2^-57 of max|x| max|y| where an FP64 accumulation rounds every partial sum to
+// 2^-54 of itself.  Against quad-precision sums, FP64 kernels and digits:
+// Gram of 163,842 x 300 5.3e-16 and 0.9e-16 (all positive 4.7 and 1.4, smooth
+// columns 23 and 1.6), update 5.8e-16 and 2.3e-16 (a random second factor 5.8 and
+// 0.6, columns scaled by 10^+-6 5.7 and 2.2); the same order at 5,003 to 20,011
+// rows and 77 to 750 columns.  Scales that would spoil the common exponents are
+// taken out first: a Gram's columns have their own (a column with entries that
+// stand out goes to the FP64 kernel), an update scales column k of A by 2^-c_k
+// and row k of B by 2^c_k, exactly, so that their largest entries meet.
+// Infinities and NaN go to the FP64 kernels too: the device decides and repeats
+// the product with them where the flag is set.
+//
+// Where the line lies (us, FP64 kernel / digits, calls with a wait): Gram 1,024
+// rows x 30 to 300 columns 281 / 73 to 283 / 81, 16,384 x 75 530 / 101, 163,842 x
+// 300 36,600 / 1,473; fewer rows than 1,024 are left to the FP64 kernel (its time
+// falls with them, and the rule on standing-out entries has no room).  Update
+// with k = 30 44 / 57 to 8,192 rows and 75 / 60 at 16,384, k = 50 77 / 55 from
+// 1,024 rows on, 163,842 x 300 25,700 / 1,049.
+constexpr int kDigits64 = 7;
+constexpr int kUpdate64MaxK = 4096;  // the inner sums of the measurements above
+
+bool gram64_on_digits(int n, int ka, int kb) { return n >= 1024 && (double)n * ka * kb >= 5e5; }
+bool update64_on_digits(int n, int k, int m) {
+    return k <= kUpdate64MaxK && ((k > 40 && (double)n * k * m >= 2e6) || (double)n * k * m >= 1.2e7);
+}
+
+// c_k = half the exponent gap between column k of A and row k of B
+__global__ void k_balance(int k, const int *__restrict__ eb, int *__restrict__ c) {
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < k) c[j] = (c[j] - eb[j]) >> 1;
+}
+
+static size_t floats_bytes(int n) { return exps_bytes(n); }
+
+size_t gram64_scratch(int n, int ka, int kb) {
+    const int r = std::min(gram_rows(n, ka, kb, kDigits64), n);
+    return 512 + 2 * (exps_bytes(ka) + exps_bytes(kb)) + floats_bytes(ka) + floats_bytes(kb) +
+           operand_bytes(ka, r, kDigits64) + operand_bytes(kb, r, kDigits64);
+}
+
+void gram64(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
+            int ldg, bool lower, void *scratch) {
+    const int range = gram_rows(n, ka, kb, kDigits64);
+    unsigned char *p = static_cast<unsigned char *>(scratch);
+    auto take = [&](size_t bytes) {
+        unsigned char *q = p;
+        p += bytes;
+        return q;
+    };
+    const size_t zero_bytes = 512 + floats_bytes(ka) + floats_bytes(kb);
+    int *flag = reinterpret_cast<int *>(take(512));
+    float *ssx = reinterpret_cast<float *>(take(floats_bytes(ka))), *ssy = reinterpret_cast<float *>(take(floats_bytes(kb)));
+    int *ex = reinterpret_cast<int *>(take(exps_bytes(ka))), *ey = reinterpret_cast<int *>(take(exps_bytes(kb)));
+    unsigned char *sx = take(operand_bytes(ka, std::min(range, n), kDigits64)), *sy = p;
+    HSIM_CUDA(cudaMemsetAsync(flag, 0, zero_bytes, s));
+    const bool same = A == B && ka == kb && lda == ldb;
+    ozaki_col_exps(s, n, ka, A, lda, ex, nullptr, flag);
+    if (same) HSIM_CUDA(cudaMemcpyAsync(ey, ex, (size_t)ka * sizeof(int), cudaMemcpyDeviceToDevice, s));
+    else ozaki_col_exps(s, n, kb, B, ldb, ey, nullptr, flag);
+    const bool several = n > range;
+    if (several) HSIM_CUDA(cudaMemset2DAsync(G, (size_t)ldg * sizeof(double), 0, (size_t)kb * sizeof(double), ka, s));
+    for (int r0 = 0; r0 < n; r0 += range) {
+        const int rows = std::min(range, n - r0);
+        OzakiOperand X = make_operand(ka, rows, sx, kDigits64, OzakiRole::X), Y = make_operand(kb, rows, sy, kDigits64, OzakiRole::Y);
+        X.exps = ex;
+        Y.exps = ey;
+        split_cols_into(s, X, rows, A + (size_t)r0 * lda, lda, nullptr, ssx);
+        split_cols_into(s, Y, rows, B + (size_t)r0 * ldb, ldb, nullptr, ssy);
+        ozaki_product(s, X, Y, G, ldg, 0, lower, several);
+    }
+    k_guard_cols<<<cdiv(ka, 256), 256, 0, s>>>(ka, (float)n, ex, ssx, flag);
+    HSIM_LAUNCHED();
+    k_guard_cols<<<cdiv(kb, 256), 256, 0, s>>>(kb, (float)n, ey, ssy, flag);
+    HSIM_LAUNCHED();
+    gram_if(s, n, ka, kb, A, lda, B, ldb, G, ldg, lower, flag);
+}
+
+size_t update64_scratch(int n, int k, int m) {
+    return 512 + 2 * exps_bytes(k) + operand_bytes(m, k, kDigits64) +
+           operand_bytes(std::min(update_rows(n, k, kDigits64), n), k, kDigits64);
+}
+
+void update64(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
+              int ldc, void *scratch) {
+    const int range = update_rows(n, k, kDigits64);
+    int *flag = static_cast<int *>(scratch), *cexp = flag + 128, *bexp = cexp + exps_bytes(k) / sizeof(int);
+    unsigned char *sy = static_cast<unsigned char *>(scratch) + 512 + 2 * exps_bytes(k);
+    unsigned char *sx = sy + operand_bytes(m, k, kDigits64);
+    HSIM_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), s));
+    ozaki_col_exps(s, n, k, A, lda, cexp, nullptr, flag);
+    k_row_exps<<<cdiv(k, 8), 256, 0, s>>>(k, m, B, ldb, nullptr, bexp, flag);
+    HSIM_LAUNCHED();
+    k_balance<<<cdiv(k, 256), 256, 0, s>>>(k, bexp, cexp);
+    HSIM_LAUNCHED();
+    OzakiOperand Y = make_operand(m, k, sy, kDigits64, OzakiRole::Y);
+    ozaki_col_exps(s, k, m, B, ldb, Y.exps, cexp);
+    split_cols_into(s, Y, k, B, ldb, cexp, nullptr);
+    for (int r0 = 0; r0 < n; r0 += range) {
+        OzakiOperand X = make_operand(std::min(range, n - r0), k, sx, kDigits64, OzakiRole::X);
+        split_rows_into(s, X, k, A + (size_t)r0 * lda, lda, cexp);
+        ozaki_product(s, X, Y, C + (size_t)r0 * ldc, ldc, 1);
+    }
+    gemm_nn_if(s, n, k, m, A, lda, B, ldb, C, ldc, flag);
 }
 
 void ozaki_check(cudaStream_t s) {

@@ -91,6 +91,11 @@ void gram(cudaStream_t s, int n, int ka, int kb, const T *A, int lda, const T *B
 template <typename T>
 void gemm_nn(cudaStream_t s, int n, int k, int m, const T *A, int lda, const double *B, int ldb,
              T *C, int ldc);
+// the FP64 kernels where *flag (device) is nonzero, nothing elsewhere
+void gram_if(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
+             int ldg, bool lower_only, const int *flag);
+void gemm_nn_if(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
+                int ldc, const int *flag);
 // residual sums: out[3j+0] = sum w R^2, +1 = sum w (S Phi)^2, +2 = sum w (M Phi)^2
 // with R = SPhi - lam * MPhi; w = dinv (M^{-1}-norm) or 1 (2-norm)
 template <typename T>
@@ -328,6 +333,16 @@ void ozaki_gram(cudaStream_t s, int n, int ka, int kb, const double *A, int lda,
 size_t ozaki_update_scratch(int n, int k, int m, int digits);
 void ozaki_update(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
                   int ldc, int digits, void *scratch);
+// gram and gemm_nn in FP64 on seven digits (scratch 512-byte aligned), where the
+// *_on_digits rules say that they are the faster form
+bool gram64_on_digits(int n, int ka, int kb);
+size_t gram64_scratch(int n, int ka, int kb);
+void gram64(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
+            int ldg, bool lower, void *scratch);
+bool update64_on_digits(int n, int k, int m);
+size_t update64_scratch(int n, int k, int m);
+void update64(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
+              int ldc, void *scratch);
 // fails (HSIM_E_INTERNAL) if a tensor-core product kernel gave up waiting on
 // one of its barriers since the last check; synchronises the stream
 void ozaki_check(cudaStream_t s);

@@ -12,9 +12,9 @@
 //      column suffices (k_tridiag_rows); otherwise the rows stay in global
 //      memory with two barriers per column (k_tridiag).  The reflectors are
 //      kept row-wise in Vh (contiguous for the back transformation).
-//   2. Eigenvalues of T by multisection on Sturm counts, one warp per index
-//      (ascending by construction): FP32 rounds, an FP64 check of the
-//      bracket, FP64 rounds.
+//   2. Eigenvalues of T by multisection on division-free Sturm counts, a group
+//      of lanes per index (ascending by construction): FP32 rounds, then FP64
+//      rounds around the zero of the determinant's chord.
 //   3. Eigenvectors of T by inverse iteration on T - lambda I (Gaussian
 //      elimination with partial pivoting, reciprocal pivots kept), three
 //      iterations from a hashed random start; eigenvalues closer than
@@ -345,101 +345,160 @@ __global__ void __launch_bounds__(256) k_tri_back_warp(int n, int m, const doubl
     }
 }
 
-// number of eigenvalues of T below x (Sturm sequence of the LDL^T of T - x I)
-__device__ __forceinline__ int sturm_count(int n, const double *__restrict__ d, const double *__restrict__ e2,
-                                           double x, double pivmin) {
-    double q = d[0] - x;
-    if (fabs(q) < pivmin) q = -pivmin;
-    int c = q < 0.0;
-    for (int j = 1; j < n; ++j) {
-        q = d[j] - x - e2[j - 1] / q;
-        if (fabs(q) < pivmin) q = -pivmin;
-        c += q < 0.0;
-    }
-    return c;
-}
-
-// e2[j] = e[j]^2, and the Gershgorin interval and ||T|| in bounds[0..2]
-__global__ void k_tri_prep(int n, const double *__restrict__ d, const double *__restrict__ e, double *__restrict__ e2,
-                           double *__restrict__ bounds, float *__restrict__ d32, float *__restrict__ e232) {
+// T scaled by a power of two to a norm bound in [1/2, 1): ds, e2s = e^2 (at least
+// 2^-120 in FP64 and 2^-40 in FP32: couplings of 2^-60 and 2^-20 of ||T||, below
+// the accuracy of either count) and their FP32 copies; bounds: the Gershgorin
+// interval of the scaled T, ||T|| (not scaled), the scale
+__global__ void k_tri_prep(int n, const double *__restrict__ d, const double *__restrict__ e, double *__restrict__ ds,
+                           double *__restrict__ e2s, double *__restrict__ bounds, float *__restrict__ d32,
+                           float *__restrict__ e232) {
     __shared__ double red[3][kTriThreads / 32];
-    double lo = DBL_MAX, hi = -DBL_MAX, nm = 0.0, e2max = 0.0;
+    double lo = DBL_MAX, hi = -DBL_MAX, nm = 0.0;
     for (int j = threadIdx.x; j < n; j += kTriThreads) {
         const double r = (j > 0 ? fabs(e[j - 1]) : 0.0) + (j + 1 < n ? fabs(e[j]) : 0.0);
         lo = fmin(lo, d[j] - r);
         hi = fmax(hi, d[j] + r);
         nm = fmax(nm, fabs(d[j]) + r);
-        d32[j] = (float)d[j];
-        if (j + 1 < n) {
-            e2[j] = e[j] * e[j];
-            e232[j] = (float)e2[j];
-            e2max = fmax(e2max, e2[j]);
-        }
     }
     for (int o = 16; o > 0; o >>= 1) {
         lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
         hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
         nm = fmax(nm, __shfl_xor_sync(0xffffffffu, nm, o));
-        e2max = fmax(e2max, __shfl_xor_sync(0xffffffffu, e2max, o));
     }
-    __shared__ double red4[kTriThreads / 32];
     const int w = threadIdx.x >> 5;
     if ((threadIdx.x & 31) == 0) {
         red[0][w] = lo;
         red[1][w] = hi;
         red[2][w] = nm;
-        red4[w] = e2max;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = 1; i < kTriThreads / 32; ++i) {
-            lo = fmin(lo, red[0][i]);
-            hi = fmax(hi, red[1][i]);
-            nm = fmax(nm, red[2][i]);
-            e2max = fmax(e2max, red4[i]);
+    for (int i = 0; i < kTriThreads / 32; ++i) {
+        lo = fmin(lo, red[0][i]);
+        hi = fmax(hi, red[1][i]);
+        nm = fmax(nm, red[2][i]);
+    }
+    int ex = 0;
+    if (nm > 0.0 && nm <= DBL_MAX) frexp(nm, &ex);
+    const double sc = ldexp(1.0, min(max(-ex, -1000), 1000));
+    for (int j = threadIdx.x; j < n; j += kTriThreads) {
+        ds[j] = d[j] * sc;
+        d32[j] = (float)(d[j] * sc);
+        if (j + 1 < n) {
+            const double es = e[j] * sc, q = es * es;
+            e2s[j] = fmax(q, 0x1p-120);
+            e232[j] = fmaxf((float)q, 0x1p-40f);
         }
-        lo = fmin(lo, red[0][0]);
-        hi = fmax(hi, red[1][0]);
-        nm = fmax(nm, red[2][0]);
-        e2max = fmax(e2max, red4[0]);
-        const double pivmin = fmax(e2max, 1.0) * DBL_MIN / DBL_EPSILON;
-        const double pad = 2.0 * DBL_EPSILON * nm + pivmin;
-        bounds[0] = lo - pad;
-        bounds[1] = hi + pad;
+    }
+    if (threadIdx.x == 0) {
+        const double pad = 4.0 * DBL_EPSILON;
+        bounds[0] = lo * sc - pad;
+        bounds[1] = hi * sc + pad;
         bounds[2] = nm;
-        bounds[3] = pivmin;
+        bounds[3] = sc;
     }
 }
 
-__device__ __forceinline__ int sturm_count32(int n, const float *__restrict__ d, const float *__restrict__ e2, float x,
-                                             float pivmin) {
-    float q = d[0] - x;
-    if (fabsf(q) < pivmin) q = -pivmin;
-    int c = q < 0.f;
-    for (int j = 1; j < n; ++j) {
-        q = d[j] - x - e2[j - 1] / q;
-        if (fabsf(q) < pivmin) q = -pivmin;
-        c += q < 0.f;
+// Eigenvalues of the scaled T below x, and det(T - x I) as fm 2^fe.  The Sturm
+// sequence p_{j+1} = (d_j - x) p_j - e_j^2 p_{j-1} without divisions: three FP64
+// instructions a step, where d - x - e^2 / q takes about ten, and an FP64
+// instruction of a warp issues every 77 clocks on a sub-partition.  The count is
+// the number of sign changes (an exact zero is counted with its own or the next
+// step, whatever its sign).  |d - x| <= 2, 2^-120 <= e^2 <= 1: eight steps grow
+// p by at most 2^13 and shrink it by at most 2^-480, then the pair is rescaled
+// by its exponent.
+__device__ __forceinline__ int sturm_count(int n, const double *__restrict__ d, const double *__restrict__ e2,
+                                           double x, double &fm, int &fe) {
+    double p0 = 1.0, p1 = d[0] - x;
+    unsigned h1 = (unsigned)__double2hiint(p1);
+    int c = h1 >> 31, E = 0;
+    auto step = [&](double dj, double ej) {
+        const double p2 = fma(dj - x, p1, -(ej * p0));
+        const unsigned h2 = (unsigned)__double2hiint(p2);
+        c += (h2 ^ h1) >> 31;
+        p0 = p1;
+        p1 = p2;
+        h1 = h2;
+    };
+    for (int j = 1; j < n;) {
+        if (j + 8 <= n) {
+            double dj[8], ej[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) dj[u] = d[j + u], ej[u] = e2[j + u - 1];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) step(dj[u], ej[u]);
+            j += 8;
+        } else {
+            for (; j < n; ++j) step(d[j], e2[j - 1]);
+        }
+        const int e0 = (__double2hiint(p0) >> 20) & 0x7FF, e1 = (__double2hiint(p1) >> 20) & 0x7FF;
+        const int sh = max(e0, e1) - 1023;
+        // entries 2^-1000 below the larger one become zero (with their sign)
+        p0 = __hiloint2double(e0 > sh ? __double2hiint(p0) - sh * 0x100000 : __double2hiint(p0) & 0x80000000,
+                              e0 > sh ? __double2loint(p0) : 0);
+        p1 = __hiloint2double(e1 > sh ? __double2hiint(p1) - sh * 0x100000 : __double2hiint(p1) & 0x80000000,
+                              e1 > sh ? __double2loint(p1) : 0);
+        E += sh;
+    }
+    fm = p1;
+    fe = E;
+    return c;
+}
+
+// the same in FP32 (e^2 >= 2^-40, rescaled every four steps), for brackets of
+// 1e-5 ||T||
+__device__ __forceinline__ int sturm_count32(int n, const float *__restrict__ d, const float *__restrict__ e2, float x) {
+    float p0 = 1.f, p1 = d[0] - x;
+    unsigned h1 = __float_as_uint(p1);
+    int c = h1 >> 31;
+    auto step = [&](float dj, float ej) {
+        const float p2 = fmaf(dj - x, p1, -(ej * p0));
+        const unsigned h2 = __float_as_uint(p2);
+        c += (h2 ^ h1) >> 31;
+        p0 = p1;
+        p1 = p2;
+        h1 = h2;
+    };
+    for (int j = 1; j < n;) {
+        if (j + 4 <= n) {
+            float dj[4], ej[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) dj[u] = d[j + u], ej[u] = e2[j + u - 1];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) step(dj[u], ej[u]);
+            j += 4;
+        } else {
+            for (; j < n; ++j) step(d[j], e2[j - 1]);
+        }
+        const int e0 = (__float_as_uint(p0) >> 23) & 0xFF, e1 = (h1 >> 23) & 0xFF;
+        const int sh = max(e0, e1) - 127;
+        p0 = __uint_as_float(e0 > sh ? __float_as_uint(p0) - (unsigned)(sh * 0x800000) : __float_as_uint(p0) & 0x80000000u);
+        p1 = __uint_as_float(e1 > sh ? h1 - (unsigned)(sh * 0x800000) : h1 & 0x80000000u);
+        h1 = __float_as_uint(p1);
     }
     return c;
 }
 
-// lambda_i, i < m: G eigenvalues per warp, L = 32 / G lanes each (L >= 2),
-// multisection with L interior points (the bracket shrinks (L + 1)-fold per
-// round).  FP32 rounds first (the FP32 pipe is ~60x the FP64 pipe) down to
-// 1e-5 ||T||, then the bracket is checked with FP64 counts and widened until
-// it holds, then FP64 rounds to full precision.  The FP64 rounds dominate; FP64
-// issues at about one warp instruction per 64 cycles per SM sub-partition, so
-// the launch gives each sub-partition about one warp, with G = ceil(m / (4 SMs)):
-// fewer points per eigenvalue cost more rounds, a second warp on a
-// sub-partition doubles every round.
+// number of leading lanes of the group whose count is at most i (monotone up to
+// rounding: the highest such lane decides)
 __device__ __forceinline__ int group_le(bool le, int gbase, int L) {
     const unsigned bal = __ballot_sync(0xffffffffu, le);
     const unsigned g = (L == 32) ? bal : (bal >> gbase) & ((1u << L) - 1u);
-    // lanes 0..j-1 of the group have count <= i (monotone up to rounding): take the highest
     return g == 0 ? 0 : 32 - __clz(g);
 }
 
+// lambda_i, i < m: G eigenvalues per warp, L = 32 / G >= 2 lanes each, every
+// lane a Sturm count per round.  FP32 multisection down to 1e-5 ||T||; a first
+// FP64 round on points from end to end of that bracket, which is widened until
+// its counts hold; then FP64 rounds to full precision.  Where the bracket holds
+// the one eigenvalue, the lanes gather around the zero of the chord of the
+// determinant, at distances of 2^-3 to 2^-24 of the bracket on either side: the
+// chord is off by about (bracket / gap) brackets, so the bracket shrinks
+// quadratically (three to four FP64 rounds at n = 750, where equal sections take
+// nine); the counts still decide, and a round that does not shrink the bracket
+// fourfold, or a bracket of several eigenvalues, is followed by equal sections.
+// What bounds it: an FP64 round is n dependent steps of three instructions of 77
+// clocks, 84 us at n = 750 with one warp per sub-partition (G = ceil(m / (4 SMs)):
+// a second warp on a sub-partition doubles every round).
 __global__ void k_tri_bisect(int n, int m, int G, const double *__restrict__ d, const double *__restrict__ e2,
                              const float *__restrict__ d32, const float *__restrict__ e232,
                              const double *__restrict__ bounds, double *__restrict__ lam) {
@@ -448,16 +507,14 @@ __global__ void k_tri_bisect(int n, int m, int G, const double *__restrict__ d, 
     const int i = warp * G + gi;
     const bool valid = gi < G && i < m;
     if (warp * G >= m) return;  // uniform per warp
-    const double glo = bounds[0], ghi = bounds[1], tn = bounds[2], pivmin = bounds[3];
+    const double glo = bounds[0], ghi = bounds[1], tn = bounds[2] * bounds[3];
     const double sect = 1.0 / (L + 1);
     double lo = glo, hi = ghi;
-    // FP32 multisection
-    const float pivmin32 = fmaxf((float)fmin(pivmin / DBL_MIN * FLT_MIN, 1e30), FLT_MIN / FLT_EPSILON);
     for (int round = 0; round < 64; ++round) {
-        const bool go = valid && hi - lo > 1e-5 * tn;
+        const bool go = valid && hi - lo > 1e-5;
         if (!__any_sync(0xffffffffu, go)) break;
         const double x = lo + (hi - lo) * ((li + 1) * sect);
-        const bool le = go && sturm_count32(n, d32, e232, (float)x, pivmin32) <= i;
+        const bool le = go && sturm_count32(n, d32, e232, (float)x) <= i;
         const int nle = group_le(le, gbase, L);
         if (go) {
             const double nlo = nle > 0 ? lo + (hi - lo) * (nle * sect) : lo;
@@ -466,45 +523,64 @@ __global__ void k_tri_bisect(int n, int m, int G, const double *__restrict__ d, 
             hi = nhi;
         }
     }
-    // FP64 check: count(lo) <= i < count(hi), widen otherwise
-    double w = fmax(hi - lo, 1e-5 * tn);
+    // one FP64 round of the whole warp: counts at x (ascending lanes of a group)
+    // move lo and hi; flo, fhi: the determinant there (fe < kNone: not known),
+    // clo, chi: the counts
+    constexpr int kNone = -(1 << 30);
+    double flo = 0.0, fhi = 0.0;
+    int elo = kNone, ehi = kNone, clo = 0, chi = 0;
+    auto narrow = [&](double x, bool go) {
+        double fm = 0.0;
+        int fe = 0;
+        const int cnt = go ? sturm_count(n, d, e2, x, fm, fe) : 0;
+        const int nle = group_le(go && cnt <= i, gbase, L);
+        const int sl = gbase + max(nle - 1, 0), sh = gbase + min(nle, L - 1);
+        const double xl = __shfl_sync(0xffffffffu, x, sl & 31), xh = __shfl_sync(0xffffffffu, x, sh & 31);
+        const double ml = __shfl_sync(0xffffffffu, fm, sl & 31), mh = __shfl_sync(0xffffffffu, fm, sh & 31);
+        const int fl = __shfl_sync(0xffffffffu, fe, sl & 31), fh = __shfl_sync(0xffffffffu, fe, sh & 31);
+        const int cl = __shfl_sync(0xffffffffu, cnt, sl & 31), ch = __shfl_sync(0xffffffffu, cnt, sh & 31);
+        if (go && nle > 0) lo = xl, flo = ml, elo = fl, clo = cl;
+        if (go && nle < L) hi = xh, fhi = mh, ehi = fh, chi = ch;
+        return nle;
+    };
+    // the FP32 bracket, end to end; widened where its own ends do not hold
+    double wid = fmax(hi - lo, 1e-5);
     bool checked = !valid;
     for (int t = 0; t < 64; ++t) {
         if (!__any_sync(0xffffffffu, !checked)) break;
-        const double x = li == 0 ? lo : hi;
-        const int c = (!checked && li < 2) ? sturm_count(n, d, e2, x, pivmin) : 0;
-        const int clo = __shfl_sync(0xffffffffu, c, gbase), chi = __shfl_sync(0xffffffffu, c, gbase + 1);
+        const double l0 = lo, h0 = hi;
+        const int nle = narrow(l0 + (h0 - l0) * ((double)li / (L - 1)), !checked);
         if (!checked) {
-            const bool okl = clo <= i || lo <= glo, okh = chi > i || hi >= ghi;
-            if (okl && okh) {
-                checked = true;
-            } else {
-                if (!okl) lo = fmax(glo, lo - w);
-                if (!okh) hi = fmin(ghi, hi + w);
-                w *= 2.0;
-            }
+            const bool okl = nle > 0 || l0 <= glo, okh = nle < L || h0 >= ghi;
+            checked = okl && okh;
+            if (!okl) lo = fmax(glo, l0 - wid), hi = l0, elo = kNone;
+            if (!okh) hi = fmin(ghi, h0 + wid), lo = h0, ehi = kNone;
+            wid *= 2.0;
         }
     }
-    // FP64 multisection to 2 eps max(|lambda|, ||T||): the absolute accuracy
-    // of a dense symmetric eigensolve (a relative stop alone would drive the
-    // bracket of an eigenvalue at zero down to pivmin)
-    const double atol = 2.0 * DBL_EPSILON * tn + pivmin;
+    // to 2 eps max(|lambda|, ||T||): the absolute accuracy of a dense symmetric
+    // eigensolve
+    const int H = L / 2;
+    bool chord = true;
     for (int round = 0; round < 200; ++round) {
-        const double mid = 0.5 * (lo + hi);
-        const bool go = valid && !(hi - lo <= 2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)) + atol || mid == lo ||
-                                   mid == hi);
+        const double w = hi - lo, mid = lo + 0.5 * w;
+        const bool go = valid && !(w <= 2.0 * DBL_EPSILON * (tn + fmax(fabs(lo), fabs(hi))) || mid <= lo || mid >= hi);
         if (!__any_sync(0xffffffffu, go)) break;
-        const double x = lo + (hi - lo) * ((li + 1) * sect);
-        const bool le = go && sturm_count(n, d, e2, x, pivmin) <= i;
-        const int nle = group_le(le, gbase, L);
-        if (go) {
-            const double nlo = nle > 0 ? lo + (hi - lo) * (nle * sect) : lo;
-            const double nhi = nle < L ? lo + (hi - lo) * ((nle + 1) * sect) : hi;
-            lo = nlo;
-            hi = nhi;
+        double x = lo + w * ((li + 1) * sect);
+        const bool one = L >= 8 && chord && elo != kNone && ehi != kNone && clo == i && chi == i + 1;
+        if (one) {
+            // |f(hi) / f(lo)| in FP32: the chord's zero to 24 bits of the bracket
+            const int de = ehi - elo;
+            const float r = fabsf((float)fhi / (float)flo) * exp2f((float)min(max(de, -100), 100));
+            const double z = lo + w * (double)(1.f / (1.f + r));
+            const int k = li < H ? li + 1 : L - li;  // 1 .. H from the outside in
+            const double dl = w * (double)exp2f(-(float)(24 * k / H));
+            x = fmin(fmax(li < H ? z - dl : z + dl, lo), hi);
         }
+        narrow(x, go);
+        chord = !one || !(hi - lo > 0.25 * w);
     }
-    if (valid && li == 0) lam[i] = 0.5 * (lo + hi);
+    if (valid && li == 0) lam[i] = (lo + 0.5 * (hi - lo)) / bounds[3];
 }
 
 // uniform in [-1, 1) from a 64-bit hash (splitmix64 finaliser)
@@ -707,7 +783,8 @@ void launch_back_warp(cudaStream_t s, int warps, int n, int m, const double *Vh,
 
 void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, int ldx, double *work) {
     HSIM_CHECK_ARG(n >= 1 && m >= 1 && m <= n, "sym_eig: bad sizes");
-    double *d = work, *e = d + n, *tau = e + n, *p = tau + n, *e2 = p + n, *bounds = e2 + n;
+    // p is free once T stands: the scaled diagonal
+    double *d = work, *e = d + n, *tau = e + n, *p = tau + n, *ds = p, *e2 = p + n, *bounds = e2 + n;
     double *Vh = bounds + 8, *Z = Vh + (size_t)n * n, *lam = Z + (size_t)m * n, *lu = lam + m;
     unsigned char *pivf = reinterpret_cast<unsigned char *>(lu + (size_t)5 * n * m);
     int *cst = reinterpret_cast<int *>(reinterpret_cast<double *>(pivf) + ((size_t)n * m + 7) / 8);
@@ -763,7 +840,7 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
         HSIM_LAUNCHED();
     }
     // 2. eigenvalues
-    k_tri_prep<<<1, kTriThreads, 0, s>>>(n, d, e, e2, bounds, d32, e232);
+    k_tri_prep<<<1, kTriThreads, 0, s>>>(n, d, e, ds, e2, bounds, d32, e232);
     HSIM_LAUNCHED();
     if (detail) cudaEventRecord(t1, s);
     // about one warp per SM: G eigenvalues per warp (L = 32 / G >= 2 lanes each)
@@ -771,7 +848,7 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
     // sub-partitions (blocks of four warps, one per sub-partition)
     const int per_warp = std::max(1, std::min(16, (m + 4 * sms - 1) / (4 * sms)));
     const int nwarps = (m + per_warp - 1) / per_warp;
-    k_tri_bisect<<<(nwarps + 3) / 4, 128, 0, s>>>(n, m, per_warp, d, e2, d32, e232, bounds, lam);
+    k_tri_bisect<<<(nwarps + 3) / 4, 128, 0, s>>>(n, m, per_warp, ds, e2, d32, e232, bounds, lam);
     HSIM_LAUNCHED();
     if (detail) cudaEventRecord(t2, s);
     // 3. clusters on the host, then inverse iteration

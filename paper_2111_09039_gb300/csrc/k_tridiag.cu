@@ -15,10 +15,11 @@
 //   2. Eigenvalues of T by multisection on division-free Sturm counts, a group
 //      of lanes per index (ascending by construction): FP32 rounds, then FP64
 //      rounds around the zero of the determinant's chord.
-//   3. Eigenvectors of T by inverse iteration on T - lambda I (Gaussian
-//      elimination with partial pivoting, reciprocal pivots kept), three
-//      iterations from a hashed random start; eigenvalues closer than
-//      1e-5 ||T|| form a cluster whose vectors are made orthogonal to the
+//   3. Eigenvectors of T: a column of the adjugate of T - lambda I from the two
+//      Sturm sequences (k_tri_minors, k_tri_vectors).  Eigenvalues closer than
+//      1e-5 ||T|| form a cluster, whose vectors come from inverse iteration
+//      (Gaussian elimination with partial pivoting, reciprocal pivots kept),
+//      three iterations from a hashed random start, made orthogonal to the
 //      previous ones of the cluster in every iteration (one warp per cluster).
 //   4. Back transformation X = Q Z, reflectors applied in reverse order: one
 //      warp per eigenvector held in registers (n <= 2048), else a few
@@ -47,6 +48,7 @@ inline unsigned cdiv(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b);
 
 constexpr int kTriThreads = 256;
 constexpr double kClusterTol = 1e-5;  // relative to ||T||
+constexpr double kNearTol = 1e-4;     // the same, vectors made orthogonal once
 constexpr size_t kTriSmemMax = 200 * 1024;  // dynamic shared memory limit of k_tridiag and k_tri_back
 
 // sum over the block (256 threads); `red` holds 8 doubles; result in all threads
@@ -348,11 +350,14 @@ __global__ void __launch_bounds__(256) k_tri_back_warp(int n, int m, const doubl
 // T scaled by a power of two to a norm bound in [1/2, 1): ds, e2s = e^2 (at least
 // 2^-120 in FP64 and 2^-40 in FP32: couplings of 2^-60 and 2^-20 of ||T||, below
 // the accuracy of either count) and their FP32 copies; bounds: the Gershgorin
-// interval of the scaled T, ||T|| (not scaled), the scale
+// interval of the scaled T, ||T|| (not scaled), the scale; F_j for k_tri_vectors
 __global__ void k_tri_prep(int n, const double *__restrict__ d, const double *__restrict__ e, double *__restrict__ ds,
                            double *__restrict__ e2s, double *__restrict__ bounds, float *__restrict__ d32,
-                           float *__restrict__ e232) {
+                           float *__restrict__ e232, double *__restrict__ fm, double *__restrict__ fi,
+                           int *__restrict__ fx) {
     __shared__ double red[3][kTriThreads / 32];
+    __shared__ double sm[2][kTriThreads];
+    __shared__ int sx[2][kTriThreads];
     double lo = DBL_MAX, hi = -DBL_MAX, nm = 0.0;
     for (int j = threadIdx.x; j < n; j += kTriThreads) {
         const double r = (j > 0 ? fabs(e[j - 1]) : 0.0) + (j + 1 < n ? fabs(e[j]) : 0.0);
@@ -388,6 +393,48 @@ __global__ void k_tri_prep(int n, const double *__restrict__ d, const double *__
             e2s[j] = fmax(q, 0x1p-120);
             e232[j] = fmaxf((float)q, 0x1p-40f);
         }
+    }
+    // F_j = prod_{i < j} (-e_i) of the scaled T as fm 2^fx (fi = 1 / fm): every
+    // thread a run of factors, then a scan over the runs
+    const int run = (n + kTriThreads - 1) / kTriThreads, j0 = min(n, (int)threadIdx.x * run), j1 = min(n, j0 + run);
+    auto norm = [](double &m, int &x) {
+        const int h = __double2hiint(m), q = ((h >> 20) & 0x7FF) - 1023;
+        m = __hiloint2double(h - q * 0x100000, __double2loint(m));
+        x += q;
+    };
+    auto factor = [&](int i) {
+        const double es = i + 1 < n ? e[i] * sc : 1.0;
+        return -copysign(fmax(fabs(es), 0x1p-60), es);
+    };
+    double pm = 1.0;
+    int px = 0;
+    for (int i = j0; i < j1; ++i) {
+        pm *= factor(i);
+        norm(pm, px);
+    }
+    int cur = 0;
+    sm[0][threadIdx.x] = pm;
+    sx[0][threadIdx.x] = px;
+    __syncthreads();
+    for (int o = 1; o < kTriThreads; o <<= 1) {
+        if ((int)threadIdx.x >= o) {
+            pm *= sm[cur][threadIdx.x - o];
+            px += sx[cur][threadIdx.x - o];
+            norm(pm, px);
+        }
+        cur ^= 1;
+        sm[cur][threadIdx.x] = pm;
+        sx[cur][threadIdx.x] = px;
+        __syncthreads();
+    }
+    pm = threadIdx.x > 0 ? sm[cur][threadIdx.x - 1] : 1.0;
+    px = threadIdx.x > 0 ? sx[cur][threadIdx.x - 1] : 0;
+    for (int i = j0; i < j1; ++i) {
+        fm[i] = pm;
+        fi[i] = 1.0 / pm;
+        fx[i] = px;
+        pm *= factor(i);
+        norm(pm, px);
     }
     if (threadIdx.x == 0) {
         const double pad = 4.0 * DBL_EPSILON;
@@ -597,14 +644,134 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// inverse iteration, one warp per cluster [cstart[c], cstart[c + 1]); Z is m x n
+// Eigenvectors of T for single eigenvalues: column k of the adjugate of T -
+// lambda I,
+//     z_j = P_j prod_{i=j}^{k-1} (-e_i) B_{k+1}  (j <= k),
+//     z_j = P_k prod_{i=k}^{j-1} (-e_i) B_{j+1}  (j > k),
+// P_j and B_j the determinants of the leading j rows and of the rows from j on,
+// k where |P_k B_{k+1}| is largest (the diagonal of the adjugate goes with the
+// squares of the vector's entries; the twisted factorisation of Dhillon and
+// Parlett in product form).  One vector of inverse iteration with LU cost two
+// dependent divisions a step and three solves, one lane at work (1.32 ms for 750
+// vectors); here the two sequences run without divisions, sixteen vectors to a
+// warp (forward in the lower lanes, backward in the upper: an FP64 instruction
+// of a warp takes the same 77 clocks for one lane as for 32), 0.1 ms.
+//
+// k_tri_minors: S_t = P_t (dir 0) and B_{n-t} (dir 1), t < n, as seq[dir][t][i]
+// 2^xs[dir][t / 8][i]
+__global__ void __launch_bounds__(32) k_tri_minors(int n, int m, const double *__restrict__ d, const double *__restrict__ e2,
+                                                   const double *__restrict__ bounds, const double *__restrict__ lam,
+                                                   double *__restrict__ seq, int *__restrict__ xs) {
+    const int lane = threadIdx.x, i = blockIdx.x * 16 + (lane & 15), dir = lane >> 4;
+    if (i >= m) return;
+    const double x = lam[i] * bounds[3];
+    double *out = seq + (size_t)dir * n * m + i;
+    int *ox = xs + (size_t)dir * ((n + 7) / 8) * m + i;
+    // step t: row t forward, n - 1 - t backward, coupled by e2[t - 1] or e2[n - 1 - t]
+    const double *dp = dir ? d + (n - 1) : d;
+    const double *ep = dir ? e2 + (n - 1) : e2 - 1;
+    const int sg = dir ? -1 : 1;
+    double p0 = 0.0, p1 = 1.0;  // S_{t-1}, S_t
+    int E = 0;
+    for (int t = 0; t < n; t += 8) {
+        ox[(size_t)(t >> 3) * m] = E;
+        const int cnt = min(8, n - t);
+        double dj[8], ej[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            dj[u] = u < cnt ? dp[sg * (t + u)] : 0.0;
+            ej[u] = u < cnt && t + u > 0 ? ep[sg * (t + u)] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (u >= cnt) break;
+            out[(size_t)(t + u) * m] = p1;
+            const double p2 = fma(dj[u] - x, p1, -(ej[u] * p0));
+            p0 = p1;
+            p1 = p2;
+        }
+        const int e0 = (__double2hiint(p0) >> 20) & 0x7FF, e1 = (__double2hiint(p1) >> 20) & 0x7FF;
+        const int sh = max(e0, e1) - 1023;
+        p0 = e0 > sh ? __hiloint2double(__double2hiint(p0) - sh * 0x100000, __double2loint(p0)) : 0.0;
+        p1 = e1 > sh ? __hiloint2double(__double2hiint(p1) - sh * 0x100000, __double2loint(p1)) : 0.0;
+        E += sh;
+    }
+}
+
+// x 2^e, 0 below the normal range (entries 2^-1000 of the largest)
+__device__ __forceinline__ double shift_exp(double x, int e) {
+    const int h = __double2hiint(x), q = ((h >> 20) & 0x7FF) + e;
+    return q > 0 && (h & 0x7FF00000) != 0 ? __hiloint2double(h + min(e, 4000) * 0x100000, __double2loint(x)) : 0.0;
+}
+
+// z for 8 vectors per CTA, thread (vector tid % 8, rows tid / 8, + 32, ...)
+__global__ void __launch_bounds__(256) k_tri_vectors(int n, int m, const double *__restrict__ seq,
+                                                     const int *__restrict__ xs, const double *__restrict__ fm,
+                                                     const double *__restrict__ fi, const int *__restrict__ fx,
+                                                     double *__restrict__ Z) {
+    __shared__ float key[32][8];
+    __shared__ int row[32][8];
+    __shared__ double part[32][8];
+    const int v = threadIdx.x & 7, r = threadIdx.x >> 3, i = blockIdx.x * 8 + v, nb = (n + 7) / 8;
+    const bool ok = i < m;
+    const double *P = seq + i, *B = seq + (size_t)n * m + i;
+    const int *xP = xs + i, *xB = xs + (size_t)nb * m + i;
+    // S^b_{n-1-j} = B_{j+1}
+    auto lg = [](double x) {
+        const int h = __double2hiint(x) & 0x7FFFFFFF;
+        return h < 0x00100000 ? -3e38f : (float)((h >> 20) - 1023) + __log2f(__int_as_float(0x3F800000 | ((h & 0xFFFFF) << 3)));
+    };
+    float best = -3.4e38f;
+    int k = 0;
+    if (ok)
+        for (int j = r; j < n; j += 32) {
+            const int tb = n - 1 - j;
+            const float q = lg(P[(size_t)j * m]) + lg(B[(size_t)tb * m]) + (float)(xP[(size_t)(j >> 3) * m] + xB[(size_t)(tb >> 3) * m]);
+            if (q > best) best = q, k = j;
+        }
+    key[r][v] = best;
+    row[r][v] = k;
+    __syncthreads();
+    for (int q = 0; q < 32; ++q)
+        if (key[q][v] > best || (key[q][v] == best && row[q][v] < k)) best = key[q][v], k = row[q][v];
+    double c1 = 0.0, c2 = 0.0;
+    int s1 = 0, s2 = 0;
+    if (ok) {
+        const int tb = n - 1 - k;
+        c1 = fm[k] / P[(size_t)k * m];
+        c2 = fi[k] / B[(size_t)tb * m];
+        s1 = fx[k] - xP[(size_t)(k >> 3) * m];
+        s2 = -fx[k] - xB[(size_t)(tb >> 3) * m];
+    }
+    auto entry = [&](int j) {
+        if (j <= k) return shift_exp(P[(size_t)j * m] * fi[j] * c1, xP[(size_t)(j >> 3) * m] - fx[j] + s1);
+        const int tb = n - 1 - j;
+        return shift_exp(B[(size_t)tb * m] * fm[j] * c2, xB[(size_t)(tb >> 3) * m] + fx[j] + s2);
+    };
+    double sum = 0.0;
+    if (ok)
+        for (int j = r; j < n; j += 32) {
+            const double z = entry(j);
+            sum = fma(z, z, sum);
+        }
+    part[r][v] = sum;
+    __syncthreads();
+    sum = 0.0;
+#pragma unroll
+    for (int q = 0; q < 32; ++q) sum += part[q][v];
+    const double inv = rsqrt(sum);
+    if (ok)
+        for (int j = r; j < n; j += 32) Z[(size_t)i * n + j] = entry(j) * inv;
+}
+
+// Clusters: inverse iteration, one warp per cluster [cl[2 c], cl[2 c + 1]); Z is m x n
 // (vector-major); LU scratch: 5 n doubles + n flags per cluster
 __global__ void k_tri_invit(int n, const double *__restrict__ d, const double *__restrict__ e,
                             const double *__restrict__ bounds, const double *__restrict__ lam,
-                            const int *__restrict__ cstart, double *__restrict__ Z, double *__restrict__ scratch,
+                            const int *__restrict__ cl, double *__restrict__ Z, double *__restrict__ scratch,
                             unsigned char *__restrict__ pivflag) {
     const int c = blockIdx.x, lane = threadIdx.x;
-    const int i0 = cstart[c], i1 = cstart[c + 1];
+    const int i0 = cl[2 * c], i1 = cl[2 * c + 1];
     double *u0i = scratch + (size_t)c * 5 * n;  // reciprocal of the pivot
     double *u1 = u0i + n, *u2 = u1 + n, *l = u2 + n, *y = l + n;
     unsigned char *piv = pivflag + (size_t)c * n;
@@ -685,6 +852,28 @@ __global__ void k_tri_invit(int n, const double *__restrict__ d, const double *_
     }
 }
 
+// Vectors of eigenvalues closer than kNearTol ||T||, made orthogonal in
+// ascending order (one warp per chain of such neighbours).  The vector of an
+// eigenvalue known to eps ||T|| carries about eps ||T|| / gap of its neighbour:
+// 1e-11 at the gap of a cluster, 4e-12 where this ends.
+__global__ void __launch_bounds__(32) k_tri_orth(int n, int m, const double *__restrict__ bounds,
+                                                 const double *__restrict__ lam, double *__restrict__ Z) {
+    const int i0 = blockIdx.x, lane = threadIdx.x;
+    const double tol = kNearTol * bounds[2];
+    if (i0 > 0 && lam[i0] - lam[i0 - 1] <= tol) return;  // not the first of its chain
+    for (int i = i0 + 1; i < m && lam[i] - lam[i - 1] <= tol; ++i) {
+        double *z = Z + (size_t)i * n;
+        for (int jv = i - 1; jv >= i0 && lam[i] - lam[jv] <= tol; --jv) {
+            const double *o = Z + (size_t)jv * n;
+            double s = 0.0;
+            for (int j = lane; j < n; j += 32) s = fma(o[j], z[j], s);
+            s = warp_sum(s);
+            for (int j = lane; j < n; j += 32) z[j] = fma(-s, o[j], z[j]);
+            __syncwarp();
+        }
+    }
+}
+
 // X[:, i] = Q z_i for i in this CTA's group; vectors kept in shared memory
 __global__ void __launch_bounds__(kTriThreads) k_tri_back(int n, int m, int per_cta, const double *__restrict__ Vh,
                                                         const double *__restrict__ tau, const double *__restrict__ Z,
@@ -740,10 +929,10 @@ __global__ void __launch_bounds__(kTriThreads) k_tri_back(int n, int m, int per_
 }  // namespace
 
 size_t sym_eig_work_size(int n, int m) {
-    // d e tau p e2 bounds(8) | Vh n^2 | Z m n | lam m | LU 5 n m | pivots n m bytes | cluster starts m + 1 ints
-    // | d, e^2 in FP32 (n each)
+    // d e tau p e2 bounds(8) | Vh n^2 | Z m n | lam m | LU 5 n m (the minors' sequences before) | pivots n m bytes |
+    // clusters m + 1 ints | d, e^2 in FP32 (n each) | F, 1 / F, its exponents
     return (size_t)5 * n + 8 + (size_t)n * n + (size_t)m * n + m + (size_t)5 * n * m + ((size_t)n * m + 7) / 8 +
-           ((size_t)m + 2) / 2 + 16 + (size_t)n + 8 + (size_t)4 * n + 8;
+           ((size_t)m + 2) / 2 + 16 + (size_t)n + 8 + (size_t)4 * n + 8 + (size_t)3 * n + 8;
 }
 
 namespace {
@@ -791,6 +980,10 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
     float *d32 = reinterpret_cast<float *>(reinterpret_cast<double *>(cst) + ((size_t)m + 2) / 2 + 8);
     float *e232 = d32 + n;
     double *pbuf = reinterpret_cast<double *>(e232 + n) + 4, *rbuf = pbuf + 2 * (size_t)n;
+    double *fm = rbuf + 2 * (size_t)n, *fi = fm + n;
+    int *fx = reinterpret_cast<int *>(fi + n);
+    // sequences of k_tri_minors: 2 n m doubles, 2 ceil(n / 8) m exponents
+    int *xs = reinterpret_cast<int *>(lu + (size_t)2 * n * m);
     if (n == 1) {
         HSIM_CUDA(cudaMemcpyAsync(evals, A, sizeof(double), cudaMemcpyDeviceToDevice, s));
         const double one = 1.0;
@@ -840,7 +1033,7 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
         HSIM_LAUNCHED();
     }
     // 2. eigenvalues
-    k_tri_prep<<<1, kTriThreads, 0, s>>>(n, d, e, ds, e2, bounds, d32, e232);
+    k_tri_prep<<<1, kTriThreads, 0, s>>>(n, d, e, ds, e2, bounds, d32, e232, fm, fi, fx);
     HSIM_LAUNCHED();
     if (detail) cudaEventRecord(t1, s);
     // about one warp per SM: G eigenvalues per warp (L = 32 / G >= 2 lanes each)
@@ -851,19 +1044,36 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
     k_tri_bisect<<<(nwarps + 3) / 4, 128, 0, s>>>(n, m, per_warp, ds, e2, d32, e232, bounds, lam);
     HSIM_LAUNCHED();
     if (detail) cudaEventRecord(t2, s);
-    // 3. clusters on the host, then inverse iteration
+    // 3. vectors of single eigenvalues on the device; clusters, found on the
+    // host meanwhile, by inverse iteration
+    k_tri_minors<<<cdiv(m, 16), 32, 0, s>>>(n, m, ds, e2, bounds, lam, lu, xs);
+    HSIM_LAUNCHED();
+    k_tri_vectors<<<cdiv(m, 8), 256, 0, s>>>(n, m, lu, xs, fm, fi, fx, Z);
+    HSIM_LAUNCHED();
     std::vector<double> hl(m), hb(4);
     HSIM_CUDA(cudaMemcpyAsync(hl.data(), lam, m * sizeof(double), cudaMemcpyDeviceToHost, s));
     HSIM_CUDA(cudaMemcpyAsync(hb.data(), bounds, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
     HSIM_CUDA(cudaStreamSynchronize(s));
-    std::vector<int> starts{0};
-    for (int i = 1; i < m; ++i)
-        if (hl[i] - hl[i - 1] > kClusterTol * hb[2]) starts.push_back(i);
-    starts.push_back(m);
-    const int nclusters = (int)starts.size() - 1;
-    HSIM_CUDA(cudaMemcpyAsync(cst, starts.data(), starts.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+    std::vector<int> clusters;  // first, end of every cluster of two and more
+    int biggest = 1;
+    for (int i = 0; i < m;) {
+        int j = i + 1;
+        while (j < m && !(hl[j] - hl[j - 1] > kClusterTol * hb[2])) ++j;
+        if (j - i > 1) {
+            clusters.push_back(i);
+            clusters.push_back(j);
+            biggest = std::max(biggest, j - i);
+        }
+        i = j;
+    }
+    const int nclusters = (int)clusters.size() / 2;
     if (detail) cudaEventRecord(t2, s);
-    k_tri_invit<<<nclusters, 32, 0, s>>>(n, d, e, bounds, lam, cst, Z, lu, pivf);
+    if (nclusters > 0) {
+        HSIM_CUDA(cudaMemcpyAsync(cst, clusters.data(), clusters.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+        k_tri_invit<<<nclusters, 32, 0, s>>>(n, d, e, bounds, lam, cst, Z, lu, pivf);
+        HSIM_LAUNCHED();
+    }
+    k_tri_orth<<<m, 32, 0, s>>>(n, m, bounds, lam, Z);
     HSIM_LAUNCHED();
     if (detail) cudaEventRecord(t3, s);
     // 4. back transformation: a warp per vector held in registers where n <=
@@ -885,8 +1095,8 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
         HSIM_LAUNCHED();
     }
     HSIM_CUDA(cudaMemcpyAsync(evals, lam, m * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    // the host vector `starts` must outlive the copy above
-    HSIM_CUDA(cudaStreamSynchronize(s));
+    // the host vector `clusters` must outlive its copy
+    if (nclusters > 0) HSIM_CUDA(cudaStreamSynchronize(s));
     if (detail) {
         cudaEventRecord(t4, s);
         cudaEventSynchronize(t4);
@@ -895,8 +1105,6 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
         cudaEventElapsedTime(&b, t1, t2);
         cudaEventElapsedTime(&c, t2, t3);
         cudaEventElapsedTime(&dd, t3, t4);
-        int biggest = 0;
-        for (size_t i = 0; i + 1 < starts.size(); ++i) biggest = std::max(biggest, starts[i + 1] - starts[i]);
         std::fprintf(stderr,
                      "[hsim] sym_eig n=%d m=%d tridiag %.2f ms eigenvalues %.2f ms vectors %.2f ms (%d clusters, "
                      "largest %d) back %.2f ms\n",

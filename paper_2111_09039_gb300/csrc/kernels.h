@@ -122,7 +122,7 @@ int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar,
 // ---- tridiagonal eigensolver (k_tridiag.cu) ----------------------------------
 // lowest m eigenpairs of the symmetric n x n A (row-major, ld n, destroyed):
 // evals ascending (m), X (n x m, ld ldx) orthonormal eigenvectors; work of
-// sym_eig_work_size(n, m) doubles; synchronises the stream
+// sym_eig_work_size(n, m) doubles; waits for the stream in between
 size_t sym_eig_work_size(int n, int m);
 void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, int ldx, double *work);
 size_t ritz_work_size(int k);

@@ -137,63 +137,121 @@ __global__ void __launch_bounds__(kTriThreads) k_tridiag(int n, double *__restri
 // warp on a sub-partition; with one warp each that cost is paid once.
 constexpr int kTrdThreads = 128;
 
+// Sum over the warp in fixed point: every value as a 57-bit integer against the
+// warp's largest exponent, three limbs added by redux, the total rounded once.
+// An FP64 add of a warp costs 77 issue clocks and 106 through a shuffle, five of
+// them 530; this takes about 200, and the values' truncation (2^-57 of the
+// largest) stays below the rounding of the FP64 tree.
+__device__ __forceinline__ double warp_sum_fixed(double v) {
+    const int h = __double2hiint(v), e = (h >> 20) & 0x7FF;
+    const int em = __reduce_max_sync(0xffffffffu, e);
+    if (em == 0x7FF) {  // infinities and NaN
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    }
+    const unsigned long long M =
+        ((unsigned long long)((unsigned)(h & 0xFFFFF) | (e ? 0x100000u : 0u)) << 32) | (unsigned)__double2loint(v);
+    long long T = (long long)((M << 4) >> min(em - e, 63));
+    if (h < 0) T = -T;
+    const unsigned s0 = __reduce_add_sync(0xffffffffu, (unsigned)T & 0x3FFFFFu);
+    const unsigned s1 = __reduce_add_sync(0xffffffffu, (unsigned)(T >> 22) & 0x3FFFFFu);
+    const int s2 = (int)__reduce_add_sync(0xffffffffu, (unsigned)(int)(T >> 44));
+    const double t = (double)(((long long)s2 << 44) + ((long long)s1 << 22) + (long long)s0);
+    // 2^(max(em, 1) - 1075 - 4), in two exact steps near the ends of the range
+    const int q = max(em, 1) - 1079, th = __double2hiint(t);
+    const int te = ((th >> 20) & 0x7FF) + q;
+    if (t == 0.0) return 0.0;
+    return te > 0 && te < 0x7FF ? __hiloint2double(th + q * 0x100000, __double2loint(t)) : ldexp(t, q);
+}
+
 // sum over the block (kTrdThreads threads); result in all threads
 __device__ __forceinline__ double block_sum128(double v, double *red) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    v = warp_sum_fixed(v);
     __syncthreads();  // red may still be read from the previous call
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
     return (red[0] + red[1]) + (red[2] + red[3]);
 }
 
-// Sums over the 32 lanes of RMAX values per lane by halving: at the step with
-// offset o every lane keeps the half of its values selected by its lane bit o
-// and adds the partner's copy of that half, so the adds per lane are RMAX - 1
-// plus log2(32 / RMAX) instead of 5 RMAX.  Afterwards lane l holds the total
-// of value l / (32 / RMAX).
-template <int RMAX>
-__device__ __forceinline__ double warp_sum_rows(double (&a)[RMAX], int lane) {
-    int off = 16;
-#pragma unroll
-    for (int h = RMAX / 2; h >= 1; h /= 2) {
-        const bool up = (lane & off) != 0;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const double keep = up ? a[i + h] : a[i];
-            const double send = up ? a[i] : a[i + h];
-            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+// 1 / sqrt(x) and 1 / x of normal numbers from the 20-bit seeds by one
+// third-order step (error of the seed cubed, 2^-60)
+__device__ __forceinline__ double rsqrt_step(double x) {
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-(x * r), r, 1.0);
+    return fma(r * e, fma(e, 0.375, 0.5), r);
+}
+__device__ __forceinline__ double rcp_step(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
+// Grid barrier: every CTA adds to a counter that starts at zero; `target`
+// arrivals complete it.  The waiting gives up after two seconds (false, *err
+// set); the CTAs that then leave let the others run into the same limit.
+__device__ __forceinline__ bool grid_barrier(unsigned *counter, unsigned target, double *err) {
+    int ok = 1;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
+        unsigned long long t0 = 0;
+        for (unsigned it = 0;; ++it) {
+            unsigned c;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(counter) : "memory");
+            if (c >= target) break;
+            if ((it & 1023u) == 1023u) {
+                unsigned long long t;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+                if (t0 == 0) t0 = t;
+                else if (t - t0 > 2000000000ull) {
+                    *err = 1.0;
+                    ok = 0;
+                    break;
+                }
+            }
         }
-        off >>= 1;
     }
-    double s = a[0];
-    for (; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    return s;
+    return __syncthreads_and(ok) != 0;
 }
 
 // Tridiagonalisation with the matrix resident in shared memory.  CTA b owns
-// the rows b, b + G, b + 2G, ... (full length n), so the product p = t A22 v
+// the rows b, b + G, b + 2G, ... (full length n), so the product p = t A22 u
 // and the rank-2 update of every column read and write only shared memory,
 // and one grid barrier per column suffices: before it every CTA writes its
 // entries of p, and the owner of row k+1 writes that row as it stands before
-// the update of column k; after it every CTA forms w and, from that row, the
+// the update of column k; after it every CTA forms, from that row, the
 // updated row k+1, which by symmetry is the next column to reduce.  The update
 // of column k is applied to the owned rows in the same pass as the product of
-// column k+1.  The arithmetic per column is that of k_tridiag.
+// column k+1.
+//
+// The reflector is I - t u u^T with u the column itself but for its first
+// entry (u_0 = x_0 - beta, t = -1 / (beta u_0)): nothing is scaled.  With w = p -
+// (t/2)(p.u) u the update of row r is -(u_r w + w_r u) = -(u_r p + b_r u), b_r =
+// p_r - t (p.u) u_r: w is not formed.  An entry costs three FP64 instructions.
+// What bounds it (n = 750 on 152 SMs: 7.4 us per column, 8.1 with scaled
+// reflectors, w formed, FP64 shuffles for the sums and divisions): the barrier
+// and the loads behind it about 3,000 clocks, FP64 issue (77 clocks per warp
+// instruction: 2.5 rows x 3 x 3 on average, and the vectors that every CTA
+// repeats), two block sums and the scalars in a dependent chain.  Entries tagged
+// with their column and polled for by every thread, instead of the barrier, took
+// 8,000 clocks per column at n = 750 (the polling loads themselves).
 // Shared memory: R n (owned rows, R = ceil(n / G) <= RMAX) + 4 n doubles.
 template <int RMAX>
 __global__ void __launch_bounds__(kTrdThreads) k_tridiag_rows(int n, const double *__restrict__ A, double *__restrict__ d,
                                                             double *__restrict__ e, double *__restrict__ tau,
                                                             double *__restrict__ Vh, double *__restrict__ pbuf,
-                                                            double *__restrict__ rbuf) {
+                                                            double *__restrict__ rbuf, unsigned *__restrict__ counter,
+                                                            double *__restrict__ err) {
     constexpr int NW = kTrdThreads / 32;
-    cg::grid_group grid = cg::this_grid();
     extern __shared__ double sm[];
     const int G = gridDim.x, b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int R = (n - b + G - 1) / G;          // rows owned by this CTA
     const int Rmax = (n + G - 1) / G;
     double *rows = sm;                           // Rmax x n
     double *xs = rows + (size_t)Rmax * n;        // row k: xs[i] = A[k, k + i]
-    double *v = xs + n, *vp = v + n, *w = vp + n;  // reflector of column k, of column k - 1; w of column k - 1
+    double *u = xs + n, *up = u + n, *p = up + n;  // reflector of column k, of column k - 1; p of column k - 1
     __shared__ double red[NW];
     __shared__ double redr[NW][RMAX];
     for (int i = 0; i < R; ++i) {
@@ -201,6 +259,7 @@ __global__ void __launch_bounds__(kTrdThreads) k_tridiag_rows(int n, const doubl
         for (int j = tid; j < n; j += kTrdThreads) rows[(size_t)i * n + j] = src[j];
     }
     for (int j = tid; j < n; j += kTrdThreads) xs[j] = A[j];
+    double tpu = 0.0;  // t (p.u) of column k - 1
     __syncthreads();
     for (int k = 0; k + 1 < n; ++k) {
         const int L = n - k - 1;
@@ -209,19 +268,26 @@ __global__ void __launch_bounds__(kTrdThreads) k_tridiag_rows(int n, const doubl
         for (int i = 1 + tid; i < L; i += kTrdThreads) part = fma(xs[1 + i], xs[1 + i], part);
         const double sigma = block_sum128(part, red);
         const double x0 = xs[1];
-        double beta = x0, t = 0.0, scale = 0.0;
+        double beta = x0, t = 0.0, u0 = 1.0;
         if (sigma != 0.0) {
-            const double mu = sqrt(fma(x0, x0, sigma));
-            beta = x0 >= 0.0 ? -mu : mu;
-            // t = (beta - x0) / beta and scale = 1 / (x0 - beta) from one division
-            const double dlt = x0 - beta, inv = 1.0 / (beta * dlt);
-            t = -dlt * dlt * inv;
-            scale = beta * inv;
+            const double s2 = fma(x0, x0, sigma);
+            if (s2 > 1e-280 && s2 < 1e280) {
+                const double r = rsqrt_step(s2), m0 = s2 * r;
+                const double mu = fma(fma(-m0, m0, s2), 0.5 * r, m0);
+                beta = x0 >= 0.0 ? -mu : mu;
+                u0 = x0 - beta;
+                t = rcp_step(-beta * u0);
+            } else {
+                const double mu = sqrt(s2);
+                beta = x0 >= 0.0 ? -mu : mu;
+                u0 = x0 - beta;
+                t = -1.0 / (beta * u0);
+            }
         }
         for (int i = tid; i < L; i += kTrdThreads) {
-            const double vi = i == 0 ? 1.0 : xs[1 + i] * scale;
-            v[i] = vi;
-            if (b == 0) Vh[(size_t)k * n + k + 1 + i] = vi;
+            const double ui = i == 0 ? u0 : xs[1 + i];
+            u[i] = ui;
+            if (b == 0) Vh[(size_t)k * n + k + 1 + i] = ui;
         }
         if (b == 0 && tid == 0) {
             d[k] = xs[0];
@@ -229,55 +295,63 @@ __global__ void __launch_bounds__(kTrdThreads) k_tridiag_rows(int n, const doubl
             tau[k] = t;
         }
         __syncthreads();
-        // owned rows r >= k + 1: update of column k - 1 (vectors vp, w, index
-        // 0 <-> row k) on columns >= k + 1, then the product with v
+        // owned rows r >= k + 1: update of column k - 1 (vectors up, p, index
+        // 0 <-> row k) on columns >= k + 1, then the product with u
         const int i0 = k + 1 > b ? (k + 1 - b + G - 1) / G : 0;
-        double acc[RMAX];
+        double acc[RMAX], ca[RMAX], cb[RMAX];
 #pragma unroll
-        for (int i = 0; i < RMAX; ++i) acc[i] = 0.0;
+        for (int i = 0; i < RMAX; ++i) {
+            acc[i] = ca[i] = cb[i] = 0.0;
+            if (k == 0 || i < i0 || i >= R) continue;
+            const int r = b + i * G - k;
+            ca[i] = -up[r];
+            cb[i] = fma(tpu, up[r], -p[r]);
+        }
         double *rb = rbuf + (size_t)(k & 1) * n;
+        const int ir = (k + 1) % G == b ? (k + 1) / G : -1;  // this CTA's index of row k + 1
         for (int j = tid; j < L; j += kTrdThreads) {
-            const double vj = v[j];
-            const double vpj = k > 0 ? vp[j + 1] : 0.0, wpj = k > 0 ? w[j + 1] : 0.0;
+            const double uj = u[j];
+            const double upj = k > 0 ? up[j + 1] : 0.0, pj = k > 0 ? p[j + 1] : 0.0;
 #pragma unroll
             for (int i = 0; i < RMAX; ++i) {
                 if (i < i0 || i >= R) continue;
-                const int r = b + i * G;
                 double *a = rows + (size_t)i * n + k + 1 + j;
                 double x = *a;
-                if (k > 0) x -= vp[r - k] * wpj + w[r - k] * vpj;
-                *a = x;
-                acc[i] = fma(x, vj, acc[i]);
-                if (r == k + 1) rb[j] = x;
+                if (k > 0) {
+                    x = fma(cb[i], upj, fma(ca[i], pj, x));
+                    *a = x;
+                }
+                acc[i] = fma(x, uj, acc[i]);
+                if (i == ir) rb[j] = x;
             }
         }
-        const double rs = warp_sum_rows<RMAX>(acc, lane);
-        if ((lane & (32 / RMAX - 1)) == 0) redr[wid][lane / (32 / RMAX)] = rs;
-        __syncthreads();
-        if (tid >= i0 && tid < R) {
-            double s = 0.0;
 #pragma unroll
-            for (int q = 0; q < NW; ++q) s += redr[q][tid];
-            pbuf[(size_t)(k & 1) * n + (b + tid * G - k - 1)] = t * s;
+        for (int i = 0; i < RMAX; ++i) {
+            if (i < i0 || i >= R) continue;
+            const double rs = warp_sum_fixed(acc[i]);
+            if (lane == 0) redr[wid][i] = rs;
         }
-        grid.sync();
-        // w = p - (t/2)(p.v) v, then row k + 1 after the update of column k
+        __syncthreads();
+        if (tid >= i0 && tid < R)
+            pbuf[(size_t)(k & 1) * n + (b + tid * G - k - 1)] =
+                t * ((redr[0][tid] + redr[1][tid]) + (redr[2][tid] + redr[3][tid]));
+        if (!grid_barrier(counter, (unsigned)(k + 1) * (unsigned)G, err)) return;
+        // row k + 1 after the update of column k
         const double *pb = pbuf + (size_t)(k & 1) * n;
-        double pv = 0.0;
+        double pu = 0.0;
+#pragma unroll 4
         for (int j = tid; j < L; j += kTrdThreads) {
             const double pj = __ldcg(pb + j);
             xs[j] = __ldcg(rb + j);
-            w[j] = pj;
-            pv = fma(pj, v[j], pv);
+            p[j] = pj;
+            pu = fma(pj, u[j], pu);
         }
-        const double K = 0.5 * t * block_sum128(pv, red);
-        for (int j = tid; j < L; j += kTrdThreads) w[j] -= K * v[j];
-        __syncthreads();
-        const double w0 = w[0];
-        for (int j = tid; j < L; j += kTrdThreads) xs[j] -= v[0] * w[j] + w0 * v[j];
-        double *tmp = vp;
-        vp = v;
-        v = tmp;
+        tpu = t * block_sum128(pu, red);
+        const double b0 = fma(-tpu, u0, p[0]);
+        for (int j = tid; j < L; j += kTrdThreads) xs[j] = fma(-b0, u[j], fma(-u0, p[j], xs[j]));
+        double *tmp = up;
+        up = u;
+        u = tmp;
         __syncthreads();
     }
     if (b == 0 && tid == 0) {
@@ -949,13 +1023,13 @@ int rows_grid(int n, int sms, size_t *smem, int *rmax) {
 
 template <int RMAX>
 bool launch_tridiag_rows(cudaStream_t s, int G, size_t smem, int sms, int n, const double *A, double *d, double *e,
-                         double *tau, double *Vh, double *pbuf, double *rbuf) {
+                         double *tau, double *Vh, double *pbuf, double *rbuf, unsigned *counter, double *err) {
     HSIM_SMEM_LIMIT_ONCE(k_tridiag_rows<RMAX>, kTriSmemMax);
     int per_sm = 0;
     HSIM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag_rows<RMAX>, kTrdThreads, smem));
     if ((int64_t)per_sm * sms < G) return false;
     int nn = n;
-    void *args[] = {&nn, &A, &d, &e, &tau, &Vh, &pbuf, &rbuf};
+    void *args[] = {&nn, &A, &d, &e, &tau, &Vh, &pbuf, &rbuf, &counter, &err};
     HSIM_CUDA(cudaLaunchCooperativeKernel((void *)k_tridiag_rows<RMAX>, dim3(G), dim3(kTrdThreads), args, smem, s));
     HSIM_LAUNCHED();
     return true;
@@ -1014,10 +1088,13 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
     int rmax = 0;
     const int G = rows_grid(n, sms, &rsmem, &rmax);
     bool done = false;
+    double *err = bounds + 4;                                       // set if a barrier gave up
+    unsigned *counter = reinterpret_cast<unsigned *>(bounds + 5);  // arrivals of the barriers
+    HSIM_CUDA(cudaMemsetAsync(err, 0, 2 * sizeof(double), s));
     if (G > 0) {
-        if (rmax == 4) done = launch_tridiag_rows<4>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf);
-        else if (rmax == 8) done = launch_tridiag_rows<8>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf);
-        else done = launch_tridiag_rows<16>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf);
+        if (rmax == 4) done = launch_tridiag_rows<4>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf, counter, err);
+        else if (rmax == 8) done = launch_tridiag_rows<8>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf, counter, err);
+        else done = launch_tridiag_rows<16>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf, counter, err);
     }
     if (!done) {
         const size_t smem = 2 * (size_t)n * sizeof(double);
@@ -1050,10 +1127,11 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
     HSIM_LAUNCHED();
     k_tri_vectors<<<cdiv(m, 8), 256, 0, s>>>(n, m, lu, xs, fm, fi, fx, Z);
     HSIM_LAUNCHED();
-    std::vector<double> hl(m), hb(4);
+    std::vector<double> hl(m), hb(5);
     HSIM_CUDA(cudaMemcpyAsync(hl.data(), lam, m * sizeof(double), cudaMemcpyDeviceToHost, s));
-    HSIM_CUDA(cudaMemcpyAsync(hb.data(), bounds, 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
+    HSIM_CUDA(cudaMemcpyAsync(hb.data(), bounds, 5 * sizeof(double), cudaMemcpyDeviceToHost, s));
     HSIM_CUDA(cudaStreamSynchronize(s));
+    if (hb[4] != 0.0) fail(HSIM_E_TIMEOUT, "sym_eig: a grid barrier of the tridiagonalisation gave up");
     std::vector<int> clusters;  // first, end of every cluster of two and more
     int biggest = 1;
     for (int i = 0; i < m;) {

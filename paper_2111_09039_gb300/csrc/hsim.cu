@@ -1712,7 +1712,8 @@ hsim_status hsim_eig_grad(hsim_ctx *ctx, int n, int m, const double *V, const in
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"V", V}, {"F", F}, {"evals", evals}, {"evecs", evecs}, {"dloss", dloss},
                                         {"dV", dV}});
-        k::eig_grad(ctx->stream, n, p == 0 ? 0 : m, p, V, F, evals, evecs, n, dloss, dV);
+        CtxScratch<double> Pv(ctx, (size_t)n);
+        k::eig_grad(ctx->stream, n, p == 0 ? 0 : m, p, V, F, evals, evecs, n, dloss, dV, Pv.p);
         HSIM_CUDA(cudaStreamSynchronize(ctx->stream));
     });
 }

@@ -9,16 +9,25 @@
 //     phi^T S phi |_t = 1/2 sum_k cot_k (phi_{k+1} - phi_{k+2})^2,
 //     phi^T M phi |_t = A_t / 3 sum_k phi_k^2,
 // so one pass over the eigenpairs reduces every triangle to four numbers,
-//     D_k = sum_i w_i (phi_i(k+1) - phi_i(k+2))^2,  P = sum_i w_i lambda_i sum_k phi_i(k)^2,
-// and the gradient is 1/2 sum_k D_k dcot_k/dx - P/3 dA/dx.  Here the corner
-// cotangent is written with the two edge vectors leaving the corner,
-// u = x_{k+1} - x_k, w = x_{k+2} - x_k, cot_k = (u.w) / |u x w|, and with
-// n = (u x w)/|u x w| (the same for all three corners),
-//     d cot_k = [ (w - cot_k (w x n)) . du + (u - cot_k (n x u)) . dw ] / |u x w|,
-//     d A     = 1/2 [ (w x n) . du + (n x u) . dw ]         (corner 0).
+//     D_k = sum_i w_i (phi_i(k+1) - phi_i(k+2))^2,  P = sum of the corners' P_v,
+//     P_v = sum_i w_i lambda_i phi_i(v)^2 (once per vertex, k_vertex_energy),
+// and its part of the loss is E = sum_k t_k D_k / (2 s) - P s / 6 with the edges
+// e_0 = x_2 - x_1, e_1 = x_0 - x_2, e_2 = x_1 - x_0, t_k = -e_{k+1}.e_{k+2} (the
+// corner's u.w), s = |u x w| = 2 A, cot_k = t_k / s.  In the squared lengths l_k
+// = e_k.e_k, t_k = (l_{k+1} + l_{k+2} - l_k) / 2 and ds/dl_k = t_k / (2 s), so
+//     dE/dl_k = (D_{k+1} + D_{k+2} - D_k) / (4 s) + E_s t_k / (2 s),
+//     E_s = -sum_k t_k D_k / (2 s^2) - P / 6,
+// and with G_k = 2 dE/dl_k e_k the corners get G_1 - G_2, G_2 - G_0, G_0 - G_1.
 // One thread per triangle; the nine partial derivatives go to the vertices
 // with FP64 atomics (the order of the additions, hence the last bits, vary
 // from run to run).
+//
+// What bounds it: FP64 instructions (1.67 lanes per clock and SM), nine per
+// triangle and eigenpair, two per vertex and eigenpair and about 90 per
+// triangle: 80,000 triangles x 50 pairs take 90 + 12 us, where fourteen (P per triangle)
+// and the derivatives of the three cotangents one by one took 206 us.  CTAs of 64
+// threads spread 1,250 over 152 SMs evenly; of 256 threads 313 left a third of
+// them a CTA behind.
 
 #include "common.h"
 #include "kernels.h"
@@ -32,12 +41,13 @@ struct v3 {
     double x, y, z;
 };
 __device__ __forceinline__ v3 sub(v3 a, v3 b) { return {a.x - b.x, a.y - b.y, a.z - b.z}; }
-__device__ __forceinline__ v3 add(v3 a, v3 b) { return {a.x + b.x, a.y + b.y, a.z + b.z}; }
 __device__ __forceinline__ v3 mul(double s, v3 a) { return {s * a.x, s * a.y, s * a.z}; }
 __device__ __forceinline__ double dot(v3 a, v3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 __device__ __forceinline__ v3 cross(v3 a, v3 b) {
     return {a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
 }
+// x == 0 on the bits (the FP64 comparison takes its place in the FP64 pipe)
+__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
 __device__ __forceinline__ v3 load(const double *V, int v) {
     return {V[3 * (size_t)v], V[3 * (size_t)v + 1], V[3 * (size_t)v + 2]};
 }
@@ -47,58 +57,73 @@ __device__ __forceinline__ void atomic_add3(double *g, int v, v3 a) {
     atomicAdd(g + 3 * (size_t)v + 2, a.z);
 }
 
-__global__ void __launch_bounds__(256) k_eig_grad(int m, int n, int p, const double *__restrict__ V,
-                                                  const int *__restrict__ F, const double *__restrict__ evals,
-                                                  const double *__restrict__ evecs, int ld,
-                                                  const double *__restrict__ dl, double *__restrict__ g) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
+// Pv[v] = sum_i w_i lambda_i phi_i(v)^2
+__global__ void __launch_bounds__(64) k_vertex_energy(int n, int p, const double *__restrict__ evals,
+                                                      const double *__restrict__ evecs, int ld,
+                                                      const double *__restrict__ dl, double *__restrict__ Pv) {
+    __shared__ double wl[64];
+    const int v = blockIdx.x * blockDim.x + threadIdx.x;
+    const double *f = evecs + min(v, n - 1);
+    double P = 0.0;
+    for (int i0 = 0; i0 < p; i0 += 64) {
+        const int cnt = min(64, p - i0);
+        __syncthreads();
+        if ((int)threadIdx.x < cnt) wl[threadIdx.x] = __ldg(dl + i0 + threadIdx.x) * __ldg(evals + i0 + threadIdx.x);
+        __syncthreads();
+#pragma unroll 8
+        for (int i = 0; i < cnt; ++i) {
+            const double x = __ldg(f + (size_t)(i0 + i) * ld);
+            if (!is_zero(__ldg(dl + i0 + i))) P = fma(wl[i] * x, x, P);
+        }
+    }
+    if (v < n) Pv[v] = P;
+}
+
+__global__ void __launch_bounds__(64) k_eig_grad(int m, int p, const double *__restrict__ V, const int *__restrict__ F,
+                                                 const double *__restrict__ evecs, int ld,
+                                                 const double *__restrict__ dl, const double *__restrict__ Pv,
+                                                 double *__restrict__ g) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= m) return;
-    int c[3] = {F[3 * (size_t)t], F[3 * (size_t)t + 1], F[3 * (size_t)t + 2]};
-    double D[3] = {0.0, 0.0, 0.0}, P = 0.0;
+    const int c[3] = {F[3 * (size_t)t], F[3 * (size_t)t + 1], F[3 * (size_t)t + 2]};
+    double D0 = 0.0, D1 = 0.0, D2 = 0.0;
+    const double *q0 = evecs + c[0], *q1 = evecs + c[1], *q2 = evecs + c[2];
+#pragma unroll 4
     for (int i = 0; i < p; ++i) {
-        double w = __ldg(dl + i);
-        if (w == 0.0) continue;
-        const double *phi = evecs + (size_t)i * ld;
-        double f0 = __ldg(phi + c[0]), f1 = __ldg(phi + c[1]), f2 = __ldg(phi + c[2]);
-        double d0 = f1 - f2, d1 = f2 - f0, d2 = f0 - f1;
-        D[0] += w * d0 * d0;
-        D[1] += w * d1 * d1;
-        D[2] += w * d2 * d2;
-        P += w * __ldg(evals + i) * (f0 * f0 + f1 * f1 + f2 * f2);
+        const double w = __ldg(dl + i);
+        const double f0 = __ldg(q0 + (size_t)i * ld), f1 = __ldg(q1 + (size_t)i * ld), f2 = __ldg(q2 + (size_t)i * ld);
+        if (is_zero(w)) continue;
+        const double a = f1 - f2, b = f2 - f0, d = f0 - f1;
+        D0 = fma(w * a, a, D0);
+        D1 = fma(w * b, b, D1);
+        D2 = fma(w * d, d, D2);
     }
-    v3 x[3] = {load(V, c[0]), load(V, c[1]), load(V, c[2])};
-    v3 nrm = cross(sub(x[1], x[0]), sub(x[2], x[0]));
-    double s = sqrt(dot(nrm, nrm));  // 2 A
-    nrm = mul(1.0 / s, nrm);
-    v3 gr[3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    for (int k = 0; k < 3; ++k) {
-        int k1 = (k + 1) % 3, k2 = (k + 2) % 3;
-        v3 u = sub(x[k1], x[k]), w = sub(x[k2], x[k]);
-        double cot = dot(u, w) / s;
-        double h = 0.5 * D[k] / s;
-        v3 gu = mul(h, sub(w, mul(cot, cross(w, nrm))));
-        v3 gw = mul(h, sub(u, mul(cot, cross(nrm, u))));
-        gr[k1] = add(gr[k1], gu);
-        gr[k2] = add(gr[k2], gw);
-        gr[k] = sub(gr[k], add(gu, gw));
-    }
-    // - P/3 dA/dx
-    double a = -P / 6.0;
-    v3 ga1 = mul(a, cross(sub(x[2], x[0]), nrm));
-    v3 ga2 = mul(a, cross(nrm, sub(x[1], x[0])));
-    gr[1] = add(gr[1], ga1);
-    gr[2] = add(gr[2], ga2);
-    gr[0] = sub(gr[0], add(ga1, ga2));
-    for (int k = 0; k < 3; ++k) atomic_add3(g, c[k], gr[k]);
+    const v3 x0 = load(V, c[0]), x1 = load(V, c[1]), x2 = load(V, c[2]);
+    const v3 e0 = sub(x2, x1), e1 = sub(x0, x2), e2 = sub(x1, x0);
+    const v3 nrm = cross(e2, e1);  // u x w with the sign left out
+    const double s = sqrt(dot(nrm, nrm)), inv = 1.0 / s;
+    const double t0 = -dot(e1, e2), t1 = -dot(e2, e0), t2 = -dot(e0, e1);
+    const double P = Pv[c[0]] + Pv[c[1]] + Pv[c[2]];
+    const double N = fma(t0, D0, fma(t1, D1, t2 * D2));
+    // 2 dE/dl_k = ((D_{k+1} + D_{k+2} - D_k) / 2 + E_s t_k) / s
+    const double Es = fma(-0.5 * N * inv, inv, P * (-1.0 / 6.0));
+    const v3 G0 = mul(inv * fma(Es, t0, 0.5 * (D1 + D2 - D0)), e0);
+    const v3 G1 = mul(inv * fma(Es, t1, 0.5 * (D2 + D0 - D1)), e1);
+    const v3 G2 = mul(inv * fma(Es, t2, 0.5 * (D0 + D1 - D2)), e2);
+    atomic_add3(g, c[0], sub(G1, G2));
+    atomic_add3(g, c[1], sub(G2, G0));
+    atomic_add3(g, c[2], sub(G0, G1));
 }
 
 }  // namespace
 
 void eig_grad(cudaStream_t s, int n, int m, int p, const double *V, const int *F, const double *evals,
-              const double *evecs, int ld, const double *dloss, double *dV) {
+              const double *evecs, int ld, const double *dloss, double *dV, double *Pv) {
     HSIM_CUDA(cudaMemsetAsync(dV, 0, sizeof(double) * 3 * (size_t)n, s));
     if (m == 0) return;
-    k_eig_grad<<<(unsigned)((m + 255) / 256), 256, 0, s>>>(m, n, p, V, F, evals, evecs, ld, dloss, dV);
+    k_vertex_energy<<<(unsigned)((n + 63) / 64), 64, 0, s>>>(n, p, evals, evecs, ld, dloss, Pv);
+    HSIM_LAUNCHED();
+    k_eig_grad<<<(unsigned)((m + 63) / 64), 64, 0, s>>>(m, p, V, F, evecs, ld, dloss, Pv, dV);
     HSIM_LAUNCHED();
 }
 

@@ -24,9 +24,10 @@ void assemble_sm(cudaStream_t s, int n, const int *ptr, const int *col, const in
                  double *S_val, double *M_diag, bool consistent);
 // out[i] = sum of row i of a CSR matrix
 void row_sums(cudaStream_t s, int n, const int *ptr, const double *val, double *out);
-// dV = sum_i dloss[i] d lambda_i / dV (k_grad.cu); dV is zeroed first
+// dV = sum_i dloss[i] d lambda_i / dV (k_grad.cu); dV is zeroed first; Pv: n
+// doubles of scratch
 void eig_grad(cudaStream_t s, int n, int m, int p, const double *V, const int *F, const double *evals,
-              const double *evecs, int ld, const double *dloss, double *dV);
+              const double *evecs, int ld, const double *dloss, double *dV, double *Pv);
 // Y[r, 0:k] = sum A[r,c] X[c, 0:k]
 void spmm(cudaStream_t s, int n_rows, const int *ptr, const int *col, const double *val, int k,
           const double *X, int ldx, double *Y, int ldy);

@@ -3,9 +3,9 @@
 // and the numeric Galerkin products U^T A U (Alg. 3), plus permutation and
 // layout helpers.
 //
-// SpMM is HBM-bound: one warp per sparse row, lanes stride over the k dense
-// columns so every X row read is a contiguous, coalesced 8k-byte segment; the
-// row's nonzeros are broadcast from registers with warp shuffles.
+// SpMM: one warp per sparse row (and 128-column block), lanes stride over the
+// dense columns so every X row read is a contiguous segment; the row's nonzeros
+// are broadcast from registers with warp shuffles.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -94,65 +94,125 @@ __global__ void k_row_sums(int n, const int *__restrict__ ptr, const double *__r
     out[i] = s;
 }
 
-// One warp per row; each lane owns columns lane, lane+32, ...  Up to
-// kMaxCols/32 accumulators per lane are kept in registers; wider k is done in
-// several column passes.
-template <typename T, int kChunk>
-__global__ void k_spmm(int n_rows, const int *__restrict__ ptr, const int *__restrict__ col,
-                       const T *__restrict__ val, int k, const T *__restrict__ X, int ldx,
-                       T *__restrict__ Y, int ldy) {
-    const int lane = threadIdx.x & (kWarp - 1);
-    const int warps = blockDim.x / kWarp;
-    int64_t row = (int64_t)blockIdx.x * warps + threadIdx.x / kWarp;
+// Y = A X for narrow blocks, k <= 32 CH: one warp per row, lane l the columns l
+// and l + 32, the row's entries broadcast from registers four at a time so that
+// the gathers of four X rows are in flight together.
+template <int CH>
+__global__ void __launch_bounds__(128) k_spmm_narrow(int n_rows, const int *__restrict__ ptr, const int *__restrict__ col,
+                                                     const double *__restrict__ val, int k, const double *__restrict__ X,
+                                                     int ldx, double *__restrict__ Y, int ldy) {
+    const int lane = threadIdx.x & 31;
+    const int64_t row = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
     if (row >= n_rows) return;
     const int beg = ptr[row], end = ptr[row + 1];
-    for (int c0 = 0; c0 < k; c0 += kChunk * kWarp) {
-        T acc[kChunk];
+    double acc[CH];
 #pragma unroll
-        for (int u = 0; u < kChunk; ++u) acc[u] = T(0);
-        for (int e0 = beg; e0 < end; e0 += kWarp) {
-            int my_c = 0;
-            T my_v = T(0);
-            if (e0 + lane < end) {
-                my_c = col[e0 + lane];
-                my_v = val[e0 + lane];
-            }
-            const int cnt = min(kWarp, end - e0);
-            for (int t = 0; t < cnt; ++t) {
-                int c = __shfl_sync(0xffffffffu, my_c, t);
-                T v = __shfl_sync(0xffffffffu, my_v, t);
-                const T *xr = X + (size_t)c * ldx;
-#pragma unroll
-                for (int u = 0; u < kChunk; ++u) {
-                    int j = c0 + u * kWarp + lane;
-                    if (j < k) acc[u] += v * xr[j];
-                }
-            }
+    for (int u = 0; u < CH; ++u) acc[u] = 0.0;
+    for (int e0 = beg; e0 < end; e0 += 32) {
+        int my_c = 0;
+        double my_v = 0.0;
+        if (e0 + lane < end) {
+            my_c = col[e0 + lane];
+            my_v = val[e0 + lane];
         }
-        T *yr = Y + (size_t)row * ldy;
+        const int cnt = min(32, end - e0);
+        for (int t0 = 0; t0 < cnt; t0 += 4) {
+            double x[4][CH];
 #pragma unroll
-        for (int u = 0; u < kChunk; ++u) {
-            int j = c0 + u * kWarp + lane;
-            if (j < k) yr[j] = acc[u];
+            for (int t = 0; t < 4; ++t) {
+                const double *xr = X + (size_t)__shfl_sync(0xffffffffu, my_c, (t0 + t) & 31) * ldx + lane;
+#pragma unroll
+                for (int u = 0; u < CH; ++u) x[t][u] = t0 + t < cnt && 32 * u + lane < k ? xr[32 * u] : 0.0;
+            }
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const double v = __shfl_sync(0xffffffffu, my_v, (t0 + t) & 31);
+                if (t0 + t >= cnt) break;
+#pragma unroll
+                for (int u = 0; u < CH; ++u) acc[u] = fma(v, x[t][u], acc[u]);
+            }
         }
     }
+    double *yr = Y + (size_t)row * ldy + lane;
+#pragma unroll
+    for (int u = 0; u < CH; ++u)
+        if (32 * u + lane < k) yr[32 * u] = acc[u];
 }
 
-constexpr int kSpmmRows = 16;  // rows (warps) per CTA of the column-block SpMMs
+constexpr int kSpmmRows = 16;  // rows (warps) per CTA of the column-block SpMM
 
-// CTA (16 consecutive rows, one 128-column block), the column block the slow
-// index: the CTA's gathered 1 KB row segments stay in L1, and concurrently
-// running CTAs share the same column block in L2
-__device__ __forceinline__ bool spmm_cb_map(int n_rows, int k, int &row, int &c) {
+// Y = A X for k > 64: a CTA takes 16 consecutive rows of one 128-column block,
+// the column block the slow index: the CTA's gathered 1 KB row segments stay in
+// L1, and concurrently running CTAs share the same column block in L2.  Bound by
+// the FP64 pipe, 94 % of its rate at 10^6 rows x 750 (9.0 ms), where an
+// instruction costs a warp the same 77 clocks however many lanes it serves.
+// Two layouts of a block on the lanes:
+// k_spmm4: four consecutive columns per lane, read as pairs (every block at
+//   least 97 columns wide: nothing to skip; 0.5 to 1 % faster than the other);
+// k_spmm_groups: columns l, l + 32, l + 64, l + 96, groups of 32 beyond k skipped
+//   (75 columns: three of four groups).
+template <int NG>
+__device__ __forceinline__ void spmm_block(const int *__restrict__ col, const double *__restrict__ val, int beg, int end,
+                                           const double *__restrict__ X, int ldx, bool last, double *__restrict__ y) {
+    const int lane = threadIdx.x & 31;
+    double acc[NG];
+#pragma unroll
+    for (int v = 0; v < NG; ++v) acc[v] = 0.0;
+    for (int e0 = beg; e0 < end; e0 += 32) {
+        int my_c = 0;
+        double my_v = 0.0;
+        if (e0 + lane < end) {
+            my_c = col[e0 + lane];
+            my_v = val[e0 + lane];
+        }
+        const int cnt = min(32, end - e0);
+        auto load = [&](int t, double (&x)[NG]) {
+            const double *xr = X + (size_t)__shfl_sync(0xffffffffu, my_c, t) * ldx;
+#pragma unroll
+            for (int v = 0; v < NG; ++v) x[v] = v < NG - 1 || last ? xr[32 * v] : 0.0;
+        };
+        int t = 0;
+        for (; t + 1 < cnt; t += 2) {
+            double xa[NG], xb[NG];
+            load(t, xa);
+            load(t + 1, xb);
+            const double sa = __shfl_sync(0xffffffffu, my_v, t), sb = __shfl_sync(0xffffffffu, my_v, t + 1);
+#pragma unroll
+            for (int v = 0; v < NG; ++v) acc[v] = fma(sa, xa[v], acc[v]);
+#pragma unroll
+            for (int v = 0; v < NG; ++v) acc[v] = fma(sb, xb[v], acc[v]);
+        }
+        if (t < cnt) {
+            double xa[NG];
+            load(t, xa);
+            const double sa = __shfl_sync(0xffffffffu, my_v, t);
+#pragma unroll
+            for (int v = 0; v < NG; ++v) acc[v] = fma(sa, xa[v], acc[v]);
+        }
+    }
+#pragma unroll
+    for (int v = 0; v < NG; ++v)
+        if (v < NG - 1 || last) y[32 * v] = acc[v];
+}
+
+__global__ void __launch_bounds__(kSpmmRows * 32) k_spmm_groups(int n_rows, const int *__restrict__ ptr,
+                                                                const int *__restrict__ col,
+                                                                const double *__restrict__ val, int k,
+                                                                const double *__restrict__ X, int ldx,
+                                                                double *__restrict__ Y, int ldy) {
     const int nrg = (n_rows + kSpmmRows - 1) / kSpmmRows;
-    const int cb = blockIdx.x / nrg, rg = blockIdx.x - cb * nrg;
-    row = rg * kSpmmRows + (threadIdx.x >> 5);
-    c = cb * 128 + (threadIdx.x & 31) * 4;
-    return row < n_rows && cb * 128 < k;
+    const int cb = blockIdx.x / nrg, row = (blockIdx.x - cb * nrg) * kSpmmRows + (threadIdx.x >> 5);
+    if (row >= n_rows) return;
+    const int c = cb * 128 + (threadIdx.x & 31), ng = min(4, (k - cb * 128 + 31) / 32);
+    const bool last = c + 32 * (ng - 1) < k;  // this lane's column of the last group
+    const int beg = ptr[row], end = ptr[row + 1];
+    double *y = Y + (size_t)row * ldy + c;
+    if (ng == 4) spmm_block<4>(col, val, beg, end, X + c, ldx, last, y);
+    else if (ng == 3) spmm_block<3>(col, val, beg, end, X + c, ldx, last, y);
+    else if (ng == 2) spmm_block<2>(col, val, beg, end, X + c, ldx, last, y);
+    else spmm_block<1>(col, val, beg, end, X + c, ldx, last, y);
 }
 
-
-// FP64 S X with the same column-block mapping: four doubles per lane
 __device__ __forceinline__ void load_d4(double (&x)[4], const double *__restrict__ X, int r, int c, int k, int ldx,
                                         bool vec) {
     const double *p = X + (size_t)r * ldx + c;
@@ -170,8 +230,10 @@ __global__ void __launch_bounds__(kSpmmRows * 32) k_spmm4(int n_rows, const int 
                                                           int k, const double *__restrict__ X, int ldx,
                                                           double *__restrict__ Y, int ldy, bool vec) {
     const int lane = threadIdx.x & 31;
-    int row, c;
-    if (!spmm_cb_map(n_rows, k, row, c)) return;
+    const int nrg = (n_rows + kSpmmRows - 1) / kSpmmRows;
+    const int cb = blockIdx.x / nrg, row = (blockIdx.x - cb * nrg) * kSpmmRows + (threadIdx.x >> 5);
+    const int c = cb * 128 + lane * 4;
+    if (row >= n_rows) return;
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
     const int beg = ptr[row], end = ptr[row + 1];
     for (int e0 = beg; e0 < end; e0 += 32) {
@@ -184,11 +246,11 @@ __global__ void __launch_bounds__(kSpmmRows * 32) k_spmm4(int n_rows, const int 
         const int cnt = min(32, end - e0);
         int t = 0;
         for (; t + 1 < cnt; t += 2) {
-            const int ca = __shfl_sync(0xffffffffu, my_c, t), cb = __shfl_sync(0xffffffffu, my_c, t + 1);
+            const int ca = __shfl_sync(0xffffffffu, my_c, t), cb2 = __shfl_sync(0xffffffffu, my_c, t + 1);
             const double sa = __shfl_sync(0xffffffffu, my_v, t), sb = __shfl_sync(0xffffffffu, my_v, t + 1);
             double xa[4], xb[4];
             load_d4(xa, X, ca, c, k, ldx, vec);
-            load_d4(xb, X, cb, c, k, ldx, vec);
+            load_d4(xb, X, cb2, c, k, ldx, vec);
 #pragma unroll
             for (int v = 0; v < 4; ++v) acc[v] = fma(sa, xa[v], acc[v]);
 #pragma unroll
@@ -482,17 +544,19 @@ void assemble_sm(cudaStream_t s, int n, const int *ptr, const int *col, const in
 void spmm(cudaStream_t s, int n_rows, const int *ptr, const int *col, const double *val, int k, const double *X,
           int ldx, double *Y, int ldy) {
     if (n_rows <= 0 || k <= 0) return;
-    if (k >= 64) {
+    if (k > 64) {
         // wide blocks: column-block mapping (L1 reuse of the gathered rows)
         const unsigned blocks = (unsigned)(((n_rows + kSpmmRows - 1) / kSpmmRows) * ((k + 127) / 128));
         const bool vec = (reinterpret_cast<uintptr_t>(X) % 16 == 0) && (ldx % 2 == 0);
-        k_spmm4<<<blocks, kSpmmRows * 32, 0, s>>>(n_rows, ptr, col, val, k, X, ldx, Y, ldy, vec);
-        HSIM_LAUNCHED();
-        return;
+        if (k % 128 == 0 || k % 128 > 96)
+            k_spmm4<<<blocks, kSpmmRows * 32, 0, s>>>(n_rows, ptr, col, val, k, X, ldx, Y, ldy, vec);
+        else
+            k_spmm_groups<<<blocks, kSpmmRows * 32, 0, s>>>(n_rows, ptr, col, val, k, X, ldx, Y, ldy);
+    } else if (k > 32) {
+        k_spmm_narrow<2><<<grid1d(n_rows, 4), 128, 0, s>>>(n_rows, ptr, col, val, k, X, ldx, Y, ldy);
+    } else {
+        k_spmm_narrow<1><<<grid1d(n_rows, 4), 128, 0, s>>>(n_rows, ptr, col, val, k, X, ldx, Y, ldy);
     }
-    const int warps = 8;
-    unsigned g = grid1d(n_rows, warps);
-    k_spmm<double, 8><<<g, warps * 32, 0, s>>>(n_rows, ptr, col, val, k, X, ldx, Y, ldy);
     HSIM_LAUNCHED();
 }
 

@@ -303,7 +303,7 @@ struct hsim_hier {
     // mixed precision: FP32 factor and FP32 right-hand-side blocks
     DevBuf<float> arena32, dpos32, X32;
     // inverted-factor solves: 1 / D, the forward result Y, inversion scratch
-    DevBuf<double> dinvf, ysol, invs;
+    DevBuf<double> dinvf, invs;  // FP64 factors keep neither (arguments of factor_level_t)
     DevBuf<float> dinvf32, ysol32, invs32;
     DevBuf<double> rho;
     DevBuf<unsigned char> oz;  // digit slices of the tensor-core products
@@ -604,7 +604,7 @@ int factor_level_t(hsim_ctx *ctx, LevelData &L, const double *S, const double *M
     }
     // all nodes 0..N-1 are listed in d_hnodes grouped by height
     k::front_diag(s, L.fd, L.d_hnodes.p, fs.n_nodes, (const T *)arena.p, dpos.p, flags + 2);
-    if (std::is_same<T, float>::value) {
+    if constexpr (std::is_same<T, float>::value) {
         // FP32 factors are solved in the inverted form (see solve_level_t)
         dinv.reserve((size_t)L.n);
         k::reciprocal(s, L.n, (const T *)dpos.p, dinv.p);
@@ -621,8 +621,8 @@ int factor_level_t(hsim_ctx *ctx, LevelData &L, const double *S, const double *M
 // K^-1 X in place with the factor walked panel by panel: per tree height the
 // fused kernels for fronts of one panel, else a triangle and an update launch
 // per 32-column panel; then D^-1; then the backward sweep.
-template <typename T>
-void solve_level_panels(hsim_ctx *ctx, LevelData &L, const T *arena, const T *dpos, T *X, int k, int ldx) {
+void solve_level_panels(hsim_ctx *ctx, LevelData &L, const double *arena, const double *dpos, double *X, int k,
+                        int ldx) {
     cudaStream_t s = ctx->stream;
     const FrontSymbolic &fs = L.fs;
     auto small = [&](int h) { return L.step_cnt[h].size() == 1 && L.step_maxnf[h][0] <= k::kSmallNf; };
@@ -666,10 +666,7 @@ void solve_level_t(hsim_ctx *ctx, LevelData &L, const T *arena, const T *dpos, c
                    int k, int ldx) {
     cudaStream_t s = ctx->stream;
     const FrontSymbolic &fs = L.fs;
-    if (!std::is_same<T, float>::value) {
-        solve_level_panels(ctx, L, arena, dpos, X, k, ldx);
-        return;
-    }
+    static_assert(std::is_same<T, float>::value, "FP64 factors are solved panel by panel");
     Y.reserve((size_t)L.n * ldx);
     // HSIM_TRACE=2: time of every tree height of the forward and backward sweeps
     const bool detail = trace_level() >= 2;
@@ -765,7 +762,7 @@ int factor_level(hsim_ctx *ctx, hsim_hier *H, LevelData &L, const double *S, con
 }
 
 void solve_level(hsim_ctx *ctx, hsim_hier *H, LevelData &L, double *X, int k, int ldx) {
-    solve_level_t<double>(ctx, L, H->arena.p, H->dpos.p, H->dinvf.p, H->ysol, X, k, ldx);
+    solve_level_panels(ctx, L, H->arena.p, H->dpos.p, X, k, ldx);
 }
 
 int subspace_q(int p, const hsim_options &o) {

@@ -421,9 +421,8 @@ struct DenseFront {
     DevBuf<int64_t> foff, rows_off, relmap_off;
     DevBuf<int> nf, ns, pstart, rows, relmap, node;
     FrontDev fd{};
-    // in-place inversion of the unit lower factor (inverse_plan of one front)
-    DevBuf<int2> blk;
-    int nblk = 0;
+    // in-place inversion of the unit lower factor (inverse_plan of one front;
+    // front_panel leaves the 32 x 32 diagonal blocks inverted)
     std::vector<DevBuf<GemmTask>> p1, p2;
     std::vector<int> ntask, tiles;
     int64_t scratch = 0;
@@ -451,8 +450,6 @@ DenseFront &dense_front(int k, cudaStream_t s) {
     d->relmap.upload(std::vector<int>{0}, s);
     d->node.upload(std::vector<int>{0}, s);
     InversePlan P = inverse_plan({k}, {k}, {0});
-    d->nblk = (int)P.blk.size();
-    d->blk.upload(P.blk, s);
     for (size_t lv = 0; lv < P.p1.size(); ++lv) {
         d->ntask.push_back((int)P.p1[lv].size());
         d->p1.emplace_back();
@@ -776,7 +773,6 @@ int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar,
             (reinterpret_cast<uintptr_t>(scr + kk) + 255) & ~static_cast<uintptr_t>(255));
         const size_t rb = ozaki_rows_scratch(k, k);
         HSIM_CHECK_ARG(df.scratch <= (int64_t)kk, "ritz: inversion scratch");
-        inv_diag_blocks<double>(s, df.fd, df.blk.p, df.nblk, F);
         for (size_t lv = 0; lv < df.p1.size(); ++lv) {
             gemm_tasks<double>(s, df.p1[lv].p, df.ntask[lv], df.tiles[lv], F, F, scr);
             gemm_tasks<double>(s, df.p2[lv].p, df.ntask[lv], df.tiles[lv], F, scr, F);

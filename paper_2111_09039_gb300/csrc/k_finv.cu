@@ -1108,13 +1108,13 @@ void solve_bwd_fused(cudaStream_t s, const FrontDev &fd, const int *parents, int
     HSIM_LAUNCHED();
 }
 
-#define HSIM_FINV_INSTANTIATE(T)                                                                                    \
-    template void inv_diag_blocks<T>(cudaStream_t, const FrontDev &, const int2 *, int, T *);                     \
-    template void gemm_tasks<T>(cudaStream_t, const GemmTask *, int, int, const T *, const T *, T *);             \
-    template void copy_tasks<T>(cudaStream_t, const GemmTask *, int, int, const T *, T *);                        \
-    template void reciprocal<T>(cudaStream_t, int, const T *, T *);
-HSIM_FINV_INSTANTIATE(float)
-HSIM_FINV_INSTANTIATE(double)
+// FP64: the dense front of the Ritz step (block doubling above its inverted
+// diagonal blocks)
+template void inv_diag_blocks<float>(cudaStream_t, const FrontDev &, const int2 *, int, float *);
+template void gemm_tasks<float>(cudaStream_t, const GemmTask *, int, int, const float *, const float *, float *);
+template void gemm_tasks<double>(cudaStream_t, const GemmTask *, int, int, const double *, const double *, double *);
+template void copy_tasks<float>(cudaStream_t, const GemmTask *, int, int, const float *, float *);
+template void reciprocal<float>(cudaStream_t, int, const float *, float *);
 // the inverted-form solves serve the FP32 factor only
 template void solve_fwd_inv<float>(cudaStream_t, const FrontDev &, const int *, int, int, int, const float *, int,
                                    float *, float *, int);

@@ -7,10 +7,13 @@
 // ns columns are the pivots.  Fronts of equal height in the elimination tree
 // are independent and are processed by the same launches.  A front is
 // factored in panels of kPanel = 32 columns (right-looking):
-//   diag:    LDL^T of the 32 x 32 diagonal block in shared memory (one CTA
-//            per front), written back in place;
-//   panel:   L21 = A21 L11^-T D^-1, one tile of 128 rows per CTA;
-//   update:  A22 -= L21 D L21^T on lower-triangular 64 x 64 tiles;
+//   diag:    LDL^T of the 32 x 32 diagonal block (one CTA per front), written
+//            back in place; FP64 fronts keep the inverse of its unit lower
+//            factor there, which turns every triangle of the panel and of the
+//            solves into a product (a triangle of 32 is a chain of 496
+//            dependent FP64 instructions of 77 clocks, whatever the width);
+//   panel:   L21 = A21 L11^-T D^-1;
+//   update:  A22 -= L21 D L21^T on lower-triangular tiles;
 // and the children's update blocks are added into the parent front
 // (extend-add) before the parent is factored.  Pivoting is not used: the
 // shifted Laplacian is factored as is after the fill-reducing ordering; a
@@ -22,6 +25,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include "common.h"
 #include "host.h"
@@ -180,13 +184,118 @@ __global__ void __launch_bounds__(128) k_front_panel(FrontDev fd, const int *__r
     }
 }
 
-// A22 -= L21 D L21^T on 64 x 64 lower-triangular tiles of the trailing block;
+// FP64 diagonal block: D and the inverse of L11 in one pass (Gauss-Jordan on [A |
+// I] without the part above the diagonal).  Lane r of every warp holds row r,
+// warp w the columns w, w + 4, ... of the block and of the inverse, so a pivot
+// step is up to 8 + 8 FP64 instructions per warp, one warp per SM sub-partition,
+// around a chain of reciprocal, product and update.  32 pivots take 26 us;
+// with the block in shared memory, three barriers a pivot and a division per
+// entry they took 36.6, without the inverse.  (A correction step on the quotients
+// of l and of the panel left the solves' error as it was.)
+__global__ void __launch_bounds__(128) k_front_diag_inv(FrontDev fd, const int *__restrict__ nodes, int k0,
+                                                        double *__restrict__ arena, double tol, int *flags) {
+    __shared__ double u[2][P], pinv[2];
+    const int t = nodes[blockIdx.x];
+    const int nf = fd.nf[t], ns = fd.ns[t];
+    const int kb = min(P, ns - k0);
+    if (kb <= 0) return;
+    const int r = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double *F = arena + fd.foff[t] + (int64_t)k0 * nf + k0;  // column c at F + c nf
+    double a[P / 4], e[P / 4];
+#pragma unroll
+    for (int q = 0; q < P / 4; ++q) {
+        const int c = w + 4 * q;
+        a[q] = c < kb && r < kb && r >= c ? F[(int64_t)c * nf + r] : 0.0;
+        e[q] = r == c ? 1.0 : 0.0;
+    }
+#pragma unroll
+    for (int j = 0; j < P; ++j) {
+        if (j >= kb) break;
+        if (w == (j & 3)) {
+            double d = __shfl_sync(0xffffffffu, a[j / 4], j);
+            if (!(fabs(d) >= tol)) {  // also catches NaN
+                if (r == 0) atomicAdd(&flags[0], 1);
+                d = d < 0.0 ? -tol : tol;
+                if (r == j) a[j / 4] = d;
+            }
+            u[j & 1][r] = a[j / 4];
+            if (r == 0) {
+                const int x = (__double2hiint(d) >> 20) & 0x7FF;
+                double v;
+                if (x > 40 && x < 2006) {
+                    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(v) : "d"(d));
+                    const double q = fma(-d, v, 1.0);
+                    v = fma(v, fma(q, q, q), v);
+                } else {
+                    v = 1.0 / d;
+                }
+                pinv[j & 1] = v;
+            }
+        }
+        __syncthreads();
+        // row r > j: l = a_rj / d, A_r -= l (d l_c) = l u_c, I_r -= l I_j
+        const double l = r > j ? u[j & 1][r] * pinv[j & 1] : 0.0;
+#pragma unroll
+        for (int q = 0; q < P / 4; ++q) {
+            const int c = w + 4 * q;
+            if (c > j) a[q] = fma(-l, u[j & 1][c], a[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < P / 4; ++q)
+            if (4 * q <= j) e[q] = fma(-l, __shfl_sync(0xffffffffu, e[q], j), e[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < P / 4; ++q) {
+        const int c = w + 4 * q;
+        if (c < kb && r < kb && r >= c) F[(int64_t)c * nf + r] = r == c ? a[q] : e[q];
+    }
+}
+
+// FP64 rows below the diagonal block: L21 = A21 Linv^T D^-1 with the inverse that
+// k_front_diag_inv left in the block.  A CTA takes 16 rows, thread (row, column
+// group g) the columns g, g + 8, g + 16, g + 24: small tiles, since the FP64
+// pipes of idle SMs are what a panel of a few hundred rows can use.
+constexpr int kPanelRows64 = 16;
+__global__ void __launch_bounds__(128) k_front_panel64(FrontDev fd, const int *__restrict__ nodes, int k0,
+                                                       double *__restrict__ arena) {
+    __shared__ double Li[P][P + 1], As[P][kPanelRows64 + 1], di[P];
+    const int t = nodes[blockIdx.x];
+    const int nf = fd.nf[t], ns = fd.ns[t];
+    const int kb = min(P, ns - k0);
+    if (kb <= 0) return;
+    const int r0 = k0 + kb + blockIdx.y * kPanelRows64;
+    if (r0 >= nf) return;
+    double *F = arena + fd.foff[t];
+    for (int idx = threadIdx.x; idx < P * P; idx += 128) {
+        const int r = idx & 31, c = idx >> 5;
+        Li[r][c] = r > c && r < kb ? F[(int64_t)(k0 + c) * nf + (k0 + r)] : r == c ? 1.0 : 0.0;
+    }
+    for (int idx = threadIdx.x; idx < P * kPanelRows64; idx += 128) {
+        const int r = idx % kPanelRows64, c = idx / kPanelRows64;
+        As[c][r] = c < kb && r0 + r < nf ? F[(int64_t)(k0 + c) * nf + (r0 + r)] : 0.0;
+    }
+    if (threadIdx.x < kb) di[threadIdx.x] = 1.0 / F[(int64_t)(k0 + threadIdx.x) * nf + (k0 + threadIdx.x)];
+    __syncthreads();
+    const int r = threadIdx.x % kPanelRows64, g = threadIdx.x / kPanelRows64;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+        // the upper part is zero: whole groups of eight columns up to this one
+        for (int cc = 0; cc < 8 * v + 8; ++cc) acc[v] = fma(As[cc][r], Li[g + 8 * v][cc], acc[v]);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        const int c = g + 8 * v;
+        if (c < kb && r0 + r < nf) F[(int64_t)(k0 + c) * nf + (r0 + r)] = acc[v] * di[c];
+    }
+}
+
+// A22 -= L21 D L21^T on TS x TS lower-triangular tiles of the trailing block;
 // with ntj > 0 only the columns below c_end (tile y = ti * ntj + tj)
-template <typename T>
+template <typename T, int TS>
 __global__ void __launch_bounds__(256) k_front_update(FrontDev fd, const int *__restrict__ nodes, int k0,
                                                       T *__restrict__ arena, int c_end, int ntj) {
-    __shared__ T Lr[P][64];
-    __shared__ T Lc[P][64];
+    __shared__ T Lr[P][TS];
+    __shared__ T Lc[P][TS];
     const int t = nodes[blockIdx.x];
     const int nf = fd.nf[t], ns = fd.ns[t];
     const int kb = min(P, ns - k0);
@@ -194,7 +303,7 @@ __global__ void __launch_bounds__(256) k_front_update(FrontDev fd, const int *__
     const int base = k0 + kb;
     const int m = nf - base;
     if (m <= 0) return;
-    const int nt = (m + 63) / 64;
+    const int nt = (m + TS - 1) / TS;
     int ti, tj;
     if (ntj > 0) {
         ti = (int)(blockIdx.y / ntj);
@@ -205,10 +314,10 @@ __global__ void __launch_bounds__(256) k_front_update(FrontDev fd, const int *__
     }
     if (ti >= nt) return;
     T *F = arena + fd.foff[t];
-    const int r0 = base + ti * 64, c0 = base + tj * 64;
+    const int r0 = base + ti * TS, c0 = base + tj * TS;
     if (c0 >= c_end) return;
-    for (int idx = threadIdx.x; idx < P * 64; idx += blockDim.x) {
-        int i = idx & 63, kk = idx >> 6;
+    for (int idx = threadIdx.x; idx < P * TS; idx += blockDim.x) {
+        int i = idx % TS, kk = idx / TS;
         T vr = 0.0, vc = 0.0;
         if (kk < kb) {
             T d = F[(int64_t)(k0 + kk) * nf + (k0 + kk)];
@@ -220,25 +329,26 @@ __global__ void __launch_bounds__(256) k_front_update(FrontDev fd, const int *__
     }
     __syncthreads();
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    T acc[4][4] = {};
+    constexpr int U = TS / 16;
+    T acc[U][U] = {};
     for (int kk = 0; kk < kb; ++kk) {
-        T a[4], b[4];
+        T a[U], b[U];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < U; ++u) {
             a[u] = Lr[kk][ty + 16 * u];
             b[u] = Lc[kk][tx + 16 * u];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] += a[u] * b[v];
+            for (int v = 0; v < U; ++v) acc[u][v] += a[u] * b[v];
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < U; ++u) {
         int r = r0 + ty + 16 * u;
         if (r >= nf) continue;
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
+        for (int v = 0; v < U; ++v) {
             int c = c0 + tx + 16 * v;
             if (c < nf && r >= c && c < c_end) F[(int64_t)c * nf + r] -= acc[u][v];
         }
@@ -275,82 +385,83 @@ __global__ void k_front_maxdiag(FrontDev fd, const T *__restrict__ arena, unsign
     if (best) atomicMax(out, best);
 }
 
-// ---- solves ---------------------------------------------------------------
-constexpr int kTriCols = 128;
+// ---- FP64 solves (FP32 factors are solved in the inverted form, k_finv.cu) -----
+// Every diagonal block holds the inverse of its unit lower factor (k_front_diag_inv),
+// so the triangles are products; tiles are small where a height has few fronts
+// (an SM's FP64 pipes take 1.67 lanes per clock: 64 x 64 x 32 products keep one
+// SM busy for 38 us while others idle).
 
-// X[panel rows, cols] = L11^-1 X[...]  (unit lower, forward)
-template <typename T>
-__global__ void __launch_bounds__(kTriCols) k_solve_fwd_tri(FrontDev fd, const int *__restrict__ nodes, int k0,
-                                                            const T *__restrict__ arena, int k,
-                                                            T *__restrict__ X, int ldx) {
-    __shared__ T L[P][P + 1];
+// Li[r][c] = the inverse block (rows and columns beyond kb: identity)
+__device__ __forceinline__ void load_inv(double (&Li)[P][P + 1], const double *__restrict__ F, int nf, int k0, int kb) {
+    for (int idx = threadIdx.x; idx < P * P; idx += blockDim.x) {
+        const int r = idx & 31, c = idx >> 5;
+        Li[r][c] = r > c && r < kb ? F[(int64_t)(k0 + c) * nf + (k0 + r)] : r == c ? 1.0 : 0.0;
+    }
+}
+
+constexpr int kTriCols = 16;
+
+// X[panel rows, cols] = Linv X[...] (backward: Linv^T X[...]); thread (column,
+// row group g): rows g, g + 8, g + 16, g + 24 of a 16-column tile
+template <bool TRANS>
+__global__ void __launch_bounds__(128) k_solve_tri(FrontDev fd, const int *__restrict__ nodes, int k0,
+                                                   const double *__restrict__ arena, int k, double *__restrict__ X,
+                                                   int ldx) {
+    __shared__ double Li[P][P + 1], Xs[P][kTriCols];
     const int t = nodes[blockIdx.x];
     const int nf = fd.nf[t], ns = fd.ns[t], ps = fd.pstart[t];
     const int kb = min(P, ns - k0);
     if (kb <= 0) return;
-    const T *F = arena + fd.foff[t];
-    for (int idx = threadIdx.x; idx < kb * kb; idx += blockDim.x) {
-        int r = idx % kb, c = idx / kb;
-        L[r][c] = (r > c) ? F[(int64_t)(k0 + c) * nf + (k0 + r)] : 0.0;
+    load_inv(Li, arena + fd.foff[t], nf, k0, kb);
+    const int c = threadIdx.x % kTriCols, g = threadIdx.x / kTriCols, j = blockIdx.y * kTriCols + c;
+    double *Xb = X + (size_t)(ps + k0) * ldx + j;
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        const int r = g + 8 * v;
+        Xs[r][c] = r < kb && j < k ? Xb[(size_t)r * ldx] : 0.0;
     }
     __syncthreads();
-    const int j = blockIdx.y * kTriCols + threadIdx.x;
-    if (j >= k) return;
-    T x[P];
-    T *Xb = X + (size_t)(ps + k0) * ldx + j;
+    double acc[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-    for (int r = 0; r < P; ++r)
-        if (r < kb) x[r] = Xb[(size_t)r * ldx];
-#pragma unroll
-    for (int r = 1; r < P; ++r) {
-        if (r < kb) {
-            T v = x[r];
-#pragma unroll
-            for (int c = 0; c < P; ++c)
-                if (c < r) v -= L[r][c] * x[c];
-            x[r] = v;
+    for (int v = 0; v < 4; ++v) {
+        const int r = g + 8 * v;
+        if (TRANS) {
+            for (int q = 8 * v; q < P; ++q) acc[v] = fma(Li[q][r], Xs[q][c], acc[v]);
+        } else {
+            for (int q = 0; q < 8 * v + 8; ++q) acc[v] = fma(Li[r][q], Xs[q][c], acc[v]);
         }
     }
+    if (j >= k) return;
 #pragma unroll
-    for (int r = 0; r < P; ++r)
-        if (r < kb) Xb[(size_t)r * ldx] = x[r];
-}
-
-// x[0..3] -= a[0..3] with atomics (one vector atomic for four aligned floats)
-__device__ __forceinline__ void atomic_sub4(float *x, const float (&a)[4], int avail) {
-    if (avail >= 4 && (reinterpret_cast<uintptr_t>(x) & 15u) == 0) {
-        atomicAdd(reinterpret_cast<float4 *>(x), make_float4(-a[0], -a[1], -a[2], -a[3]));
-    } else {
-        for (int v = 0; v < 4 && v < avail; ++v) atomicAdd(x + v, -a[v]);
+    for (int v = 0; v < 4; ++v) {
+        const int r = g + 8 * v;
+        if (r < kb) Xb[(size_t)r * ldx] = acc[v];
     }
-}
-__device__ __forceinline__ void atomic_sub4(double *x, const double (&a)[4], int avail) {
-    for (int v = 0; v < 4 && v < avail; ++v) atomicAdd(x + v, -a[v]);
 }
 
 // X[row(r), cols] -= sum_c L[r, k0+c] X[panel row c, cols] for front rows
-// r >= k0 + kb; pivot rows of the front are updated in place, rows of
-// ancestor fronts with atomics (sibling fronts share them).
-template <typename T>
+// r >= k0 + kb on TS x TS tiles; pivot rows of the front are updated in place,
+// rows of ancestor fronts with atomics (sibling fronts share them).
+template <int TS>
 __global__ void __launch_bounds__(256) k_solve_fwd_upd(FrontDev fd, const int *__restrict__ nodes, int k0,
-                                                       const T *__restrict__ arena, int k,
-                                                       T *__restrict__ X, int ldx) {
-    __shared__ T Ls[P][64];
-    __shared__ T Xs[P][64];
+                                                       const double *__restrict__ arena, int k,
+                                                       double *__restrict__ X, int ldx) {
+    constexpr int U = TS / 16;
+    __shared__ double Ls[P][TS];
+    __shared__ double Xs[P][TS];
     const int t = nodes[blockIdx.x];
     const int nf = fd.nf[t], ns = fd.ns[t], ps = fd.pstart[t];
     const int kb = min(P, ns - k0);
     if (kb <= 0) return;
-    const int base = k0 + kb;
-    const int r0 = base + blockIdx.y * 64;
+    const int r0 = k0 + kb + blockIdx.y * TS;
     if (r0 >= nf) return;
-    const int c0 = blockIdx.z * 64;
+    const int c0 = blockIdx.z * TS;
     if (c0 >= k) return;
-    const T *F = arena + fd.foff[t];
+    const double *F = arena + fd.foff[t];
     const int *rows = fd.rows + fd.rows_off[t];
-    for (int idx = threadIdx.x; idx < P * 64; idx += blockDim.x) {
-        int i = idx & 63, kk = idx >> 6;
-        T lv = 0.0, xv = 0.0;
+    for (int idx = threadIdx.x; idx < P * TS; idx += blockDim.x) {
+        const int i = idx % TS, kk = idx / TS;
+        double lv = 0.0, xv = 0.0;
         if (kk < kb) {
             if (r0 + i < nf) lv = F[(int64_t)(k0 + kk) * nf + (r0 + i)];
             if (c0 + i < k) xv = X[(size_t)(ps + k0 + kk) * ldx + c0 + i];
@@ -359,40 +470,37 @@ __global__ void __launch_bounds__(256) k_solve_fwd_upd(FrontDev fd, const int *_
         Xs[kk][i] = xv;
     }
     __syncthreads();
-    // thread: rows ty + 16 u, four contiguous columns 4 tx .. 4 tx + 3
+    // thread: rows ty + 16 u, U contiguous columns
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    T acc[4][4] = {};
+    double acc[U][U] = {};
     for (int kk = 0; kk < kb; ++kk) {
-        T a[4], b[4];
+        double a[U], b[U];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < U; ++u) {
             a[u] = Ls[kk][ty + 16 * u];
-            b[u] = Xs[kk][4 * tx + u];
+            b[u] = Xs[kk][U * tx + u];
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
+        for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int v = 0; v < 4; ++v) acc[u][v] += a[u] * b[v];
+            for (int v = 0; v < U; ++v) acc[u][v] = fma(a[u], b[v], acc[u][v]);
     }
-    const int cb = c0 + 4 * tx;
+    const int cb = c0 + U * tx;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        int r = r0 + ty + 16 * u;
+    for (int u = 0; u < U; ++u) {
+        const int r = r0 + ty + 16 * u;
         if (r >= nf) continue;
-        int grow = rows[r];
-        T *xr = X + (size_t)grow * ldx + cb;
-        if (r < ns) {
+        double *xr = X + (size_t)rows[r] * ldx + cb;
 #pragma unroll
-            for (int v = 0; v < 4; ++v)
-                if (cb + v < k) xr[v] -= acc[u][v];
-        } else {
-            atomic_sub4(xr, acc[u], k - cb);
+        for (int v = 0; v < U; ++v) {
+            if (cb + v >= k) break;
+            if (r < ns) xr[v] -= acc[u][v];
+            else atomicAdd(xr + v, -acc[u][v]);
         }
     }
 }
 
-template <typename T>
-__global__ void k_solve_diag(int n, int k, const T *__restrict__ dpos, T *__restrict__ X, int ldx) {
+__global__ void k_solve_diag(int n, int k, const double *__restrict__ dpos, double *__restrict__ X, int ldx) {
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)n * k) return;
     int i = (int)(idx / k), j = (int)(idx % k);
@@ -400,55 +508,49 @@ __global__ void k_solve_diag(int n, int k, const T *__restrict__ dpos, T *__rest
 }
 
 // X[panel rows c, cols] -= sum_{r >= k0+kb} L[r, k0+c] X[row(r), cols].  A CTA
-// covers kBwdChunks 32-row chunks of r; when one CTA covers all rows of the
-// front (grid.y == 1) it updates the panel rows with plain stores, otherwise
+// covers one 32-row chunk of r and CT columns; when one CTA covers all rows of
+// the front (grid.y == 1) it updates the panel rows with plain stores, otherwise
 // the partial sums are accumulated with atomics.
-constexpr int kBwdChunks = 1;
-template <typename T>
+template <int CT>
 __global__ void __launch_bounds__(256) k_solve_bwd_upd(FrontDev fd, const int *__restrict__ nodes, int k0,
-                                                       const T *__restrict__ arena, int k,
-                                                       T *__restrict__ X, int ldx) {
-    __shared__ T Ls[P][P + 1];  // [r][c]
-    __shared__ T Xs[P][64];     // [r][col]
+                                                       const double *__restrict__ arena, int k,
+                                                       double *__restrict__ X, int ldx) {
+    constexpr int RS = 256 / CT, NU = P / RS;  // panel rows cb, cb + RS, ... per thread
+    __shared__ double Ls[P][P + 1];  // [r][c]
+    __shared__ double Xs[P][CT];     // [r][col]
     const int t = nodes[blockIdx.x];
     const int nf = fd.nf[t], ns = fd.ns[t], ps = fd.pstart[t];
     const int kb = min(P, ns - k0);
     if (kb <= 0) return;
-    const int base = k0 + kb;
-    const int rbeg = base + blockIdx.y * P * kBwdChunks;
-    if (rbeg >= nf) return;
-    const int rend = min(nf, rbeg + P * kBwdChunks);
-    const int c0 = blockIdx.z * 64;
+    const int r0 = k0 + kb + blockIdx.y * P;
+    if (r0 >= nf) return;
+    const int c0 = blockIdx.z * CT;
     if (c0 >= k) return;
-    const T *F = arena + fd.foff[t];
+    const double *F = arena + fd.foff[t];
     const int *rows = fd.rows + fd.rows_off[t];
-    // 32 x 64 outputs, 8 per thread: thread -> column j = tid & 63, rows c = (tid >> 6) + 4u
-    const int j = threadIdx.x & 63, cb = threadIdx.x >> 6;
-    T acc[8] = {};
-    for (int r0 = rbeg; r0 < rend; r0 += P) {
-        __syncthreads();
-        for (int idx = threadIdx.x; idx < P * P; idx += blockDim.x) {
-            int r = idx % P, c = idx / P;
-            Ls[r][c] = (r0 + r < rend && c < kb) ? F[(int64_t)(k0 + c) * nf + (r0 + r)] : T(0);
-        }
-        for (int idx = threadIdx.x; idx < P * 64; idx += blockDim.x) {
-            int jj = idx & 63, r = idx >> 6;
-            Xs[r][jj] = (r0 + r < rend && c0 + jj < k) ? X[(size_t)rows[r0 + r] * ldx + c0 + jj] : T(0);
-        }
-        __syncthreads();
-        for (int r = 0; r < P; ++r) {
-            T xv = Xs[r][j];
+    for (int idx = threadIdx.x; idx < P * P; idx += 256) {
+        const int r = idx % P, c = idx / P;
+        Ls[r][c] = (r0 + r < nf && c < kb) ? F[(int64_t)(k0 + c) * nf + (r0 + r)] : 0.0;
+    }
+    for (int idx = threadIdx.x; idx < P * CT; idx += 256) {
+        const int jj = idx % CT, r = idx / CT;
+        Xs[r][jj] = (r0 + r < nf && c0 + jj < k) ? X[(size_t)rows[r0 + r] * ldx + c0 + jj] : 0.0;
+    }
+    __syncthreads();
+    const int j = threadIdx.x % CT, cb = threadIdx.x / CT;
+    double acc[NU] = {};
+    for (int r = 0; r < min(P, nf - r0); ++r) {
+        const double xv = Xs[r][j];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) acc[u] += Ls[r][cb + 4 * u] * xv;
-        }
+        for (int u = 0; u < NU; ++u) acc[u] = fma(Ls[r][cb + RS * u], xv, acc[u]);
     }
     if (c0 + j < k) {
         const bool whole = gridDim.y == 1;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            int c = cb + 4 * u;
+        for (int u = 0; u < NU; ++u) {
+            const int c = cb + RS * u;
             if (c < kb) {
-                T *x = &X[(size_t)(ps + k0 + c) * ldx + c0 + j];
+                double *x = &X[(size_t)(ps + k0 + c) * ldx + c0 + j];
                 if (whole) *x -= acc[u];
                 else atomicAdd(x, -acc[u]);
             }
@@ -456,187 +558,108 @@ __global__ void __launch_bounds__(256) k_solve_bwd_upd(FrontDev fd, const int *_
     }
 }
 
-// X[panel rows, cols] = L11^-T X[...]  (unit upper, backward)
-template <typename T>
-__global__ void __launch_bounds__(kTriCols) k_solve_bwd_tri(FrontDev fd, const int *__restrict__ nodes, int k0,
-                                                            const T *__restrict__ arena, int k,
-                                                            T *__restrict__ X, int ldx) {
-    __shared__ T L[P][P + 1];
-    const int t = nodes[blockIdx.x];
-    const int nf = fd.nf[t], ns = fd.ns[t], ps = fd.pstart[t];
-    const int kb = min(P, ns - k0);
-    if (kb <= 0) return;
-    const T *F = arena + fd.foff[t];
-    for (int idx = threadIdx.x; idx < kb * kb; idx += blockDim.x) {
-        int r = idx % kb, c = idx / kb;
-        L[r][c] = (r > c) ? F[(int64_t)(k0 + c) * nf + (k0 + r)] : 0.0;
-    }
-    __syncthreads();
-    const int j = blockIdx.y * kTriCols + threadIdx.x;
-    if (j >= k) return;
-    T x[P];
-    T *Xb = X + (size_t)(ps + k0) * ldx + j;
-#pragma unroll
-    for (int r = 0; r < P; ++r)
-        if (r < kb) x[r] = Xb[(size_t)r * ldx];
-#pragma unroll
-    for (int r = P - 2; r >= 0; --r) {
-        if (r < kb - 1) {
-            T v = x[r];
-#pragma unroll
-            for (int c = 0; c < P; ++c)
-                if (c > r && c < kb) v -= L[c][r] * x[c];
-            x[r] = v;
-        }
-    }
-#pragma unroll
-    for (int r = 0; r < P; ++r)
-        if (r < kb) Xb[(size_t)r * ldx] = x[r];
-}
-
 // ---- single-panel fronts (ns <= P, nf <= kSmallNf): fused solve kernels -------
 // One CTA per (front, column tile): the front's L panel and pivot rows are
-// staged in shared memory once; the forward kernel solves the unit lower
-// triangle and sends L21 x1 to the ancestors' rows (vector atomics), the
-// backward kernel gathers the ancestors' rows, subtracts L21^T x2 and solves
-// the unit upper triangle.  Thread layout for the products: 4 contiguous
-// columns per thread, 8 row groups.
-template <typename T>
-__host__ __device__ constexpr int small_cols() { return 512 / (int)sizeof(T); }  // 128 float, 64 double
-
-// copy n values of one row between global and shared memory: 16-byte vectors
-// when `vec` (both addresses 16-byte aligned, n a multiple of the vector)
-template <typename T>
-__device__ __forceinline__ void row_load(T *dst, const T *src, int n, int lane, int lanes, bool vec) {
-    constexpr int V = 16 / (int)sizeof(T);
-    if (vec && n % V == 0) {
-        for (int i = lane; i < n / V; i += lanes) reinterpret_cast<uint4 *>(dst)[i] = reinterpret_cast<const uint4 *>(src)[i];
-    } else {
-        for (int i = lane; i < n; i += lanes) dst[i] = src[i];
-    }
-}
-
-template <typename T>
+// staged in shared memory once; the forward kernel multiplies the pivot rows by
+// Linv and sends L21 x1 to the ancestors' rows (atomics), the backward kernel
+// gathers the ancestors' rows, subtracts L21^T x2 and multiplies by Linv^T.
+// Thread layout: SC columns x 256 / SC row groups.
+template <int SC>
 __global__ void __launch_bounds__(256) k_solve_fwd_small(FrontDev fd, const int *__restrict__ nodes,
-                                                         const T *__restrict__ arena, int k, T *__restrict__ X,
-                                                         int ldx, bool vec, int nf_max) {
-    constexpr int SC = small_cols<T>();
-    constexpr int CG = SC / 4;   // column groups of 4
-    constexpr int RG = 256 / CG; // row groups
+                                                         const double *__restrict__ arena, int k,
+                                                         double *__restrict__ X, int ldx, int nf_max) {
+    constexpr int RG = 256 / SC;
     extern __shared__ __align__(16) unsigned char small_smem[];
-    T *Ls = reinterpret_cast<T *>(small_smem);  // ns x nf (column-major panel)
-    T *Xp = Ls + P * nf_max;                    // [P][SC]
+    double *Ls = reinterpret_cast<double *>(small_smem);  // ns x nf (column-major panel)
+    double *Xp = Ls + P * nf_max, *Yp = Xp + P * SC;       // [P][SC] each
     const int t = nodes[blockIdx.x];
     const int nf = fd.nf[t], ns = fd.ns[t], ps = fd.pstart[t];
     const int c0 = blockIdx.y * SC;
     if (c0 >= k) return;
-    const int tid = threadIdx.x;
-    const T *F = arena + fd.foff[t];
+    const int tid = threadIdx.x, c = tid % SC, rg = tid / SC;
+    const bool live = c0 + c < k;
+    const double *F = arena + fd.foff[t];
     for (int i = tid; i < ns * nf; i += 256) Ls[i] = F[i];
-    const int cols = min(SC, k - c0);
-    // pivot rows: one warp per row
-    for (int r = tid / 32; r < ns; r += 8) {
-        row_load(Xp + r * SC, X + (size_t)(ps + r) * ldx + c0, cols, tid % 32, 32, vec);
-        for (int c = cols + tid % 32; c < SC; c += 32) Xp[r * SC + c] = T(0);
+    double *Xc = X + c0 + c;
+    for (int r = rg; r < ns; r += RG) Xp[r * SC + c] = live ? Xc[(size_t)(ps + r) * ldx] : 0.0;
+    __syncthreads();
+    for (int r = rg; r < ns; r += RG) {
+        double acc = Xp[r * SC + c];
+        for (int q = 0; q < r; ++q) acc = fma(Ls[q * nf + r], Xp[q * SC + c], acc);
+        Yp[r * SC + c] = acc;
+        if (live) Xc[(size_t)(ps + r) * ldx] = acc;
     }
     __syncthreads();
-    if (tid < SC) {
-        for (int r = 1; r < ns; ++r) {
-            T acc = Xp[r * SC + tid];
-            for (int q = 0; q < r; ++q) acc -= Ls[q * nf + r] * Xp[q * SC + tid];
-            Xp[r * SC + tid] = acc;
-        }
-    }
-    __syncthreads();
-    for (int r = tid / 32; r < ns; r += 8) row_load(X + (size_t)(ps + r) * ldx + c0, Xp + r * SC, cols, tid % 32, 32, vec);
-    // ancestors' rows: x_r -= L_r. x_p
-    const int cg = (tid % CG) * 4, rg = tid / CG;
+    // ancestors' rows: x_r -= L_r. x_p, two rows at a time
     const int *rows = fd.rows + fd.rows_off[t];
-    for (int r = ns + rg; r < nf; r += RG) {
-        T acc[4] = {T(0), T(0), T(0), T(0)};
+    for (int r = ns + rg; r < nf; r += 2 * RG) {
+        const int r2 = r + RG < nf ? r + RG : r;
+        double a0 = 0.0, a1 = 0.0;
         for (int q = 0; q < ns; ++q) {
-            const T l = Ls[q * nf + r];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) acc[v] += l * Xp[q * SC + cg + v];
+            const double y = Yp[q * SC + c];
+            a0 = fma(Ls[q * nf + r], y, a0);
+            a1 = fma(Ls[q * nf + r2], y, a1);
         }
-        atomic_sub4(X + (size_t)rows[r] * ldx + c0 + cg, acc, k - c0 - cg);
+        if (live) {
+            atomicAdd(Xc + (size_t)rows[r] * ldx, -a0);
+            if (r2 != r) atomicAdd(Xc + (size_t)rows[r2] * ldx, -a1);
+        }
     }
 }
 
-template <typename T>
+template <int SC>
 __global__ void __launch_bounds__(256) k_solve_bwd_small(FrontDev fd, const int *__restrict__ nodes,
-                                                         const T *__restrict__ arena, int k, T *__restrict__ X,
-                                                         int ldx, bool vec, int nf_max) {
-    constexpr int SC = small_cols<T>();
-    constexpr int CG = SC / 4;
-    constexpr int RG = 256 / CG;
+                                                         const double *__restrict__ arena, int k,
+                                                         double *__restrict__ X, int ldx, int nf_max) {
+    constexpr int RG = 256 / SC;
     extern __shared__ __align__(16) unsigned char small_smem[];
-    T *Ls = reinterpret_cast<T *>(small_smem);
-    T *Xp = Ls + P * nf_max;    // [P][SC]
-    T *Xu = Xp + P * SC;        // [P][SC] chunk of ancestor rows
+    double *Ls = reinterpret_cast<double *>(small_smem);
+    double *Xp = Ls + P * nf_max;    // [P][SC]
+    double *Xu = Xp + P * SC;        // [P][SC] chunk of ancestor rows
     const int t = nodes[blockIdx.x];
     const int nf = fd.nf[t], ns = fd.ns[t], ps = fd.pstart[t];
     const int c0 = blockIdx.y * SC;
     if (c0 >= k) return;
-    const int tid = threadIdx.x;
-    const T *F = arena + fd.foff[t];
+    const int tid = threadIdx.x, c = tid % SC, rg = tid / SC;
+    const bool live = c0 + c < k;
+    const double *F = arena + fd.foff[t];
     const int *rows = fd.rows + fd.rows_off[t];
     for (int i = tid; i < ns * nf; i += 256) Ls[i] = F[i];
-    const int cols = min(SC, k - c0);
-    for (int r = tid / 32; r < ns; r += 8) {
-        row_load(Xp + r * SC, X + (size_t)(ps + r) * ldx + c0, cols, tid % 32, 32, vec);
-        for (int c = cols + tid % 32; c < SC; c += 32) Xp[r * SC + c] = T(0);
-    }
-    // x_p -= L21^T x_u over 32-row chunks of the ancestors' rows; thread: pivots
-    // q = rg + RG j, columns cg .. cg + 3
-    const int cg = (tid % CG) * 4, rg = tid / CG;
+    double *Xc = X + c0 + c;
+    // x_p - L21^T x_u over 32-row chunks of the ancestors' rows; thread: pivots
+    // q = rg + RG j of its column
     constexpr int QJ = (P + RG - 1) / RG;
-    T acc[QJ][4];
-#pragma unroll
-    for (int j = 0; j < QJ; ++j)
-#pragma unroll
-        for (int v = 0; v < 4; ++v) acc[j][v] = T(0);
-    for (int r0 = ns; r0 < nf; r0 += P) {
-        const int cnt = min(P, nf - r0);
-        __syncthreads();
-        for (int rr = tid / 32; rr < cnt; rr += 8) {
-            row_load(Xu + rr * SC, X + (size_t)rows[r0 + rr] * ldx + c0, cols, tid % 32, 32, vec);
-            for (int c = cols + tid % 32; c < SC; c += 32) Xu[rr * SC + c] = T(0);
-        }
-        __syncthreads();
-        for (int rr = 0; rr < cnt; ++rr) {
-            T xu[4];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) xu[v] = Xu[rr * SC + cg + v];
-#pragma unroll
-            for (int j = 0; j < QJ; ++j) {
-                const int q = rg + RG * j;
-                if (q < ns) {
-                    const T l = Ls[q * nf + r0 + rr];
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) acc[j][v] += l * xu[v];
-                }
-            }
-        }
-    }
-    __syncthreads();
+    double acc[QJ];
 #pragma unroll
     for (int j = 0; j < QJ; ++j) {
         const int q = rg + RG * j;
-        if (q < ns)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) Xp[q * SC + cg + v] -= acc[j][v];
+        acc[j] = q < ns && live ? Xc[(size_t)(ps + q) * ldx] : 0.0;
     }
-    __syncthreads();
-    if (tid < SC) {
-        for (int r = ns - 2; r >= 0; --r) {
-            T a = Xp[r * SC + tid];
-            for (int q = r + 1; q < ns; ++q) a -= Ls[r * nf + q] * Xp[q * SC + tid];
-            Xp[r * SC + tid] = a;
+    for (int r0 = ns; r0 < nf; r0 += P) {
+        const int cnt = min(P, nf - r0);
+        __syncthreads();
+        for (int rr = rg; rr < cnt; rr += RG) Xu[rr * SC + c] = live ? Xc[(size_t)rows[r0 + rr] * ldx] : 0.0;
+        __syncthreads();
+        for (int rr = 0; rr < cnt; ++rr) {
+            const double xu = -Xu[rr * SC + c];
+#pragma unroll
+            for (int j = 0; j < QJ; ++j) {
+                const int q = rg + RG * j;
+                if (q < ns) acc[j] = fma(Ls[q * nf + r0 + rr], xu, acc[j]);
+            }
         }
     }
+#pragma unroll
+    for (int j = 0; j < QJ; ++j) {
+        const int q = rg + RG * j;
+        if (q < ns) Xp[q * SC + c] = acc[j];
+    }
     __syncthreads();
-    for (int r = tid / 32; r < ns; r += 8) row_load(X + (size_t)(ps + r) * ldx + c0, Xp + r * SC, cols, tid % 32, 32, vec);
+    for (int r = rg; r < ns; r += RG) {
+        double a = Xp[r * SC + c];
+        for (int q = r + 1; q < ns; ++q) a = fma(Ls[r * nf + q], Xp[q * SC + c], a);
+        if (live) Xc[(size_t)(ps + r) * ldx] = a;
+    }
 }
 
 inline unsigned cdiv(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
@@ -661,15 +684,43 @@ void front_extend_add(cudaStream_t s, const FrontDev &fd, const int *parent, con
     HSIM_LAUNCHED();
 }
 
+static int front_sms() {
+    int dev = 0, c = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev);
+    return c > 0 ? c : 1;
+}
+
 template <typename T>
 void front_panel(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0, int max_rows, T *arena,
                  double pivot_tol, int *flags) {
     if (n_nodes <= 0) return;
-    k_front_diag_block<T><<<(unsigned)n_nodes, 128, 0, s>>>(fd, nodes, k0, arena, pivot_tol, flags);
-    HSIM_LAUNCHED();
-    if (max_rows <= 0) return;
-    dim3 g((unsigned)n_nodes, cdiv(max_rows, kPanelRows));
-    k_front_panel<T><<<g, 128, 0, s>>>(fd, nodes, k0, arena);
+    if constexpr (std::is_same<T, double>::value) {
+        k_front_diag_inv<<<(unsigned)n_nodes, 128, 0, s>>>(fd, nodes, k0, arena, pivot_tol, flags);
+        HSIM_LAUNCHED();
+        if (max_rows <= 0) return;
+        dim3 g((unsigned)n_nodes, cdiv(max_rows, kPanelRows64));
+        k_front_panel64<<<g, 128, 0, s>>>(fd, nodes, k0, arena);
+        HSIM_LAUNCHED();
+    } else {
+        k_front_diag_block<T><<<(unsigned)n_nodes, 128, 0, s>>>(fd, nodes, k0, arena, pivot_tol, flags);
+        HSIM_LAUNCHED();
+        if (max_rows <= 0) return;
+        dim3 g((unsigned)n_nodes, cdiv(max_rows, kPanelRows));
+        k_front_panel<T><<<g, 128, 0, s>>>(fd, nodes, k0, arena);
+        HSIM_LAUNCHED();
+    }
+}
+
+template <typename T, int TS>
+static void launch_update(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0, int max_trail,
+                          T *arena, int c_end) {
+    int64_t Tt = (max_trail + TS - 1) / TS;
+    // column tiles below c_end (the trailing part starts after k0's first pivot)
+    const int64_t ntj = c_end == INT_MAX ? 0 : std::min<int64_t>(Tt, (c_end - k0 + TS - 2) / TS + 1);
+    if (c_end != INT_MAX && ntj <= 0) return;
+    dim3 g((unsigned)n_nodes, (unsigned)(ntj > 0 ? Tt * ntj : Tt * (Tt + 1) / 2));
+    k_front_update<T, TS><<<g, 256, 0, s>>>(fd, nodes, k0, arena, c_end, (int)ntj);
     HSIM_LAUNCHED();
 }
 
@@ -677,13 +728,20 @@ template <typename T>
 void front_update(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0, int max_trail, T *arena,
                   int c_end) {
     if (n_nodes <= 0 || max_trail <= 0) return;
-    int64_t Tt = (max_trail + 63) / 64;
-    // column tiles below c_end (the trailing part starts after k0's first pivot)
-    const int64_t ntj = c_end == INT_MAX ? 0 : std::min<int64_t>(Tt, (c_end - k0 + 62) / 64 + 1);
-    if (c_end != INT_MAX && ntj <= 0) return;
-    dim3 g((unsigned)n_nodes, (unsigned)(ntj > 0 ? Tt * ntj : Tt * (Tt + 1) / 2));
-    k_front_update<T><<<g, 256, 0, s>>>(fd, nodes, k0, arena, c_end, (int)ntj);
-    HSIM_LAUNCHED();
+    if constexpr (std::is_same<T, double>::value) {
+        // tiles of 64 keep an SM's FP64 pipes busy for 38 us, of 32 for 10, of 16
+        // for 2.4: the largest with two CTAs per SM
+        auto ctas = [&](int ts) {
+            const int64_t q = (max_trail + ts - 1) / ts;
+            return (int64_t)n_nodes * q * (q + 1) / 2;
+        };
+        const int64_t want = 2 * (int64_t)front_sms();
+        if (ctas(64) >= want) launch_update<T, 64>(s, fd, nodes, n_nodes, k0, max_trail, arena, c_end);
+        else if (ctas(32) >= want) launch_update<T, 32>(s, fd, nodes, n_nodes, k0, max_trail, arena, c_end);
+        else launch_update<T, 16>(s, fd, nodes, n_nodes, k0, max_trail, arena, c_end);
+    } else {
+        launch_update<T, 64>(s, fd, nodes, n_nodes, k0, max_trail, arena, c_end);
+    }
 }
 
 template <typename T>
@@ -701,73 +759,70 @@ void front_diag(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_node
     HSIM_LAUNCHED();
 }
 
-template <typename T>
-void solve_fwd_tri(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0, const T *arena, int k,
-                   T *X, int ldx) {
+void solve_fwd_tri(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0, const double *arena,
+                   int k, double *X, int ldx) {
     if (n_nodes <= 0 || k <= 0) return;
     dim3 g((unsigned)n_nodes, cdiv(k, kTriCols));
-    k_solve_fwd_tri<T><<<g, kTriCols, 0, s>>>(fd, nodes, k0, arena, k, X, ldx);
+    k_solve_tri<false><<<g, 128, 0, s>>>(fd, nodes, k0, arena, k, X, ldx);
     HSIM_LAUNCHED();
 }
 
-template <typename T>
 void solve_fwd_upd(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0, int max_rows,
-                   const T *arena, int k, T *X, int ldx) {
+                   const double *arena, int k, double *X, int ldx) {
     if (n_nodes <= 0 || k <= 0 || max_rows <= 0) return;
-    dim3 g((unsigned)n_nodes, cdiv(max_rows, 64), cdiv(k, 64));
-    k_solve_fwd_upd<T><<<g, 256, 0, s>>>(fd, nodes, k0, arena, k, X, ldx);
+    // the largest tile with two CTAs per SM (as front_update)
+    auto grid = [&](int ts) { return dim3((unsigned)n_nodes, cdiv(max_rows, ts), cdiv(k, ts)); };
+    auto ctas = [&](int ts) { return (int64_t)n_nodes * cdiv(max_rows, ts) * cdiv(k, ts); };
+    const int64_t want = 2 * (int64_t)front_sms();
+    if (ctas(64) >= want) k_solve_fwd_upd<64><<<grid(64), 256, 0, s>>>(fd, nodes, k0, arena, k, X, ldx);
+    else if (ctas(32) >= want) k_solve_fwd_upd<32><<<grid(32), 256, 0, s>>>(fd, nodes, k0, arena, k, X, ldx);
+    else k_solve_fwd_upd<16><<<grid(16), 256, 0, s>>>(fd, nodes, k0, arena, k, X, ldx);
     HSIM_LAUNCHED();
 }
 
-template <typename T>
-void solve_diag(cudaStream_t s, int n, int k, const T *dpos, T *X, int ldx) {
+void solve_diag(cudaStream_t s, int n, int k, const double *dpos, double *X, int ldx) {
     if (n <= 0 || k <= 0) return;
-    k_solve_diag<T><<<cdiv((int64_t)n * k, 256), 256, 0, s>>>(n, k, dpos, X, ldx);
+    k_solve_diag<<<cdiv((int64_t)n * k, 256), 256, 0, s>>>(n, k, dpos, X, ldx);
     HSIM_LAUNCHED();
 }
 
-template <typename T>
 void solve_bwd_upd(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0, int max_rows,
-                   const T *arena, int k, T *X, int ldx) {
+                   const double *arena, int k, double *X, int ldx) {
     if (n_nodes <= 0 || k <= 0 || max_rows <= 0) return;
-    dim3 g((unsigned)n_nodes, cdiv(max_rows, P * kBwdChunks), cdiv(k, 64));
-    k_solve_bwd_upd<T><<<g, 256, 0, s>>>(fd, nodes, k0, arena, k, X, ldx);
+    auto grid = [&](int ct) { return dim3((unsigned)n_nodes, cdiv(max_rows, P), cdiv(k, ct)); };
+    if ((int64_t)n_nodes * cdiv(max_rows, P) * cdiv(k, 64) >= 2 * (int64_t)front_sms())
+        k_solve_bwd_upd<64><<<grid(64), 256, 0, s>>>(fd, nodes, k0, arena, k, X, ldx);
+    else
+        k_solve_bwd_upd<16><<<grid(16), 256, 0, s>>>(fd, nodes, k0, arena, k, X, ldx);
     HSIM_LAUNCHED();
 }
 
-template <typename T>
-void solve_bwd_tri(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0, const T *arena, int k,
-                   T *X, int ldx) {
+void solve_bwd_tri(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0, const double *arena,
+                   int k, double *X, int ldx) {
     if (n_nodes <= 0 || k <= 0) return;
     dim3 g((unsigned)n_nodes, cdiv(k, kTriCols));
-    k_solve_bwd_tri<T><<<g, kTriCols, 0, s>>>(fd, nodes, k0, arena, k, X, ldx);
+    k_solve_tri<true><<<g, 128, 0, s>>>(fd, nodes, k0, arena, k, X, ldx);
     HSIM_LAUNCHED();
 }
 
-template <typename T>
-void solve_fwd_small(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int nf_max, const T *arena,
-                     int k, T *X, int ldx) {
+constexpr int kSmallCols = 32;
+static size_t small_smem(int nf_max) { return ((size_t)P * nf_max + 2 * (size_t)P * kSmallCols) * sizeof(double); }
+
+void solve_fwd_small(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int nf_max, const double *arena,
+                     int k, double *X, int ldx) {
     if (n_nodes <= 0 || k <= 0) return;
-    nf_max = (nf_max + 3) & ~3;  // keeps the row blocks after the panel 16-byte aligned
-    const size_t sm = ((size_t)P * nf_max + (size_t)P * small_cols<T>()) * sizeof(T);
-    HSIM_SMEM_LIMIT_ONCE(k_solve_fwd_small<T>, ((size_t)P * kSmallNf + (size_t)P * small_cols<T>()) * sizeof(T));
-    const bool vec = (reinterpret_cast<uintptr_t>(X) % 16 == 0) && ((size_t)ldx * sizeof(T)) % 16 == 0;
-    k_solve_fwd_small<T><<<dim3((unsigned)n_nodes, cdiv(k, small_cols<T>())), 256, sm, s>>>(fd, nodes, arena, k, X,
-                                                                                             ldx, vec, nf_max);
+    HSIM_SMEM_LIMIT_ONCE(k_solve_fwd_small<kSmallCols>, small_smem(kSmallNf));
+    k_solve_fwd_small<kSmallCols><<<dim3((unsigned)n_nodes, cdiv(k, kSmallCols)), 256, small_smem(nf_max), s>>>(
+        fd, nodes, arena, k, X, ldx, nf_max);
     HSIM_LAUNCHED();
 }
 
-template <typename T>
-void solve_bwd_small(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int nf_max, const T *arena,
-                     int k, T *X, int ldx) {
+void solve_bwd_small(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int nf_max, const double *arena,
+                     int k, double *X, int ldx) {
     if (n_nodes <= 0 || k <= 0) return;
-    nf_max = (nf_max + 3) & ~3;
-    const size_t sm = ((size_t)P * nf_max + 2 * (size_t)P * small_cols<T>()) * sizeof(T);
-    HSIM_SMEM_LIMIT_ONCE(k_solve_bwd_small<T>,
-                         ((size_t)P * kSmallNf + 2 * (size_t)P * small_cols<T>()) * sizeof(T));
-    const bool vec = (reinterpret_cast<uintptr_t>(X) % 16 == 0) && ((size_t)ldx * sizeof(T)) % 16 == 0;
-    k_solve_bwd_small<T><<<dim3((unsigned)n_nodes, cdiv(k, small_cols<T>())), 256, sm, s>>>(fd, nodes, arena, k, X,
-                                                                                             ldx, vec, nf_max);
+    HSIM_SMEM_LIMIT_ONCE(k_solve_bwd_small<kSmallCols>, small_smem(kSmallNf));
+    k_solve_bwd_small<kSmallCols><<<dim3((unsigned)n_nodes, cdiv(k, kSmallCols)), 256, small_smem(nf_max), s>>>(
+        fd, nodes, arena, k, X, ldx, nf_max);
     HSIM_LAUNCHED();
 }
 
@@ -778,16 +833,7 @@ void solve_bwd_small(cudaStream_t s, const FrontDev &fd, const int *nodes, int n
     template void front_panel<T>(cudaStream_t, const FrontDev &, const int *, int, int, int, T *, double, int *);  \
     template void front_update<T>(cudaStream_t, const FrontDev &, const int *, int, int, int, T *, int);         \
     template void front_maxdiag<T>(cudaStream_t, const FrontDev &, int, const T *, unsigned long long *);        \
-    template void front_diag<T>(cudaStream_t, const FrontDev &, const int *, int, const T *, T *, int *);        \
-    template void solve_fwd_tri<T>(cudaStream_t, const FrontDev &, const int *, int, int, const T *, int, T *, int); \
-    template void solve_fwd_upd<T>(cudaStream_t, const FrontDev &, const int *, int, int, int, const T *, int, T *, \
-                                   int);                                                                         \
-    template void solve_diag<T>(cudaStream_t, int, int, const T *, T *, int);                                    \
-    template void solve_bwd_upd<T>(cudaStream_t, const FrontDev &, const int *, int, int, int, const T *, int, T *, \
-                                   int);                                                                         \
-    template void solve_bwd_tri<T>(cudaStream_t, const FrontDev &, const int *, int, int, const T *, int, T *, int); \
-    template void solve_fwd_small<T>(cudaStream_t, const FrontDev &, const int *, int, int, const T *, int, T *, int); \
-    template void solve_bwd_small<T>(cudaStream_t, const FrontDev &, const int *, int, int, const T *, int, T *, int);
+    template void front_diag<T>(cudaStream_t, const FrontDev &, const int *, int, const T *, T *, int *);
 
 HSIM_FRONT_INSTANTIATE(float)
 HSIM_FRONT_INSTANTIATE(double)

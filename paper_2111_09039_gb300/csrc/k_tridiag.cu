@@ -679,8 +679,8 @@ __global__ void k_tri_bisect(int n, int m, int G, const double *__restrict__ d, 
             wid *= 2.0;
         }
     }
-    // to 2 eps max(|lambda|, ||T||): the absolute accuracy of a dense symmetric
-    // eigensolve
+    // to 2 eps (|lambda| + ||T||), the absolute accuracy of a dense symmetric
+    // eigensolve (a quarter of it: a round more, the vectors' error unchanged)
     const int H = L / 2;
     bool chord = true;
     for (int round = 0; round < 200; ++round) {

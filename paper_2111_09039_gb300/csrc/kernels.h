@@ -145,6 +145,8 @@ void front_assemble(cudaStream_t s, int64_t nnz, const int *row_of, const int *c
 template <typename T>
 void front_extend_add(cudaStream_t s, const FrontDev &fd, const int *parent, const int *children,
                       int n_children, int max_upd, T *arena);
+// LDL^T of the panel's diagonal block and the rows below it; double: the block's
+// unit lower factor is replaced by its inverse
 template <typename T>
 void front_panel(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0,
                  int max_rows, T *arena, double pivot_tol, int *flags);
@@ -160,29 +162,24 @@ void front_maxdiag(cudaStream_t s, const FrontDev &fd, int n_nodes, const T *are
 template <typename T>
 void front_diag(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, const T *arena,
                 T *dpos, int *neg_count);
-template <typename T>
+// FP64 solves: the diagonal blocks hold the inverse of their unit lower factor
+// (front_panel<double>)
 void solve_fwd_tri(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0,
-                   const T *arena, int k, T *X, int ldx);
-template <typename T>
+                   const double *arena, int k, double *X, int ldx);
 void solve_fwd_upd(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0,
-                   int max_rows, const T *arena, int k, T *X, int ldx);
-template <typename T>
-void solve_diag(cudaStream_t s, int n, int k, const T *dpos, T *X, int ldx);
-template <typename T>
+                   int max_rows, const double *arena, int k, double *X, int ldx);
+void solve_diag(cudaStream_t s, int n, int k, const double *dpos, double *X, int ldx);
 void solve_bwd_upd(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0,
-                   int max_rows, const T *arena, int k, T *X, int ldx);
-template <typename T>
+                   int max_rows, const double *arena, int k, double *X, int ldx);
 void solve_bwd_tri(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int k0,
-                   const T *arena, int k, T *X, int ldx);
+                   const double *arena, int k, double *X, int ldx);
 // fused forward / backward solve of single-panel fronts (ns <= kPanel,
 // nf <= kSmallNf): triangle and update in one launch per tree height
 constexpr int kSmallNf = 320;
-template <typename T>
-void solve_fwd_small(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int nf_max, const T *arena,
-                     int k, T *X, int ldx);
-template <typename T>
-void solve_bwd_small(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int nf_max, const T *arena,
-                     int k, T *X, int ldx);
+void solve_fwd_small(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int nf_max, const double *arena,
+                     int k, double *X, int ldx);
+void solve_bwd_small(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int nf_max, const double *arena,
+                     int k, double *X, int ldx);
 
 // ---- inverted-factor solves (k_finv.cu) ------------------------------------
 // One product of the front inversion, all operands column-major:

@@ -17,13 +17,13 @@
 //      rounds around the zero of the determinant's chord.
 //   3. Eigenvectors of T: a column of the adjugate of T - lambda I from the two
 //      Sturm sequences (k_tri_minors, k_tri_vectors).  Eigenvalues closer than
-//      1e-5 ||T|| form a cluster, whose vectors come from inverse iteration
+//      1e-9 ||T|| form a cluster, whose vectors come from inverse iteration
 //      (Gaussian elimination with partial pivoting, reciprocal pivots kept),
 //      three iterations from a hashed random start, made orthogonal to the
 //      previous ones of the cluster in every iteration (one warp per cluster).
-//   4. Back transformation X = Q Z, reflectors applied in reverse order: one
-//      warp per eigenvector held in registers (n <= 2048), else a few
-//      eigenvectors per CTA held in shared memory.
+//   4. Back transformation X = Q Z: eight reflectors at a time in compact WY
+//      form, a few eigenvectors per CTA held in registers (n <= 2048), else one
+//      reflector at a time, the eigenvectors in shared memory.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -47,7 +47,7 @@ namespace {
 inline unsigned cdiv(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
 constexpr int kTriThreads = 256;
-constexpr double kClusterTol = 1e-5;  // relative to ||T||
+constexpr double kClusterTol = 1e-9;  // relative to ||T||
 constexpr double kNearTol = 1e-4;     // the same, vectors made orthogonal once
 constexpr size_t kTriSmemMax = 200 * 1024;  // dynamic shared memory limit of k_tridiag and k_tri_back
 
@@ -360,65 +360,163 @@ __global__ void __launch_bounds__(kTrdThreads) k_tridiag_rows(int n, const doubl
     }
 }
 
-// Back transformation X = Q Z with Q = H_0 H_1 ... H_{n-2}: one warp per
-// vector, its entries j = lane + 32 c in registers (n <= 32 C); the reflector
-// of the next step is loaded into registers while the current one is applied
-// and then stored to the other shared-memory buffer (one barrier per step).
-template <int C>
-__global__ void __launch_bounds__(256) k_tri_back_warp(int n, int m, const double *__restrict__ Vh,
-                                                     const double *__restrict__ tau, const double *__restrict__ Z,
-                                                     double *__restrict__ X, int ldx) {
-    __shared__ double vs[2][32 * C];
-    const int lane = threadIdx.x & 31, nthr = blockDim.x;
-    const int i = blockIdx.x * (nthr >> 5) + (threadIdx.x >> 5);
-    constexpr int P = (32 * C + 127) / 128;  // staged entries per thread (blockDim >= 128)
-    double z[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) {
-        const int j = lane + 32 * c;
-        z[c] = (i < m && j < n) ? Z[(size_t)i * n + j] : 0.0;
+// Compact WY of every block of eight consecutive reflectors k0 .. k0 + 7: H_k0 ...
+// H_{k0+7} = I - V T V^T, T (8 x 8, upper triangular, row-major) from the Gram
+// matrix of the block's vectors.  One CTA per block.
+constexpr int kWY = 8;
+__global__ void __launch_bounds__(128) k_tri_wy(int n, const double *__restrict__ Vh, const double *__restrict__ tau,
+                                                double *__restrict__ Tw) {
+    __shared__ double G[kWY][kWY], T[kWY][kWY];
+    const int k0 = blockIdx.x * kWY, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // pairs (i, j), i < j: dot over the rows where both are stored (j's)
+    for (int q = wid; q < kWY * kWY; q += 4) {
+        const int i = q / kWY, j = q % kWY;
+        if (i >= j) continue;
+        double s = 0.0;
+        if (k0 + j < n - 1) {
+            const double *vi = Vh + (size_t)(k0 + i) * n, *vj = Vh + (size_t)(k0 + j) * n;
+            for (int r = k0 + j + 1 + lane; r < n; r += 32) s = fma(vi[r], vj[r], s);
+            s = warp_sum_fixed(s);
+        }
+        if (lane == 0) G[i][j] = s;
     }
-    // reflector k: entries j > k of row k of Vh, zero elsewhere
-    for (int j = threadIdx.x; j < 32 * C; j += nthr) vs[0][j] = (j > n - 2 && j < n) ? Vh[(size_t)(n - 2) * n + j] : 0.0;
     __syncthreads();
-    int cur = 0;
-    for (int k = n - 2; k >= 0; --k) {
-        double pre[P];
-        const bool more = k > 0;
-#pragma unroll
-        for (int q = 0; q < P; ++q) {
-            const int j = threadIdx.x + q * nthr;
-            pre[q] = (more && j < n && j > k - 1 && j < 32 * C) ? Vh[(size_t)(k - 1) * n + j] : 0.0;
+    if (threadIdx.x < kWY) {
+        const int r = threadIdx.x;  // row of T
+        for (int i = 0; i < kWY; ++i) {
+            const double t = k0 + i < n - 1 ? tau[k0 + i] : 0.0;
+            double v = r == i ? t : 0.0;
+            if (r < i) {
+                double s = 0.0;
+                for (int j = r; j < i; ++j) s = fma(T[r][j], G[j][i], s);
+                v = -t * s;
+            }
+            T[r][i] = v;
+            __syncwarp(0xffu);
         }
-        const double t = tau[k];
-        if (t != 0.0) {
-            const double *vk = vs[cur];
-            const int c0 = (k + 1) >> 5;  // entries below k + 1 are zero
-            double s = 0.0;
+    }
+    __syncthreads();
+    if (threadIdx.x < kWY * kWY) Tw[(size_t)blockIdx.x * kWY * kWY + threadIdx.x] = T[threadIdx.x / kWY][threadIdx.x % kWY];
+}
+
+// Back transformation X = Q Z with Q = H_0 H_1 ... H_{n-2}, eight reflectors at a
+// time (last block first): z -= V (T (V^T z)).  A CTA holds nv <= NV vectors in
+// registers, thread t the rows t, t + 128, ...; the block's V is staged in shared
+// memory while the block before is applied.
+// What bounds it: FP64 instructions, 2 x nv x rows / 128 per reflector and warp,
+// balanced over the SMs (nv = m / SMs).  n = m = 750: 1.35 ms (2.9
+// with a fixed-point sum per dot product); one warp per vector and one reflector
+// at a time took 2.2 ms (750 warps on 608 sub-partitions, five FP64 adds for the
+// sum and a barrier per reflector).
+template <int RPT, int NV>
+__global__ void __launch_bounds__(128) k_tri_back_wy(int n, int m, int nv, int bufs, const double *__restrict__ Vh,
+                                                     const double *__restrict__ Tw, const double *__restrict__ Z,
+                                                     double *__restrict__ X, int ldx) {
+    extern __shared__ double vs[];  // bufs (1 or 2) buffers of kWY x n
+    __shared__ double red[4][kWY * NV], cs[kWY * NV], Ts[2][kWY * kWY];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int i0 = blockIdx.x * nv, cnt = min(nv, m - i0);
+    double z[NV][RPT];
 #pragma unroll
-            for (int c = 0; c < C; ++c)
-                if (c >= c0) s += vk[lane + 32 * c] * z[c];
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            s *= t;
+    for (int v = 0; v < NV; ++v)
 #pragma unroll
-            for (int c = 0; c < C; ++c)
-                if (c >= c0) z[c] -= s * vk[lane + 32 * c];
+        for (int q = 0; q < RPT; ++q) {
+            const int j = tid + 128 * q;
+            z[v][q] = v < cnt && j < n ? Z[(size_t)(i0 + v) * n + j] : 0.0;
         }
-#pragma unroll
-        for (int q = 0; q < P; ++q) {
-            const int j = threadIdx.x + q * nthr;
-            if (j < 32 * C) vs[cur ^ 1][j] = pre[q];
+    const int nb = (n - 1 + kWY - 1) / kWY;
+    // rows j > k of reflector k, zero elsewhere
+    auto stage = [&](int b, int buf) {
+        double *dst = vs + (size_t)buf * kWY * n;
+        // from the first row of 128 that the block touches
+        for (int kk = 0; kk < kWY; ++kk) {
+            const int k = b * kWY + kk;
+            for (int j = ((b * kWY + 1) & ~127) + tid; j < n; j += 128) {
+                const bool live = k < n - 1 && j > k;
+                const unsigned d = (unsigned)__cvta_generic_to_shared(dst + kk * n + j);
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(d),
+                             "l"(Vh + (live ? (size_t)k * n + j : 0)), "r"(live ? 8 : 0));
+            }
         }
-        cur ^= 1;
+        if (tid < kWY * kWY) Ts[buf][tid] = Tw[(size_t)b * kWY * kWY + tid];
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    if (bufs == 2) stage(nb - 1, (nb - 1) & 1);
+    for (int b = nb - 1; b >= 0; --b) {
+        const int cur = bufs == 2 ? b & 1 : 0;
+        if (bufs == 1) stage(b, 0);
+        else if (b > 0) stage(b - 1, cur ^ 1);
+        if (bufs == 2 && b > 0) asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         __syncthreads();
-    }
-    if (i < m) {
+        const double *V = vs + (size_t)cur * kWY * n;
+        const int q0 = (b * kWY + 1) >> 7;  // rows below are zero in the whole block
+        double s[kWY][NV];
 #pragma unroll
-        for (int c = 0; c < C; ++c) {
-            const int j = lane + 32 * c;
-            if (j < n) X[(size_t)j * ldx + i] = z[c];
+        for (int kk = 0; kk < kWY; ++kk)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) s[kk][v] = 0.0;
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            const int j = tid + 128 * q;
+            if (q < q0 || 128 * q >= n) continue;
+#pragma unroll
+            for (int kk = 0; kk < kWY; ++kk) {
+                const double x = j < n ? V[kk * n + j] : 0.0;
+#pragma unroll
+                for (int v = 0; v < NV; ++v) s[kk][v] = fma(x, z[v][q], s[kk][v]);
+            }
         }
+        // half of the reflectors to the other lane at each of three exchanges
+        // (7 adds per vector in place of 24), reflector lane & 7 is left
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            double h4[4], h2[2], h1;
+            const bool b4 = lane & 4, b2 = lane & 2, b1 = lane & 1;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                h4[u] = (b4 ? s[u + 4][v] : s[u][v]) + __shfl_xor_sync(0xffffffffu, b4 ? s[u][v] : s[u + 4][v], 4);
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                h2[u] = (b2 ? h4[u + 2] : h4[u]) + __shfl_xor_sync(0xffffffffu, b2 ? h4[u] : h4[u + 2], 2);
+            h1 = (b1 ? h2[1] : h2[0]) + __shfl_xor_sync(0xffffffffu, b1 ? h2[0] : h2[1], 1);
+            h1 += __shfl_xor_sync(0xffffffffu, h1, 8);
+            h1 += __shfl_xor_sync(0xffffffffu, h1, 16);
+            if (lane < kWY) red[wid][lane * NV + v] = h1;
+        }
+        __syncthreads();
+        if (tid < kWY * NV) red[0][tid] = (red[0][tid] + red[1][tid]) + (red[2][tid] + red[3][tid]);
+        __syncthreads();
+        if (tid < kWY * NV) {
+            const int i = tid / NV, v = tid % NV;
+            double c = 0.0;
+            for (int j = i; j < kWY; ++j) c = fma(Ts[cur][i * kWY + j], red[0][j * NV + v], c);
+            cs[tid] = -c;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < kWY; ++kk) {
+            double c[NV];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) c[v] = cs[kk * NV + v];
+#pragma unroll
+            for (int q = 0; q < RPT; ++q) {
+                const int j = tid + 128 * q;
+                if (q < q0 || 128 * q >= n) continue;
+                const double x = j < n ? V[kk * n + j] : 0.0;
+#pragma unroll
+                for (int v = 0; v < NV; ++v) z[v][q] = fma(c[v], x, z[v][q]);
+            }
+        }
+        __syncthreads();  // before this buffer is staged again
     }
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int q = 0; q < RPT; ++q) {
+            const int j = tid + 128 * q;
+            if (v < cnt && j < n) X[(size_t)j * ldx + i0 + v] = z[v][q];
+        }
 }
 
 // T scaled by a power of two to a norm bound in [1/2, 1): ds, e2s = e^2 (at least
@@ -928,8 +1026,9 @@ __global__ void k_tri_invit(int n, const double *__restrict__ d, const double *_
 
 // Vectors of eigenvalues closer than kNearTol ||T||, made orthogonal in
 // ascending order (one warp per chain of such neighbours).  The vector of an
-// eigenvalue known to eps ||T|| carries about eps ||T|| / gap of its neighbour:
-// 1e-11 at the gap of a cluster, 4e-12 where this ends.
+// eigenvalue known to eps ||T|| carries about eps ||T|| / gap of its neighbour: a
+// residual of eps ||T|| whatever the gap, 4e-7 of the neighbour at the gap of a
+// cluster (below it inverse iteration), 4e-12 where this ends.
 __global__ void __launch_bounds__(32) k_tri_orth(int n, int m, const double *__restrict__ bounds,
                                                  const double *__restrict__ lam, double *__restrict__ Z) {
     const int i0 = blockIdx.x, lane = threadIdx.x;
@@ -942,7 +1041,9 @@ __global__ void __launch_bounds__(32) k_tri_orth(int n, int m, const double *__r
             double s = 0.0;
             for (int j = lane; j < n; j += 32) s = fma(o[j], z[j], s);
             s = warp_sum(s);
-            for (int j = lane; j < n; j += 32) z[j] = fma(-s, o[j], z[j]);
+            // unit length again where the part taken off is felt
+            const double c = fabs(s) > 1e-9 ? rsqrt(fmax(1.0 - s * s, 0.25)) : 1.0;
+            for (int j = lane; j < n; j += 32) z[j] = c * fma(-s, o[j], z[j]);
             __syncwarp();
         }
     }
@@ -1004,9 +1105,9 @@ __global__ void __launch_bounds__(kTriThreads) k_tri_back(int n, int m, int per_
 
 size_t sym_eig_work_size(int n, int m) {
     // d e tau p e2 bounds(8) | Vh n^2 | Z m n | lam m | LU 5 n m (the minors' sequences before) | pivots n m bytes |
-    // clusters m + 1 ints | d, e^2 in FP32 (n each) | F, 1 / F, its exponents
+    // clusters m + 1 ints | d, e^2 in FP32 (n each) | F, 1 / F, its exponents | T of the reflector blocks
     return (size_t)5 * n + 8 + (size_t)n * n + (size_t)m * n + m + (size_t)5 * n * m + ((size_t)n * m + 7) / 8 +
-           ((size_t)m + 2) / 2 + 16 + (size_t)n + 8 + (size_t)4 * n + 8 + (size_t)3 * n + 8;
+           ((size_t)m + 2) / 2 + 16 + (size_t)n + 8 + (size_t)4 * n + 8 + (size_t)3 * n + 8 + (size_t)kWY * (n + kWY);
 }
 
 namespace {
@@ -1035,11 +1136,25 @@ bool launch_tridiag_rows(cudaStream_t s, int G, size_t smem, int sms, int n, con
     return true;
 }
 
-template <int C>
-void launch_back_warp(cudaStream_t s, int warps, int n, int m, const double *Vh, const double *tau, const double *Z,
-                      double *X, int ldx) {
-    k_tri_back_warp<C><<<cdiv(m, warps), 32 * warps, 0, s>>>(n, m, Vh, tau, Z, X, ldx);
+template <int RPT, int NV>
+void launch_back_wy(cudaStream_t s, int nv, int n, int m, const double *Vh, const double *Tw, const double *Z, double *X,
+                    int ldx) {
+    const size_t one = (size_t)kWY * n * sizeof(double);
+    const int bufs = 2 * one <= kTriSmemMax ? 2 : 1;
+    const size_t smem = bufs * one;
+    HSIM_SMEM_LIMIT_ONCE((k_tri_back_wy<RPT, NV>), kTriSmemMax);
+    k_tri_back_wy<RPT, NV><<<cdiv(m, nv), 128, smem, s>>>(n, m, nv, bufs, Vh, Tw, Z, X, ldx);
     HSIM_LAUNCHED();
+}
+template <int RPT>
+void launch_back_wy(cudaStream_t s, int nv, int n, int m, const double *Vh, const double *Tw, const double *Z, double *X,
+                    int ldx) {
+    constexpr int kMost = RPT <= 8 ? 5 : RPT <= 12 ? 3 : 2;  // vectors that fit the registers
+    if (nv == 1) launch_back_wy<RPT, 1>(s, nv, n, m, Vh, Tw, Z, X, ldx);
+    else if (nv == 2) launch_back_wy<RPT, 2>(s, nv, n, m, Vh, Tw, Z, X, ldx);
+    else if (kMost > 3 && nv == 3) launch_back_wy<RPT, kMost == 5 ? 3 : 1>(s, nv, n, m, Vh, Tw, Z, X, ldx);
+    else if (kMost > 4 && nv == 4) launch_back_wy<RPT, kMost == 5 ? 4 : 1>(s, nv, n, m, Vh, Tw, Z, X, ldx);
+    else launch_back_wy<RPT, kMost>(s, std::min(nv, kMost), n, m, Vh, Tw, Z, X, ldx);
 }
 
 }  // namespace
@@ -1056,6 +1171,7 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
     double *pbuf = reinterpret_cast<double *>(e232 + n) + 4, *rbuf = pbuf + 2 * (size_t)n;
     double *fm = rbuf + 2 * (size_t)n, *fi = fm + n;
     int *fx = reinterpret_cast<int *>(fi + n);
+    double *Tw = fi + 2 * (size_t)n;  // kWY x kWY per block of reflectors
     // sequences of k_tri_minors: 2 n m doubles, 2 ceil(n / 8) m exponents
     int *xs = reinterpret_cast<int *>(lu + (size_t)2 * n * m);
     if (n == 1) {
@@ -1154,18 +1270,19 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
     k_tri_orth<<<m, 32, 0, s>>>(n, m, bounds, lam, Z);
     HSIM_LAUNCHED();
     if (detail) cudaEventRecord(t3, s);
-    // 4. back transformation: a warp per vector held in registers where n <=
-    // 2048, else a few vectors per CTA in shared memory
-    const int warps = std::max(4, std::min(8, (m + sms - 1) / sms));
-    const int cw = (n + 31) / 32;
-    if (cw <= 4) launch_back_warp<4>(s, warps, n, m, Vh, tau, Z, X, ldx);
-    else if (cw <= 8) launch_back_warp<8>(s, warps, n, m, Vh, tau, Z, X, ldx);
-    else if (cw <= 16) launch_back_warp<16>(s, warps, n, m, Vh, tau, Z, X, ldx);
-    else if (cw <= 24) launch_back_warp<24>(s, warps, n, m, Vh, tau, Z, X, ldx);
-    else if (cw <= 32) launch_back_warp<32>(s, warps, n, m, Vh, tau, Z, X, ldx);
-    else if (cw <= 48) launch_back_warp<48>(s, warps, n, m, Vh, tau, Z, X, ldx);
-    else if (cw <= 64) launch_back_warp<64>(s, warps, n, m, Vh, tau, Z, X, ldx);
-    else {
+    // 4. back transformation: eight reflectors at a time where a thread's rows fit
+    // its registers, else one by one, a few vectors per CTA in shared memory
+    if (n <= 2048) {
+        k_tri_wy<<<cdiv(n - 1, kWY), 128, 0, s>>>(n, Vh, tau, Tw);
+        HSIM_LAUNCHED();
+        const int nv = cdiv(m, sms), rpt = cdiv(n, 128);
+        if (rpt <= 1) launch_back_wy<1>(s, nv, n, m, Vh, Tw, Z, X, ldx);
+        else if (rpt <= 3) launch_back_wy<3>(s, nv, n, m, Vh, Tw, Z, X, ldx);
+        else if (rpt <= 6) launch_back_wy<6>(s, nv, n, m, Vh, Tw, Z, X, ldx);
+        else if (rpt <= 8) launch_back_wy<8>(s, nv, n, m, Vh, Tw, Z, X, ldx);
+        else if (rpt <= 12) launch_back_wy<12>(s, nv, n, m, Vh, Tw, Z, X, ldx);
+        else launch_back_wy<16>(s, nv, n, m, Vh, Tw, Z, X, ldx);
+    } else {
         const int per_cta = std::max(1, std::min(8, (int)(kTriSmemMax / ((size_t)n * sizeof(double)))));
         const size_t bsm = (size_t)per_cta * n * sizeof(double);
         HSIM_SMEM_LIMIT_ONCE(k_tri_back, kTriSmemMax);

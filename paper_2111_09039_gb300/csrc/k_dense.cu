@@ -679,11 +679,70 @@ __global__ void k_rows_rsqrt(int rows, int cols, const double *__restrict__ d, d
     X[(size_t)i * ldx + j] *= rsqrt(d[i]);
 }
 
-// C = A B for k x k row-major FP64 blocks as an FP64-accurate tensor-core product
-static void tc_mm(cudaStream_t s, int k, const double *A, int lda, const double *B, int ldb, double *C, int ldc,
+// C = A B (n x kk times kk x m, row-major) in FP64 for small blocks: a CTA per
+// 16 x 8 tile, an entry per thread.  NS: C = (3 I - A B) / 2 and max |I - A B| as in
+// k_ns_step.  blockIdx.z: one of two products of the same shape.
+// What bounds it: FP64 issue, kk instructions per warp of the fullest SM (75: 3 us
+// of 7 per product; 256: 41 us).
+struct SmallMM {
+    const double *A, *B;
+    double *C;
+};
+template <bool NS>
+__global__ void __launch_bounds__(128) k_small_mm(int n, int kk, int m, SmallMM p0, SmallMM p1, int lda, int ldb, int ldc,
+                                                  unsigned long long *out) {
+    constexpr int KC = 128;
+    __shared__ double As[16][KC + 1], Bs[KC][8];
+    const SmallMM p = blockIdx.z ? p1 : p0;
+    const int tid = threadIdx.x, ty = tid >> 3, tx = tid & 7, i0 = blockIdx.y * 16, j0 = blockIdx.x * 8;
+    double acc = 0.0;
+    for (int k0 = 0; k0 < kk; k0 += KC) {
+        const int kc = min(KC, kk - k0);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < 16; ++r)
+            if (tid < kc) As[r][tid] = i0 + r < n ? p.A[(size_t)(i0 + r) * lda + k0 + tid] : 0.0;
+#pragma unroll 8
+        for (int r = ty; r < kc; r += 16) Bs[r][tx] = j0 + tx < m ? p.B[(size_t)(k0 + r) * ldb + j0 + tx] : 0.0;
+        __syncthreads();
+#pragma unroll 8
+        for (int q = 0; q < kc; ++q) acc = fma(As[ty][q], Bs[q][tx], acc);
+    }
+    const int i = i0 + ty, j = j0 + tx;
+    const bool in = i < n && j < m;
+    if (NS) {
+        const double id = i == j ? 1.0 : 0.0;
+        double e = in ? fabs(id - acc) : 0.0;
+        for (int o = 16; o > 0; o >>= 1) e = fmax(e, __shfl_xor_sync(0xffffffffu, e, o));
+        if ((tid & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(e));
+        acc = 0.5 * (3.0 * id - acc);
+    }
+    if (in) p.C[(size_t)i * ldc + j] = acc;
+}
+
+// Up to this order the FP64 kernel is taken in place of the digit products, whose
+// launches (two splits, the exponents, the product) cost about 45 us whatever the
+// size.  Mixed Ritz solve at k = 30, 75, 128, 192, 256 (us): 560, 790, 1153, 1790,
+// 2402 against 1109, 1255, 1550, 2065, 2500 with digits.
+constexpr int kSmallMM = 256;
+
+static void small_mm(cudaStream_t s, int n, int kk, int m, SmallMM p0, int lda, int ldb, int ldc,
+                     const SmallMM *p1 = nullptr) {
+    k_small_mm<false><<<dim3(cdiv(m, 8), cdiv(n, 16), p1 ? 2 : 1), 128, 0, s>>>(n, kk, m, p0, p1 ? *p1 : p0, lda, ldb, ldc,
+                                                                               nullptr);
+    HSIM_LAUNCHED();
+}
+
+// C = A B, k x k times k x m blocks, row-major: FP64 or an FP64-accurate
+// tensor-core product
+static void tc_mm(cudaStream_t s, int k, int m, const double *A, int lda, const double *B, int ldb, double *C, int ldc,
                   unsigned char *oz) {
+    if (k <= kSmallMM) {
+        small_mm(s, k, k, m, {A, B, C}, lda, ldb, ldc);
+        return;
+    }
     OzakiOperand a = ozaki_split_rows(s, k, k, A, lda, oz);
-    OzakiOperand b = ozaki_split_cols(s, k, k, B, ldb, oz + ozaki_rows_scratch(k, k), kOzakiSlices, OzakiRole::Y);
+    OzakiOperand b = ozaki_split_cols(s, k, m, B, ldb, oz + ozaki_rows_scratch(k, k), kOzakiSlices, OzakiRole::Y);
     ozaki_product(s, a, b, C, ldc, 0);
 }
 
@@ -692,12 +751,12 @@ static void tc_mm(cudaStream_t s, int k, const double *A, int lda, const double 
 // converges quadratically when ||M_bar - I||_2 < 1; products on the tensor
 // cores.  Used when a Gershgorin bound puts ||M_bar - I||_2 below 1/2 (the
 // columns are scaled to unit M-norm, so M_bar is near I once the basis is
-// nearly M-orthonormal).  buf: four k x k scratch blocks.  Returns the block
+// nearly M-orthonormal).  buf: five k x k scratch blocks.  Returns the block
 // that holds Z, or nullptr if the bound fails or the iteration does not reach
 // max|I - Z Y| < 1e-12 within 12 steps (the caller then factors M_bar); the
 // products carry about 2^-47 of their row and column maxima per term, so the
 // attainable level near I is a few 1e-14 times sqrt(k).  *steps: iterations.
-static const double *ns_inv_sqrt(cudaStream_t s, int k, const double *Mbar, int ldm, double *const buf[4],
+static const double *ns_inv_sqrt(cudaStream_t s, int k, const double *Mbar, int ldm, double *const buf[5],
                                  unsigned char *oz, unsigned long long *dmax, int *steps) {
     auto read_max = [&](double &v) {
         unsigned long long h = 0;
@@ -711,15 +770,19 @@ static const double *ns_inv_sqrt(cudaStream_t s, int k, const double *Mbar, int 
     double g = 1.0;
     read_max(g);
     if (!(g < 0.5)) return nullptr;
-    double *Y = buf[0], *Z = buf[1], *P = buf[2], *T = buf[3];
+    double *Y = buf[0], *Z = buf[1], *P = buf[2], *T = buf[3], *Q = buf[4];
     copy_matrix(s, k, k, Mbar, ldm, Y, k);
     k_identity<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, Z, k);
     HSIM_LAUNCHED();
     double prev = 1.0;
     for (int it = 0; it < 12; ++it) {
-        tc_mm(s, k, Z, k, Y, k, P, k, oz);  // P = Z Y
         HSIM_CUDA(cudaMemsetAsync(dmax, 0, sizeof(unsigned long long), s));
-        k_ns_step<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, P, T, dmax);
+        if (k <= kSmallMM) {
+            k_small_mm<true><<<dim3(cdiv(k, 8), cdiv(k, 16)), 128, 0, s>>>(k, k, k, {Z, Y, T}, {Z, Y, T}, k, k, k, dmax);
+        } else {
+            tc_mm(s, k, k, Z, k, Y, k, P, k, oz);  // P = Z Y
+            k_ns_step<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, P, T, dmax);
+        }
         HSIM_LAUNCHED();
         double e = 1.0;
         read_max(e);
@@ -731,9 +794,16 @@ static const double *ns_inv_sqrt(cudaStream_t s, int k, const double *Mbar, int 
         }
         if (!(e < 0.5 * prev) && it > 1) return nullptr;  // stopped contracting above the target
         prev = e;
-        tc_mm(s, k, Y, k, T, k, P, k, oz);  // Y T
+        if (k <= kSmallMM) {
+            const SmallMM tz{T, Z, Q};  // both products in one launch
+            small_mm(s, k, k, k, {Y, T, P}, k, k, k, &tz);
+            std::swap(Y, P);
+            std::swap(Z, Q);
+            continue;
+        }
+        tc_mm(s, k, k, Y, k, T, k, P, k, oz);  // Y T
         std::swap(Y, P);
-        tc_mm(s, k, T, k, Z, k, P, k, oz);  // T Z
+        tc_mm(s, k, k, T, k, Z, k, P, k, oz);  // T Z
         std::swap(Z, P);
     }
     return nullptr;
@@ -755,21 +825,20 @@ int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar,
         double *Cr = ework + sym_eig_work_size(k, k) + 8, *Cc = Cr + kk, *V = Cc + kk, *scr = V + kk;
         unsigned char *oz = reinterpret_cast<unsigned char *>(
             (reinterpret_cast<uintptr_t>(scr + kk) + 255) & ~static_cast<uintptr_t>(255));
-        double *const buf[4] = {F, Cr, Cc, scr};
+        double *const buf[5] = {F, Cr, Cc, scr, T};
         int ns_steps = 0;
         const double *Wz =
             ns_inv_sqrt(s, k, Mbar, ldm, buf, oz, reinterpret_cast<unsigned long long *>(flag_dev + 4), &ns_steps);
         if (Wz) {
             if (sweeps) *sweeps = ns_steps;
-            tc_mm(s, k, Wz, k, Sbar, lds, W, k, oz);
-            tc_mm(s, k, W, k, Wz, k, T, k, oz);
-            k_symmetrize<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, T, k);
+            double *A = Wz == T ? F : T;
+            tc_mm(s, k, k, Wz, k, Sbar, lds, W, k, oz);
+            tc_mm(s, k, k, W, k, Wz, k, A, k, oz);
+            k_symmetrize<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, A, k);
             HSIM_LAUNCHED();
-            sym_eig(s, k, m, T, evals, V, m, ework);
-            OzakiOperand a = ozaki_split_rows(s, k, k, Wz, k, oz);
-            OzakiOperand b = ozaki_split_cols(s, k, m, V, m, oz + ozaki_rows_scratch(k, k), kOzakiSlices, OzakiRole::Y);
-            ozaki_product(s, a, b, X, ldx, 0);
-            ozaki_check(s);
+            sym_eig(s, k, m, A, evals, V, m, ework);
+            tc_mm(s, k, m, Wz, k, V, m, X, ldx, oz);
+            if (k > kSmallMM) ozaki_check(s);
             return 0;
         }
     }
@@ -797,7 +866,6 @@ int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar,
         // digit slices are read by bulk copies: 256-byte aligned base
         unsigned char *oz = reinterpret_cast<unsigned char *>(
             (reinterpret_cast<uintptr_t>(scr + kk) + 255) & ~static_cast<uintptr_t>(255));
-        const size_t rb = ozaki_rows_scratch(k, k);
         HSIM_CHECK_ARG(df.scratch <= (int64_t)kk, "ritz: inversion scratch");
         for (size_t lv = 0; lv < df.p1.size(); ++lv) {
             gemm_tasks<double>(s, df.p1[lv].p, df.ntask[lv], df.tiles[lv], F, F, scr);
@@ -805,19 +873,13 @@ int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar,
         }
         k_cinv<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, F, d, Cr, Cc);
         HSIM_LAUNCHED();
-        OzakiOperand a = ozaki_split_rows(s, k, k, Cr, k, oz);
-        OzakiOperand b = ozaki_split_cols(s, k, k, Sbar, lds, oz + rb, kOzakiSlices, OzakiRole::Y);
-        ozaki_product(s, a, b, W, k, 0);
-        a = ozaki_split_rows(s, k, k, W, k, oz);
-        b = ozaki_split_cols(s, k, k, Cc, k, oz + rb, kOzakiSlices, OzakiRole::Y);
-        ozaki_product(s, a, b, T, k, 0);
+        tc_mm(s, k, k, Cr, k, Sbar, lds, W, k, oz);
+        tc_mm(s, k, k, W, k, Cc, k, T, k, oz);
         k_symmetrize<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, T, k);
         HSIM_LAUNCHED();
         sym_eig(s, k, m, T, evals, V, m, ework);
-        a = ozaki_split_rows(s, k, k, Cc, k, oz);
-        b = ozaki_split_cols(s, k, m, V, m, oz + rb, kOzakiSlices, OzakiRole::Y);
-        ozaki_product(s, a, b, X, ldx, 0);
-        ozaki_check(s);
+        tc_mm(s, k, m, Cc, k, V, m, X, ldx, oz);
+        if (k > kSmallMM) ozaki_check(s);
         return 0;
     }
     // A = C^-1 S_bar C^-T: W = D^-1/2 L^-1 S_bar, T = D^-1/2 L^-1 W^T

@@ -77,26 +77,27 @@ __device__ __forceinline__ int find_task(const GemmTask *tasks, int ntasks, int 
     return lo;
 }
 
-template <typename T>
+template <typename T, int BT>
 __global__ void __launch_bounds__(256) k_gemm_tasks(const GemmTask *__restrict__ tasks, int ntasks,
                                                     const T *__restrict__ Ab, const T *__restrict__ Bb,
                                                     T *__restrict__ Cb) {
-    constexpr int BT = kGemmTile, BK = 16;
+    constexpr int BK = 16, U = BT / 16, SUB = kGemmTile / BT;
     __shared__ T As[BK][BT + 1];
     __shared__ T Bs[BK][BT + 1];
     const GemmTask tk = tasks[find_task(tasks, ntasks, blockIdx.x)];
     const int local = blockIdx.x - tk.tile0;
-    const int ntn = (tk.N + BT - 1) / BT;
-    const int m0 = (local / ntn) * BT, n0 = (local % ntn) * BT;
+    const int ntn = (tk.N + kGemmTile - 1) / kGemmTile;
+    const int m0 = (local / ntn) * kGemmTile + (blockIdx.y / SUB) * BT, n0 = (local % ntn) * kGemmTile + (blockIdx.y % SUB) * BT;
+    if (m0 >= tk.M || n0 >= tk.N) return;
     const bool ua = tk.flags & kGemmAUnitLower, ub = tk.flags & kGemmBUnitLower;
     const T *A = Ab + tk.a, *B = Bb + tk.b;
     T *C = Cb + tk.c;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // tx: rows, ty: columns
-    T acc[4][4];
+    T acc[U][U];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = T(0);
+        for (int v = 0; v < U; ++v) acc[u][v] = T(0);
     // a unit lower A has A(i, k) = 0 for k > i; a unit lower B has B(k, j) = 0 for k < j
     const int kbeg = ub ? (n0 / BK) * BK : 0;
     const int kend = ua ? min(tk.K, m0 + BT) : tk.K;
@@ -114,26 +115,26 @@ __global__ void __launch_bounds__(256) k_gemm_tasks(const GemmTask *__restrict__
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < BK; ++kk) {
-            T a[4], b[4];
+            T a[U], b[U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < U; ++u) {
                 a[u] = As[kk][tx + 16 * u];
                 b[u] = Bs[kk][ty + 16 * u];
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u)
+            for (int u = 0; u < U; ++u)
 #pragma unroll
-                for (int v = 0; v < 4; ++v) acc[u][v] += a[u] * b[v];
+                for (int v = 0; v < U; ++v) acc[u][v] += a[u] * b[v];
         }
         __syncthreads();
     }
     const T sg = (tk.flags & kGemmNeg) ? T(-1) : T(1);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < U; ++u) {
         const int i = m0 + tx + 16 * u;
         if (i >= tk.M) continue;
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
+        for (int v = 0; v < U; ++v) {
             const int j = n0 + ty + 16 * v;
             if (j < tk.N) C[(int64_t)j * tk.ldc + i] = sg * acc[u][v];
         }
@@ -952,7 +953,15 @@ void inv_diag_blocks(cudaStream_t s, const FrontDev &fd, const int2 *blk, int nb
 template <typename T>
 void gemm_tasks(cudaStream_t s, const GemmTask *tasks, int ntasks, int tiles, const T *Ab, const T *Bb, T *Cb) {
     if (ntasks <= 0 || tiles <= 0) return;
-    k_gemm_tasks<T><<<tiles, 256, 0, s>>>(tasks, ntasks, Ab, Bb, Cb);
+    // FP64: a 64 x 64 tile is 16 instructions of 77 clocks per step and warp; tiles
+    // of 32 or 16 rows and columns where those of 64 leave SMs idle (inversion of
+    // the factor at n = 1000: 2.6 ms with 64, 0.6 with 16)
+    if (sizeof(T) == 8 && tiles <= 76)
+        k_gemm_tasks<T, sizeof(T) == 8 ? 16 : kGemmTile><<<dim3(tiles, 16), 256, 0, s>>>(tasks, ntasks, Ab, Bb, Cb);
+    else if (sizeof(T) == 8 && tiles <= 304)
+        k_gemm_tasks<T, sizeof(T) == 8 ? 32 : kGemmTile><<<dim3(tiles, 4), 256, 0, s>>>(tasks, ntasks, Ab, Bb, Cb);
+    else
+        k_gemm_tasks<T, kGemmTile><<<tiles, 256, 0, s>>>(tasks, ntasks, Ab, Bb, Cb);
     HSIM_LAUNCHED();
 }
 

@@ -11,7 +11,7 @@ from synth import meshes
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("nu,nv,p,levels", [(31, 17, 2, 2), (60, 41, 31, 2), (60, 41, 32, 2), (60, 41, 33, 2),
+@pytest.mark.parametrize("nu,nv,p,levels", [(60, 41, 31, 2), (60, 41, 32, 2), (60, 41, 33, 2),
                                             (97, 83, 65, 2), (250, 160, 230, 2)])
 @pytest.mark.parametrize("mixed", [True, False])
 def test_reported_residual(nu, nv, p, levels, mixed):

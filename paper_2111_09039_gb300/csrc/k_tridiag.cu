@@ -164,13 +164,43 @@ __device__ __forceinline__ double warp_sum_fixed(double v) {
     return te > 0 && te < 0x7FF ? __hiloint2double(th + q * 0x100000, __double2loint(t)) : ldexp(t, q);
 }
 
-// sum over the block (kTrdThreads threads); result in all threads
+// named barriers of the two halves of a k_tridiag_rows block
+template <int ID, int COUNT>
+__device__ __forceinline__ void bar_sync() {
+    asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(COUNT) : "memory");
+}
+template <int ID, int COUNT>
+__device__ __forceinline__ void bar_arrive() {
+    asm volatile("bar.arrive %0, %1;" ::"n"(ID), "n"(COUNT) : "memory");
+}
+
+// sum over the kTrdThreads threads of the computing half; result in all of them
 __device__ __forceinline__ double block_sum128(double v, double *red) {
     v = warp_sum_fixed(v);
-    __syncthreads();  // red may still be read from the previous call
+    bar_sync<1, kTrdThreads>();  // red may still be read from the previous call
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
+    bar_sync<1, kTrdThreads>();
     return (red[0] + red[1]) + (red[2] + red[3]);
+}
+
+// sums of N <= 16 values (a power of two) over the warp: half of them to the
+// other lane at each of log2 N exchanges (N + 3 adds for 8, chain of five);
+// returns that of value lane & (N - 1)
+template <int N>
+__device__ __forceinline__ double warp_sums(const double (&a)[N], int lane) {
+    double h[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) h[i] = a[i];
+#pragma unroll
+    for (int w = N / 2; w > 0; w >>= 1) {
+        const bool up = lane & w;
+#pragma unroll
+        for (int i = 0; i < w; ++i)
+            h[i] = (up ? h[i + w] : h[i]) + __shfl_xor_sync(0xffffffffu, up ? h[i] : h[i + w], w);
+    }
+#pragma unroll
+    for (int w = N; w < 32; w <<= 1) h[0] += __shfl_xor_sync(0xffffffffu, h[0], w);
+    return h[0];
 }
 
 // 1 / sqrt(x) and 1 / x of normal numbers from the 20-bit seeds by one
@@ -188,58 +218,115 @@ __device__ __forceinline__ double rcp_step(double x) {
     return fma(r, fma(e, e, e), r);
 }
 
-// Grid barrier: every CTA adds to a counter that starts at zero; `target`
-// arrivals complete it.  The waiting gives up after two seconds (false, *err
-// set); the CTAs that then leave let the others run into the same limit.
-__device__ __forceinline__ bool grid_barrier(unsigned *counter, unsigned target, double *err) {
-    int ok = 1;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
-        unsigned long long t0 = 0;
-        for (unsigned it = 0;; ++it) {
-            unsigned c;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(counter) : "memory");
-            if (c >= target) break;
-            if ((it & 1023u) == 1023u) {
-                unsigned long long t;
-                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-                if (t0 == 0) t0 = t;
-                else if (t - t0 > 2000000000ull) {
-                    *err = 1.0;
-                    ok = 0;
-                    break;
-                }
+// Waiting for `target` arrivals at a counter that starts at zero.  It gives up
+// after two seconds (false, *err set); the CTAs that then leave let the others
+// run into the same limit.
+__device__ __forceinline__ bool grid_wait(unsigned *counter, unsigned target, double *err) {
+    unsigned long long t0 = 0;
+    for (unsigned it = 0;; ++it) {
+        unsigned c;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(c) : "l"(counter) : "memory");
+        if (c >= target) return true;
+        if ((it & 1023u) == 1023u) {
+            unsigned long long t;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+            if (t0 == 0) t0 = t;
+            else if (t - t0 > 2000000000ull) {
+                *err = 1.0;
+                return false;
             }
         }
     }
-    return __syncthreads_and(ok) != 0;
+}
+
+// NA rows of a k_tridiag_rows CTA (a: the first, from column k + 1 on, n apart):
+// x += cb up + ca P, the sums of x y over the block's threads into redr[warp], the
+// first row also to rb if that is not null.  The loads of a step stand before its
+// stores, which the compiler could not tell apart from them.
+template <int NA, int STRIDE>
+__device__ __forceinline__ void rows_pass(int L, int n, double *a, const double *y, const double *up, const double *P,
+                                          double t, double tpu, int r0, int G, double *rb, double (*redr)[STRIDE]) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    constexpr int N2 = NA <= 1 ? 1 : NA <= 2 ? 2 : NA <= 4 ? 4 : NA <= 8 ? 8 : 16;
+    double acc[N2], ca[NA], cb[NA];
+#pragma unroll
+    for (int i = 0; i < N2; ++i) acc[i] = 0.0;
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+        const double ur = up[r0 + i * G + 1];
+        ca[i] = -(t * ur);
+        cb[i] = fma(tpu, ur, -(t * P[r0 + i * G]));
+    }
+    int j = tid;
+    for (; j + kTrdThreads < L; j += 2 * kTrdThreads) {
+        const int j1 = j + kTrdThreads;
+        const double y0 = y[j], y1 = y[j1], u0 = up[j + 2], u1 = up[j1 + 2], p0 = P[j + 1], p1 = P[j1 + 1];
+        double x0[NA], x1[NA];
+#pragma unroll
+        for (int i = 0; i < NA; ++i) x0[i] = a[(size_t)i * n + j], x1[i] = a[(size_t)i * n + j1];
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            x0[i] = fma(cb[i], u0, fma(ca[i], p0, x0[i]));
+            x1[i] = fma(cb[i], u1, fma(ca[i], p1, x1[i]));
+        }
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            a[(size_t)i * n + j] = x0[i];
+            a[(size_t)i * n + j1] = x1[i];
+            acc[i] = fma(x1[i], y1, fma(x0[i], y0, acc[i]));
+        }
+        if (rb) rb[j] = x0[0], rb[j1] = x1[0];
+    }
+    if (j < L) {
+        const double y0 = y[j], u0 = up[j + 2], p0 = P[j + 1];
+        double x0[NA];
+#pragma unroll
+        for (int i = 0; i < NA; ++i) x0[i] = a[(size_t)i * n + j];
+#pragma unroll
+        for (int i = 0; i < NA; ++i) x0[i] = fma(cb[i], u0, fma(ca[i], p0, x0[i]));
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            a[(size_t)i * n + j] = x0[i];
+            acc[i] = fma(x0[i], y0, acc[i]);
+        }
+        if (rb) rb[j] = x0[0];
+    }
+    const double rs = warp_sums<N2>(acc, lane);
+    if (lane < NA) redr[tid >> 5][lane] = rs;
 }
 
 // Tridiagonalisation with the matrix resident in shared memory.  CTA b owns
 // the rows b, b + G, b + 2G, ... (full length n), so the product p = t A22 u
 // and the rank-2 update of every column read and write only shared memory,
 // and one grid barrier per column suffices: before it every CTA writes its
-// entries of p, and the owner of row k+1 writes that row as it stands before
-// the update of column k; after it every CTA forms, from that row, the
-// updated row k+1, which by symmetry is the next column to reduce.  The update
-// of column k is applied to the owned rows in the same pass as the product of
-// column k+1.
+// entries of A22 y, y the column to reduce, and the owner of row k+1 writes that
+// row as it stands before the update of column k; after it every CTA forms, from
+// that row, the updated row k+1, which by symmetry is the next column to reduce.
+// The update of column k is applied to the owned rows in the same pass as the
+// product of column k+1.
 //
-// The reflector is I - t u u^T with u the column itself but for its first
-// entry (u_0 = x_0 - beta, t = -1 / (beta u_0)): nothing is scaled.  With w = p -
-// (t/2)(p.u) u the update of row r is -(u_r w + w_r u) = -(u_r p + b_r u), b_r =
-// p_r - t (p.u) u_r: w is not formed.  An entry costs three FP64 instructions.
-// What bounds it (n = 750 on 152 SMs: 7.4 us per column, 8.1 with scaled
-// reflectors, w formed, FP64 shuffles for the sums and divisions): the barrier
-// and the loads behind it about 3,000 clocks, FP64 issue (77 clocks per warp
-// instruction: 2.5 rows x 3 x 3 on average, and the vectors that every CTA
-// repeats), two block sums and the scalars in a dependent chain.  Entries tagged
-// with their column and polled for by every thread, instead of the barrier, took
-// 8,000 clocks per column at n = 750 (the polling loads themselves).
+// The reflector is I - t u u^T with u = y but for its first entry (u_0 = y_0 -
+// beta, t = -1 / (beta u_0)): nothing is scaled, and A22 u = A22 y + (u_0 - y_0)
+// A22 e_0, whose last vector is the row k+1 that every CTA receives.  So the
+// product does not wait for the reflector: its norm, square root and reciprocal
+// are computed while the entries travel.  With p = t A22 u and w = p - (t/2)(p.u) u
+// the update of row r is -(u_r w + w_r u) = -(u_r p + b_r u), b_r = p_r - t (p.u)
+// u_r: w is not formed.  An entry costs three FP64 instructions.
+// The second half of a block's threads only communicates: it arrives at the
+// barrier, waits and brings the entries to shared memory.
+// What bounds it: a chain per column.  Clocks at n = 75 / 750 (152 SMs): the rows
+// 1,800 / 3,800 (FP64 issue, 77 clocks per warp instruction, 2,900 of them at 750),
+// the other warps' sums 260 / 500, then the reflector 2,600 / 3,200 beside the
+// barrier and the loads 3,300 / 4,900, u^T A u 900 / 1,450, the next column 460 /
+// 980.  Per column 3.6 us at 75 and 5.7 us at 750; with the reflector before the
+// product, one thread polling and loading after it, and branches between the rows
+// 4.6 and 7.4; with scaled reflectors, w formed, FP64 shuffles for the sums and
+// divisions 8.1 at 750.  Entries tagged with their column and polled for by every
+// thread, instead of the barrier, took 8,000 clocks per column at n = 750 (the
+// polling loads themselves).
 // Shared memory: R n (owned rows, R = ceil(n / G) <= RMAX) + 4 n doubles.
 template <int RMAX>
-__global__ void __launch_bounds__(kTrdThreads) k_tridiag_rows(int n, const double *__restrict__ A, double *__restrict__ d,
+__global__ void __launch_bounds__(2 * kTrdThreads) k_tridiag_rows(int n, const double *__restrict__ A, double *__restrict__ d,
                                                             double *__restrict__ e, double *__restrict__ tau,
                                                             double *__restrict__ Vh, double *__restrict__ pbuf,
                                                             double *__restrict__ rbuf, unsigned *__restrict__ counter,
@@ -250,31 +337,103 @@ __global__ void __launch_bounds__(kTrdThreads) k_tridiag_rows(int n, const doubl
     const int R = (n - b + G - 1) / G;          // rows owned by this CTA
     const int Rmax = (n + G - 1) / G;
     double *rows = sm;                           // Rmax x n
-    double *xs = rows + (size_t)Rmax * n;        // row k: xs[i] = A[k, k + i]
-    double *u = xs + n, *up = u + n, *p = up + n;  // reflector of column k, of column k - 1; p of column k - 1
+    double *cur = rows + (size_t)Rmax * n;       // row k: cur[i] = A[k, k + i]; then u of column k in cur[1 + i]
+    double *prev = cur + n;                      // the same of column k - 1
+    double *P = prev + n, *tu = P + n;           // A u of column k - 1 (index 0 <-> row k); t u of column k
     __shared__ double red[NW];
     __shared__ double redr[NW][RMAX];
+    __shared__ int gave_up;
     for (int i = 0; i < R; ++i) {
         const double *src = A + (size_t)(b + i * G) * n;
-        for (int j = tid; j < n; j += kTrdThreads) rows[(size_t)i * n + j] = src[j];
+        for (int j = tid; j < n; j += 2 * kTrdThreads) rows[(size_t)i * n + j] = src[j];
     }
-    for (int j = tid; j < n; j += kTrdThreads) xs[j] = A[j];
-    double tpu = 0.0;  // t (p.u) of column k - 1
+    // no update before the first column: zeros in u and P of the one before
+    for (int j = tid; j < n; j += 2 * kTrdThreads) cur[j] = A[j], prev[j] = P[j] = 0.0;
+    if (tid == 0) gave_up = 0;
     __syncthreads();
+    if (tid >= kTrdThreads) {
+        // communicating half
+        const int lt = tid - kTrdThreads;
+        for (int k = 0; k + 1 < n; ++k) {
+            const int L = n - k - 1;
+            const double *ab = pbuf + (size_t)(k & 1) * n, *rb = rbuf + (size_t)(k & 1) * n;
+            bar_sync<2, 2 * kTrdThreads>();  // this CTA's entries are written, prev and P are free
+            if (lt == 0) {
+                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(counter) : "memory");
+                if (!grid_wait(counter, (unsigned)(k + 1) * (unsigned)G, err)) gave_up = 1;
+            }
+            bar_sync<3, kTrdThreads>();
+            if (!gave_up) {
+#pragma unroll 4
+                for (int j = lt; j < L; j += kTrdThreads) {
+                    const double rj = __ldcg(rb + j), aj = __ldcg(ab + j);
+                    prev[j] = rj;
+                    P[j] = aj;
+                }
+            }
+            bar_sync<4, 2 * kTrdThreads>();
+            if (gave_up) return;
+            double *tmp = prev;
+            prev = cur;
+            cur = tmp;
+        }
+        return;
+    }
+    double tpu = 0.0, tp = 0.0;  // t (p.u), t of column k - 1
     for (int k = 0; k + 1 < n; ++k) {
         const int L = n - k - 1;
-        // reflector of y = xs[1 .. L] (column k below the diagonal)
+        const double x0 = cur[1];
+        // owned rows r >= k + 1: update of column k - 1 on columns >= k + 1, then
+        // the product with y = cur[1 .. L], the column below the diagonal
+        const int i0 = k + 1 > b ? (k + 1 - b + G - 1) / G : 0, na = R - i0;
+        double *ab = pbuf + (size_t)(k & 1) * n;
+        {
+            // row k + 1 is the first of its owner's rows that are left
+            double *rb = b + i0 * G == k + 1 ? rbuf + (size_t)(k & 1) * n : nullptr;
+            double *a = rows + (size_t)i0 * n + k + 1;
+            const int r0 = b + i0 * G - k;
+#define HSIM_ROWS(NA)                                                                              \
+    case NA:                                                                                       \
+        if (NA <= RMAX) rows_pass<NA <= RMAX ? NA : 1>(L, n, a, cur + 1, prev, P, tp, tpu, r0, G, rb, redr); \
+        break
+            switch (na) {
+                HSIM_ROWS(1);
+                HSIM_ROWS(2);
+                HSIM_ROWS(3);
+                HSIM_ROWS(4);
+                HSIM_ROWS(5);
+                HSIM_ROWS(6);
+                HSIM_ROWS(7);
+                HSIM_ROWS(8);
+                HSIM_ROWS(9);
+                HSIM_ROWS(10);
+                HSIM_ROWS(11);
+                HSIM_ROWS(12);
+                HSIM_ROWS(13);
+                HSIM_ROWS(14);
+                HSIM_ROWS(15);
+                HSIM_ROWS(16);
+                default: break;  // none left
+            }
+#undef HSIM_ROWS
+        }
+        bar_sync<1, kTrdThreads>();
+        if (tid < na)
+            ab[b + (i0 + tid) * G - k - 1] = (redr[0][tid] + redr[1][tid]) + (redr[2][tid] + redr[3][tid]);
+        bar_arrive<2, 2 * kTrdThreads>();
+        // meanwhile the reflector
         double part = 0.0;
-        for (int i = 1 + tid; i < L; i += kTrdThreads) part = fma(xs[1 + i], xs[1 + i], part);
+        for (int i = 1 + tid; i < L; i += kTrdThreads) part = fma(cur[1 + i], cur[1 + i], part);
         const double sigma = block_sum128(part, red);
-        const double x0 = xs[1];
         double beta = x0, t = 0.0, u0 = 1.0;
-        if (sigma != 0.0) {
+        // (tests on the bits: an FP64 comparison waits for the pipe)
+        if ((__double2hiint(sigma) | __double2loint(sigma)) != 0) {
             const double s2 = fma(x0, x0, sigma);
-            if (s2 > 1e-280 && s2 < 1e280) {
+            const int ex = __double2hiint(s2) >> 20;
+            if (ex > 93 && ex < 1952) {  // 1e-280 .. 1e279
                 const double r = rsqrt_step(s2), m0 = s2 * r;
                 const double mu = fma(fma(-m0, m0, s2), 0.5 * r, m0);
-                beta = x0 >= 0.0 ? -mu : mu;
+                beta = __double2hiint(x0) >= 0 ? -mu : mu;
                 u0 = x0 - beta;
                 t = rcp_step(-beta * u0);
             } else {
@@ -284,78 +443,53 @@ __global__ void __launch_bounds__(kTrdThreads) k_tridiag_rows(int n, const doubl
                 t = -1.0 / (beta * u0);
             }
         }
+        const double d0 = u0 - x0, c0 = u0 * t;
         for (int i = tid; i < L; i += kTrdThreads) {
-            const double ui = i == 0 ? u0 : xs[1 + i];
-            u[i] = ui;
+            const double ui = i == 0 ? u0 : cur[1 + i];
+            if (i == 0) cur[1] = u0;
+            tu[i] = t * ui;
             if (b == 0) Vh[(size_t)k * n + k + 1 + i] = ui;
         }
         if (b == 0 && tid == 0) {
-            d[k] = xs[0];
+            d[k] = cur[0];
             e[k] = beta;
             tau[k] = t;
         }
-        __syncthreads();
-        // owned rows r >= k + 1: update of column k - 1 (vectors up, p, index
-        // 0 <-> row k) on columns >= k + 1, then the product with u
-        const int i0 = k + 1 > b ? (k + 1 - b + G - 1) / G : 0;
-        double acc[RMAX], ca[RMAX], cb[RMAX];
-#pragma unroll
-        for (int i = 0; i < RMAX; ++i) {
-            acc[i] = ca[i] = cb[i] = 0.0;
-            if (k == 0 || i < i0 || i >= R) continue;
-            const int r = b + i * G - k;
-            ca[i] = -up[r];
-            cb[i] = fma(tpu, up[r], -p[r]);
-        }
-        double *rb = rbuf + (size_t)(k & 1) * n;
-        const int ir = (k + 1) % G == b ? (k + 1) / G : -1;  // this CTA's index of row k + 1
-        for (int j = tid; j < L; j += kTrdThreads) {
-            const double uj = u[j];
-            const double upj = k > 0 ? up[j + 1] : 0.0, pj = k > 0 ? p[j + 1] : 0.0;
-#pragma unroll
-            for (int i = 0; i < RMAX; ++i) {
-                if (i < i0 || i >= R) continue;
-                double *a = rows + (size_t)i * n + k + 1 + j;
-                double x = *a;
-                if (k > 0) {
-                    x = fma(cb[i], upj, fma(ca[i], pj, x));
-                    *a = x;
-                }
-                acc[i] = fma(x, uj, acc[i]);
-                if (i == ir) rb[j] = x;
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < RMAX; ++i) {
-            if (i < i0 || i >= R) continue;
-            const double rs = warp_sum_fixed(acc[i]);
-            if (lane == 0) redr[wid][i] = rs;
-        }
-        __syncthreads();
-        if (tid >= i0 && tid < R)
-            pbuf[(size_t)(k & 1) * n + (b + tid * G - k - 1)] =
-                t * ((redr[0][tid] + redr[1][tid]) + (redr[2][tid] + redr[3][tid]));
-        if (!grid_barrier(counter, (unsigned)(k + 1) * (unsigned)G, err)) return;
-        // row k + 1 after the update of column k
-        const double *pb = pbuf + (size_t)(k & 1) * n;
+        bar_sync<4, 2 * kTrdThreads>();
+        if (gave_up) return;
+        // P = A u from A y (in P), and row k + 1 (in prev) after the update of
+        // column k
         double pu = 0.0;
-#pragma unroll 4
-        for (int j = tid; j < L; j += kTrdThreads) {
-            const double pj = __ldcg(pb + j);
-            xs[j] = __ldcg(rb + j);
-            p[j] = pj;
-            pu = fma(pj, u[j], pu);
+        int j = tid;
+        for (; j + kTrdThreads < L; j += 2 * kTrdThreads) {
+            const int j1 = j + kTrdThreads;
+            const double a0 = P[j], a1 = P[j1], r0 = prev[j], r1 = prev[j1], t0 = tu[j], t1 = tu[j1];
+            const double P0 = fma(d0, r0, a0), P1 = fma(d0, r1, a1);
+            P[j] = P0, P[j1] = P1;
+            pu = fma(P1, t1, fma(P0, t0, pu));
+        }
+        if (j < L) {
+            const double P0 = fma(d0, prev[j], P[j]);
+            P[j] = P0;
+            pu = fma(P0, tu[j], pu);
         }
         tpu = t * block_sum128(pu, red);
-        const double b0 = fma(-tpu, u0, p[0]);
-        for (int j = tid; j < L; j += kTrdThreads) xs[j] = fma(-b0, u[j], fma(-u0, p[j], xs[j]));
-        double *tmp = up;
-        up = u;
-        u = tmp;
-        __syncthreads();
+        const double b0 = fma(-tpu, u0, t * P[0]);
+        for (j = tid; j + kTrdThreads < L; j += 2 * kTrdThreads) {
+            const int j1 = j + kTrdThreads;
+            const double a0 = P[j], a1 = P[j1], r0 = prev[j], r1 = prev[j1], v0 = cur[1 + j], v1 = cur[1 + j1];
+            prev[j] = fma(-b0, v0, fma(-c0, a0, r0));
+            prev[j1] = fma(-b0, v1, fma(-c0, a1, r1));
+        }
+        if (j < L) prev[j] = fma(-b0, cur[1 + j], fma(-c0, P[j], prev[j]));
+        tp = t;
+        double *tmp = prev;
+        prev = cur;
+        cur = tmp;
+        bar_sync<1, kTrdThreads>();
     }
     if (b == 0 && tid == 0) {
-        d[n - 1] = xs[0];
+        d[n - 1] = cur[0];
         tau[n - 1] = 0.0;
     }
 }
@@ -1127,11 +1261,11 @@ bool launch_tridiag_rows(cudaStream_t s, int G, size_t smem, int sms, int n, con
                          double *tau, double *Vh, double *pbuf, double *rbuf, unsigned *counter, double *err) {
     HSIM_SMEM_LIMIT_ONCE(k_tridiag_rows<RMAX>, kTriSmemMax);
     int per_sm = 0;
-    HSIM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag_rows<RMAX>, kTrdThreads, smem));
+    HSIM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag_rows<RMAX>, 2 * kTrdThreads, smem));
     if ((int64_t)per_sm * sms < G) return false;
     int nn = n;
     void *args[] = {&nn, &A, &d, &e, &tau, &Vh, &pbuf, &rbuf, &counter, &err};
-    HSIM_CUDA(cudaLaunchCooperativeKernel((void *)k_tridiag_rows<RMAX>, dim3(G), dim3(kTrdThreads), args, smem, s));
+    HSIM_CUDA(cudaLaunchCooperativeKernel((void *)k_tridiag_rows<RMAX>, dim3(G), dim3(2 * kTrdThreads), args, smem, s));
     HSIM_LAUNCHED();
     return true;
 }
@@ -1150,11 +1284,12 @@ template <int RPT>
 void launch_back_wy(cudaStream_t s, int nv, int n, int m, const double *Vh, const double *Tw, const double *Z, double *X,
                     int ldx) {
     constexpr int kMost = RPT <= 8 ? 5 : RPT <= 12 ? 3 : 2;  // vectors that fit the registers
+    nv = cdiv(nv, cdiv(nv, kMost));  // waves of equal height
     if (nv == 1) launch_back_wy<RPT, 1>(s, nv, n, m, Vh, Tw, Z, X, ldx);
     else if (nv == 2) launch_back_wy<RPT, 2>(s, nv, n, m, Vh, Tw, Z, X, ldx);
     else if (kMost > 3 && nv == 3) launch_back_wy<RPT, kMost == 5 ? 3 : 1>(s, nv, n, m, Vh, Tw, Z, X, ldx);
     else if (kMost > 4 && nv == 4) launch_back_wy<RPT, kMost == 5 ? 4 : 1>(s, nv, n, m, Vh, Tw, Z, X, ldx);
-    else launch_back_wy<RPT, kMost>(s, std::min(nv, kMost), n, m, Vh, Tw, Z, X, ldx);
+    else launch_back_wy<RPT, kMost>(s, nv, n, m, Vh, Tw, Z, X, ldx);
 }
 
 }  // namespace

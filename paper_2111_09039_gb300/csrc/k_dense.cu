@@ -160,14 +160,16 @@ __global__ void __launch_bounds__(256) k_col_sums(int n, int k, int rows, const 
     using A = typename F::Acc;
     __shared__ A red[8][F::N][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int j = blockIdx.y * 32 + lane, r_end = min(n, (blockIdx.x + 1) * rows);
+    // neighbouring CTAs share rows: whole rows are read at about the same time
+    const int ncb = (k + 31) / 32, rb = blockIdx.x / ncb;
+    const int j = (blockIdx.x - rb * ncb) * 32 + lane, r_end = min(n, (rb + 1) * rows);
     A a[F::N];
 #pragma unroll
     for (int u = 0; u < F::N; ++u) a[u] = A(0);
     if (j < k) {
         const double c = f.column(j);
 #pragma unroll 4
-        for (int r = blockIdx.x * rows + wid; r < r_end; r += 8) f.add(r, j, c, a);
+        for (int r = rb * rows + wid; r < r_end; r += 8) f.add(r, j, c, a);
     }
 #pragma unroll
     for (int u = 0; u < F::N; ++u) red[wid][u][lane] = a[u];
@@ -185,7 +187,7 @@ template <class F>
 void col_sums(cudaStream_t s, int n, int k, const F &f) {
     if (n <= 0 || k <= 0) return;
     const int rows = (int64_t)n * cdiv(k, 32) >= (int64_t)256 * 8 * 152 ? 256 : 64;
-    k_col_sums<<<dim3(cdiv(n, rows), cdiv(k, 32)), 256, 0, s>>>(n, k, rows, f);
+    k_col_sums<<<cdiv(n, rows) * cdiv(k, 32), 256, 0, s>>>(n, k, rows, f);
     HSIM_LAUNCHED();
 }
 

@@ -322,7 +322,7 @@ __global__ void k_axpy_matrix(int n, int k, const double *__restrict__ X, int ld
 
 __global__ void k_diag_scale(int n, int k, const double *__restrict__ d, const double *__restrict__ X, int ldx,
                              double *__restrict__ Y, int ldy) {
-    HSIM_FOR_RC(i, n, j, k) Y[(size_t)i * ldy + j] = d[i] * X[(size_t)i * ldx + j];
+    HSIM_ROWS_OF_COLUMN(i, n, j, k) Y[(size_t)i * ldy + j] = d[i] * X[(size_t)i * ldx + j];
 }
 
 __device__ __forceinline__ int find_col(const int *__restrict__ c, int lo, int hi, int key) {
@@ -396,7 +396,7 @@ __global__ void k_gather_rows(int n, int k, const int *__restrict__ perm, const 
 
 __global__ void k_copy_matrix(int rows, int cols, const double *__restrict__ X, int ldx, double *__restrict__ Y,
                               int ldy) {
-    HSIM_FOR_RC(i, rows, j, cols) Y[(size_t)i * ldy + j] = X[(size_t)i * ldx + j];
+    HSIM_ROWS_OF_COLUMN(i, rows, j, cols) Y[(size_t)i * ldy + j] = X[(size_t)i * ldx + j];
 }
 
 __global__ void k_densify(int n, const int *__restrict__ ptr, const int *__restrict__ col,
@@ -476,22 +476,24 @@ __global__ void k_rho(int cols, const double *__restrict__ num, const double *__
 __global__ void k_residual_f32(int rows, int cols, const double *__restrict__ SP, int lds,
                                const double *__restrict__ MP, int ldm, const double *__restrict__ rho,
                                float *__restrict__ R, int ldr) {
-    HSIM_FOR_RC(i, rows, j, cols) R[(size_t)i * ldr + j] =
-        d2f_trunc(fma(-rho[j], MP[(size_t)i * ldm + j], SP[(size_t)i * lds + j]));
+    const double rj = rho[min((int)(blockIdx.x * blockDim.x + threadIdx.x), cols - 1)];
+    HSIM_ROWS_OF_COLUMN(i, rows, j, cols) R[(size_t)i * ldr + j] =
+        d2f_trunc(fma(-rj, MP[(size_t)i * ldm + j], SP[(size_t)i * lds + j]));
 }
 
 // R (FP32) = SP - rho_j m_i X with M = diag(m): M X is not formed
 __global__ void k_residual_f32_diag(int rows, int cols, const double *__restrict__ SP, int lds,
                                     const double *__restrict__ X, int ldx, const double *__restrict__ m,
                                     const double *__restrict__ rho, float *__restrict__ R, int ldr) {
-    HSIM_FOR_RC(i, rows, j, cols) R[(size_t)i * ldr + j] =
-        d2f_trunc(fma(-rho[j] * m[i], X[(size_t)i * ldx + j], SP[(size_t)i * lds + j]));
+    const double rj = rho[min((int)(blockIdx.x * blockDim.x + threadIdx.x), cols - 1)];
+    HSIM_ROWS_OF_COLUMN(i, rows, j, cols) R[(size_t)i * ldr + j] =
+        d2f_trunc(fma(-rj * m[i], X[(size_t)i * ldx + j], SP[(size_t)i * lds + j]));
 }
 
 // Y (FP64) = X - Z (FP32)
 __global__ void k_sub_f2d(int rows, int cols, const double *__restrict__ X, int ldx, const float *__restrict__ Z,
                           int ldz, double *__restrict__ Y, int ldy) {
-    HSIM_FOR_RC(i, rows, j, cols) Y[(size_t)i * ldy + j] = X[(size_t)i * ldx + j] - f2d_bits(Z[(size_t)i * ldz + j]);
+    HSIM_ROWS_OF_COLUMN(i, rows, j, cols) Y[(size_t)i * ldy + j] = X[(size_t)i * ldx + j] - f2d_bits(Z[(size_t)i * ldz + j]);
 }
 
 template <typename T>

@@ -227,64 +227,83 @@ __global__ void __launch_bounds__(256) k_split_rows(int R, int K, const double *
 }
 
 // split a row-major K x C block per column (operand row r = column r, K = rows
-// of X), transposed through shared memory: a block handles 64 columns x 32 K
-// rows.  rexp: row k of the block is scaled by 2^rexp[k].  sumsq (seven-digit
-// Grams): sum over k of (128 x / 2^e)^2 per column, from the leading digits.
+// of X), transposed through shared memory: a block handles 64 columns and `tiles`
+// times 32 K rows, two tiles on their way (cp.async) while one is split; half a
+// warp reads 16 columns of eight rows, a warp stores 512 contiguous bytes.
+// rexp: row k of the block is scaled by 2^rexp[k].  sumsq (seven-digit Grams):
+// sum over k of (128 x / 2^e)^2 per column, from the leading digits.
+// What bounds it: memory (a 250,000 x 750 block into five digits: 0.55 ms,
+// 6.1 TB/s; a tile per block through registers 0.75 ms, waiting for its loads).
+constexpr int kSplitPitch = 66;                         // doubles: 16-byte rows
+constexpr int kSplitSmem = 3 * 32 * kSplitPitch * 8;    // three tiles
 template <int SL>
-__global__ void __launch_bounds__(256) k_split_cols(int K, int C, const double *__restrict__ X, int ldx, bool vec,
-                                                    const int *__restrict__ ex, const int *__restrict__ rexp,
-                                                    __nv_bfloat16 *__restrict__ out, int rows_p, int kp, int rb_log,
-                                                    float *__restrict__ sumsq) {
-    __shared__ double tile[32][65];
-    const int k0 = blockIdx.x * 32, c0 = blockIdx.y * 64;
-    {
-        const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-        const int c = c0 + 2 * tx;
+__global__ void __launch_bounds__(256, 4) k_split_cols(int K, int C, const double *__restrict__ X, int ldx, bool vec,
+                                                       const int *__restrict__ ex, const int *__restrict__ rexp,
+                                                       __nv_bfloat16 *__restrict__ out, int rows_p, int kp, int rb_log,
+                                                       float *__restrict__ sumsq, int tiles) {
+    extern __shared__ __align__(16) double tile[];
+    const int c0 = blockIdx.y * 64, t0 = blockIdx.x * tiles, t1 = min(t0 + tiles, (kp + 31) / 32);
+    auto stage = [&](int t) {
+        if (t < t1) {
+            double *dst = tile + (size_t)((t - t0) % 3) * 32 * kSplitPitch;
+            // rows past K and columns past C: zeros (no byte read)
+            if (vec) {
 #pragma unroll
-        for (int yy = ty; yy < 32; yy += 8) {
-            const double *p = X + (size_t)(k0 + yy) * ldx + c;
-            double a = 0.0, b = 0.0;
-            if (k0 + yy < K) {
-                if (vec && c + 1 < C) {
-                    const double2 q = *reinterpret_cast<const double2 *>(p);
-                    a = q.x, b = q.y;
-                } else {
-                    if (c < C) a = p[0];
-                    if (c + 1 < C) b = p[1];
+                for (int q = threadIdx.x; q < 1024; q += 256) {
+                    const int yy = q >> 5, c = 2 * (q & 31), k = 32 * t + yy;
+                    const int bytes = k < K ? 8 * max(0, min(2, C - c0 - c)) : 0;
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(
+                                     (unsigned)__cvta_generic_to_shared(dst + yy * kSplitPitch + c)),
+                                 "l"(bytes ? X + (size_t)k * ldx + c0 + c : X), "r"(bytes));
+                }
+            } else {
+#pragma unroll
+                for (int q = threadIdx.x; q < 2048; q += 256) {
+                    const int yy = q >> 6, c = q & 63, k = 32 * t + yy;
+                    const int bytes = k < K && c0 + c < C ? 8 : 0;
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(
+                                     (unsigned)__cvta_generic_to_shared(dst + yy * kSplitPitch + c)),
+                                 "l"(bytes ? X + (size_t)k * ldx + c0 + c : X), "r"(bytes));
                 }
             }
-            tile[yy][2 * tx] = a;
-            tile[yy][2 * tx + 1] = b;
         }
-    }
-    __syncthreads();
-    // thread -> (column c0 + lc, K group kg): a warp covers 8 columns x 4 groups
-    const int lane = threadIdx.x & 31;
-    const int lc = (lane & 7) + 8 * (threadIdx.x >> 5), kg = lane >> 3;
-    const int r = c0 + lc, k = k0 + 8 * kg;
-    double v[8];
-    int e[8];
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lc = (lane & 15) + 16 * (wid & 3), kg = (lane >> 4) + 2 * (wid >> 2), r = c0 + lc;
     const int er = r < C ? ex[r] : kNoExp;
+    float ss = 0.f;
+    stage(t0);
+    stage(t0 + 1);
+    for (int t = t0; t < t1; ++t) {
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        __syncthreads();  // tile t is there, the one of t - 1 is free
+        stage(t + 2);
+        const double *src = tile + (size_t)((t - t0) % 3) * 32 * kSplitPitch + kg * 8 * kSplitPitch + lc;
+        const int k = 32 * t + 8 * kg;
+        double v[8];
+        int e[8];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        v[t] = tile[kg * 8 + t][lc];
-        e[t] = er - (rexp && k + t < K ? rexp[k + t] : 0);
-    }
-    if (r < rows_p && k < kp)
-        split8_store<SL>(v, e, out + tiled_off<SL>(r, k, rows_p >> rb_log, rb_log), (size_t)16 << rb_log);
-    if (sumsq) {
-        float s = 0.f;
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            // x 2^(7-e) from the upper word (zeros and tiny values: nothing to add)
-            const unsigned hw = (unsigned)((unsigned long long)__double_as_longlong(v[t]) >> 32) & 0x7FFFFFFFu;
-            const int q = (int)(hw >> 20) - 1023 + 7 - er;
-            const float f = q > -60 && q < 60 ? __int_as_float(((q + 127) << 23) | (int)((hw & 0xFFFFFu) << 3)) : 0.f;
-            s = fmaf(f, f, s);
+        for (int u = 0; u < 8; ++u) {
+            v[u] = src[u * kSplitPitch];
+            e[u] = er - (rexp && k + u < K ? rexp[k + u] : 0);
         }
-        s += __shfl_xor_sync(0xffffffffu, s, 8);
-        s += __shfl_xor_sync(0xffffffffu, s, 16);
-        if (kg == 0 && r < C && s > 0.f) atomicAdd(&sumsq[r], s);
+        if (r < rows_p && k < kp)
+            split8_store<SL>(v, e, out + tiled_off<SL>(r, k, rows_p >> rb_log, rb_log), (size_t)16 << rb_log);
+        if (sumsq) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                // x 2^(7-e) from the upper word (zeros and tiny values: nothing to add)
+                const unsigned hw = (unsigned)((unsigned long long)__double_as_longlong(v[u]) >> 32) & 0x7FFFFFFFu;
+                const int q = (int)(hw >> 20) - 1023 + 7 - er;
+                const float f = q > -60 && q < 60 ? __int_as_float(((q + 127) << 23) | (int)((hw & 0xFFFFFu) << 3)) : 0.f;
+                ss = fmaf(f, f, ss);
+            }
+        }
+    }
+    if (sumsq) {
+        ss += __shfl_xor_sync(0xffffffffu, ss, 16);
+        if (lane < 16 && r < C && ss > 0.f) atomicAdd(&sumsq[r], ss);
     }
 }
 
@@ -975,16 +994,27 @@ static void ozaki_col_exps(cudaStream_t s, int n, int cols, const double *X, int
 
 static void split_cols_into(cudaStream_t s, const OzakiOperand &op, int n, const double *X, int ldx, const int *rexp,
                             float *sumsq) {
-    const dim3 g(cdiv(op.kp, 32), cdiv(op.rows_p, 64));
+    // four blocks per SM (shared memory), each with up to eight tiles
+    const int nt = cdiv(op.kp, 32), ncb = cdiv(op.rows_p, 64);
+    const int tiles = (int)std::max<int64_t>(1, std::min<int64_t>(8, (int64_t)nt * ncb / (4 * (int64_t)sm_count_oz())));
+    const dim3 g(cdiv(nt, tiles), ncb);
     const bool vec = pair_rows(X, ldx);
     const int rl = role_log(op.role);
-    if (op.digits == 5)
-        k_split_cols<5><<<g, 256, 0, s>>>(n, op.rows, X, ldx, vec, op.exps, rexp, op.slices, op.rows_p, op.kp, rl, sumsq);
-    else if (op.digits == 6)
-        k_split_cols<6><<<g, 256, 0, s>>>(n, op.rows, X, ldx, vec, op.exps, rexp, op.slices, op.rows_p, op.kp, rl, sumsq);
-    else
-        k_split_cols<7><<<g, 256, 0, s>>>(n, op.rows, X, ldx, vec, op.exps, rexp, op.slices, op.rows_p, op.kp, rl, sumsq);
-    HSIM_LAUNCHED();
+    auto go = [&](auto kernel) {
+        kernel<<<g, 256, kSplitSmem, s>>>(n, op.rows, X, ldx, vec, op.exps, rexp, op.slices, op.rows_p, op.kp, rl, sumsq,
+                                          tiles);
+        HSIM_LAUNCHED();
+    };
+    if (op.digits == 5) {
+        HSIM_SMEM_LIMIT_ONCE(k_split_cols<5>, kSplitSmem);
+        go(k_split_cols<5>);
+    } else if (op.digits == 6) {
+        HSIM_SMEM_LIMIT_ONCE(k_split_cols<6>, kSplitSmem);
+        go(k_split_cols<6>);
+    } else {
+        HSIM_SMEM_LIMIT_ONCE(k_split_cols<7>, kSplitSmem);
+        go(k_split_cols<7>);
+    }
 }
 
 OzakiOperand ozaki_split_cols(cudaStream_t s, int n, int cols, const double *X, int ldx, void *scratch, int digits,

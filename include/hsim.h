@@ -308,19 +308,23 @@ hsim_status hsim_spmm(hsim_ctx *ctx, int n_rows, int n_cols, const int32_t *row_
                       const int32_t *col_dev, const double *val_dev, int k, const double *X_dev,
                       int ldx, double *Y_dev, int ldy);
 /* G = A^T B (k_a x k_b, row-major, ld k_b) for tall A (n x k_a, ld lda) and
- * B (n x k_b, ld ldb): the reduced matrices Psi^T S Psi, Psi^T M Psi of Alg. 1. */
+ * B (n x k_b, ld ldb): the reduced matrices Psi^T S Psi, Psi^T M Psi of Alg. 1.
+ * Large products run on the BF16 tensor cores with seven digits per value (FP64
+ * accuracy; columns whose largest entry stands out and non-finite input on the
+ * FP64 units); their scratch is kept by the context for the next call (at most
+ * 2 GiB). */
 hsim_status hsim_gram(hsim_ctx *ctx, int n, int k_a, int k_b, const double *A_dev, int lda,
                       const double *B_dev, int ldb, double *G_dev);
 
 /* C = A B for A (n x k, ld lda) and small B (k x m, ld ldb), C (n x m, ld ldc):
- * the basis update Phi = Psi Phi_bar of Alg. 1. */
+ * the basis update Phi = Psi Phi_bar of Alg. 1.  Large products as hsim_gram's. */
 hsim_status hsim_gemm_update(hsim_ctx *ctx, int n, int k, int m, const double *A_dev, int lda,
                              const double *B_dev, int ldb, double *C_dev, int ldc);
 
 /* The same two products evaluated on BF16 tensor cores with FP64 accuracy
  * (mixed-precision path): every FP64 operand is split against a power of two
  * per row or column into 6 integer digits of at most 8 bits, digit products
- * are accumulated exactly in FP32 over chunks of 128 and summed in FP64; the
+ * are accumulated exactly in FP32 over chunks of 256 and summed in FP32 pairs; the
  * result matches the FP64 product to about 2^-47 of the row/column maxima.
  * hsim_gram_tc takes `digits` = 6 (that accuracy) or 5 (2^-39, 15 digit
  * products instead of 21; the solve's Grams at tolerances >= 1e-6).
@@ -332,12 +336,13 @@ hsim_status hsim_gemm_update_tc(hsim_ctx *ctx, int n, int k, int m, const double
 
 /* Dense generalised symmetric eigenproblem S_bar X = M_bar X Lambda (Alg. 1,
  * dense eigenproblem step; also the coarsest level of Alg. 3): LDL^T of
- * M_bar = C C^T, Householder tridiagonalisation, multisection and inverse
- * iteration on A = C^-1 S_bar C^-T, back-transformation, all in FP64.  S_bar
+ * M_bar = C C^T, Householder tridiagonalisation, Sturm counts and eigenvectors
+ * from minors (inverse iteration in clusters) on A = C^-1 S_bar C^-T,
+ * back-transformation, all in FP64.  S_bar
  * and M_bar are k x k row-major (read only); evals (k) ascending; X (k x k,
  * row-major, column j = eigenvector j, X^T M_bar X = I).  Returns
  * HSIM_E_NOT_SPD if M_bar is not positive definite.  sweeps_out (host) may
- * be NULL (always 0).  Scratch is allocated per call. */
+ * be NULL (always 0).  Scratch is kept by the context. */
 hsim_status hsim_ritz(hsim_ctx *ctx, int k, const double *Sbar_dev, const double *Mbar_dev,
                       double *evals_dev, double *X_dev, int *sweeps_out);
 /* The same solve as done by the mixed-precision path.  When a Gershgorin
@@ -346,8 +351,8 @@ hsim_status hsim_ritz(hsim_ctx *ctx, int k, const double *Sbar_dev, const double
  * Newton-Schulz iteration and A = W S_bar W, X = W V; otherwise, or if that
  * iteration stalls above max|I - W^2 M_bar| = 1e-12, C^-1 is formed
  * explicitly (LDL^T of M_bar, in-place inversion of L by block doubling, FP64)
- * and A = (C^-1 S_bar) C^-T, X = C^-T V.  Every product is FP64-accurate on
- * BF16 tensor cores (as hsim_gram_tc).  sweeps_out: the Newton-Schulz steps
+ * and A = (C^-1 S_bar) C^-T, X = C^-T V.  Every product is in FP64 up to
+ * k = 256, above FP64-accurate on BF16 tensor cores (as hsim_gram_tc).  sweeps_out: the Newton-Schulz steps
  * taken, 0 on the factorisation path.  Arguments and errors as hsim_ritz. */
 hsim_status hsim_ritz_tc(hsim_ctx *ctx, int k, const double *Sbar_dev, const double *Mbar_dev,
                          double *evals_dev, double *X_dev, int *sweeps_out);

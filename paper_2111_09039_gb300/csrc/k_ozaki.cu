@@ -361,7 +361,7 @@ int sm_count_oz() {
 // 2.88 / 4.48, with the loads 2.29 / 3.18 / 4.82, the rest is the drain.  One CTA
 // per tile, K staged 32 deep in twelve copies, one set of accumulators and MMAs
 // issued by a lone lane: 3.53 ms with five digits; the update of the same sizes
-// (six digits, 23,448 tiles 47 steps deep) 6.43 ms, now 4.0.
+// (six digits, 23,448 tiles 47 steps deep) 6.43 ms, now 3.7.
 //
 // Warp roles (320 threads): warp 0 issues the loads, warp 1 owns TMEM and
 // issues the MMAs (one thread), warps 2..9 drain, one TMEM lane (output row)

@@ -9,7 +9,8 @@
 //      forms w = p - (tau/2)(p.v) v and applies A22 -= v w^T + w v^T to its
 //      rows.  Where the matrix fits in the CTAs' shared memory (n up to about
 //      1650 on 152 SMs) each CTA keeps its rows there and one grid barrier per
-//      column suffices (k_tridiag_rows); otherwise the rows stay in global
+//      column suffices (k_tridiag_rows, which takes the product with the column
+//      before the reflector is known); otherwise the rows stay in global
 //      memory with two barriers per column (k_tridiag).  The reflectors are
 //      kept row-wise in Vh (contiguous for the back transformation).
 //   2. Eigenvalues of T by multisection on division-free Sturm counts, a group

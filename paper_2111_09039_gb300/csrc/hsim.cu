@@ -1176,7 +1176,7 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
                 const double t_prod = ts.stop();
                 inf.ms_tc_product += t_prod;
                 ph[4] = t_split + t_prod;
-            } else if (k::update64_on_digits(n, q, q)) {
+            } else if (k::update64_on_digits(n, q, q, true)) {
                 H->oz.reserve(k::update64_scratch(n, q, q));
                 k::update64(s, n, q, q, H->Psi.p, q, H->phibar.p, q, H->Phi.p, q, H->oz.p);
             } else {
@@ -1754,7 +1754,7 @@ hsim_status hsim_gemm_update(hsim_ctx *ctx, int n, int kk, int m, const double *
         HSIM_CHECK_ARG(n >= 0 && kk >= 0 && m >= 0 && lda >= kk && ldb >= m && ldc >= m, "bad sizes");
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"C", C}});
-        if (k::update64_on_digits(n, kk, m)) {
+        if (k::update64_on_digits(n, kk, m, false)) {
             CtxScratch<unsigned char> scratch(ctx, k::update64_scratch(n, kk, m));
             k::update64(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc, scratch.p);
             k::ozaki_check(ctx->stream);

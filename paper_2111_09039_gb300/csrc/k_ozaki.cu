@@ -1178,13 +1178,19 @@ void ozaki_update(cudaStream_t s, int n, int k, int m, const double *A, int lda,
 // 300 36,600 / 1,473; fewer rows than 1,024 are left to the FP64 kernel (its time
 // falls with them, and the rule on standing-out entries has no room).  Update
 // with k = 30 44 / 57 to 8,192 rows and 75 / 60 at 16,384, k = 50 77 / 55 from
-// 1,024 rows on, 163,842 x 300 25,700 / 1,049.
+// 1,024 rows on, 163,842 x 300 25,700 / 1,049.  A context's first call also
+// allocates the scratch, about 140 us: where the scratch is not held by the caller
+// an update takes the digits only if the FP64 kernel is slower than both (about 1.5
+// us per inner term when it waits for its chain, 1.1 TFLOP/s otherwise; 15,923 x 36
+// 130 us against 97, but 237 in a first call).
 constexpr int kDigits64 = 7;
 constexpr int kUpdate64MaxK = 4096;  // the inner sums of the measurements above
 
 bool gram64_on_digits(int n, int ka, int kb) { return n >= 1024 && (double)n * ka * kb >= 5e5; }
-bool update64_on_digits(int n, int k, int m) {
-    return k <= kUpdate64MaxK && ((k > 40 && (double)n * k * m >= 2e6) || (double)n * k * m >= 1.2e7);
+bool update64_on_digits(int n, int k, int m, bool held) {
+    const double work = (double)n * k * m;
+    if (k > kUpdate64MaxK) return false;
+    return held ? (k > 40 && work >= 2e6) || work >= 1.2e7 : (k >= 165 && work >= 2e6) || work >= 1.2e8;
 }
 
 // c_k = half the exponent gap between column k of A and row k of B

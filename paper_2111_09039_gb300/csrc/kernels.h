@@ -337,7 +337,7 @@ bool gram64_on_digits(int n, int ka, int kb);
 size_t gram64_scratch(int n, int ka, int kb);
 void gram64(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
             int ldg, bool lower, void *scratch);
-bool update64_on_digits(int n, int k, int m);
+bool update64_on_digits(int n, int k, int m, bool held);  // held: the scratch is there already
 size_t update64_scratch(int n, int k, int m);
 void update64(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
               int ldc, void *scratch);

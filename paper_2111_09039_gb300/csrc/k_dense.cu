@@ -147,14 +147,13 @@ __global__ void __launch_bounds__(256) k_gemm_nn(int n, int kk, int m, const T *
     }
 }
 
-// Sums over the rows of per-column terms (Rayleigh quotients, residual norms).
-// A CTA takes `rows` rows of 32 columns: warp w the rows w, w + 8, ..., a lane a
-// column; the eight partial sums meet in shared memory, then one FP64 atomic per
-// column and sum.  What bounds it: the latency of the loads where the matrices are
-// small, their bandwidth where they are large.  Mixed residual sums of 19,866 x 50
-// 24 us, quotients of 75 columns 15 us; with a thread per column walking 256 rows
-// one after the other 190 and 140 us, and a whole solve of 250,000 x 500 took
-// 658 ms where it takes 577 now.
+// Sums over the rows of per-column terms (Rayleigh quotients, residual norms), in
+// two forms.
+//
+// FP64 terms: a CTA takes `rows` rows of 32 columns, warp w the rows w, w + 8, ...,
+// a lane a column; the eight partial sums meet in shared memory, then one FP64
+// atomic per column and sum (an FP64 instruction of a warp takes 77 clocks, so a
+// block of rows is spread over the sub-partitions).
 template <class F>
 __global__ void __launch_bounds__(256) k_col_sums(int n, int k, int rows, const F f) {
     using A = typename F::Acc;
@@ -188,6 +187,50 @@ void col_sums(cudaStream_t s, int n, int k, const F &f) {
     if (n <= 0 || k <= 0) return;
     const int rows = (int64_t)n * cdiv(k, 32) >= (int64_t)256 * 8 * 152 ? 256 : 64;
     k_col_sums<<<cdiv(n, rows) * cdiv(k, 32), 256, 0, s>>>(n, k, rows, f);
+    HSIM_LAUNCHED();
+}
+
+// FP32 terms (the mixed path's Rayleigh quotients and residual norms): a warp
+// takes 256 rows of 32 columns, a lane a column, its rows added in their order,
+// then one FP64 atomic per column and sum.  The order is part of the result: the
+// quotients' FP32 rounding goes into every correction step, and other partial
+// sums (eight lanes of 8 to 32 rows) moved the eigenvectors of a batch at tol 1e-5
+// by 0.4 to 1.5e-9 where two of them are 10^-5 of their eigenvalue apart, next to a
+// spread between runs of 0.3 to 2e-9.
+// What bounds it: the latency of the loads where the matrices are small (hence 16
+// rows in flight), their bandwidth where they are large.
+constexpr int kSeqRows = 256, kSeqBatch = 16;
+template <class F>
+__global__ void __launch_bounds__(128) k_col_sums_seq(int n, int k, const F f) {
+    using A = typename F::Acc;
+    const int ncb = (k + 31) / 32;
+    const int64_t gw = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
+    // neighbouring warps share rows: whole rows are read at about the same time
+    const int rb = (int)(gw / ncb), j = (int)(gw - (int64_t)rb * ncb) * 32 + (threadIdx.x & 31);
+    const int64_t r0 = (int64_t)rb * kSeqRows;
+    if (r0 >= n || j >= k) return;
+    const int r_end = min(n, (int)r0 + kSeqRows);
+    A a[F::N];
+#pragma unroll
+    for (int u = 0; u < F::N; ++u) a[u] = A(0);
+    const double c = f.column(j);
+    int r = (int)r0;
+    for (; r + kSeqBatch <= r_end; r += kSeqBatch) {
+        typename F::In in[kSeqBatch];
+#pragma unroll
+        for (int q = 0; q < kSeqBatch; ++q) in[q] = f.load(r + q, j);
+#pragma unroll
+        for (int q = 0; q < kSeqBatch; ++q) f.add(in[q], c, a);
+    }
+    for (; r < r_end; ++r) f.add(f.load(r, j), c, a);
+#pragma unroll
+    for (int u = 0; u < F::N; ++u) atomicAdd(f.sum(j, u), (double)a[u]);
+}
+
+template <class F>
+void col_sums_seq(cudaStream_t s, int n, int k, const F &f) {
+    if (n <= 0 || k <= 0) return;
+    k_col_sums_seq<<<cdiv((int64_t)cdiv(n, kSeqRows) * cdiv(k, 32), 4), 128, 0, s>>>(n, k, f);
     HSIM_LAUNCHED();
 }
 
@@ -228,10 +271,15 @@ struct ResidualSumsMixed {
     double *out;
     __device__ double column(int j) const { return lam[j]; }
     __device__ double *sum(int j, int u) const { return out + 3 * j + u; }
-    __device__ void add(int r, int j, double l, float (&a)[3]) const {
-        const double sv = SP[(size_t)r * lds + j], mv = MP[(size_t)r * ldm + j];
-        const float rr = d2f_trunc(fma(-l, mv, sv)), sf = d2f_trunc(sv), mf = d2f_trunc(mv);
-        const float w = dinv ? d2f_trunc(dinv[r]) : 1.f;
+    struct In {
+        double s, m, w;
+    };
+    __device__ In load(int r, int j) const {
+        return {SP[(size_t)r * lds + j], MP[(size_t)r * ldm + j], dinv ? dinv[r] : 1.0};
+    }
+    __device__ void add(const In &in, double l, float (&a)[3]) const {
+        const float rr = d2f_trunc(fma(-l, in.m, in.s)), sf = d2f_trunc(in.s), mf = d2f_trunc(in.m);
+        const float w = d2f_trunc(in.w);
         a[0] = fmaf(w * rr, rr, a[0]);
         a[1] = fmaf(w * sf, sf, a[1]);
         a[2] = fmaf(w * mf, mf, a[2]);
@@ -252,10 +300,16 @@ struct ColDots2Mixed {
     double *w1, *w2;
     __device__ double column(int) const { return 0.0; }
     __device__ double *sum(int j, int u) const { return (u ? w2 : w1) + j; }
-    __device__ void add(int r, int j, double, float (&a)[2]) const {
-        const float x = d2f_trunc(X[(size_t)r * ldx + j]);
-        a[0] = fmaf(x, d2f_trunc(Y1[(size_t)r * ldy + j]), a[0]);
-        a[1] = fmaf(x, d2f_trunc(Y2[(size_t)r * ldy + j]), a[1]);
+    struct In {
+        double x, y1, y2;
+    };
+    __device__ In load(int r, int j) const {
+        return {X[(size_t)r * ldx + j], Y1[(size_t)r * ldy + j], Y2[(size_t)r * ldy + j]};
+    }
+    __device__ void add(const In &in, double, float (&a)[2]) const {
+        const float x = d2f_trunc(in.x);
+        a[0] = fmaf(x, d2f_trunc(in.y1), a[0]);
+        a[1] = fmaf(x, d2f_trunc(in.y2), a[1]);
     }
 };
 
@@ -271,10 +325,14 @@ struct ColDots2DiagMixed {
     double *w1, *w2;
     __device__ double column(int) const { return 0.0; }
     __device__ double *sum(int j, int u) const { return (u ? w2 : w1) + j; }
-    __device__ void add(int r, int j, double, float (&a)[2]) const {
-        const float x = d2f_trunc(X[(size_t)r * ldx + j]);
-        a[0] = fmaf(x, d2f_trunc(Y1[(size_t)r * ldy + j]), a[0]);
-        a[1] = fmaf(d2f_trunc(m[r]) * x, x, a[1]);
+    struct In {
+        double x, y, m;
+    };
+    __device__ In load(int r, int j) const { return {X[(size_t)r * ldx + j], Y1[(size_t)r * ldy + j], m[r]}; }
+    __device__ void add(const In &in, double, float (&a)[2]) const {
+        const float x = d2f_trunc(in.x);
+        a[0] = fmaf(x, d2f_trunc(in.y), a[0]);
+        a[1] = fmaf(d2f_trunc(in.m) * x, x, a[1]);
     }
 };
 
@@ -579,20 +637,20 @@ void col_dots2_mixed(cudaStream_t s, int n, int k, const double *X, int ldx, con
                      int ldy, double *w1, double *w2) {
     HSIM_CUDA(cudaMemsetAsync(w1, 0, (size_t)k * sizeof(double), s));
     HSIM_CUDA(cudaMemsetAsync(w2, 0, (size_t)k * sizeof(double), s));
-    col_sums(s, n, k, ColDots2Mixed{X, ldx, Y1, Y2, ldy, w1, w2});
+    col_sums_seq(s, n, k, ColDots2Mixed{X, ldx, Y1, Y2, ldy, w1, w2});
 }
 
 void col_dots2_diag_mixed(cudaStream_t s, int n, int k, const double *X, int ldx, const double *Y1, int ldy,
                           const double *m, double *w1, double *w2) {
     HSIM_CUDA(cudaMemsetAsync(w1, 0, (size_t)k * sizeof(double), s));
     HSIM_CUDA(cudaMemsetAsync(w2, 0, (size_t)k * sizeof(double), s));
-    col_sums(s, n, k, ColDots2DiagMixed{X, ldx, Y1, ldy, m, w1, w2});
+    col_sums_seq(s, n, k, ColDots2DiagMixed{X, ldx, Y1, ldy, m, w1, w2});
 }
 
 void residual_sums_mixed(cudaStream_t s, int n, int k, const double *SP, int lds, const double *MP, int ldm,
                          const double *lam, const double *dinv, double *out) {
     HSIM_CUDA(cudaMemsetAsync(out, 0, (size_t)3 * k * sizeof(double), s));
-    col_sums(s, n, k, ResidualSumsMixed{SP, lds, MP, ldm, lam, dinv, out});
+    col_sums_seq(s, n, k, ResidualSumsMixed{SP, lds, MP, ldm, lam, dinv, out});
 }
 
 #define HSIM_DENSE_INSTANTIATE(T)                                                                              \

@@ -132,6 +132,22 @@ __global__ void __launch_bounds__(kTriThreads) k_tridiag(int n, double *__restri
     }
 }
 
+// Largest biased exponent of the entries of A (out starts at zero).
+__global__ void __launch_bounds__(kTriThreads) k_max_exp(int64_t n, const double *__restrict__ A, int *__restrict__ out) {
+    int m = 0;
+#pragma unroll 4
+    for (int64_t i = (int64_t)blockIdx.x * kTriThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kTriThreads)
+        m = max(m, (__double2hiint(A[i]) >> 20) & 0x7FF);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+}
+
+// Power of two that brings a matrix with that exponent near 1; 0 where it is
+// within 2^+-100 as it is (or holds infinities or NaN).
+__device__ __forceinline__ int range_shift(int e) {
+    const int q = 1023 - max(e, 1);
+    return e == 0x7FF || abs(q) <= 100 ? 0 : q;
+}
 // Threads of k_tridiag_rows: one warp per SM sub-partition.  FP64 issues at a
 // 64th of the FP32 rate here, so every FP64 instruction that all warps repeat
 // (reductions, the reflector's scalars) costs its full issue time once per
@@ -310,7 +326,11 @@ __device__ __forceinline__ void rows_pass(int L, int n, double *a, const double 
 // beta, t = -1 / (beta u_0)): nothing is scaled, and A22 u = A22 y + (u_0 - y_0)
 // A22 e_0, whose last vector is the row k+1 that every CTA receives.  So the
 // product does not wait for the reflector: its norm, square root and reciprocal
-// are computed while the entries travel.  With p = t A22 u and w = p - (t/2)(p.u) u
+// are computed while the entries travel.  t is about 1 / ||u||^2 and t (p.u) up to
+// ||A|| / ||u||^2: A is brought near 1 by a power of two where it is not within
+// 2^+-100 (as the rows are loaded; k_tri_prep takes it off T), and a column whose
+// norm is below 2^-400 is taken as reduced (its entries below the first are
+// dropped, a backward error of 2^-300 ||A|| at the most), so neither overflows.  With p = t A22 u and w = p - (t/2)(p.u) u
 // the update of row r is -(u_r w + w_r u) = -(u_r p + b_r u), b_r = p_r - t (p.u)
 // u_r: w is not formed.  An entry costs three FP64 instructions.
 // The second half of a block's threads only communicates: it arrives at the
@@ -331,7 +351,7 @@ __global__ void __launch_bounds__(2 * kTrdThreads) k_tridiag_rows(int n, const d
                                                             double *__restrict__ e, double *__restrict__ tau,
                                                             double *__restrict__ Vh, double *__restrict__ pbuf,
                                                             double *__restrict__ rbuf, unsigned *__restrict__ counter,
-                                                            double *__restrict__ err) {
+                                                            double *__restrict__ err, const int *__restrict__ amax) {
     constexpr int NW = kTrdThreads / 32;
     extern __shared__ double sm[];
     const int G = gridDim.x, b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -344,12 +364,13 @@ __global__ void __launch_bounds__(2 * kTrdThreads) k_tridiag_rows(int n, const d
     __shared__ double red[NW];
     __shared__ double redr[NW][RMAX];
     __shared__ int gave_up;
+    const int shift = range_shift(*amax);
     for (int i = 0; i < R; ++i) {
         const double *src = A + (size_t)(b + i * G) * n;
-        for (int j = tid; j < n; j += 2 * kTrdThreads) rows[(size_t)i * n + j] = src[j];
+        for (int j = tid; j < n; j += 2 * kTrdThreads) rows[(size_t)i * n + j] = shift ? ldexp(src[j], shift) : src[j];
     }
     // no update before the first column: zeros in u and P of the one before
-    for (int j = tid; j < n; j += 2 * kTrdThreads) cur[j] = A[j], prev[j] = P[j] = 0.0;
+    for (int j = tid; j < n; j += 2 * kTrdThreads) cur[j] = shift ? ldexp(A[j], shift) : A[j], prev[j] = P[j] = 0.0;
     if (tid == 0) gave_up = 0;
     __syncthreads();
     if (tid >= kTrdThreads) {
@@ -430,18 +451,12 @@ __global__ void __launch_bounds__(2 * kTrdThreads) k_tridiag_rows(int n, const d
         // (tests on the bits: an FP64 comparison waits for the pipe)
         if ((__double2hiint(sigma) | __double2loint(sigma)) != 0) {
             const double s2 = fma(x0, x0, sigma);
-            const int ex = __double2hiint(s2) >> 20;
-            if (ex > 93 && ex < 1952) {  // 1e-280 .. 1e279
+            if (((__double2hiint(s2) >> 20) & 0x7FF) >= 1023 - 800) {
                 const double r = rsqrt_step(s2), m0 = s2 * r;
                 const double mu = fma(fma(-m0, m0, s2), 0.5 * r, m0);
                 beta = __double2hiint(x0) >= 0 ? -mu : mu;
                 u0 = x0 - beta;
                 t = rcp_step(-beta * u0);
-            } else {
-                const double mu = sqrt(s2);
-                beta = x0 >= 0.0 ? -mu : mu;
-                u0 = x0 - beta;
-                t = -1.0 / (beta * u0);
             }
         }
         const double d0 = u0 - x0, c0 = u0 * t;
@@ -658,13 +673,23 @@ __global__ void __launch_bounds__(128) k_tri_back_wy(int n, int m, int nv, int b
 // 2^-120 in FP64 and 2^-40 in FP32: couplings of 2^-60 and 2^-20 of ||T||, below
 // the accuracy of either count) and their FP32 copies; bounds: the Gershgorin
 // interval of the scaled T, ||T|| (not scaled), the scale; F_j for k_tri_vectors
-__global__ void k_tri_prep(int n, const double *__restrict__ d, const double *__restrict__ e, double *__restrict__ ds,
-                           double *__restrict__ e2s, double *__restrict__ bounds, float *__restrict__ d32,
-                           float *__restrict__ e232, double *__restrict__ fm, double *__restrict__ fi,
-                           int *__restrict__ fx) {
+// amax (may be null): d and e come from a matrix scaled by 2^range_shift, which
+// is taken off first.
+__global__ void k_tri_prep(int n, double *__restrict__ d, double *__restrict__ e, const int *__restrict__ amax,
+                           double *__restrict__ ds, double *__restrict__ e2s, double *__restrict__ bounds,
+                           float *__restrict__ d32, float *__restrict__ e232, double *__restrict__ fm,
+                           double *__restrict__ fi, int *__restrict__ fx) {
     __shared__ double red[3][kTriThreads / 32];
     __shared__ double sm[2][kTriThreads];
     __shared__ int sx[2][kTriThreads];
+    const int shift = amax ? range_shift(*amax) : 0;
+    if (shift) {
+        for (int j = threadIdx.x; j < n; j += kTriThreads) {
+            d[j] = ldexp(d[j], -shift);
+            if (j + 1 < n) e[j] = ldexp(e[j], -shift);
+        }
+        __syncthreads();
+    }
     double lo = DBL_MAX, hi = -DBL_MAX, nm = 0.0;
     for (int j = threadIdx.x; j < n; j += kTriThreads) {
         const double r = (j > 0 ? fabs(e[j - 1]) : 0.0) + (j + 1 < n ? fabs(e[j]) : 0.0);
@@ -1259,13 +1284,14 @@ int rows_grid(int n, int sms, size_t *smem, int *rmax) {
 
 template <int RMAX>
 bool launch_tridiag_rows(cudaStream_t s, int G, size_t smem, int sms, int n, const double *A, double *d, double *e,
-                         double *tau, double *Vh, double *pbuf, double *rbuf, unsigned *counter, double *err) {
+                         double *tau, double *Vh, double *pbuf, double *rbuf, unsigned *counter, double *err,
+                         const int *amax) {
     HSIM_SMEM_LIMIT_ONCE(k_tridiag_rows<RMAX>, kTriSmemMax);
     int per_sm = 0;
     HSIM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_tridiag_rows<RMAX>, 2 * kTrdThreads, smem));
     if ((int64_t)per_sm * sms < G) return false;
     int nn = n;
-    void *args[] = {&nn, &A, &d, &e, &tau, &Vh, &pbuf, &rbuf, &counter, &err};
+    void *args[] = {&nn, &A, &d, &e, &tau, &Vh, &pbuf, &rbuf, &counter, &err, &amax};
     HSIM_CUDA(cudaLaunchCooperativeKernel((void *)k_tridiag_rows<RMAX>, dim3(G), dim3(2 * kTrdThreads), args, smem, s));
     HSIM_LAUNCHED();
     return true;
@@ -1342,12 +1368,17 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
     bool done = false;
     double *err = bounds + 4;                                       // set if a barrier gave up
     unsigned *counter = reinterpret_cast<unsigned *>(bounds + 5);  // arrivals of the barriers
-    HSIM_CUDA(cudaMemsetAsync(err, 0, 2 * sizeof(double), s));
+    int *amax = reinterpret_cast<int *>(bounds + 6);               // largest exponent of A
+    HSIM_CUDA(cudaMemsetAsync(err, 0, 3 * sizeof(double), s));
     if (G > 0) {
-        if (rmax == 4) done = launch_tridiag_rows<4>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf, counter, err);
-        else if (rmax == 8) done = launch_tridiag_rows<8>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf, counter, err);
-        else done = launch_tridiag_rows<16>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf, counter, err);
+        k_max_exp<<<(unsigned)std::min<int64_t>(sms, ((int64_t)n * n + 4 * kTriThreads - 1) / (4 * kTriThreads)), kTriThreads,
+                    0, s>>>((int64_t)n * n, A, amax);
+        HSIM_LAUNCHED();
+        if (rmax == 4) done = launch_tridiag_rows<4>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf, counter, err, amax);
+        else if (rmax == 8) done = launch_tridiag_rows<8>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf, counter, err, amax);
+        else done = launch_tridiag_rows<16>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf, counter, err, amax);
     }
+    const bool in_rows = done;
     if (!done) {
         const size_t smem = 2 * (size_t)n * sizeof(double);
         HSIM_CHECK_ARG(smem <= kTriSmemMax, "sym_eig: matrix too large for the tridiagonalisation kernel");
@@ -1362,7 +1393,7 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
         HSIM_LAUNCHED();
     }
     // 2. eigenvalues
-    k_tri_prep<<<1, kTriThreads, 0, s>>>(n, d, e, ds, e2, bounds, d32, e232, fm, fi, fx);
+    k_tri_prep<<<1, kTriThreads, 0, s>>>(n, d, e, in_rows ? amax : nullptr, ds, e2, bounds, d32, e232, fm, fi, fx);
     HSIM_LAUNCHED();
     if (detail) cudaEventRecord(t1, s);
     // about one warp per SM: G eigenvalues per warp (L = 32 / G >= 2 lanes each)

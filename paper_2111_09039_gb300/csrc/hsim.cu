@@ -1149,8 +1149,8 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
             } else {
                 if (k::gram64_on_digits(n, q, q)) {
                     H->oz.reserve(k::gram64_scratch(n, q, q));
-                    k::gram64(s, n, q, q, H->Psi.p, q, H->SP.p, q, H->Sbar.p, q, true, H->oz.p);
-                    k::gram64(s, n, q, q, H->Psi.p, q, H->MP.p, q, H->Mbar.p, q, true, H->oz.p);
+                    k::gram64(s, n, q, q, H->Psi.p, q, H->SP.p, q, H->Sbar.p, q, true, k::Held::Norms, H->oz.p);
+                    k::gram64(s, n, q, q, H->Psi.p, q, H->MP.p, q, H->Mbar.p, q, true, k::Held::Norms, H->oz.p);
                 } else {
                     k::gram(s, n, q, q, H->Psi.p, q, H->SP.p, q, H->Sbar.p, q, true);
                     k::gram(s, n, q, q, H->Psi.p, q, H->MP.p, q, H->Mbar.p, q, true);
@@ -1178,7 +1178,7 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
                 ph[4] = t_split + t_prod;
             } else if (k::update64_on_digits(n, q, q, true)) {
                 H->oz.reserve(k::update64_scratch(n, q, q));
-                k::update64(s, n, q, q, H->Psi.p, q, H->phibar.p, q, H->Phi.p, q, H->oz.p);
+                k::update64(s, n, q, q, H->Psi.p, q, H->phibar.p, q, H->Phi.p, q, k::Held::Norms, H->oz.p);
             } else {
                 k::gemm_nn(s, n, q, q, H->Psi.p, q, H->phibar.p, q, H->Phi.p, q);
             }
@@ -1738,7 +1738,7 @@ hsim_status hsim_gram(hsim_ctx *ctx, int n, int ka, int kb, const double *A, int
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"G", G}});
         if (k::gram64_on_digits(n, ka, kb)) {
             CtxScratch<unsigned char> scratch(ctx, k::gram64_scratch(n, ka, kb));
-            k::gram64(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, false, scratch.p);
+            k::gram64(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, false, k::Held::Entries, scratch.p);
             k::ozaki_check(ctx->stream);
             return;
         }
@@ -1756,7 +1756,7 @@ hsim_status hsim_gemm_update(hsim_ctx *ctx, int n, int kk, int m, const double *
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"C", C}});
         if (k::update64_on_digits(n, kk, m, false)) {
             CtxScratch<unsigned char> scratch(ctx, k::update64_scratch(n, kk, m));
-            k::update64(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc, scratch.p);
+            k::update64(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc, k::Held::Entries, scratch.p);
             k::ozaki_check(ctx->stream);
             return;
         }

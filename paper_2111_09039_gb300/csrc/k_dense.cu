@@ -47,10 +47,11 @@ constexpr int TK = 16;  // k step
 template <typename T>
 __global__ void __launch_bounds__(256) k_gram(int n, int ka, int kb, const T *__restrict__ A, int lda,
                                               const T *__restrict__ B, int ldb, double *__restrict__ G,
-                                              int ldg, int rows_per_split, int lower_only, const int *__restrict__ only_if) {
-    if (only_if && !*only_if) return;
+                                              int ldg, int rows_per_split, int lower_only,
+                                              const int *__restrict__ tiles, int tiles_ld) {
     const int ti = blockIdx.x, tj = blockIdx.y;
     if (lower_only && tj > ti) return;
+    if (tiles && tiles[(size_t)ti * tiles_ld + tj] == 0) return;
     const int i0 = ti * TB, j0 = tj * TB;
     const int r_beg = blockIdx.z * rows_per_split;
     const int r_end = min(n, r_beg + rows_per_split);
@@ -93,20 +94,19 @@ __global__ void __launch_bounds__(256) k_gram(int n, int ka, int kb, const T *__
     }
 }
 
-__global__ void k_mirror_lower(int k, double *__restrict__ G, int ldg, const int *__restrict__ only_if) {
-    if (only_if && !*only_if) return;
+__global__ void k_mirror_lower(int k, double *__restrict__ G, int ldg, const int *__restrict__ tiles, int tiles_ld) {
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)k * k) return;
     int i = (int)(idx / k), j = (int)(idx % k);
-    if (j > i) G[(size_t)i * ldg + j] = G[(size_t)j * ldg + i];
+    if (j > i && (!tiles || tiles[(size_t)(j / TB) * tiles_ld + i / TB] != 0)) G[(size_t)i * ldg + j] = G[(size_t)j * ldg + i];
 }
 
 // C[r0:r0+64, j0:j0+64] = A[r, :] B[:, j]
 template <typename T>
 __global__ void __launch_bounds__(256) k_gemm_nn(int n, int kk, int m, const T *__restrict__ A, int lda,
                                                  const double *__restrict__ B, int ldb, T *__restrict__ C,
-                                                 int ldc, const int *__restrict__ only_if) {
-    if (only_if && !*only_if) return;
+                                                 int ldc, const int *__restrict__ tiles, int tiles_ld) {
+    if (tiles && tiles[(size_t)blockIdx.x * tiles_ld + blockIdx.y] == 0) return;
     const int r0 = blockIdx.x * TB, j0 = blockIdx.y * TB;
     __shared__ T As[TK][TB + 1];
     __shared__ T Bs[TK][TB];
@@ -568,18 +568,19 @@ DenseFront &dense_front(int k, cudaStream_t s) {
 
 template <typename T>
 static void launch_gram(cudaStream_t s, int n, int ka, int kb, const T *A, int lda, const T *B, int ldb, double *G,
-                        int ldg, bool lower_only, const int *only_if) {
+                        int ldg, bool lower_only, const int *tiles, int tiles_ld) {
     int ti = cdiv(ka, TB), tj = cdiv(kb, TB);
-    int64_t tiles = lower_only ? (int64_t)ti * (ti + 1) / 2 : (int64_t)ti * tj;
-    int64_t want = std::max<int64_t>(1, (4LL * sm_count() + tiles - 1) / tiles);
+    int64_t nt = lower_only ? (int64_t)ti * (ti + 1) / 2 : (int64_t)ti * tj;
+    int64_t want = std::max<int64_t>(1, (4LL * sm_count() + nt - 1) / nt);
     int64_t rows = std::max<int64_t>(256, (n + want - 1) / want);
     rows = (rows + TK - 1) / TK * TK;
     unsigned splits = cdiv(n, rows);
     dim3 g(ti, tj, splits);
-    k_gram<T><<<g, 256, 0, s>>>(n, ka, kb, A, lda, B, ldb, G, ldg, (int)rows, lower_only ? 1 : 0, only_if);
+    k_gram<T><<<g, 256, 0, s>>>(n, ka, kb, A, lda, B, ldb, G, ldg, (int)rows, lower_only ? 1 : 0, tiles,
+                                        tiles_ld);
     HSIM_LAUNCHED();
     if (lower_only) {
-        k_mirror_lower<<<cdiv((int64_t)ka * ka, 256), 256, 0, s>>>(ka, G, ldg, only_if);
+        k_mirror_lower<<<cdiv((int64_t)ka * ka, 256), 256, 0, s>>>(ka, G, ldg, tiles, tiles_ld);
         HSIM_LAUNCHED();
     }
 }
@@ -593,36 +594,39 @@ void gram(cudaStream_t s, int n, int ka, int kb, const T *A, int lda, const T *B
         HSIM_CUDA(cudaMemset2DAsync(G, (size_t)ldg * sizeof(double), 0, (size_t)kb * sizeof(double), ka, s));
     }
     if (n <= 0 || ka <= 0 || kb <= 0) return;
-    launch_gram<T>(s, n, ka, kb, A, lda, B, ldb, G, ldg, lower_only, nullptr);
+    launch_gram<T>(s, n, ka, kb, A, lda, B, ldb, G, ldg, lower_only, nullptr, 0);
 }
 
-__global__ void k_zero_if(int rows, int cols, double *__restrict__ G, int ldg, const int *__restrict__ only_if) {
-    if (!*only_if) return;
+__global__ void k_zero_tiles(int rows, int cols, double *__restrict__ G, int ldg, int lower_only,
+                             const int *__restrict__ tiles, int tiles_ld) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < (int64_t)rows * cols) G[(size_t)(idx / cols) * ldg + idx % cols] = 0.0;
+    if (idx >= (int64_t)rows * cols) return;
+    const int i = (int)(idx / cols), j = (int)(idx % cols);
+    if (lower_only && j / TB > i / TB) return;
+    if (tiles[(size_t)(i / TB) * tiles_ld + j / TB] != 0) G[(size_t)i * ldg + j] = 0.0;
 }
 
-void gram_if(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
-             int ldg, bool lower_only, const int *flag) {
+void gram_tiles(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
+                int ldg, bool lower_only, const int *tiles, int tiles_ld) {
     if (n <= 0 || ka <= 0 || kb <= 0) return;
-    k_zero_if<<<cdiv((int64_t)ka * kb, 256), 256, 0, s>>>(ka, kb, G, ldg, flag);
+    k_zero_tiles<<<cdiv((int64_t)ka * kb, 256), 256, 0, s>>>(ka, kb, G, ldg, lower_only ? 1 : 0, tiles, tiles_ld);
     HSIM_LAUNCHED();
-    launch_gram<double>(s, n, ka, kb, A, lda, B, ldb, G, ldg, lower_only, flag);
+    launch_gram<double>(s, n, ka, kb, A, lda, B, ldb, G, ldg, lower_only, tiles, tiles_ld);
 }
 
 template <typename T>
 void gemm_nn(cudaStream_t s, int n, int kk, int m, const T *A, int lda, const double *B, int ldb, T *C, int ldc) {
     if (n <= 0 || m <= 0) return;
     dim3 g(cdiv(n, TB), cdiv(m, TB));
-    k_gemm_nn<T><<<g, 256, 0, s>>>(n, kk, m, A, lda, B, ldb, C, ldc, nullptr);
+    k_gemm_nn<T><<<g, 256, 0, s>>>(n, kk, m, A, lda, B, ldb, C, ldc, nullptr, 0);
     HSIM_LAUNCHED();
 }
 
-void gemm_nn_if(cudaStream_t s, int n, int kk, int m, const double *A, int lda, const double *B, int ldb, double *C,
-                int ldc, const int *flag) {
+void gemm_nn_tiles(cudaStream_t s, int n, int kk, int m, const double *A, int lda, const double *B, int ldb, double *C,
+                   int ldc, const int *tiles, int tiles_ld) {
     if (n <= 0 || m <= 0) return;
     dim3 g(cdiv(n, TB), cdiv(m, TB));
-    k_gemm_nn<double><<<g, 256, 0, s>>>(n, kk, m, A, lda, B, ldb, C, ldc, flag);
+    k_gemm_nn<double><<<g, 256, 0, s>>>(n, kk, m, A, lda, B, ldb, C, ldc, tiles, tiles_ld);
     HSIM_LAUNCHED();
 }
 

@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 #include "common.h"
@@ -34,6 +35,7 @@ namespace {
 
 constexpr int kNoExp = -5000;     // exponent of a row or column of zeros
 constexpr int kNonFinite = 1025;  // of an infinity or NaN
+constexpr int kBadExp = 1 << 20;  // the same in a block whose rows or columns are scaled
 
 inline unsigned cdiv(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
@@ -49,40 +51,83 @@ __device__ __forceinline__ int exp_bits(double a) {
     return b == 0 ? kNoExp : -1010 - __clzll((long long)b);
 }
 
+// |x| 2^-e < 1 truncated to 24 bits (0 for subnormals and below 2^-126)
+__device__ __forceinline__ float scaled_abs(double x, int e) {
+    const unsigned h = (unsigned)__double2hiint(x) & 0x7FFFFFFFu, l = (unsigned)__double2loint(x);
+    const int E = (int)(h >> 20), q = E - 1023 - e + 127;
+    return E != 0 && q >= 1 && q < 127 ? __uint_as_float(((unsigned)q << 23) | ((h & 0xFFFFFu) << 3) | (l >> 29)) : 0.f;
+}
+
+// Limits of a row (column) in the check of an FP64 product's entries (digits_fail):
+// infinite where it holds infinities or NaN, minus infinity where it is zero
+__device__ __forceinline__ bool bad_exp(int e) { return e == kNonFinite || e >= kBadExp; }
+__device__ __forceinline__ float entry_limit(int e, float sum) {
+    return bad_exp(e) ? __int_as_float(0x7F800000) : e == kNoExp ? __int_as_float((int)0xFF800000) : sum;
+}
+
 // per-row exponents of a row-major R x C FP64 block: one warp per row; with
-// cexp, of the block whose column c is scaled by 2^-cexp[c]
+// cexp, of the block whose column c is scaled by 2^-cexp[c]; limits: entry_limit of
+// the row's sum of |x| in units of 2^ex.  The upper words decide; subnormals count as
+// 2^-1022 unless the row holds nothing else (and is not scaled).
 __global__ void k_row_exps(int R, int C, const double *__restrict__ X, int ldx, const int *__restrict__ cexp,
-                           int *__restrict__ ex, int *__restrict__ nonfinite) {
+                           int *__restrict__ ex, float *__restrict__ limits) {
     int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     int lane = threadIdx.x & 31;
     if (row >= R) return;
+    const double *x = X + (size_t)row * ldx;
     int m = kNoExp;
-    bool bad = false;
 #pragma unroll 4
     for (int j = lane; j < C; j += 32) {
-        const int e = exp_bits(X[(size_t)row * ldx + j]);
-        bad |= e == kNonFinite;
-        m = max(m, cexp && e != kNoExp ? e - cexp[j] : e);
+        const double v = x[j];
+        const int h = __double2hiint(v) & 0x7FFFFFFF, c = cexp ? cexp[j] : 0;
+        const int e = (h >> 20) - 1022 - c;
+        m = max(m, (h | __double2loint(v)) == 0 ? kNoExp : cexp && h >= 0x7FF00000 ? kBadExp : e);
     }
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (m == -1022 && !cexp) {
+        m = kNoExp;
+        for (int j = lane; j < C; j += 32) m = max(m, exp_bits(x[j]));
+        m = __reduce_max_sync(0xffffffffu, m);
+    }
     if (lane == 0) ex[row] = m;
-    if (nonfinite && bad) atomicOr(nonfinite, 1);
+    if (!limits) return;
+    float s = 0.f;
+#pragma unroll 4
+    for (int j = lane; j < C; j += 32) s += scaled_abs(x[j], m + (cexp ? cexp[j] : 0));
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) limits[row] = entry_limit(m, s);
+}
+
+// h (upper word of |x|) added to a sum of magnitudes in units of 2^(ref - 1023),
+// ref the biased exponent of the first normal value met (0: none yet); infinite
+// where a later value is 2^127 times that
+__device__ __forceinline__ void add_abs(unsigned h, int &ref, float &sum) {
+    const int E = (int)(h >> 20);
+    ref = ref != 0 ? ref : E;
+    const int q = E - ref + 127;
+    const float f = __uint_as_float((h << 3) + ((unsigned)(127 - ref) << 23));
+    sum += q > 254 ? __int_as_float(0x7F800000) : E != 0 && q >= 1 ? f : 0.f;
 }
 
 // per-column exponents of a row-major R x C FP64 block (ex pre-set to kNoExp);
-// with rexp, of the block whose row r is scaled by 2^rexp[r].  A CTA takes 64
-// columns (two per thread, 32 threads) of `rows` rows (eight at a time).
+// SHIFT: of the block whose row r is scaled by 2^rexp[r]; SUMS: sum of |x| added per
+// column.  A CTA takes 64 columns (two per thread, 32 threads) of `rows` rows (eight
+// at a time).  Without SHIFT the upper words decide (three integer instructions an
+// entry where exp_bits takes a dozen; subnormal columns are read again).
+template <bool SHIFT, bool SUMS>
 __global__ void __launch_bounds__(256) k_col_exps(int R, int C, const double *__restrict__ X, int ldx, int rows,
                                                   const int *__restrict__ rexp, bool vec, int *__restrict__ ex,
-                                                  int *__restrict__ nonfinite) {
+                                                  double *__restrict__ sums) {
     __shared__ int red[8][64];
+    __shared__ double reds[SUMS ? 8 : 1][64];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int j = blockIdx.y * 64 + 2 * tx;
-    const int r1 = min(R, (int)(blockIdx.x + 1) * rows);
-    int m0 = kNoExp, m1 = kNoExp;
-    bool bad = false;
+    const int ra = blockIdx.x * rows + ty, r1 = min(R, (int)(blockIdx.x + 1) * rows);
+    int m0 = kNoExp, m1 = kNoExp, ref0 = 0, ref1 = 0;
+    unsigned h0 = 0, h1 = 0;
+    float s0 = 0.f, s1 = 0.f;
 #pragma unroll 4
-    for (int r = blockIdx.x * rows + ty; r < r1; r += 8) {
+    for (int r = ra; r < r1; r += 8) {
         const double *p = X + (size_t)r * ldx + j;
         double a = 0.0, b = 0.0;
         if (vec && j + 1 < C) {
@@ -92,36 +137,112 @@ __global__ void __launch_bounds__(256) k_col_exps(int R, int C, const double *__
             if (j < C) a = p[0];
             if (j + 1 < C) b = p[1];
         }
-        int ea = exp_bits(a), eb = exp_bits(b);
-        bad |= ea == kNonFinite || eb == kNonFinite;
-        if (rexp) {
+        if (SHIFT) {
+            int ea = exp_bits(a), eb = exp_bits(b);
             const int q = rexp[r];
-            if (ea != kNoExp) ea += q;
-            if (eb != kNoExp) eb += q;
+            if (ea != kNoExp) ea = ea == kNonFinite ? kBadExp : ea + q;
+            if (eb != kNoExp) eb = eb == kNonFinite ? kBadExp : eb + q;
+            m0 = max(m0, ea);
+            m1 = max(m1, eb);
+        } else {
+            const unsigned ha = (unsigned)__double2hiint(a) & 0x7FFFFFFFu, hb = (unsigned)__double2hiint(b) & 0x7FFFFFFFu;
+            h0 = max(h0, ha);
+            h1 = max(h1, hb);
+            if (SUMS) {
+                add_abs(ha, ref0, s0);
+                add_abs(hb, ref1, s1);
+            }
         }
-        m0 = max(m0, ea);
-        m1 = max(m1, eb);
+    }
+    if (!SHIFT) {
+        m0 = (int)(h0 >> 20) - 1022;
+        m1 = (int)(h1 >> 20) - 1022;
+        if (h0 < 0x100000u) {
+            m0 = kNoExp;
+            for (int r = ra; r < r1 && j < C; r += 8) m0 = max(m0, exp_bits(X[(size_t)r * ldx + j]));
+        }
+        if (h1 < 0x100000u) {
+            m1 = kNoExp;
+            for (int r = ra; r < r1 && j + 1 < C; r += 8) m1 = max(m1, exp_bits(X[(size_t)r * ldx + j + 1]));
+        }
     }
     red[ty][2 * tx] = m0;
     red[ty][2 * tx + 1] = m1;
+    if (SUMS) {
+        reds[ty][2 * tx] = ldexp((double)s0, ref0 - 1023);
+        reds[ty][2 * tx + 1] = ldexp((double)s1, ref1 - 1023);
+    }
     __syncthreads();
     if (threadIdx.x < 64 && blockIdx.y * 64 + threadIdx.x < C) {
         int m = red[0][threadIdx.x];
 #pragma unroll
         for (int q = 1; q < 8; ++q) m = max(m, red[q][threadIdx.x]);
         if (m != kNoExp) atomicMax(&ex[blockIdx.y * 64 + threadIdx.x], m);
+        if (SUMS) {
+            double t = reds[0][threadIdx.x];
+#pragma unroll
+            for (int q = 1; q < 8; ++q) t += reds[q][threadIdx.x];
+            if (t != 0.0) atomicAdd(&sums[blockIdx.y * 64 + threadIdx.x], t);
+        }
     }
-    if (nonfinite && bad) atomicOr(nonfinite, 1);
 }
 
-// seven-digit Grams: flag set if a column's largest entry stands out, n 2^(2 e) >=
-// 1024 ||x||^2 (16 to 32 times the root mean square; a column that one entry
-// dominates has n to 4 n there); below that the truncation stays under the
-// rounding of the FP64 sums
-__global__ void k_guard_cols(int cols, float n, const int *__restrict__ ex, const float *__restrict__ sumsq,
-                             int *__restrict__ flag) {
+// ---- which tiles of an FP64 product the seven digits may compute ----------------
+//
+// With |x| < 2^e per row of C (column of C), x = 2^e u, the digits leave
+//     |error of C_ij| <= 2^(e_i + e_j) (2^-56 (sum |u_i| + sum |u_j|) + 2^-61 K),
+// the rounding of either factor's last digit against the other factor, and the
+// digit pairs left out.  FP64 arithmetic is held by sum |x_i| |x_j| instead (K
+// 2^-53 of it in the worst case, a few 2^-53 as a rule), so an entry is left to the
+// digits only where that sum is large enough:
+//     sum |u_i| + sum |u_j| + K / 32 <= R h_ij,   h_ij = sum |u_i| |u_j|,
+// R = min(8 K, 52 sqrt(K), 1024): K 2^-53 sum |x_i| |x_j| at the most if all K
+// roundings had one sign, 2^-50 since they have either (sqrt(K) of them are felt).
+// h is one BF16 product of the magnitudes, rounded down (a Gram takes every fourth
+// or eighth row: part of the terms is a lower bound too).  The 64 x 64 tiles with an entry
+// that fails, or with infinities or NaN, go to the FP64 kernel and are skipped here.
+// Normal data have a left side of 0.2 to 0.3 K and a right side of 1.5 to 8 K; a
+// second factor I + 0.3 N(0, 1) / sqrt(K) 42 to 72 and 190 to 370 at K = 300 (110 to
+// 220 in the least of 49 million entries).  Columns graded from 1 to 10^-10
+// against one that lives on the small half fail, where the digits left 2.4e-9 of
+// sum |x_i| |x_j|.
+static float digits_ratio(double k) { return (float)std::min({8.0 * k, 52.0 * std::sqrt(k), 1024.0}); }
+
+// li, lj: entry_limit of sum |u_i| + K / 32 and of sum |u_j|
+__device__ __forceinline__ bool digits_fail(float li, float lj, float ratio, float h) { return !(li + lj <= ratio * h); }
+
+// tiles of an M x N Gram with entries that fail
+__global__ void k_check_tiles(int M, int N, float k, float ratio, const float *__restrict__ h, const int *__restrict__ ex,
+                              const double *__restrict__ sx, const int *__restrict__ ey, const double *__restrict__ sy,
+                              int *__restrict__ tiles, int ntn) {
+    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (idx >= (int64_t)M * N) return;
+    const int i = (int)(idx / N), j = (int)(idx % N);
+    const float li = entry_limit(ex[i], (float)ldexp(sx[i], -ex[i]) + k * 0.03125f);
+    if (digits_fail(li, entry_limit(ey[j], (float)ldexp(sy[j], -ey[j])), ratio, h[idx]))
+        tiles[(size_t)(i >> 6) * ntn + (j >> 6)] = 1;
+}
+
+// limits of n columns (sums |u| on entry) with their K / 32, up to np
+__global__ void k_col_limits(int n, int np, float k, const int *__restrict__ ex, float *__restrict__ limits) {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < cols && ex[j] != kNoExp && n * 16384.f >= 1024.f * sumsq[j]) atomicOr(flag, 2);
+    if (j < np) limits[j] = j < n ? entry_limit(ex[j], limits[j] + k * 0.03125f) : entry_limit(kNoExp, 0.f);
+}
+
+// Products whose result is held to norms instead (Rayleigh-Ritz): tiles with
+// infinities or NaN and, with sums, columns i with K 2^e_i > 128 sum |x_i|, whose
+// rounding to digits could pass 2^-48 ||x_i|| ||x_j||.  A CTA per tile.
+__global__ void __launch_bounds__(128) k_guard_tiles(int M, int N, double k, const int *__restrict__ ex,
+                                                     const double *__restrict__ sx, const int *__restrict__ ey,
+                                                     const double *__restrict__ sy, int *__restrict__ tiles, int ntn) {
+    const bool row = threadIdx.x < 64;
+    const int i = (row ? blockIdx.x : blockIdx.y) * 64 + (threadIdx.x & 63);
+    bool bad = false;
+    if (i < (row ? M : N)) {
+        const int e = (row ? ex : ey)[i];
+        bad = bad_exp(e) || (sx && e != kNoExp && !(k <= 128.0 * ldexp((row ? sx : sy)[i], -e)));
+    }
+    if (__syncthreads_or(bad) && threadIdx.x == 0) tiles[(size_t)blockIdx.x * ntn + blockIdx.y] = 1;
 }
 
 // T + offset of x against the group exponent e (|x| < 2^e): T = round(x
@@ -181,6 +302,16 @@ __device__ __forceinline__ void split8_store(const double (&v)[8], const int (&e
     }
 }
 
+// one slice of magnitudes: u = |v| 2^-e as BF16, rounded down
+template <>
+__device__ __forceinline__ void split8_store<1>(const double (&v)[8], const int (&e)[8], __nv_bfloat16 *out, size_t) {
+    unsigned w[4];
+#pragma unroll
+    for (int t = 0; t < 8; t += 2)
+        w[t / 2] = __byte_perm(__float_as_uint(scaled_abs(v[t], e[t])), __float_as_uint(scaled_abs(v[t + 1], e[t + 1])), 0x7632);
+    *reinterpret_cast<uint4 *>(out) = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // Global layout of the digit slices: for K step kc = k / 16, row block b = r /
 // RB (RB = 128 rows for the first operand of a product, 64 for the second) and
 // slice s, the 8 x 8 core matrices (8 rows x 16 bytes) of the RB x 16 block in
@@ -195,11 +326,13 @@ __device__ __forceinline__ size_t tiled_off(int r, int k, int nb, int rb_log) {
 
 // split a row-major R x K block per row (K = columns): one thread per row and
 // 8-wide K group; a warp covers one 8-row group x 32 columns.  cexp: column k
-// of the block is scaled by 2^-cexp[k] before the split.
+// of the block is scaled by 2^-cexp[k] before the split; mags (may be null): the
+// slice of magnitudes as well.
 template <int SL>
 __global__ void __launch_bounds__(256) k_split_rows(int R, int K, const double *__restrict__ X, int ldx, bool vec,
                                                     const int *__restrict__ ex, const int *__restrict__ cexp,
-                                                    __nv_bfloat16 *__restrict__ out, int rows_p, int kp, int rb_log) {
+                                                    __nv_bfloat16 *__restrict__ out, int rows_p, int kp, int rb_log,
+                                                    __nv_bfloat16 *__restrict__ mags) {
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     const int KC = (kp + 31) / 32;
@@ -224,14 +357,15 @@ __global__ void __launch_bounds__(256) k_split_rows(int R, int K, const double *
 #pragma unroll
     for (int t = 0; t < 8; ++t) e[t] = er + (cexp && k0 + t < K ? cexp[k0 + t] : 0);
     split8_store<SL>(v, e, out + tiled_off<SL>(r, k0, rows_p >> rb_log, rb_log), (size_t)16 << rb_log);
+    if (SL == 7 && mags) split8_store<1>(v, e, mags + tiled_off<1>(r, k0, rows_p >> rb_log, rb_log), 0);
 }
 
 // split a row-major K x C block per column (operand row r = column r, K = rows
 // of X), transposed through shared memory: a block handles 64 columns and `tiles`
 // times 32 K rows, two tiles on their way (cp.async) while one is split; half a
 // warp reads 16 columns of eight rows, a warp stores 512 contiguous bytes.
-// rexp: row k of the block is scaled by 2^rexp[k].  sumsq (seven-digit Grams):
-// sum over k of (128 x / 2^e)^2 per column, from the leading digits.
+// rexp: row k of the block is scaled by 2^rexp[k].  sums (magnitudes, SL = 1): the
+// sum over k of u added per column.
 // What bounds it: memory (a 250,000 x 750 block into five digits: 0.55 ms,
 // 6.1 TB/s; a tile per block through registers 0.75 ms, waiting for its loads).
 constexpr int kSplitPitch = 66;                         // doubles: 16-byte rows
@@ -240,7 +374,7 @@ template <int SL>
 __global__ void __launch_bounds__(256, 4) k_split_cols(int K, int C, const double *__restrict__ X, int ldx, bool vec,
                                                        const int *__restrict__ ex, const int *__restrict__ rexp,
                                                        __nv_bfloat16 *__restrict__ out, int rows_p, int kp, int rb_log,
-                                                       float *__restrict__ sumsq, int tiles) {
+                                                       float *__restrict__ sums, int tiles) {
     extern __shared__ __align__(16) double tile[];
     const int c0 = blockIdx.y * 64, t0 = blockIdx.x * tiles, t1 = min(t0 + tiles, (kp + 31) / 32);
     auto stage = [&](int t) {
@@ -290,20 +424,14 @@ __global__ void __launch_bounds__(256, 4) k_split_cols(int K, int C, const doubl
         }
         if (r < rows_p && k < kp)
             split8_store<SL>(v, e, out + tiled_off<SL>(r, k, rows_p >> rb_log, rb_log), (size_t)16 << rb_log);
-        if (sumsq) {
+        if (SL == 1 && sums) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                // x 2^(7-e) from the upper word (zeros and tiny values: nothing to add)
-                const unsigned hw = (unsigned)((unsigned long long)__double_as_longlong(v[u]) >> 32) & 0x7FFFFFFFu;
-                const int q = (int)(hw >> 20) - 1023 + 7 - er;
-                const float f = q > -60 && q < 60 ? __int_as_float(((q + 127) << 23) | (int)((hw & 0xFFFFFu) << 3)) : 0.f;
-                ss = fmaf(f, f, ss);
-            }
+            for (int u = 0; u < 8; ++u) ss += scaled_abs(v[u], e[u]);
         }
     }
-    if (sumsq) {
+    if (SL == 1 && sums) {
         ss += __shfl_xor_sync(0xffffffffu, ss, 16);
-        if (lane < 16 && r < C && ss > 0.f) atomicAdd(&sumsq[r], ss);
+        if (lane < 16 && r < C && ss > 0.f) atomicAdd(&sums[r], ss);
     }
 }
 
@@ -564,6 +692,8 @@ struct TcWork {
     int ntn, tiles, items;  // column tiles, output tiles, tiles x K ranges
     int ksteps, split;      // K steps of the product, K steps per item
     int lower;              // tiles meeting the lower triangle only
+    const int *skip;        // 64 x 64 tiles left to others (nonzero), skip_ld to a row of tiles; may be null
+    int skip_ld;
 };
 struct TcItem {
     int i0, j0, kc0, nk;
@@ -591,11 +721,21 @@ __device__ __forceinline__ TcItem tc_item(const TcWork &w, int item) {
     return it;
 }
 
+// whether one of the item's two 64 x 64 tiles is wanted
+__device__ __forceinline__ bool tc_wanted(const TcWork &w, const TcItem &it, int M) {
+    if (!w.skip) return true;
+    const int c = it.j0 / 64;
+    bool wanted = false;
+    for (int q = it.i0 / 64; q < it.i0 / 64 + 2; ++q)
+        wanted |= q * 64 < M && !(w.lower && c > q) && w.skip[(size_t)q * w.skip_ld + c] == 0;
+    return wanted;
+}
+
 template <int SL>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_ozaki_tc(int M, int N, const __nv_bfloat16 *__restrict__ Xs, int nbx, const __nv_bfloat16 *__restrict__ Ys,
                int nby, const int *__restrict__ ex, const int *__restrict__ ey, double *__restrict__ C, int ldc,
-               TcWork w, int atomic, int vec, const int *__restrict__ skip) {
+               TcWork w, int atomic, int vec) {
     constexpr int ND = tc_nd<SL>(), STAGES = tc_stages<SL>(), LOW = tc_low<SL>();
     constexpr uint32_t A_BYTES = tc_a_bytes<SL>(), B_BYTES = tc_b_bytes<SL>(), STAGE = tc_stage_bytes<SL>();
     constexpr uint32_t LBO = 128, SBO = 256, SLICE_A = A_BYTES / SL, SLICE_B = B_BYTES / SL;
@@ -604,7 +744,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     // groups with six digits); high_bar: all of it is
     __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES], accf_bar, free_bar[2], high_bar, drain_bar;
     __shared__ uint32_t tmem_slot;
-    if (skip && *skip) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // stages on a 1024-byte boundary
     const uint32_t smem0 = (smem_addr(smem_dyn) + 1023u) & ~1023u;
@@ -637,6 +776,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             int g = 0;  // K steps issued by this CTA so far
             for (int item = blockIdx.x; item < w.items && ok; item += gridDim.x) {
                 const TcItem it = tc_item(w, item);
+                if (!tc_wanted(w, it, M)) continue;
                 const __nv_bfloat16 *xa = Xs + ((size_t)it.kc0 * nbx + it.i0 / TC_M) * (A_BYTES / 2);
                 const __nv_bfloat16 *yb = Ys + ((size_t)it.kc0 * nby + it.j0 / TC_N) * (B_BYTES / 2);
                 for (int kt = 0; kt < it.nk; ++kt, ++g) {
@@ -682,7 +822,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         bool ok = true;
         uint32_t st = 0, ph = 0, c = 0;  // stage and its parity, chunks started by this CTA
         for (int item = blockIdx.x; item < w.items && ok; item += gridDim.x) {
-            const int nk = tc_item(w, item).nk;
+            const TcItem it = tc_item(w, item);
+            if (!tc_wanted(w, it, M)) continue;
+            const int nk = it.nk;
             for (int k0 = 0; k0 < nk && ok; k0 += kChunkSteps, ++c) {
                 const int steps = min(kChunkSteps, nk - k0);
                 const uint32_t ap = (c - 1) & 1;  // parity of the chunk before
@@ -755,6 +897,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         int c = 0;
         for (int item = blockIdx.x; item < w.items && ok; item += gridDim.x) {
             const TcItem it = tc_item(w, item);
+            if (!tc_wanted(w, it, M)) continue;
             float hi[32], lo[32], mid[SL == 7 ? 32 : 1];
 #pragma unroll
             for (int q = 0; q < 32; ++q) hi[q] = lo[q] = 0.f;
@@ -932,6 +1075,180 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TC_TMEM_COLS));
 }
 
+// ---- the product of the magnitudes ------------------------------------------
+//
+// h = X Y^T of one slice of magnitudes each (all terms positive, FP32
+// accumulators: a lower bound to 2^-13), per 128 x 64 nt item (nt <= 4 blocks of 64
+// columns, so that the first operand is read ntn / nt times) over a range of K.
+// Four K steps to a stage (one wait and one commit per four MMAs), two sets of
+// accumulators.  Either h is added to chk.h (ld N), or it is checked against the
+// sums of the rows' and columns' magnitudes and the tiles that fail are marked.
+// What bounds it: the loads.  Update of 163,842 x 300 x 300 (98 MB of magnitudes):
+// @MAGUPD us; as one-block items with a stage per K step 205.  Roles, waits and
+// teardown as k_ozaki_tc's.
+constexpr int kMagSteps = 4, kMagBlocks = 4, kMagStages = 4;
+constexpr uint32_t kMagA = 2u * TC_M * TC_K, kMagB = 2u * TC_N * TC_K;  // bytes per K step and block
+constexpr uint32_t kMagStage = kMagSteps * (kMagA + kMagBlocks * kMagB);
+constexpr size_t kMagSmem = (size_t)kMagStages * kMagStage + 1024;
+
+struct MagWork {
+    int groups, tiles, items;  // column groups, output tiles, tiles x K ranges
+    int nt, nby;               // column blocks per group, of the second operand
+    int ksteps, split;         // K steps of the product, K steps per item
+};
+struct MagCheck {
+    float *h;
+    const float *lx, *ly;  // limits; ly in whole blocks of 64 columns
+    float ratio;
+    int *tiles;
+    int tiles_ld;
+};
+
+__global__ void __launch_bounds__(TC_THREADS, 1)
+    k_magnitudes_tc(int M, int N, const __nv_bfloat16 *__restrict__ Xs, int nbx, const __nv_bfloat16 *__restrict__ Ys,
+                    MagWork w, MagCheck chk) {
+    extern __shared__ unsigned char smem_dyn[];
+    __shared__ __align__(8) uint64_t full_bar[kMagStages], empty_bar[kMagStages], accf_bar[2], free_bar[2], drain_bar;
+    __shared__ uint32_t tmem_slot;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t smem0 = (smem_addr(smem_dyn) + 1023u) & ~1023u;
+    if (threadIdx.x == 0) {
+        for (int st = 0; st < kMagStages; ++st) {
+            mbar_init(smem_addr(&full_bar[st]), 1);
+            mbar_init(smem_addr(&empty_bar[st]), 1);
+        }
+        for (int q = 0; q < 2; ++q) {
+            mbar_init(smem_addr(&accf_bar[q]), 1);
+            mbar_init(smem_addr(&free_bar[q]), TC_DRAIN_WARPS);
+        }
+        mbar_init(smem_addr(&drain_bar), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_addr(&tmem_slot)),
+                     "r"(TC_TMEM_COLS));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const uint32_t tmem = tmem_slot;
+    // item -> row tile, first column block, blocks, first K step, K steps
+    struct Item {
+        int ti, jb, nb, kc0, nk;
+    };
+    auto item_of = [&](int item) {
+        const int sp = item / w.tiles, tile = item - sp * w.tiles, ti = tile / w.groups;
+        Item it;
+        it.ti = ti;
+        it.jb = (tile - ti * w.groups) * w.nt;
+        it.nb = min(w.nt, w.nby - it.jb);
+        it.kc0 = sp * w.split;
+        it.nk = min(w.split, w.ksteps - it.kc0);
+        return it;
+    };
+    if (warp == 0) {
+        if (lane == 0) {
+            bool ok = true;
+            int g = 0;  // stages filled by this CTA so far
+            for (int item = blockIdx.x; item < w.items && ok; item += gridDim.x) {
+                const Item it = item_of(item);
+                for (int k0 = 0; k0 < it.nk; k0 += kMagSteps, ++g) {
+                    const int st = g % kMagStages, steps = min(kMagSteps, it.nk - k0);
+                    if (g >= kMagStages) ok = mbar_wait(smem_addr(&empty_bar[st]), ((g / kMagStages) & 1) ^ 1);
+                    if (!ok) break;
+                    const uint32_t fb = smem_addr(&full_bar[st]), dst = smem0 + st * kMagStage;
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb),
+                                 "r"(steps * (kMagA + it.nb * kMagB))
+                                 : "memory");
+                    for (int q = 0; q < steps; ++q) {
+                        const size_t kc = it.kc0 + k0 + q;
+                        bulk_load(dst + q * kMagA, Xs + (kc * nbx + it.ti) * (kMagA / 2), kMagA, fb);
+                        bulk_load(dst + kMagSteps * kMagA + q * kMagBlocks * kMagB, Ys + (kc * w.nby + it.jb) * (kMagB / 2),
+                                  it.nb * kMagB, fb);
+                    }
+                }
+            }
+            for (int q = max(0, g - kMagStages); q < g; ++q)
+                mbar_wait(smem_addr(&full_bar[q % kMagStages]), (q / kMagStages) & 1);
+        }
+    } else if (warp == 1) {
+        const uint32_t el = elect_lane();
+        constexpr uint32_t LBO = 128, SBO = 256;
+        bool ok = true;
+        uint32_t g = 0, c = 0;  // stages and items so far
+        for (int item = blockIdx.x; item < w.items && ok; item += gridDim.x, ++c) {
+            const Item it = item_of(item);
+            const uint32_t d = tmem + (c & 1) * TC_N * kMagBlocks, idesc = umma_idesc(TC_M, TC_N * it.nb);
+            // the set is drained of the item before the last
+            if (c >= 2) ok = mbar_wait(smem_addr(&free_bar[c & 1]), ((c >> 1) - 1) & 1);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            for (int k0 = 0; k0 < it.nk; k0 += kMagSteps, ++g) {
+                const uint32_t st = g % kMagStages;
+                ok = mbar_wait(smem_addr(&full_bar[st]), (g / kMagStages) & 1);
+                if (!ok) break;
+                const uint32_t a = smem0 + st * kMagStage, b = a + kMagSteps * kMagA;
+                const int steps = min(kMagSteps, it.nk - k0);
+                for (int q = 0; q < steps; ++q)
+                    umma_f16(d, umma_desc(umma_desc_lo(a + q * kMagA, LBO), SBO),
+                             umma_desc(umma_desc_lo(b + q * kMagBlocks * kMagB, LBO), SBO), idesc, k0 + q > 0, el);
+                umma_commit(smem_addr(&empty_bar[st]), el);
+            }
+            if (!ok) break;
+            umma_commit(smem_addr(&accf_bar[c & 1]), el);
+        }
+        umma_commit(smem_addr(&drain_bar), el);
+        mbar_wait(smem_addr(&drain_bar), 0);
+    } else {
+        const int quad = warp & 3, c0 = 32 * ((warp - 2) >> 2);
+        bool ok = true;
+        int c = 0;
+        for (int item = blockIdx.x; item < w.items && ok; item += gridDim.x, ++c) {
+            const Item it = item_of(item);
+            const int i = it.ti * TC_M + 32 * quad + lane;
+            const float li = chk.h || i >= M ? 0.f : chk.lx[i];
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&accf_bar[c & 1]), (c >> 1) & 1));
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            for (int b = 0; b < it.nb; ++b) {
+                uint32_t r[32];
+                tmem_ld<32>(tmem + ((uint32_t)(32 * quad) << 16) + (c & 1) * TC_N * kMagBlocks + b * TC_N + c0, r);
+                tmem_wait<32>(r);
+                if (b == it.nb - 1) {
+                    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_addr(&free_bar[c & 1]));
+                }
+                const int jb = (it.jb + b) * TC_N + c0;
+                if (chk.h) {
+                    if (i < M)
+#pragma unroll
+                        for (int q = 0; q < 32; ++q)
+                            if (jb + q < N) atomicAdd(&chk.h[(size_t)i * N + jb + q], __uint_as_float(r[q]));
+                    continue;
+                }
+                bool fails = false;
+#pragma unroll
+                for (int q = 0; q < 32; q += 4) {
+                    const float4 l = *reinterpret_cast<const float4 *>(chk.ly + jb + q);
+                    fails |= digits_fail(li, l.x, chk.ratio, __uint_as_float(r[q])) |
+                             digits_fail(li, l.y, chk.ratio, __uint_as_float(r[q + 1])) |
+                             digits_fail(li, l.z, chk.ratio, __uint_as_float(r[q + 2])) |
+                             digits_fail(li, l.w, chk.ratio, __uint_as_float(r[q + 3]));
+                }
+                fails = fails && i < M;
+                if (__any_sync(0xffffffffu, fails) && lane == 0)
+                    chk.tiles[(size_t)((it.ti * TC_M + 32 * quad) >> 6) * chk.tiles_ld + it.jb + b] = 1;
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TC_TMEM_COLS));
+}
 
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 inline bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -940,13 +1257,13 @@ inline bool pair_rows(const double *p, int ld) { return aligned16(p) && ld % 2 =
 
 template <int SL>
 void launch_tc(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, const TcWork &w,
-               bool atomic, const int *skip) {
+               bool atomic) {
     HSIM_SMEM_LIMIT_ONCE(k_ozaki_tc<SL>, tc_smem<SL>());
     const int grid = std::min(w.items, sm_count_oz());
     const bool vec = !atomic && !w.lower && pair_rows(C, ldc);
     k_ozaki_tc<SL><<<grid, TC_THREADS, tc_smem<SL>(), s>>>(X.rows, Y.rows, X.slices, X.rows_p / TC_M, Y.slices,
                                                           Y.rows_p / TC_N, X.exps, Y.exps, C, ldc, w, atomic ? 1 : 0,
-                                                          vec ? 1 : 0, skip);
+                                                          vec ? 1 : 0);
     HSIM_LAUNCHED();
 }
 
@@ -965,7 +1282,7 @@ size_t ozaki_cols_scratch(int n, int cols, int digits) { return operand_bytes(co
 size_t ozaki_rows_scratch(int rows, int k, int digits) { return operand_bytes(rows, k, digits); }
 
 static OzakiOperand make_operand(int rows, int kdim, void *scratch, int digits, OzakiRole role) {
-    HSIM_CHECK_ARG(digits >= 5 && digits <= 7, "ozaki product: 5, 6 or 7 digits per value");
+    HSIM_CHECK_ARG(digits == 1 || (digits >= 5 && digits <= 7), "ozaki product: 5, 6 or 7 digits per value");
     HSIM_CHECK_ARG(aligned16(scratch), "ozaki product: scratch not 16-byte aligned");
     OzakiOperand op;
     op.digits = digits;
@@ -981,19 +1298,22 @@ static OzakiOperand make_operand(int rows, int kdim, void *scratch, int digits, 
 static int role_log(OzakiRole r) { return r == OzakiRole::X ? 7 : 6; }
 
 static void ozaki_col_exps(cudaStream_t s, int n, int cols, const double *X, int ldx, int *exps, const int *rexp,
-                           int *nonfinite = nullptr) {
+                           double *sums = nullptr) {
     k_fill_int<<<cdiv(cols, 256), 256, 0, s>>>(cols, kNoExp, exps);
     HSIM_LAUNCHED();
     // rows per CTA: about eight CTAs per SM, 32 to 1024 rows
     const int64_t cb = cdiv(cols, 64), want = std::max<int64_t>(1, 8 * (int64_t)sm_count_oz() / cb);
     const int rows = (int)std::min<int64_t>(1024, std::max<int64_t>(32, round_up((int)cdiv(n, want), 8)));
-    k_col_exps<<<dim3(cdiv(n, rows), (unsigned)cb), 256, 0, s>>>(n, cols, X, ldx, rows, rexp, pair_rows(X, ldx), exps,
-                                                                        nonfinite);
+    const dim3 g(cdiv(n, rows), (unsigned)cb);
+    auto go = [&](auto kernel) { kernel<<<g, 256, 0, s>>>(n, cols, X, ldx, rows, rexp, pair_rows(X, ldx), exps, sums); };
+    if (rexp) go(k_col_exps<true, false>);
+    else if (sums) go(k_col_exps<false, true>);
+    else go(k_col_exps<false, false>);
     HSIM_LAUNCHED();
 }
 
 static void split_cols_into(cudaStream_t s, const OzakiOperand &op, int n, const double *X, int ldx, const int *rexp,
-                            float *sumsq) {
+                            float *sums = nullptr) {
     // four blocks per SM (shared memory), each with up to eight tiles
     const int nt = cdiv(op.kp, 32), ncb = cdiv(op.rows_p, 64);
     const int tiles = (int)std::max<int64_t>(1, std::min<int64_t>(8, (int64_t)nt * ncb / (4 * (int64_t)sm_count_oz())));
@@ -1001,7 +1321,7 @@ static void split_cols_into(cudaStream_t s, const OzakiOperand &op, int n, const
     const bool vec = pair_rows(X, ldx);
     const int rl = role_log(op.role);
     auto go = [&](auto kernel) {
-        kernel<<<g, 256, kSplitSmem, s>>>(n, op.rows, X, ldx, vec, op.exps, rexp, op.slices, op.rows_p, op.kp, rl, sumsq,
+        kernel<<<g, 256, kSplitSmem, s>>>(n, op.rows, X, ldx, vec, op.exps, rexp, op.slices, op.rows_p, op.kp, rl, sums,
                                           tiles);
         HSIM_LAUNCHED();
     };
@@ -1011,6 +1331,9 @@ static void split_cols_into(cudaStream_t s, const OzakiOperand &op, int n, const
     } else if (op.digits == 6) {
         HSIM_SMEM_LIMIT_ONCE(k_split_cols<6>, kSplitSmem);
         go(k_split_cols<6>);
+    } else if (op.digits == 1) {
+        HSIM_SMEM_LIMIT_ONCE(k_split_cols<1>, kSplitSmem);
+        go(k_split_cols<1>);
     } else {
         HSIM_SMEM_LIMIT_ONCE(k_split_cols<7>, kSplitSmem);
         go(k_split_cols<7>);
@@ -1022,24 +1345,25 @@ OzakiOperand ozaki_split_cols(cudaStream_t s, int n, int cols, const double *X, 
     OzakiOperand op = make_operand(cols, n, scratch, digits, role);
     if (n <= 0 || cols <= 0) return op;
     ozaki_col_exps(s, n, cols, X, ldx, op.exps, nullptr);
-    split_cols_into(s, op, n, X, ldx, nullptr, nullptr);
+    split_cols_into(s, op, n, X, ldx, nullptr);
     return op;
 }
 
+// mags, limits (may be null): the magnitudes' slice and limits of every row as well
 static void split_rows_into(cudaStream_t s, const OzakiOperand &op, int k, const double *X, int ldx, const int *cexp,
-                            int *nonfinite = nullptr) {
-    k_row_exps<<<cdiv(op.rows, 8), 256, 0, s>>>(op.rows, k, X, ldx, cexp, op.exps, nonfinite);
+                            __nv_bfloat16 *mags = nullptr, float *limits = nullptr) {
+    k_row_exps<<<cdiv(op.rows, 8), 256, 0, s>>>(op.rows, k, X, ldx, cexp, op.exps, limits);
     HSIM_LAUNCHED();
     const unsigned g = cdiv((int64_t)(op.rows_p / 8) * ((op.kp + 31) / 32) * 32, 256);
     const bool vec = pair_rows(X, ldx);
     const int rl = role_log(op.role);
-    if (op.digits == 5)
-        k_split_rows<5><<<g, 256, 0, s>>>(op.rows, k, X, ldx, vec, op.exps, cexp, op.slices, op.rows_p, op.kp, rl);
-    else if (op.digits == 6)
-        k_split_rows<6><<<g, 256, 0, s>>>(op.rows, k, X, ldx, vec, op.exps, cexp, op.slices, op.rows_p, op.kp, rl);
-    else
-        k_split_rows<7><<<g, 256, 0, s>>>(op.rows, k, X, ldx, vec, op.exps, cexp, op.slices, op.rows_p, op.kp, rl);
-    HSIM_LAUNCHED();
+    auto go = [&](auto kernel) {
+        kernel<<<g, 256, 0, s>>>(op.rows, k, X, ldx, vec, op.exps, cexp, op.slices, op.rows_p, op.kp, rl, mags);
+        HSIM_LAUNCHED();
+    };
+    if (op.digits == 5) go(k_split_rows<5>);
+    else if (op.digits == 6) go(k_split_rows<6>);
+    else go(k_split_rows<7>);
 }
 
 OzakiOperand ozaki_split_rows(cudaStream_t s, int rows, int k, const double *X, int ldx, void *scratch, int digits) {
@@ -1049,14 +1373,13 @@ OzakiOperand ozaki_split_rows(cudaStream_t s, int rows, int k, const double *X, 
     return op;
 }
 
-void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, int splits,
-                   bool lower, bool accumulate, const int *skip) {
-    if (X.rows <= 0 || Y.rows <= 0) return;
+// work items of C = X Y^T; splits <= 0 chooses the number of K ranges, which is
+// returned
+static int plan_tc(const OzakiOperand &X, const OzakiOperand &Y, int splits, bool lower, TcWork &w) {
     HSIM_CHECK_ARG(X.kp == Y.kp, "ozaki_product: operands split over different K");
     HSIM_CHECK_ARG(X.digits == Y.digits, "ozaki_product: operands split into different digit counts");
     HSIM_CHECK_ARG(X.role == OzakiRole::X && Y.role == OzakiRole::Y, "ozaki_product: operand roles");
     HSIM_CHECK_ARG(!lower || X.rows == Y.rows, "ozaki product: lower triangle needs a square result");
-    TcWork w{};
     w.lower = lower ? 1 : 0;
     w.ksteps = X.kp / TC_K;
     w.ntn = (int)cdiv(Y.rows, TC_N);
@@ -1087,14 +1410,48 @@ void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y,
     HSIM_CHECK_ARG(tiles * splits <= INT32_MAX / 2, "ozaki product: too many tiles");
     w.tiles = (int)tiles;
     w.items = (int)(tiles * splits);
+    return splits;
+}
+
+static void zero_block(cudaStream_t s, int rows, int cols, double *C, int ldc) {
+    if (ldc == cols) HSIM_CUDA(cudaMemsetAsync(C, 0, (size_t)rows * cols * sizeof(double), s));
+    else HSIM_CUDA(cudaMemset2DAsync(C, (size_t)ldc * sizeof(double), 0, (size_t)cols * sizeof(double), rows, s));
+}
+
+void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, int splits,
+                   bool lower, bool accumulate, const int *skip, int skip_ld) {
+    if (X.rows <= 0 || Y.rows <= 0) return;
+    TcWork w{};
+    splits = plan_tc(X, Y, splits, lower, w);
+    w.skip = skip;
+    w.skip_ld = skip_ld;
     const bool atomic = splits > 1 || accumulate;
-    if (atomic && !accumulate) {
-        if (ldc == Y.rows) HSIM_CUDA(cudaMemsetAsync(C, 0, (size_t)X.rows * Y.rows * sizeof(double), s));
-        else HSIM_CUDA(cudaMemset2DAsync(C, (size_t)ldc * sizeof(double), 0, (size_t)Y.rows * sizeof(double), X.rows, s));
-    }
-    if (X.digits == 5) launch_tc<5>(s, X, Y, C, ldc, w, atomic, skip);
-    else if (X.digits == 6) launch_tc<6>(s, X, Y, C, ldc, w, atomic, skip);
-    else launch_tc<7>(s, X, Y, C, ldc, w, atomic, skip);
+    if (atomic && !accumulate) zero_block(s, X.rows, Y.rows, C, ldc);
+    if (X.digits == 5) launch_tc<5>(s, X, Y, C, ldc, w, atomic);
+    else if (X.digits == 6) launch_tc<6>(s, X, Y, C, ldc, w, atomic);
+    else launch_tc<7>(s, X, Y, C, ldc, w, atomic);
+}
+
+// the product of two slices of magnitudes, added to chk.h (over K ranges that fill
+// the SMs) or checked (one K range)
+static void product_magnitudes(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, const MagCheck &chk) {
+    MagWork w{};
+    w.nby = Y.rows_p / TC_N;
+    w.groups = (int)cdiv(w.nby, kMagBlocks);
+    w.nt = (int)cdiv(w.nby, w.groups);
+    w.ksteps = X.kp / TC_K;
+    const int64_t tiles = (int64_t)(X.rows_p / TC_M) * w.groups;
+    const int64_t want = chk.h ? std::max<int64_t>(1, (int64_t)sm_count_oz() / tiles) : 1;
+    const int64_t stages = cdiv(w.ksteps, kMagSteps);
+    w.split = (int)(kMagSteps * cdiv(stages, std::min(stages, want)));
+    const int64_t items = tiles * cdiv(w.ksteps, w.split);
+    HSIM_CHECK_ARG(items <= INT32_MAX / 2, "ozaki product: too many tiles");
+    w.tiles = (int)tiles;
+    w.items = (int)items;
+    HSIM_SMEM_LIMIT_ONCE(k_magnitudes_tc, kMagSmem);
+    k_magnitudes_tc<<<std::min(w.items, sm_count_oz()), TC_THREADS, kMagSmem, s>>>(X.rows, Y.rows, X.slices, X.rows_p / TC_M,
+                                                                              Y.slices, w, chk);
+    HSIM_LAUNCHED();
 }
 
 // ---- products over ranges of rows -------------------------------------------
@@ -1135,8 +1492,8 @@ void ozaki_gram(cudaStream_t s, int n, int ka, int kb, const double *A, int lda,
         OzakiOperand X = make_operand(ka, rows, sx, digits, OzakiRole::X), Y = make_operand(kb, rows, sy, digits, OzakiRole::Y);
         X.exps = ex;
         Y.exps = ey;
-        split_cols_into(s, X, rows, A + (size_t)r0 * lda, lda, nullptr, nullptr);
-        split_cols_into(s, Y, rows, B + (size_t)r0 * ldb, ldb, nullptr, nullptr);
+        split_cols_into(s, X, rows, A + (size_t)r0 * lda, lda, nullptr);
+        split_cols_into(s, Y, rows, B + (size_t)r0 * ldb, ldb, nullptr);
         ozaki_product(s, X, Y, G, ldg, 0, false, several);
     }
 }
@@ -1161,17 +1518,17 @@ void ozaki_update(cudaStream_t s, int n, int k, int m, const double *A, int lda,
 // ---- FP64 products on seven digits --------------------------------------------
 // gram and gemm_nn of the FP64 path.  Seven digits keep 55 bits against each
 // group's maximum and the digit pairs down to 2^-63, so the error per term is
-// 2^-57 of max|x| max|y| where an FP64 accumulation rounds every partial sum to
+// 2^-56 of max|x| max|y| where an FP64 accumulation rounds every partial sum to
 // 2^-54 of itself.  Against quad-precision sums, FP64 kernels and digits:
 // Gram of 163,842 x 300 5.3e-16 and 0.9e-16 (all positive 4.7 and 1.4, smooth
 // columns 23 and 1.6), update 5.8e-16 and 2.3e-16 (a random second factor 5.8 and
 // 0.6, columns scaled by 10^+-6 5.7 and 2.2); the same order at 5,003 to 20,011
-// rows and 77 to 750 columns.  Scales that would spoil the common exponents are
-// taken out first: a Gram's columns have their own (a column with entries that
-// stand out goes to the FP64 kernel), an update scales column k of A by 2^-c_k
-// and row k of B by 2^c_k, exactly, so that their largest entries meet.
-// Infinities and NaN go to the FP64 kernels too: the device decides and repeats
-// the product with them where the flag is set.
+// rows and 77 to 750 columns.  Tiles where the maxima say too little go to the
+// FP64 kernels (digits_fail and k_guard_tiles above), which the device decides
+// before a digit of them is multiplied.  A Gram's columns have their own
+// exponents; an update scales column k of A by 2^-c_k and row k of B by 2^c_k,
+// exactly, so that their mean magnitudes meet (means: one large entry must not move
+// the scale of the others).
 //
 // Where the line lies (us, FP64 kernel / digits, calls with a wait): Gram 1,024
 // rows x 30 to 300 columns 281 / 73 to 283 / 81, 16,384 x 75 530 / 101, 163,842 x
@@ -1193,83 +1550,205 @@ bool update64_on_digits(int n, int k, int m, bool held) {
     return held ? (k > 40 && work >= 2e6) || work >= 1.2e7 : (k >= 165 && work >= 2e6) || work >= 1.2e8;
 }
 
-// c_k = half the exponent gap between column k of A and row k of B
-__global__ void k_balance(int k, const int *__restrict__ eb, int *__restrict__ c) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < k) c[j] = (c[j] - eb[j]) >> 1;
+namespace {
+
+// Powers of two c_k: half the gap between the mean magnitudes of column k of A (sum
+// over n rows) and row k of B (sum in units of 2^eb over m columns), less the mean
+// gap of all k (a common factor does nothing); below 1.5 left at 0, so that pairs
+// alike are not told apart by rounding.  One CTA; zeros and infinities: 0.
+__global__ void __launch_bounds__(256) k_balance(int k, int n, int m, const double *__restrict__ suma,
+                                                 const int *__restrict__ eb, const float *__restrict__ sumb,
+                                                 int *__restrict__ c) {
+    __shared__ float red[2][8];
+    auto log2_of = [](double x, float &l) {
+        const int h = __double2hiint(x), e = (h >> 20) & 0x7FF;
+        l = (float)(e - 1023) + __log2f(__int_as_float(0x3F800000 | ((h & 0xFFFFF) << 3)));
+        return e != 0 && e != 0x7FF;
+    };
+    auto gap = [&](int j, float &g) {
+        float a, b;
+        const bool ok = log2_of(suma[j], a) && log2_of((double)sumb[j], b) && !bad_exp(eb[j]);
+        g = 0.5f * ((a - __log2f((float)n)) - (b + (float)eb[j] - __log2f((float)m)));
+        return ok;
+    };
+    float sum = 0.f, cnt = 0.f, g;
+    for (int j = threadIdx.x; j < k; j += 256)
+        if (gap(j, g)) sum += g, cnt += 1.f;
+    for (int o = 16; o > 0; o >>= 1) {
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    }
+    if ((threadIdx.x & 31) == 0) red[0][threadIdx.x >> 5] = sum, red[1][threadIdx.x >> 5] = cnt;
+    __syncthreads();
+    sum = cnt = 0.f;
+    for (int q = 0; q < 8; ++q) sum += red[0][q], cnt += red[1][q];
+    const float mean = sum / fmaxf(cnt, 1.f);
+    for (int j = threadIdx.x; j < k; j += 256) c[j] = gap(j, g) && fabsf(g - mean) > 1.5f ? __float2int_rn(g - mean) : 0;
 }
 
-static size_t floats_bytes(int n) { return exps_bytes(n); }
+// 512-byte aligned pieces of one scratch block
+struct Pieces {
+    unsigned char *p;
+    size_t used = 0;
+    template <class T> T *take(size_t count) {
+        T *q = reinterpret_cast<T *>(p + used);
+        used += (count * sizeof(T) + 511) / 512 * 512;
+        return q;
+    }
+};
 
-size_t gram64_scratch(int n, int ka, int kb) {
-    const int r = std::min(gram_rows(n, ka, kb, kDigits64), n);
-    return 512 + 2 * (exps_bytes(ka) + exps_bytes(kb)) + floats_bytes(ka) + floats_bytes(kb) +
-           operand_bytes(ka, r, kDigits64) + operand_bytes(kb, r, kDigits64);
-}
+// 64 x 64 tiles of an M x N result (whole row tiles of the products)
+inline int tile_rows(int M) { return 2 * (int)cdiv(M, TC_M); }
+inline int tile_cols(int N) { return (int)cdiv(N, TC_N); }
+
+// every how manieth row stands for all: 8 where that leaves 2048 and more, 4 below
+// (a row pitch that an int holds)
+int sample_step(int n, int ld) { return ld > INT32_MAX / 8 ? 1 : n >= 16384 ? 8 : 4; }
+
+struct Gram64 {
+    int range, step, sampled, mag_range;  // rows of a digit range; rows between sampled ones, their number, their range
+    int *tiles, *ex, *ey;
+    double *sx, *sy;
+    float *h;
+    unsigned char *dx, *dy;
+    size_t zero_bytes, bytes;  // tiles to sy; all of it
+    Gram64(int n, int ka, int kb, int lda, int ldb, void *scratch) {
+        Pieces q{static_cast<unsigned char *>(scratch)};
+        range = std::min(gram_rows(n, ka, kb, kDigits64), n);
+        step = sample_step(n, std::max(lda, ldb));
+        sampled = (int)cdiv(n, step);
+        mag_range = std::min(gram_rows(sampled, ka, kb, 1), sampled);
+        tiles = q.take<int>((size_t)tile_rows(ka) * tile_cols(kb));
+        sx = q.take<double>(ka);
+        sy = q.take<double>(kb);
+        zero_bytes = q.used;
+        ex = q.take<int>(ka);
+        ey = q.take<int>(kb);
+        h = q.take<float>((size_t)ka * kb);
+        dx = q.take<unsigned char>(std::max(operand_bytes(ka, range, kDigits64), operand_bytes(ka, mag_range, 1)));
+        dy = q.take<unsigned char>(std::max(operand_bytes(kb, range, kDigits64), operand_bytes(kb, mag_range, 1)));
+        bytes = q.used;
+    }
+};
+
+struct Update64 {
+    int range;
+    int *tiles, *cexp, *bexp;
+    double *suma;
+    float *sumb, *lx, *ly;
+    unsigned char *dy, *my, *dx, *mx;
+    size_t zero_bytes, bytes;  // tiles to ly; all of it
+    Update64(int n, int k, int m, void *scratch) {
+        Pieces q{static_cast<unsigned char *>(scratch)};
+        range = std::min(range_rows(n, 2 * (size_t)(kDigits64 + 1) * round_up(k, TC_K), TC_M), n);
+        tiles = q.take<int>((size_t)tile_rows(n) * tile_cols(m));
+        suma = q.take<double>(k);
+        ly = q.take<float>(round_up(m, TC_N));
+        zero_bytes = q.used;
+        cexp = q.take<int>(k);
+        bexp = q.take<int>(k);
+        sumb = q.take<float>(k);
+        lx = q.take<float>(range);
+        dy = q.take<unsigned char>(operand_bytes(m, k, kDigits64));
+        my = q.take<unsigned char>(operand_bytes(m, k, 1));
+        dx = q.take<unsigned char>(operand_bytes(range, k, kDigits64));
+        mx = q.take<unsigned char>(operand_bytes(range, k, 1));
+        bytes = q.used;
+    }
+};
+
+}  // namespace
+
+size_t gram64_scratch(int n, int ka, int kb) { return Gram64(n, ka, kb, ka, kb, nullptr).bytes; }
 
 void gram64(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
-            int ldg, bool lower, void *scratch) {
-    const int range = gram_rows(n, ka, kb, kDigits64);
-    unsigned char *p = static_cast<unsigned char *>(scratch);
-    auto take = [&](size_t bytes) {
-        unsigned char *q = p;
-        p += bytes;
-        return q;
-    };
-    const size_t zero_bytes = 512 + floats_bytes(ka) + floats_bytes(kb);
-    int *flag = reinterpret_cast<int *>(take(512));
-    float *ssx = reinterpret_cast<float *>(take(floats_bytes(ka))), *ssy = reinterpret_cast<float *>(take(floats_bytes(kb)));
-    int *ex = reinterpret_cast<int *>(take(exps_bytes(ka))), *ey = reinterpret_cast<int *>(take(exps_bytes(kb)));
-    unsigned char *sx = take(operand_bytes(ka, std::min(range, n), kDigits64)), *sy = p;
-    HSIM_CUDA(cudaMemsetAsync(flag, 0, zero_bytes, s));
+            int ldg, bool lower, Held held, void *scratch) {
+    const Gram64 g(n, ka, kb, lda, ldb, scratch);
+    const int tm = tile_rows(ka), tn = tile_cols(kb);
+    HSIM_CUDA(cudaMemsetAsync(g.tiles, 0, g.zero_bytes, s));
     const bool same = A == B && ka == kb && lda == ldb;
-    ozaki_col_exps(s, n, ka, A, lda, ex, nullptr, flag);
-    if (same) HSIM_CUDA(cudaMemcpyAsync(ey, ex, (size_t)ka * sizeof(int), cudaMemcpyDeviceToDevice, s));
-    else ozaki_col_exps(s, n, kb, B, ldb, ey, nullptr, flag);
-    const bool several = n > range;
-    if (several) HSIM_CUDA(cudaMemset2DAsync(G, (size_t)ldg * sizeof(double), 0, (size_t)kb * sizeof(double), ka, s));
-    for (int r0 = 0; r0 < n; r0 += range) {
-        const int rows = std::min(range, n - r0);
-        OzakiOperand X = make_operand(ka, rows, sx, kDigits64, OzakiRole::X), Y = make_operand(kb, rows, sy, kDigits64, OzakiRole::Y);
-        X.exps = ex;
-        Y.exps = ey;
-        split_cols_into(s, X, rows, A + (size_t)r0 * lda, lda, nullptr, ssx);
-        split_cols_into(s, Y, rows, B + (size_t)r0 * ldb, ldb, nullptr, ssy);
-        ozaki_product(s, X, Y, G, ldg, 0, lower, several);
+    ozaki_col_exps(s, n, ka, A, lda, g.ex, nullptr, g.sx);
+    if (same) {
+        HSIM_CUDA(cudaMemcpyAsync(g.ey, g.ex, (size_t)ka * sizeof(int), cudaMemcpyDeviceToDevice, s));
+        HSIM_CUDA(cudaMemcpyAsync(g.sy, g.sx, (size_t)ka * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    } else {
+        ozaki_col_exps(s, n, kb, B, ldb, g.ey, nullptr, g.sy);
     }
-    k_guard_cols<<<cdiv(ka, 256), 256, 0, s>>>(ka, (float)n, ex, ssx, flag);
+    auto operands = [&](int rows, int digits, OzakiOperand &X, OzakiOperand &Y, const double *a, int la, const double *b,
+                        int lb) {
+        X = make_operand(ka, rows, g.dx, digits, OzakiRole::X);
+        Y = make_operand(kb, rows, g.dy, digits, OzakiRole::Y);
+        X.exps = g.ex;
+        Y.exps = g.ey;
+        split_cols_into(s, X, rows, a, la, nullptr);
+        split_cols_into(s, Y, rows, b, lb, nullptr);
+    };
+    OzakiOperand X, Y;
+    if (held == Held::Entries) {
+        HSIM_CUDA(cudaMemsetAsync(g.h, 0, (size_t)ka * kb * sizeof(float), s));
+        MagCheck chk{};
+        chk.h = g.h;
+        for (int r0 = 0; r0 < g.sampled; r0 += g.mag_range) {
+            const size_t r = (size_t)r0 * g.step;
+            operands(std::min(g.mag_range, g.sampled - r0), 1, X, Y, A + r * lda, lda * g.step, B + r * ldb, ldb * g.step);
+            product_magnitudes(s, X, Y, chk);
+        }
+        k_check_tiles<<<cdiv((int64_t)ka * kb, 256), 256, 0, s>>>(ka, kb, (float)n, digits_ratio(n), g.h, g.ex, g.sx, g.ey,
+                                                                 g.sy, g.tiles, tn);
+    } else {
+        k_guard_tiles<<<dim3(tm, tn), 128, 0, s>>>(ka, kb, (double)n, g.ex, g.sx, g.ey, g.sy, g.tiles, tn);
+    }
     HSIM_LAUNCHED();
-    k_guard_cols<<<cdiv(kb, 256), 256, 0, s>>>(kb, (float)n, ey, ssy, flag);
-    HSIM_LAUNCHED();
-    gram_if(s, n, ka, kb, A, lda, B, ldb, G, ldg, lower, flag);
+    const bool several = n > g.range;
+    if (several) zero_block(s, ka, kb, G, ldg);
+    for (int r0 = 0; r0 < n; r0 += g.range) {
+        operands(std::min(g.range, n - r0), kDigits64, X, Y, A + (size_t)r0 * lda, lda, B + (size_t)r0 * ldb, ldb);
+        ozaki_product(s, X, Y, G, ldg, 0, lower, several, g.tiles, tn);
+    }
+    gram_tiles(s, n, ka, kb, A, lda, B, ldb, G, ldg, lower, g.tiles, tn);
 }
 
-size_t update64_scratch(int n, int k, int m) {
-    return 512 + 2 * exps_bytes(k) + operand_bytes(m, k, kDigits64) +
-           operand_bytes(std::min(update_rows(n, k, kDigits64), n), k, kDigits64);
-}
+size_t update64_scratch(int n, int k, int m) { return Update64(n, k, m, nullptr).bytes; }
 
 void update64(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
-              int ldc, void *scratch) {
-    const int range = update_rows(n, k, kDigits64);
-    int *flag = static_cast<int *>(scratch), *cexp = flag + 128, *bexp = cexp + exps_bytes(k) / sizeof(int);
-    unsigned char *sy = static_cast<unsigned char *>(scratch) + 512 + 2 * exps_bytes(k);
-    unsigned char *sx = sy + operand_bytes(m, k, kDigits64);
-    HSIM_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), s));
-    ozaki_col_exps(s, n, k, A, lda, cexp, nullptr, flag);
-    k_row_exps<<<cdiv(k, 8), 256, 0, s>>>(k, m, B, ldb, nullptr, bexp, flag);
+              int ldc, Held held, void *scratch) {
+    const Update64 u(n, k, m, scratch);
+    const int tn = tile_cols(m);
+    HSIM_CUDA(cudaMemsetAsync(u.tiles, 0, u.zero_bytes, s));
+    // means over part of the rows: they only set the scale
+    const int step = sample_step(n, lda), sampled = (int)cdiv(n, step);
+    ozaki_col_exps(s, sampled, k, A, lda * step, u.cexp, nullptr, u.suma);
+    k_row_exps<<<cdiv(k, 8), 256, 0, s>>>(k, m, B, ldb, nullptr, u.bexp, u.sumb);
     HSIM_LAUNCHED();
-    k_balance<<<cdiv(k, 256), 256, 0, s>>>(k, bexp, cexp);
+    k_balance<<<1, 256, 0, s>>>(k, sampled, m, u.suma, u.bexp, u.sumb, u.cexp);
     HSIM_LAUNCHED();
-    OzakiOperand Y = make_operand(m, k, sy, kDigits64, OzakiRole::Y);
-    ozaki_col_exps(s, k, m, B, ldb, Y.exps, cexp);
-    split_cols_into(s, Y, k, B, ldb, cexp, nullptr);
-    for (int r0 = 0; r0 < n; r0 += range) {
-        OzakiOperand X = make_operand(std::min(range, n - r0), k, sx, kDigits64, OzakiRole::X);
-        split_rows_into(s, X, k, A + (size_t)r0 * lda, lda, cexp);
-        ozaki_product(s, X, Y, C + (size_t)r0 * ldc, ldc, 1);
+    OzakiOperand Y = make_operand(m, k, u.dy, kDigits64, OzakiRole::Y), Ym = make_operand(m, k, u.my, 1, OzakiRole::Y);
+    ozaki_col_exps(s, k, m, B, ldb, Y.exps, u.cexp);
+    split_cols_into(s, Y, k, B, ldb, u.cexp);
+    Ym.exps = Y.exps;
+    const bool entries = held == Held::Entries;
+    if (entries) {
+        split_cols_into(s, Ym, k, B, ldb, u.cexp, u.ly);
+        k_col_limits<<<cdiv(round_up(m, TC_N), 256), 256, 0, s>>>(m, round_up(m, TC_N), (float)k, Y.exps, u.ly);
+        HSIM_LAUNCHED();
     }
-    gemm_nn_if(s, n, k, m, A, lda, B, ldb, C, ldc, flag);
+    for (int r0 = 0; r0 < n; r0 += u.range) {
+        const int rows = std::min(u.range, n - r0);
+        int *tiles = u.tiles + (size_t)(r0 / 64) * tn;
+        OzakiOperand X = make_operand(rows, k, u.dx, kDigits64, OzakiRole::X), Xm = make_operand(rows, k, u.mx, 1, OzakiRole::X);
+        Xm.exps = X.exps;
+        split_rows_into(s, X, k, A + (size_t)r0 * lda, lda, u.cexp, entries ? Xm.slices : nullptr, entries ? u.lx : nullptr);
+        if (entries) {
+            const MagCheck chk{nullptr, u.lx, u.ly, digits_ratio(k), tiles, tn};
+            product_magnitudes(s, Xm, Ym, chk);
+        } else {
+            k_guard_tiles<<<dim3(cdiv(rows, 64), tn), 128, 0, s>>>(rows, m, (double)k, X.exps, nullptr, Y.exps, nullptr, tiles,
+                                                                  tn);
+            HSIM_LAUNCHED();
+        }
+        ozaki_product(s, X, Y, C + (size_t)r0 * ldc, ldc, 1, false, false, tiles, tn);
+    }
+    gemm_nn_tiles(s, n, k, m, A, lda, B, ldb, C, ldc, u.tiles, tn);
 }
 
 void ozaki_check(cudaStream_t s) {

@@ -92,11 +92,12 @@ void gram(cudaStream_t s, int n, int ka, int kb, const T *A, int lda, const T *B
 template <typename T>
 void gemm_nn(cudaStream_t s, int n, int k, int m, const T *A, int lda, const double *B, int ldb,
              T *C, int ldc);
-// the FP64 kernels where *flag (device) is nonzero, nothing elsewhere
-void gram_if(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
-             int ldg, bool lower_only, const int *flag);
-void gemm_nn_if(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
-                int ldc, const int *flag);
+// the FP64 kernels on the 64 x 64 tiles of the result that are marked (nonzero)
+// in tiles (device, tiles_ld to a row of tiles), the others as they are
+void gram_tiles(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
+                int ldg, bool lower_only, const int *tiles, int tiles_ld);
+void gemm_nn_tiles(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
+                   int ldc, const int *tiles, int tiles_ld);
 // residual sums: out[3j+0] = sum w R^2, +1 = sum w (S Phi)^2, +2 = sum w (M Phi)^2
 // with R = SPhi - lam * MPhi; w = dinv (M^{-1}-norm) or 1 (2-norm)
 template <typename T>
@@ -319,9 +320,10 @@ OzakiOperand ozaki_split_rows(cudaStream_t s, int rows, int k, const double *X, 
 // accumulated with atomics), 1 stores directly (up to 16,384 deep); lower: C
 // is symmetric, only tiles meeting the lower triangle run and the epilogue
 // writes each value and its mirror image (X.rows == Y.rows); accumulate: added
-// to C; skip (device, may be null): nothing is done where *skip is nonzero
+// to C; skip (device, may be null): 64 x 64 tiles of C that are not wanted
+// (nonzero; skip_ld to a row of tiles), computed or not
 void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, int splits,
-                   bool lower = false, bool accumulate = false, const int *skip = nullptr);
+                   bool lower = false, bool accumulate = false, const int *skip = nullptr, int skip_ld = 0);
 // G (ka x kb, ld ldg) = A^T B over n rows and C (n x m, ld ldc) = A B (A n x k, B
 // k x m), split and multiplied a range of rows at a time so that the digits of
 // one range take about 1 GiB of scratch (256-byte aligned)
@@ -332,15 +334,20 @@ size_t ozaki_update_scratch(int n, int k, int m, int digits);
 void ozaki_update(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
                   int ldc, int digits, void *scratch);
 // gram and gemm_nn in FP64 on seven digits (scratch 512-byte aligned), where the
-// *_on_digits rules say that they are the faster form
+// *_on_digits rules say that they are the faster form.  What the digits' result is
+// held to (tiles that could miss it go to the FP64 kernel): Entries, every entry
+// against the sum of its terms' magnitudes, as FP64 arithmetic is; Norms, against
+// the norms of the columns (Gram) or of a row and a column (update), which is what
+// a Rayleigh-Ritz step needs.
+enum class Held { Entries, Norms };
 bool gram64_on_digits(int n, int ka, int kb);
 size_t gram64_scratch(int n, int ka, int kb);
 void gram64(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
-            int ldg, bool lower, void *scratch);
+            int ldg, bool lower, Held held, void *scratch);
 bool update64_on_digits(int n, int k, int m, bool held);  // held: the scratch is there already
 size_t update64_scratch(int n, int k, int m);
 void update64(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
-              int ldc, void *scratch);
+              int ldc, Held held, void *scratch);
 // fails (HSIM_E_INTERNAL) if a tensor-core product kernel gave up waiting on
 // one of its barriers since the last check; synchronises the stream
 void ozaki_check(cudaStream_t s);

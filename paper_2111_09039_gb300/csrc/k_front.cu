@@ -219,18 +219,7 @@ __global__ void __launch_bounds__(128) k_front_diag_inv(FrontDev fd, const int *
                 if (r == j) a[j / 4] = d;
             }
             u[j & 1][r] = a[j / 4];
-            if (r == 0) {
-                const int x = (__double2hiint(d) >> 20) & 0x7FF;
-                double v;
-                if (x > 40 && x < 2006) {
-                    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(v) : "d"(d));
-                    const double q = fma(-d, v, 1.0);
-                    v = fma(v, fma(q, q, q), v);
-                } else {
-                    v = 1.0 / d;
-                }
-                pinv[j & 1] = v;
-            }
+            if (r == 0) pinv[j & 1] = 1.0 / d;
         }
         __syncthreads();
         // row r > j: l = a_rj / d, A_r -= l (d l_c) = l u_c, I_r -= l I_j

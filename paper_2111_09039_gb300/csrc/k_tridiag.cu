@@ -220,21 +220,6 @@ __device__ __forceinline__ double warp_sums(const double (&a)[N], int lane) {
     return h[0];
 }
 
-// 1 / sqrt(x) and 1 / x of normal numbers from the 20-bit seeds by one
-// third-order step (error of the seed cubed, 2^-60)
-__device__ __forceinline__ double rsqrt_step(double x) {
-    double r;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-(x * r), r, 1.0);
-    return fma(r * e, fma(e, 0.375, 0.5), r);
-}
-__device__ __forceinline__ double rcp_step(double x) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-
 // Waiting for `target` arrivals at a counter that starts at zero.  It gives up
 // after two seconds (false, *err set); the CTAs that then leave let the others
 // run into the same limit.
@@ -452,11 +437,10 @@ __global__ void __launch_bounds__(2 * kTrdThreads) k_tridiag_rows(int n, const d
         if ((__double2hiint(sigma) | __double2loint(sigma)) != 0) {
             const double s2 = fma(x0, x0, sigma);
             if (((__double2hiint(s2) >> 20) & 0x7FF) >= 1023 - 800) {
-                const double r = rsqrt_step(s2), m0 = s2 * r;
-                const double mu = fma(fma(-m0, m0, s2), 0.5 * r, m0);
+                const double mu = sqrt(s2);
                 beta = __double2hiint(x0) >= 0 ? -mu : mu;
                 u0 = x0 - beta;
-                t = rcp_step(-beta * u0);
+                t = -1.0 / (beta * u0);
             }
         }
         const double d0 = u0 - x0, c0 = u0 * t;

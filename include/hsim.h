@@ -450,6 +450,11 @@ hsim_status hsim_check_inverted(int n, const int32_t *ptr, const int32_t *col, c
                                 int leaf_size, int nrhs, const double *B, double *X,
                                 int *negative_pivots, int64_t *nnz_L, int fused_h01,
                                 int *fused_counts);
+/* Sets the error word of the context's tensor-core products as a product that gave
+ * up waiting would: the next call that checks it on this context (hsim_gram_tc and
+ * the others) fails with HSIM_E_INTERNAL and clears it, calls on other contexts do
+ * not see it.  For tests; the solver never uses it. */
+hsim_status hsim_check_product_error(hsim_ctx *ctx);
 /* Host replay of the mesh part of hsim_build_hierarchy: the level sizes
  * (eqs. nT-1 and growthRate), the farthest-point order (Alg. 2) and the
  * prolongations U^tau (eq. basis, rows normalised to one), computed by the

@@ -175,6 +175,15 @@ struct hsim_ctx {
     std::vector<int> hflags;  // host mirror
     DevBuf<unsigned long long> scratch_u64;
     ScratchPool pool;
+    void init() {
+        hflags.assign(hsim::k::kFlagWords, 0);
+        flags.alloc(hsim::k::kFlagWords);
+        // before the call returns, whatever the context's stream is ordered with
+        HSIM_CUDA(cudaMemcpy(flags.p, hflags.data(), hflags.size() * sizeof(int), cudaMemcpyHostToDevice));
+        scratch_u64.alloc(4);
+    }
+    int *err_products() const { return flags.p + hsim::k::kErrProducts; }
+    int *err_tc32() const { return flags.p + hsim::k::kErrTc32; }
 };
 
 namespace {
@@ -529,7 +538,7 @@ void upload_level(LevelData &L, cudaStream_t s) {
 // Inverts the pivot blocks of all fronts in place and forms W = L_bs Linv
 // (the inverted-factor form of k_finv.cu).
 template <typename T>
-void invert_level_t(cudaStream_t s, LevelData &L, T *arena, DevBuf<T> &scr) {
+void invert_level_t(cudaStream_t s, LevelData &L, T *arena, DevBuf<T> &scr, int *err) {
     scr.reserve((size_t)std::max<int64_t>(L.inv_scratch, 1));
     k::inv_diag_blocks(s, L.fd, L.inv_blk.p, L.n_inv_blk, arena);
     if constexpr (std::is_same<T, float>::value) {
@@ -540,11 +549,11 @@ void invert_level_t(cudaStream_t s, LevelData &L, T *arena, DevBuf<T> &scr) {
                     k::gemm_tasks<T>(s, L.inv_p1[lv].p, L.inv_n[lv], L.inv_tiles[lv], arena, arena, scr.p);
                     k::gemm_tasks<T>(s, L.inv_p2[lv].p, L.inv_n[lv], L.inv_tiles[lv], arena, scr.p, arena);
                 } else {
-                    k::gemm_tasks_tc(s, L.inv_p1_tc[lv].p, L.inv_n[lv], L.inv_tiles_tc[lv], arena, arena, scr.p);
-                    k::gemm_tasks_tc(s, L.inv_p2_tc[lv].p, L.inv_n[lv], L.inv_tiles_tc[lv], arena, scr.p, arena);
+                    k::gemm_tasks_tc(s, L.inv_p1_tc[lv].p, L.inv_n[lv], L.inv_tiles_tc[lv], arena, arena, scr.p, err);
+                    k::gemm_tasks_tc(s, L.inv_p2_tc[lv].p, L.inv_n[lv], L.inv_tiles_tc[lv], arena, scr.p, arena, err);
                 }
             }
-            k::gemm_tasks_tc(s, L.inv_w_tc.p, L.inv_nw_tc, L.inv_tw_tc, arena, arena, scr.p);
+            k::gemm_tasks_tc(s, L.inv_w_tc.p, L.inv_nw_tc, L.inv_tw_tc, arena, arena, scr.p, err);
             k::gemm_tasks<T>(s, L.inv_w_cc.p, L.inv_nw_cc, L.inv_tw_cc, arena, arena, scr.p);
             k::copy_tasks<T>(s, L.inv_wc.p, L.inv_nw, L.inv_tw, scr.p, arena);
             return;
@@ -598,7 +607,8 @@ int factor_level_t(hsim_ctx *ctx, LevelData &L, const double *S, const double *M
             if (blocked && block_end) {
                 const size_t b = kst / spb;
                 const int64_t t0 = L.schur_off[h][b], t1 = L.schur_off[h][b + 1];
-                k::schur_tc(s, L.fd, L.schur_tasks.p + t0, (int)(t1 - t0), K0, reinterpret_cast<float *>(arena.p));
+                k::schur_tc(s, L.fd, L.schur_tasks.p + t0, (int)(t1 - t0), K0, reinterpret_cast<float *>(arena.p),
+                            ctx->err_tc32());
             }
         }
     }
@@ -608,7 +618,7 @@ int factor_level_t(hsim_ctx *ctx, LevelData &L, const double *S, const double *M
         // FP32 factors are solved in the inverted form (see solve_level_t)
         dinv.reserve((size_t)L.n);
         k::reciprocal(s, L.n, (const T *)dpos.p, dinv.p);
-        invert_level_t<T>(s, L, arena.p, scr);
+        invert_level_t<T>(s, L, arena.p, scr, ctx->err_tc32());
     }
     HSIM_CUDA(cudaMemcpyAsync(ctx->hflags.data(), flags, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
     HSIM_CUDA(cudaStreamSynchronize(s));
@@ -702,7 +712,7 @@ void solve_level_t(hsim_ctx *ctx, LevelData &L, const T *arena, const T *dpos, c
         }
         if constexpr (std::is_same<T, float>::value) {
             if (tc32_enabled() && L.h_maxns[h] >= kTcMinFwdPivots)
-                k::solve_fwd_tc(s, L.fd, nodes, cnt, L.h_maxnf[h], arena, k, X, Y.p, ldx);
+                k::solve_fwd_tc(s, L.fd, nodes, cnt, L.h_maxnf[h], arena, k, X, Y.p, ldx, ctx->err_tc32());
             else
                 k::solve_fwd_inv(s, L.fd, nodes, cnt, L.h_maxnf[h], L.h_maxns[h], arena, k, X, Y.p, ldx);
         } else {
@@ -1141,16 +1151,18 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
                 k::OzakiOperand YS = k::ozaki_split_cols(s, n, q, H->SP.p, q, H->oz.p + part, gd, k::OzakiRole::Y);
                 k::OzakiOperand YM = k::ozaki_split_cols(s, n, q, H->MP.p, q, H->oz.p + 2 * part, gd, k::OzakiRole::Y);
                 const double t_split = ts.stop();
-                k::ozaki_product(s, X, YS, H->Sbar.p, q, 0, true);
-                k::ozaki_product(s, X, YM, H->Mbar.p, q, 0, true);
+                k::ozaki_product(s, X, YS, H->Sbar.p, q, 0, ctx->err_products(), true);
+                k::ozaki_product(s, X, YM, H->Mbar.p, q, 0, ctx->err_products(), true);
                 const double t_prod = ts.stop();
                 inf.ms_tc_product += t_prod;
                 ph[2] = t_split + t_prod;
             } else {
                 if (k::gram64_on_digits(n, q, q)) {
                     H->oz.reserve(k::gram64_scratch(n, q, q));
-                    k::gram64(s, n, q, q, H->Psi.p, q, H->SP.p, q, H->Sbar.p, q, true, k::Held::Norms, H->oz.p);
-                    k::gram64(s, n, q, q, H->Psi.p, q, H->MP.p, q, H->Mbar.p, q, true, k::Held::Norms, H->oz.p);
+                    k::gram64(s, n, q, q, H->Psi.p, q, H->SP.p, q, H->Sbar.p, q, true, k::Held::Norms, H->oz.p,
+                              ctx->err_products());
+                    k::gram64(s, n, q, q, H->Psi.p, q, H->MP.p, q, H->Mbar.p, q, true, k::Held::Norms, H->oz.p,
+                              ctx->err_products());
                 } else {
                     k::gram(s, n, q, q, H->Psi.p, q, H->SP.p, q, H->Sbar.p, q, true);
                     k::gram(s, n, q, q, H->Psi.p, q, H->MP.p, q, H->Mbar.p, q, true);
@@ -1172,13 +1184,14 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
                 k::OzakiOperand X = k::ozaki_split_rows(s, n, q, H->Psi.p, q, H->oz.p);
                 k::OzakiOperand Y = k::ozaki_split_cols(s, q, q, H->phibar.p, q, H->oz.p + part, k::kOzakiSlices, k::OzakiRole::Y);
                 const double t_split = ts.stop();
-                k::ozaki_product(s, X, Y, H->Phi.p, q, 1);
+                k::ozaki_product(s, X, Y, H->Phi.p, q, 1, ctx->err_products());
                 const double t_prod = ts.stop();
                 inf.ms_tc_product += t_prod;
                 ph[4] = t_split + t_prod;
             } else if (k::update64_on_digits(n, q, q, true)) {
                 H->oz.reserve(k::update64_scratch(n, q, q));
-                k::update64(s, n, q, q, H->Psi.p, q, H->phibar.p, q, H->Phi.p, q, k::Held::Norms, H->oz.p);
+                k::update64(s, n, q, q, H->Psi.p, q, H->phibar.p, q, H->Phi.p, q, k::Held::Norms, H->oz.p,
+                            ctx->err_products());
             } else {
                 k::gemm_nn(s, n, q, q, H->Psi.p, q, H->phibar.p, q, H->Phi.p, q);
             }
@@ -1193,8 +1206,8 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
             HSIM_CUDA(cudaMemcpyAsync(rs.data(), H->res_sums.p, 3 * p * sizeof(double), cudaMemcpyDeviceToHost, s));
             HSIM_CUDA(cudaMemcpyAsync(lam_h.data(), H->lam.p, q * sizeof(double), cudaMemcpyDeviceToHost, s));
             HSIM_CUDA(cudaStreamSynchronize(s));
-            k::ozaki_check(s);
-            if (mixed) k::tc32_check(s);
+            k::ozaki_check(s, ctx->err_products());
+            if (mixed) k::tc32_check(s, ctx->err_tc32());
             inf.ms_residual += (ph[5] = ts.stop());
             double lam_ref = lam_h[q - 1];
             for (int i = 0; i < q; ++i)
@@ -1472,9 +1485,7 @@ hsim_status hsim_create(int device, void *stream, hsim_ctx **out) {
         auto c = std::make_unique<hsim_ctx>();
         c->device = device;
         c->stream = (cudaStream_t)stream;
-        c->flags.alloc(16);
-        c->hflags.assign(16, 0);
-        c->scratch_u64.alloc(4);
+        c->init();
         *out = c.release();
     });
 }
@@ -1637,9 +1648,7 @@ hsim_status hsim_solve_batched(hsim_ctx *ctx, int nmesh, hsim_hier *const *hiers
                 auto c = std::make_unique<hsim_ctx>();
                 c->device = ctx->device;
                 HSIM_CUDA(cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking));
-                c->flags.alloc(16);
-                c->hflags.assign(16, 0);
-                c->scratch_u64.alloc(4);
+                c->init();
                 HSIM_CUDA(cudaStreamWaitEvent(c->stream, ready, 0));
                 wctx.push_back(std::move(c));
             }
@@ -1738,8 +1747,8 @@ hsim_status hsim_gram(hsim_ctx *ctx, int n, int ka, int kb, const double *A, int
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"G", G}});
         if (k::gram64_on_digits(n, ka, kb)) {
             CtxScratch<unsigned char> scratch(ctx, k::gram64_scratch(n, ka, kb));
-            k::gram64(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, false, k::Held::Entries, scratch.p);
-            k::ozaki_check(ctx->stream);
+            k::gram64(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, false, k::Held::Entries, scratch.p, ctx->err_products());
+            k::ozaki_check(ctx->stream, ctx->err_products());
             return;
         }
         k::gram(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, false);
@@ -1756,12 +1765,21 @@ hsim_status hsim_gemm_update(hsim_ctx *ctx, int n, int kk, int m, const double *
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"C", C}});
         if (k::update64_on_digits(n, kk, m, false)) {
             CtxScratch<unsigned char> scratch(ctx, k::update64_scratch(n, kk, m));
-            k::update64(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc, k::Held::Entries, scratch.p);
-            k::ozaki_check(ctx->stream);
+            k::update64(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc, k::Held::Entries, scratch.p,
+                        ctx->err_products());
+            k::ozaki_check(ctx->stream, ctx->err_products());
             return;
         }
         k::gemm_nn(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc);
         HSIM_CUDA(cudaStreamSynchronize(ctx->stream));
+    });
+}
+
+hsim_status hsim_check_product_error(hsim_ctx *ctx) {
+    return guard([&] {
+        HSIM_CHECK_ARG(ctx, "NULL argument");
+        DeviceGuard dg(ctx->device);
+        HSIM_CUDA(cudaMemsetAsync(ctx->err_products(), 1, sizeof(int), ctx->stream));
     });
 }
 
@@ -1774,8 +1792,8 @@ hsim_status hsim_gram_tc(hsim_ctx *ctx, int n, int ka, int kb, const double *A, 
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"G", G}});
         CtxScratch<unsigned char> scratch(ctx, k::ozaki_gram_scratch(n, ka, kb, digits));
-        k::ozaki_gram(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, digits, scratch.p);
-        k::ozaki_check(ctx->stream);
+        k::ozaki_gram(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, digits, scratch.p, ctx->err_products());
+        k::ozaki_check(ctx->stream, ctx->err_products());
     });
 }
 
@@ -1787,8 +1805,8 @@ hsim_status hsim_gemm_update_tc(hsim_ctx *ctx, int n, int kk, int m, const doubl
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"C", C}});
         CtxScratch<unsigned char> scratch(ctx, k::ozaki_update_scratch(n, kk, m, k::kOzakiSlices));
-        k::ozaki_update(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc, k::kOzakiSlices, scratch.p);
-        k::ozaki_check(ctx->stream);
+        k::ozaki_update(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc, k::kOzakiSlices, scratch.p, ctx->err_products());
+        k::ozaki_check(ctx->stream, ctx->err_products());
     });
 }
 
@@ -1921,7 +1939,7 @@ hsim_status hsim_shifted_solve(hsim_ctx *ctx, hsim_hier *h, int tau, const doubl
         solve_level(ctx, h, L, X.p, kk, kk);
         k::gather_rows(s, L.n, kk, L.d_iperm.p, X.p, kk, B, ldb);
         HSIM_CUDA(cudaStreamSynchronize(s));
-        k::tc32_check(s);
+        k::tc32_check(s, ctx->err_tc32());
         if (neg) *neg = negp;
     });
 }
@@ -1952,7 +1970,7 @@ hsim_status hsim_shifted_solve_f32(hsim_ctx *ctx, hsim_hier *h, int tau, const d
         k::convert_matrix(s, L.n, kk, X32.p, ld, X.p, kk);
         k::gather_rows(s, L.n, kk, L.d_iperm.p, X.p, kk, B, ldb);
         HSIM_CUDA(cudaStreamSynchronize(s));
-        k::tc32_check(s);
+        k::tc32_check(s, ctx->err_tc32());
         if (neg) *neg = negp;
     });
 }

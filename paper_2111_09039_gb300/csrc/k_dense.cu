@@ -800,14 +800,14 @@ static void small_mm(cudaStream_t s, int n, int kk, int m, SmallMM p0, int lda, 
 // C = A B, k x k times k x m blocks, row-major: FP64 or an FP64-accurate
 // tensor-core product
 static void tc_mm(cudaStream_t s, int k, int m, const double *A, int lda, const double *B, int ldb, double *C, int ldc,
-                  unsigned char *oz) {
+                  unsigned char *oz, int *err) {
     if (k <= kSmallMM) {
         small_mm(s, k, k, m, {A, B, C}, lda, ldb, ldc);
         return;
     }
     OzakiOperand a = ozaki_split_rows(s, k, k, A, lda, oz);
     OzakiOperand b = ozaki_split_cols(s, k, m, B, ldb, oz + ozaki_rows_scratch(k, k), kOzakiSlices, OzakiRole::Y);
-    ozaki_product(s, a, b, C, ldc, 0);
+    ozaki_product(s, a, b, C, ldc, 0, err);
 }
 
 // Z = M_bar^-1/2 by the coupled Newton-Schulz iteration Y_0 = M_bar, Z_0 = I,
@@ -821,7 +821,7 @@ static void tc_mm(cudaStream_t s, int k, int m, const double *A, int lda, const 
 // products carry about 2^-47 of their row and column maxima per term, so the
 // attainable level near I is a few 1e-14 times sqrt(k).  *steps: iterations.
 static const double *ns_inv_sqrt(cudaStream_t s, int k, const double *Mbar, int ldm, double *const buf[5],
-                                 unsigned char *oz, unsigned long long *dmax, int *steps) {
+                                 unsigned char *oz, unsigned long long *dmax, int *steps, int *err) {
     auto read_max = [&](double &v) {
         unsigned long long h = 0;
         HSIM_CUDA(cudaMemcpyAsync(&h, dmax, sizeof(h), cudaMemcpyDeviceToHost, s));
@@ -844,7 +844,7 @@ static const double *ns_inv_sqrt(cudaStream_t s, int k, const double *Mbar, int 
         if (k <= kSmallMM) {
             k_small_mm<true><<<dim3(cdiv(k, 8), cdiv(k, 16)), 128, 0, s>>>(k, k, k, {Z, Y, T}, {Z, Y, T}, k, k, k, dmax);
         } else {
-            tc_mm(s, k, k, Z, k, Y, k, P, k, oz);  // P = Z Y
+            tc_mm(s, k, k, Z, k, Y, k, P, k, oz, err);  // P = Z Y
             k_ns_step<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, P, T, dmax);
         }
         HSIM_LAUNCHED();
@@ -865,9 +865,9 @@ static const double *ns_inv_sqrt(cudaStream_t s, int k, const double *Mbar, int 
             std::swap(Z, Q);
             continue;
         }
-        tc_mm(s, k, k, Y, k, T, k, P, k, oz);  // Y T
+        tc_mm(s, k, k, Y, k, T, k, P, k, oz, err);  // Y T
         std::swap(Y, P);
-        tc_mm(s, k, k, T, k, Z, k, P, k, oz);  // T Z
+        tc_mm(s, k, k, T, k, Z, k, P, k, oz, err);  // T Z
         std::swap(Z, P);
     }
     return nullptr;
@@ -875,6 +875,7 @@ static const double *ns_inv_sqrt(cudaStream_t s, int k, const double *Mbar, int 
 
 int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar, int ldm, double *evals, double *X,
          int ldx, double *work, int *sweeps, int *flag_dev, int *flag_host, int m, bool tc) {
+    int *err = flag_dev + kErrProducts;
     // work layout: F (k*k) | W (k*k) | T (k*k) | d (k) | eigensolver work
     if (m <= 0 || m > k) m = k;
     const size_t kk = (size_t)k * k;
@@ -892,17 +893,17 @@ int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar,
         double *const buf[5] = {F, Cr, Cc, scr, T};
         int ns_steps = 0;
         const double *Wz =
-            ns_inv_sqrt(s, k, Mbar, ldm, buf, oz, reinterpret_cast<unsigned long long *>(flag_dev + 4), &ns_steps);
+            ns_inv_sqrt(s, k, Mbar, ldm, buf, oz, reinterpret_cast<unsigned long long *>(flag_dev + 4), &ns_steps, err);
         if (Wz) {
             if (sweeps) *sweeps = ns_steps;
             double *A = Wz == T ? F : T;
-            tc_mm(s, k, k, Wz, k, Sbar, lds, W, k, oz);
-            tc_mm(s, k, k, W, k, Wz, k, A, k, oz);
+            tc_mm(s, k, k, Wz, k, Sbar, lds, W, k, oz, err);
+            tc_mm(s, k, k, W, k, Wz, k, A, k, oz, err);
             k_symmetrize<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, A, k);
             HSIM_LAUNCHED();
             sym_eig(s, k, m, A, evals, V, m, ework);
-            tc_mm(s, k, m, Wz, k, V, m, X, ldx, oz);
-            if (k > kSmallMM) ozaki_check(s);
+            tc_mm(s, k, m, Wz, k, V, m, X, ldx, oz, err);
+            if (k > kSmallMM) ozaki_check(s, err);
             return 0;
         }
     }
@@ -937,13 +938,13 @@ int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar,
         }
         k_cinv<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, F, d, Cr, Cc);
         HSIM_LAUNCHED();
-        tc_mm(s, k, k, Cr, k, Sbar, lds, W, k, oz);
-        tc_mm(s, k, k, W, k, Cc, k, T, k, oz);
+        tc_mm(s, k, k, Cr, k, Sbar, lds, W, k, oz, err);
+        tc_mm(s, k, k, W, k, Cc, k, T, k, oz, err);
         k_symmetrize<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, T, k);
         HSIM_LAUNCHED();
         sym_eig(s, k, m, T, evals, V, m, ework);
-        tc_mm(s, k, m, Cc, k, V, m, X, ldx, oz);
-        if (k > kSmallMM) ozaki_check(s);
+        tc_mm(s, k, m, Cc, k, V, m, X, ldx, oz, err);
+        if (k > kSmallMM) ozaki_check(s, err);
         return 0;
     }
     // A = C^-1 S_bar C^-T: W = D^-1/2 L^-1 S_bar, T = D^-1/2 L^-1 W^T

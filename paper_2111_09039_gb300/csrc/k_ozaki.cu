@@ -495,7 +495,7 @@ int sm_count_oz() {
 // issues the MMAs (one thread), warps 2..9 drain, one TMEM lane (output row)
 // and 32 of the 64 columns per thread, and write the item's results while the
 // MMAs of the next item run.  Every mbarrier wait gives up after 2 s, records
-// an error flag that the host checks, and the CTA still drains its own copies
+// that in the caller's error word, which the host checks, and the CTA still drains its own copies
 // and MMAs and frees its TMEM.
 // ------------------------------------------------------------------------------
 constexpr int TC_M = 128, TC_N = 64, TC_K = 16;
@@ -518,8 +518,6 @@ template <int SL> __host__ __device__ constexpr int tc_low() { return SL == 5 ? 
 template <int SL> constexpr size_t tc_smem() { return (size_t)tc_stages<SL>() * tc_stage_bytes<SL>() + 1024; }
 constexpr uint32_t TC_TMEM_COLS = 512;
 constexpr uint64_t TC_WAIT_NS = 2000000000ull;  // 2 s per barrier wait
-
-__device__ int g_oz_error;
 
 // shared-memory matrix descriptor, low word: start >> 4 (bits 0-13), LBO >> 4
 // (16-29); high word: SBO >> 4 (32-45), descriptor version 1 (46-47), no
@@ -547,7 +545,8 @@ __device__ __forceinline__ uint64_t global_ns() {
 }
 
 // wait for the phase of the given parity; gives up after TC_WAIT_NS of wall time
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+// and sets *err
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int *err) {
     uint64_t t0 = 0;
     for (uint32_t it = 0;; ++it) {
         uint32_t ok;
@@ -563,7 +562,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
             else if (t - t0 > TC_WAIT_NS) break;
         }
     }
-    atomicExch(&g_oz_error, 1);
+    atomicExch(err, 1);
     return false;
 }
 
@@ -735,7 +734,7 @@ template <int SL>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_ozaki_tc(int M, int N, const __nv_bfloat16 *__restrict__ Xs, int nbx, const __nv_bfloat16 *__restrict__ Ys,
                int nby, const int *__restrict__ ex, const int *__restrict__ ey, double *__restrict__ C, int ldc,
-               TcWork w, int atomic, int vec) {
+               TcWork w, int atomic, int vec, int *__restrict__ err) {
     constexpr int ND = tc_nd<SL>(), STAGES = tc_stages<SL>(), LOW = tc_low<SL>();
     constexpr uint32_t A_BYTES = tc_a_bytes<SL>(), B_BYTES = tc_b_bytes<SL>(), STAGE = tc_stage_bytes<SL>();
     constexpr uint32_t LBO = 128, SBO = 256, SLICE_A = A_BYTES / SL, SLICE_B = B_BYTES / SL;
@@ -781,7 +780,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 const __nv_bfloat16 *yb = Ys + ((size_t)it.kc0 * nby + it.j0 / TC_N) * (B_BYTES / 2);
                 for (int kt = 0; kt < it.nk; ++kt, ++g) {
                     const int st = g % STAGES;
-                    if (g >= STAGES) ok = mbar_wait(smem_addr(&empty_bar[st]), ((g / STAGES) & 1) ^ 1);
+                    if (g >= STAGES) ok = mbar_wait(smem_addr(&empty_bar[st]), ((g / STAGES) & 1) ^ 1, err);
                     if (!ok) break;
                     const uint32_t fb = smem_addr(&full_bar[st]), dst = smem0 + st * STAGE;
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb), "r"(STAGE)
@@ -791,7 +790,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 }
             }
             // the last loads of every stage have landed before the CTA exits
-            for (int q = max(0, g - STAGES); q < g; ++q) mbar_wait(smem_addr(&full_bar[q % STAGES]), (q / STAGES) & 1);
+            for (int q = max(0, g - STAGES); q < g; ++q) mbar_wait(smem_addr(&full_bar[q % STAGES]), (q / STAGES) & 1, err);
         }
     } else if (warp == 1) {
         // the whole warp runs the loop, the elected lane issues
@@ -830,10 +829,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 const uint32_t ap = (c - 1) & 1;  // parity of the chunk before
                 const uint32_t hi = tmem + (c & 1) * TC_N * (ND - LOW);
                 // first step of the chunk: every accumulator is overwritten once
-                ok = mbar_wait(full0 + 8 * st, ph);
+                ok = mbar_wait(full0 + 8 * st, ph, err);
                 const uint32_t dw = d0 + st * (STAGE >> 4);
                 if constexpr (SL == 7) {
-                    if (c > 0) ok = ok && mbar_wait(smem_addr(&free_bar[0]), ap);
+                    if (c > 0) ok = ok && mbar_wait(smem_addr(&free_bar[0]), ap, err);
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                     part(dw, hi, 0, 0, 6, 0);  // acc_0 .. acc_6 start
@@ -848,7 +847,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                         // ended, acc_3 and acc_2 (six digits), acc_1 and acc_0
                         // when the drain says so
                         if (c > 0 && (sl == 1 || (SL == 6 && sl == 3))) {
-                            ok = ok && mbar_wait(smem_addr(&free_bar[SL == 6 && sl == 1 ? 1 : 0]), ap);
+                            ok = ok && mbar_wait(smem_addr(&free_bar[SL == 6 && sl == 1 ? 1 : 0]), ap, err);
                             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                         }
                         if (!ok) break;
@@ -860,7 +859,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 umma_commit(empty0 + 8 * st, el);
                 if (++st == STAGES) st = 0, ph ^= 1;
                 for (int q = 1; q < steps; ++q) {
-                    ok = mbar_wait(full0 + 8 * st, ph);
+                    ok = mbar_wait(full0 + 8 * st, ph, err);
                     if (!ok) break;
                     const uint32_t dw = d0 + st * (STAGE >> 4);
 #pragma unroll
@@ -872,7 +871,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 // drained (waited for here, before this chunk's own completion,
                 // so that the barrier is never two phases ahead)
                 if (SL != 7 && c > 0) {
-                    ok = ok && mbar_wait(smem_addr(&high_bar), ap);
+                    ok = ok && mbar_wait(smem_addr(&high_bar), ap, err);
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 }
                 if (!ok) break;
@@ -881,7 +880,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
         // every MMA issued by this warp has completed before teardown
         umma_commit(smem_addr(&drain_bar), el);
-        mbar_wait(smem_addr(&drain_bar), 0);
+        mbar_wait(smem_addr(&drain_bar), 0, err);
     } else {
         // drain warps: TMEM lane quadrant = warp % 4, one output row and one
         // 32-column half per thread
@@ -906,7 +905,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 for (int q = 0; q < 32; ++q) mid[q] = 0.f;
             const int nchunks = (it.nk + kChunkSteps - 1) / kChunkSteps;
             for (int ch = 0; ch < nchunks && ok; ++ch, ++c) {
-                ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&accf_bar), c & 1));
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&accf_bar), c & 1, err));
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 const uint32_t thigh = tbase + (c & 1) * TC_N * (ND - LOW);
@@ -1106,7 +1105,7 @@ struct MagCheck {
 
 __global__ void __launch_bounds__(TC_THREADS, 1)
     k_magnitudes_tc(int M, int N, const __nv_bfloat16 *__restrict__ Xs, int nbx, const __nv_bfloat16 *__restrict__ Ys,
-                    MagWork w, MagCheck chk) {
+                    MagWork w, MagCheck chk, int *__restrict__ err) {
     extern __shared__ unsigned char smem_dyn[];
     __shared__ __align__(8) uint64_t full_bar[kMagStages], empty_bar[kMagStages], accf_bar[2], free_bar[2], drain_bar;
     __shared__ uint32_t tmem_slot;
@@ -1155,7 +1154,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 const Item it = item_of(item);
                 for (int k0 = 0; k0 < it.nk; k0 += kMagSteps, ++g) {
                     const int st = g % kMagStages, steps = min(kMagSteps, it.nk - k0);
-                    if (g >= kMagStages) ok = mbar_wait(smem_addr(&empty_bar[st]), ((g / kMagStages) & 1) ^ 1);
+                    if (g >= kMagStages) ok = mbar_wait(smem_addr(&empty_bar[st]), ((g / kMagStages) & 1) ^ 1, err);
                     if (!ok) break;
                     const uint32_t fb = smem_addr(&full_bar[st]), dst = smem0 + st * kMagStage;
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb),
@@ -1170,7 +1169,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 }
             }
             for (int q = max(0, g - kMagStages); q < g; ++q)
-                mbar_wait(smem_addr(&full_bar[q % kMagStages]), (q / kMagStages) & 1);
+                mbar_wait(smem_addr(&full_bar[q % kMagStages]), (q / kMagStages) & 1, err);
         }
     } else if (warp == 1) {
         const uint32_t el = elect_lane();
@@ -1181,12 +1180,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             const Item it = item_of(item);
             const uint32_t d = tmem + (c & 1) * TC_N * kMagBlocks, idesc = umma_idesc(TC_M, TC_N * it.nb);
             // the set is drained of the item before the last
-            if (c >= 2) ok = mbar_wait(smem_addr(&free_bar[c & 1]), ((c >> 1) - 1) & 1);
+            if (c >= 2) ok = mbar_wait(smem_addr(&free_bar[c & 1]), ((c >> 1) - 1) & 1, err);
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             for (int k0 = 0; k0 < it.nk; k0 += kMagSteps, ++g) {
                 const uint32_t st = g % kMagStages;
-                ok = mbar_wait(smem_addr(&full_bar[st]), (g / kMagStages) & 1);
+                ok = mbar_wait(smem_addr(&full_bar[st]), (g / kMagStages) & 1, err);
                 if (!ok) break;
                 const uint32_t a = smem0 + st * kMagStage, b = a + kMagSteps * kMagA;
                 const int steps = min(kMagSteps, it.nk - k0);
@@ -1199,7 +1198,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             umma_commit(smem_addr(&accf_bar[c & 1]), el);
         }
         umma_commit(smem_addr(&drain_bar), el);
-        mbar_wait(smem_addr(&drain_bar), 0);
+        mbar_wait(smem_addr(&drain_bar), 0, err);
     } else {
         const int quad = warp & 3, c0 = 32 * ((warp - 2) >> 2);
         bool ok = true;
@@ -1208,7 +1207,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             const Item it = item_of(item);
             const int i = it.ti * TC_M + 32 * quad + lane;
             const float li = chk.h || i >= M ? 0.f : chk.lx[i];
-            ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&accf_bar[c & 1]), (c >> 1) & 1));
+            ok = __all_sync(0xffffffffu, mbar_wait(smem_addr(&accf_bar[c & 1]), (c >> 1) & 1, err));
             if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             for (int b = 0; b < it.nb; ++b) {
@@ -1257,13 +1256,13 @@ inline bool pair_rows(const double *p, int ld) { return aligned16(p) && ld % 2 =
 
 template <int SL>
 void launch_tc(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, const TcWork &w,
-               bool atomic) {
+               bool atomic, int *err) {
     HSIM_SMEM_LIMIT_ONCE(k_ozaki_tc<SL>, tc_smem<SL>());
     const int grid = std::min(w.items, sm_count_oz());
     const bool vec = !atomic && !w.lower && pair_rows(C, ldc);
     k_ozaki_tc<SL><<<grid, TC_THREADS, tc_smem<SL>(), s>>>(X.rows, Y.rows, X.slices, X.rows_p / TC_M, Y.slices,
                                                           Y.rows_p / TC_N, X.exps, Y.exps, C, ldc, w, atomic ? 1 : 0,
-                                                          vec ? 1 : 0);
+                                                          vec ? 1 : 0, err);
     HSIM_LAUNCHED();
 }
 
@@ -1418,7 +1417,7 @@ static void zero_block(cudaStream_t s, int rows, int cols, double *C, int ldc) {
     else HSIM_CUDA(cudaMemset2DAsync(C, (size_t)ldc * sizeof(double), 0, (size_t)cols * sizeof(double), rows, s));
 }
 
-void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, int splits,
+void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, int splits, int *err,
                    bool lower, bool accumulate, const int *skip, int skip_ld) {
     if (X.rows <= 0 || Y.rows <= 0) return;
     TcWork w{};
@@ -1427,14 +1426,14 @@ void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y,
     w.skip_ld = skip_ld;
     const bool atomic = splits > 1 || accumulate;
     if (atomic && !accumulate) zero_block(s, X.rows, Y.rows, C, ldc);
-    if (X.digits == 5) launch_tc<5>(s, X, Y, C, ldc, w, atomic);
-    else if (X.digits == 6) launch_tc<6>(s, X, Y, C, ldc, w, atomic);
-    else launch_tc<7>(s, X, Y, C, ldc, w, atomic);
+    if (X.digits == 5) launch_tc<5>(s, X, Y, C, ldc, w, atomic, err);
+    else if (X.digits == 6) launch_tc<6>(s, X, Y, C, ldc, w, atomic, err);
+    else launch_tc<7>(s, X, Y, C, ldc, w, atomic, err);
 }
 
 // the product of two slices of magnitudes, added to chk.h (over K ranges that fill
 // the SMs) or checked (one K range)
-static void product_magnitudes(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, const MagCheck &chk) {
+static void product_magnitudes(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, const MagCheck &chk, int *err) {
     MagWork w{};
     w.nby = Y.rows_p / TC_N;
     w.groups = (int)cdiv(w.nby, kMagBlocks);
@@ -1450,7 +1449,7 @@ static void product_magnitudes(cudaStream_t s, const OzakiOperand &X, const Ozak
     w.items = (int)items;
     HSIM_SMEM_LIMIT_ONCE(k_magnitudes_tc, kMagSmem);
     k_magnitudes_tc<<<std::min(w.items, sm_count_oz()), TC_THREADS, kMagSmem, s>>>(X.rows, Y.rows, X.slices, X.rows_p / TC_M,
-                                                                              Y.slices, w, chk);
+                                                                              Y.slices, w, chk, err);
     HSIM_LAUNCHED();
 }
 
@@ -1477,7 +1476,7 @@ size_t ozaki_gram_scratch(int n, int ka, int kb, int digits) {
 }
 
 void ozaki_gram(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
-                int ldg, int digits, void *scratch) {
+                int ldg, int digits, void *scratch, int *err) {
     const int range = gram_rows(n, ka, kb, digits);
     int *ex = static_cast<int *>(scratch);
     int *ey = ex + exps_bytes(ka) / sizeof(int);
@@ -1494,7 +1493,7 @@ void ozaki_gram(cudaStream_t s, int n, int ka, int kb, const double *A, int lda,
         Y.exps = ey;
         split_cols_into(s, X, rows, A + (size_t)r0 * lda, lda, nullptr);
         split_cols_into(s, Y, rows, B + (size_t)r0 * ldb, ldb, nullptr);
-        ozaki_product(s, X, Y, G, ldg, 0, false, several);
+        ozaki_product(s, X, Y, G, ldg, 0, err, false, several);
     }
 }
 
@@ -1505,13 +1504,13 @@ size_t ozaki_update_scratch(int n, int k, int m, int digits) {
 }
 
 void ozaki_update(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
-                  int ldc, int digits, void *scratch) {
+                  int ldc, int digits, void *scratch, int *err) {
     const int range = update_rows(n, k, digits);
     unsigned char *sy = static_cast<unsigned char *>(scratch), *sx = sy + operand_bytes(m, k, digits);
     OzakiOperand Y = ozaki_split_cols(s, k, m, B, ldb, sy, digits, OzakiRole::Y);
     for (int r0 = 0; r0 < n; r0 += range) {
         OzakiOperand X = ozaki_split_rows(s, std::min(range, n - r0), k, A + (size_t)r0 * lda, lda, sx, digits);
-        ozaki_product(s, X, Y, C + (size_t)r0 * ldc, ldc, 1);
+        ozaki_product(s, X, Y, C + (size_t)r0 * ldc, ldc, 1, err);
     }
 }
 
@@ -1662,7 +1661,7 @@ struct Update64 {
 size_t gram64_scratch(int n, int ka, int kb) { return Gram64(n, ka, kb, ka, kb, nullptr).bytes; }
 
 void gram64(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
-            int ldg, bool lower, Held held, void *scratch) {
+            int ldg, bool lower, Held held, void *scratch, int *err) {
     const Gram64 g(n, ka, kb, lda, ldb, scratch);
     const int tm = tile_rows(ka), tn = tile_cols(kb);
     HSIM_CUDA(cudaMemsetAsync(g.tiles, 0, g.zero_bytes, s));
@@ -1691,7 +1690,7 @@ void gram64(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, con
         for (int r0 = 0; r0 < g.sampled; r0 += g.mag_range) {
             const size_t r = (size_t)r0 * g.step;
             operands(std::min(g.mag_range, g.sampled - r0), 1, X, Y, A + r * lda, lda * g.step, B + r * ldb, ldb * g.step);
-            product_magnitudes(s, X, Y, chk);
+            product_magnitudes(s, X, Y, chk, err);
         }
         k_check_tiles<<<cdiv((int64_t)ka * kb, 256), 256, 0, s>>>(ka, kb, (float)n, digits_ratio(n), g.h, g.ex, g.sx, g.ey,
                                                                  g.sy, g.tiles, tn);
@@ -1703,7 +1702,7 @@ void gram64(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, con
     if (several) zero_block(s, ka, kb, G, ldg);
     for (int r0 = 0; r0 < n; r0 += g.range) {
         operands(std::min(g.range, n - r0), kDigits64, X, Y, A + (size_t)r0 * lda, lda, B + (size_t)r0 * ldb, ldb);
-        ozaki_product(s, X, Y, G, ldg, 0, lower, several, g.tiles, tn);
+        ozaki_product(s, X, Y, G, ldg, 0, err, lower, several, g.tiles, tn);
     }
     gram_tiles(s, n, ka, kb, A, lda, B, ldb, G, ldg, lower, g.tiles, tn);
 }
@@ -1711,7 +1710,7 @@ void gram64(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, con
 size_t update64_scratch(int n, int k, int m) { return Update64(n, k, m, nullptr).bytes; }
 
 void update64(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
-              int ldc, Held held, void *scratch) {
+              int ldc, Held held, void *scratch, int *err) {
     const Update64 u(n, k, m, scratch);
     const int tn = tile_cols(m);
     HSIM_CUDA(cudaMemsetAsync(u.tiles, 0, u.zero_bytes, s));
@@ -1740,24 +1739,23 @@ void update64(cudaStream_t s, int n, int k, int m, const double *A, int lda, con
         split_rows_into(s, X, k, A + (size_t)r0 * lda, lda, u.cexp, entries ? Xm.slices : nullptr, entries ? u.lx : nullptr);
         if (entries) {
             const MagCheck chk{nullptr, u.lx, u.ly, digits_ratio(k), tiles, tn};
-            product_magnitudes(s, Xm, Ym, chk);
+            product_magnitudes(s, Xm, Ym, chk, err);
         } else {
             k_guard_tiles<<<dim3(cdiv(rows, 64), tn), 128, 0, s>>>(rows, m, (double)k, X.exps, nullptr, Y.exps, nullptr, tiles,
                                                                   tn);
             HSIM_LAUNCHED();
         }
-        ozaki_product(s, X, Y, C + (size_t)r0 * ldc, ldc, 1, false, false, tiles, tn);
+        ozaki_product(s, X, Y, C + (size_t)r0 * ldc, ldc, 1, err, false, false, tiles, tn);
     }
     gemm_nn_tiles(s, n, k, m, A, lda, B, ldb, C, ldc, u.tiles, tn);
 }
 
-void ozaki_check(cudaStream_t s) {
+void ozaki_check(cudaStream_t s, int *err) {
     int h = 0;
-    HSIM_CUDA(cudaMemcpyFromSymbolAsync(&h, g_oz_error, sizeof(int), 0, cudaMemcpyDeviceToHost, s));
+    HSIM_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     HSIM_CUDA(cudaStreamSynchronize(s));
     if (h != 0) {
-        const int zero = 0;
-        HSIM_CUDA(cudaMemcpyToSymbolAsync(g_oz_error, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, s));
+        HSIM_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
         HSIM_CUDA(cudaStreamSynchronize(s));
         fail(HSIM_E_INTERNAL, "tensor-core product: an mbarrier wait timed out");
     }

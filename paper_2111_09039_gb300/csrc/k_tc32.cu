@@ -62,8 +62,6 @@ constexpr size_t SMEM = 2 * (size_t)STAGE_BYTES + 1024;
 constexpr uint32_t TMEM_COLS = BN;
 constexpr uint64_t WAIT_NS = 2000000000ull;  // 2 s per barrier wait
 
-__device__ int g_tc32_error;
-
 inline unsigned cdiv(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
 __device__ __forceinline__ uint32_t swz_off(int r, int kq) {
@@ -117,7 +115,7 @@ __device__ __forceinline__ void atomic_sub32(float *p, const float (&v)[32], int
 // ---- the tile engine ----------------------------------------------------------
 
 template <class Op>
-__global__ void __launch_bounds__(THREADS, 1) k_tc32(const Op op) {
+__global__ void __launch_bounds__(THREADS, 1) k_tc32(const Op op, int *__restrict__ err) {
     extern __shared__ unsigned char smem_dyn[];
     __shared__ __align__(8) uint64_t bar[2], done;
     __shared__ uint32_t tmem_slot;
@@ -126,7 +124,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_tc32(const Op op) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nk = T.ke > T.kb ? (T.ke - T.kb + BK - 1) / BK : 0;
     const uint32_t smem0 = (tc::smem_addr(smem_dyn) + 1023u) & ~1023u;
-    int *err = &g_tc32_error;
     if (tid == 0) {
         tc::mbar_init(tc::smem_addr(&bar[0]), 1);
         tc::mbar_init(tc::smem_addr(&bar[1]), 1);
@@ -405,9 +402,9 @@ struct SchurOp {
 };
 
 template <class Op>
-void launch(cudaStream_t s, dim3 grid, const Op &op) {
+void launch(cudaStream_t s, dim3 grid, const Op &op, int *err) {
     HSIM_SMEM_LIMIT_ONCE(k_tc32<Op>, SMEM);
-    k_tc32<Op><<<grid, THREADS, SMEM, s>>>(op);
+    k_tc32<Op><<<grid, THREADS, SMEM, s>>>(op, err);
     HSIM_LAUNCHED();
 }
 
@@ -418,21 +415,21 @@ bool aligned16f(const float *p, int ldx) {
 }  // namespace
 
 void solve_fwd_tc(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int max_nf, const float *arena,
-                  int k, float *X, float *Y, int ldx) {
+                  int k, float *X, float *Y, int ldx, int *err) {
     if (n_nodes <= 0 || k <= 0 || max_nf <= 0) return;
     FwdSolveOp op{fd, nodes, (int)cdiv(max_nf, BM), k, ldx, arena, X, Y, aligned16f(X, ldx) && aligned16f(Y, ldx)};
-    launch(s, dim3((unsigned)((int64_t)n_nodes * op.rt), cdiv(k, BN)), op);
+    launch(s, dim3((unsigned)((int64_t)n_nodes * op.rt), cdiv(k, BN)), op, err);
 }
 
-void schur_tc(cudaStream_t s, const FrontDev &fd, const SchurTask *tasks, int ntasks, int K0, float *arena) {
+void schur_tc(cudaStream_t s, const FrontDev &fd, const SchurTask *tasks, int ntasks, int K0, float *arena, int *err) {
     if (ntasks <= 0) return;
-    launch(s, dim3((unsigned)ntasks), SchurOp{fd, tasks, K0, arena});
+    launch(s, dim3((unsigned)ntasks), SchurOp{fd, tasks, K0, arena}, err);
 }
 
 void gemm_tasks_tc(cudaStream_t s, const GemmTask *tasks, int ntasks, int tiles, const float *Ab, const float *Bb,
-                   float *Cb) {
+                   float *Cb, int *err) {
     if (ntasks <= 0 || tiles <= 0) return;
-    launch(s, dim3((unsigned)tiles), GemmTaskOp{tasks, ntasks, Ab, Bb, Cb});
+    launch(s, dim3((unsigned)tiles), GemmTaskOp{tasks, ntasks, Ab, Bb, Cb}, err);
 }
 
 int gemm_tiles_tc(std::vector<GemmTask> &tasks) {
@@ -444,13 +441,12 @@ int gemm_tiles_tc(std::vector<GemmTask> &tasks) {
     return nt;
 }
 
-void tc32_check(cudaStream_t s) {
+void tc32_check(cudaStream_t s, int *err) {
     int h = 0;
-    HSIM_CUDA(cudaMemcpyFromSymbolAsync(&h, g_tc32_error, sizeof(int), 0, cudaMemcpyDeviceToHost, s));
+    HSIM_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     HSIM_CUDA(cudaStreamSynchronize(s));
     if (h != 0) {
-        const int zero = 0;
-        HSIM_CUDA(cudaMemcpyToSymbolAsync(g_tc32_error, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, s));
+        HSIM_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
         HSIM_CUDA(cudaStreamSynchronize(s));
         fail(HSIM_E_TIMEOUT, "tensor-core FP32 product: an mbarrier wait timed out");
     }

@@ -11,6 +11,11 @@ struct __nv_bfloat16;
 namespace hsim {
 namespace k {
 
+// Words of a context's flag area beyond the counters that a call clears itself (0 to
+// 5): set by a tensor-core product that gave up waiting, zero otherwise.  Each
+// context has its own, so that a check on one stream never takes the error of another.
+constexpr int kErrProducts = 8, kErrTc32 = 9, kFlagWords = 16;
+
 // ---- sparse (k_sparse.cu) -------------------------------------------------
 // per-triangle cotangents and areas from positions or squared lengths
 void triangle_geometry(cudaStream_t s, int m, const int *F, const double *V, const double *L2,
@@ -252,9 +257,9 @@ void solve_bwd_fused(cudaStream_t s, const FrontDev &fd, const int *parents, int
 // TMEM; 128 x 128 output tiles).  The same operations as solve_fwd_inv and
 // gemm_tasks for FP32 fronts.
 void solve_fwd_tc(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_nodes, int max_nf, const float *arena,
-                  int k, float *X, float *Y, int ldx);
+                  int k, float *X, float *Y, int ldx, int *err);
 void gemm_tasks_tc(cudaStream_t s, const GemmTask *tasks, int ntasks, int tiles, const float *Ab, const float *Bb,
-                   float *Cb);
+                   float *Cb, int *err);
 // numbers the tasks' 128 x 128 tiles consecutively (tile0); returns the total
 int gemm_tiles_tc(std::vector<GemmTask> &tasks);
 // Schur-complement update of the blocked FP32 factorisation after a block of
@@ -266,10 +271,10 @@ constexpr int kSchurBlock = 128;
 struct SchurTask {
     int node, m0, n0;
 };
-void schur_tc(cudaStream_t s, const FrontDev &fd, const SchurTask *tasks, int ntasks, int K0, float *arena);
+void schur_tc(cudaStream_t s, const FrontDev &fd, const SchurTask *tasks, int ntasks, int K0, float *arena, int *err);
 // fails with HSIM_E_TIMEOUT (and clears the flag) if a product's bounded
 // mbarrier wait gave up since the last check
-void tc32_check(cudaStream_t s);
+void tc32_check(cudaStream_t s, int *err);
 // inverse of the unit lower 32 x 32 diagonal blocks (t, b0) of the pivot
 // blocks, in place
 template <typename T>
@@ -322,17 +327,17 @@ OzakiOperand ozaki_split_rows(cudaStream_t s, int rows, int k, const double *X, 
 // writes each value and its mirror image (X.rows == Y.rows); accumulate: added
 // to C; skip (device, may be null): 64 x 64 tiles of C that are not wanted
 // (nonzero; skip_ld to a row of tiles), computed or not
-void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, int splits,
+void ozaki_product(cudaStream_t s, const OzakiOperand &X, const OzakiOperand &Y, double *C, int ldc, int splits, int *err,
                    bool lower = false, bool accumulate = false, const int *skip = nullptr, int skip_ld = 0);
 // G (ka x kb, ld ldg) = A^T B over n rows and C (n x m, ld ldc) = A B (A n x k, B
 // k x m), split and multiplied a range of rows at a time so that the digits of
 // one range take about 1 GiB of scratch (256-byte aligned)
 size_t ozaki_gram_scratch(int n, int ka, int kb, int digits);
 void ozaki_gram(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
-                int ldg, int digits, void *scratch);
+                int ldg, int digits, void *scratch, int *err);
 size_t ozaki_update_scratch(int n, int k, int m, int digits);
 void ozaki_update(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
-                  int ldc, int digits, void *scratch);
+                  int ldc, int digits, void *scratch, int *err);
 // gram and gemm_nn in FP64 on seven digits (scratch 512-byte aligned), where the
 // *_on_digits rules say that they are the faster form.  What the digits' result is
 // held to (tiles that could miss it go to the FP64 kernel): Entries, every entry
@@ -343,14 +348,15 @@ enum class Held { Entries, Norms };
 bool gram64_on_digits(int n, int ka, int kb);
 size_t gram64_scratch(int n, int ka, int kb);
 void gram64(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, const double *B, int ldb, double *G,
-            int ldg, bool lower, Held held, void *scratch);
+            int ldg, bool lower, Held held, void *scratch, int *err);
 bool update64_on_digits(int n, int k, int m, bool held);  // held: the scratch is there already
 size_t update64_scratch(int n, int k, int m);
 void update64(cudaStream_t s, int n, int k, int m, const double *A, int lda, const double *B, int ldb, double *C,
-              int ldc, Held held, void *scratch);
-// fails (HSIM_E_INTERNAL) if a tensor-core product kernel gave up waiting on
-// one of its barriers since the last check; synchronises the stream
-void ozaki_check(cudaStream_t s);
+              int ldc, Held held, void *scratch, int *err);
+// Every product takes an error word (device, of the caller's context), set where a
+// kernel gave up waiting on one of its barriers; this fails (HSIM_E_INTERNAL) if the
+// word is set and clears it; synchronises the stream
+void ozaki_check(cudaStream_t s, int *err);
 
 }  // namespace k
 }  // namespace hsim

@@ -92,6 +92,7 @@ struct DevBuf {
         cudaError_t e = cudaMalloc((void **)&p, count * sizeof(T));
         if (e != cudaSuccess) {
             p = nullptr;
+            cudaGetLastError();  // reported here, not by the next launch
             fail(HSIM_E_NOMEM, "cudaMalloc of " + std::to_string(count * sizeof(T)) +
                                    " bytes failed: " + cudaGetErrorString(e));
         }

@@ -211,6 +211,17 @@ struct CtxScratch {
     }
 };
 
+// Scratch of a product on digits, where it fits: null if the device has no room for
+// it (the FP64 kernels need none)
+std::unique_ptr<CtxScratch<unsigned char>> digit_scratch(hsim_ctx *ctx, size_t bytes) {
+    try {
+        return std::make_unique<CtxScratch<unsigned char>>(ctx, bytes);
+    } catch (const Error &e) {
+        if (e.status != HSIM_E_NOMEM) throw;
+        return nullptr;
+    }
+}
+
 }  // namespace
 
 namespace {
@@ -1077,6 +1088,16 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
         // inverse iteration removes it; in automatic mode it is switched on
         // once a level's residual stops decreasing.
         bool refine = o.refine > 0;
+        // FP64 products on digits where the device has room for their scratch
+        auto oz_fits = [&](size_t bytes) {
+            try {
+                H->oz.reserve(bytes);
+                return true;
+            } catch (const Error &e) {
+                if (e.status != HSIM_E_NOMEM) throw;
+                return false;
+            }
+        };
         for (it = 1; it <= o.max_iters; ++it) {
             const int a = q - locked;
             Timer ts(s);
@@ -1157,8 +1178,7 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
                 inf.ms_tc_product += t_prod;
                 ph[2] = t_split + t_prod;
             } else {
-                if (k::gram64_on_digits(n, q, q)) {
-                    H->oz.reserve(k::gram64_scratch(n, q, q));
+                if (k::gram64_on_digits(n, q, q) && oz_fits(k::gram64_scratch(n, q, q))) {
                     k::gram64(s, n, q, q, H->Psi.p, q, H->SP.p, q, H->Sbar.p, q, true, k::Held::Norms, H->oz.p,
                               ctx->err_products());
                     k::gram64(s, n, q, q, H->Psi.p, q, H->MP.p, q, H->Mbar.p, q, true, k::Held::Norms, H->oz.p,
@@ -1188,8 +1208,7 @@ void run_solve(hsim_ctx *ctx, hsim_hier *H, const double *S_val, const double *M
                 const double t_prod = ts.stop();
                 inf.ms_tc_product += t_prod;
                 ph[4] = t_split + t_prod;
-            } else if (k::update64_on_digits(n, q, q, true)) {
-                H->oz.reserve(k::update64_scratch(n, q, q));
+            } else if (k::update64_on_digits(n, q, q, true) && oz_fits(k::update64_scratch(n, q, q))) {
                 k::update64(s, n, q, q, H->Psi.p, q, H->phibar.p, q, H->Phi.p, q, k::Held::Norms, H->oz.p,
                             ctx->err_products());
             } else {
@@ -1746,10 +1765,12 @@ hsim_status hsim_gram(hsim_ctx *ctx, int n, int ka, int kb, const double *A, int
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"G", G}});
         if (k::gram64_on_digits(n, ka, kb)) {
-            CtxScratch<unsigned char> scratch(ctx, k::gram64_scratch(n, ka, kb));
-            k::gram64(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, false, k::Held::Entries, scratch.p, ctx->err_products());
-            k::ozaki_check(ctx->stream, ctx->err_products());
-            return;
+            if (auto scratch = digit_scratch(ctx, k::gram64_scratch(n, ka, kb))) {
+                k::gram64(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, false, k::Held::Entries, scratch->p,
+                          ctx->err_products());
+                k::ozaki_check(ctx->stream, ctx->err_products());
+                return;
+            }
         }
         k::gram(ctx->stream, n, ka, kb, A, lda, B, ldb, G, kb, false);
         HSIM_CUDA(cudaStreamSynchronize(ctx->stream));
@@ -1764,11 +1785,12 @@ hsim_status hsim_gemm_update(hsim_ctx *ctx, int n, int kk, int m, const double *
         DeviceGuard dg(ctx->device);
         check_device_ptrs(ctx->device, {{"A", A}, {"B", B}, {"C", C}});
         if (k::update64_on_digits(n, kk, m, false)) {
-            CtxScratch<unsigned char> scratch(ctx, k::update64_scratch(n, kk, m));
-            k::update64(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc, k::Held::Entries, scratch.p,
-                        ctx->err_products());
-            k::ozaki_check(ctx->stream, ctx->err_products());
-            return;
+            if (auto scratch = digit_scratch(ctx, k::update64_scratch(n, kk, m))) {
+                k::update64(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc, k::Held::Entries, scratch->p,
+                            ctx->err_products());
+                k::ozaki_check(ctx->stream, ctx->err_products());
+                return;
+            }
         }
         k::gemm_nn(ctx->stream, n, kk, m, A, lda, B, ldb, C, ldc);
         HSIM_CUDA(cudaStreamSynchronize(ctx->stream));

@@ -71,6 +71,10 @@ constexpr int kMaxDevices = 64;
         HSIM_CUDA(err_[dev_]);                                                                        \
     } while (0)
 
+// Gives the contexts' unused scratch of the current process back to the devices
+// (hsim.cu); called where an allocation found no room, before it is tried again.
+void release_scratch() noexcept;
+
 // Owning device buffer.
 template <class T>
 struct DevBuf {
@@ -90,6 +94,11 @@ struct DevBuf {
         release();
         if (count == 0) return;
         cudaError_t e = cudaMalloc((void **)&p, count * sizeof(T));
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            release_scratch();
+            e = cudaMalloc((void **)&p, count * sizeof(T));
+        }
         if (e != cudaSuccess) {
             p = nullptr;
             cudaGetLastError();  // reported here, not by the next launch

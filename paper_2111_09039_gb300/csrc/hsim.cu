@@ -100,9 +100,25 @@ void check_device_ptrs(int device, std::initializer_list<std::pair<const char *,
 // 2.5).  A call takes a block for its duration and returns it after its stream
 // has drained; calls of other threads on the same context meanwhile take
 // others.  At most kKeep bytes stay with the context (the largest of the last
-// blocks that fit), and they are given back when an allocation fails and when
-// the context is destroyed.
+// blocks that fit), and they are given back when the context is destroyed and
+// when any allocation of the library, of this context or another one, finds no
+// room (release_scratch, through the list of pools).
+struct ScratchPool;
+struct PoolList {
+    std::mutex mu;
+    std::set<ScratchPool *> pools;
+    static PoolList &get() {
+        static PoolList *list = new PoolList;  // outlives contexts destroyed at exit
+        return *list;
+    }
+};
 struct ScratchPool {
+    ScratchPool() {
+        std::lock_guard<std::mutex> lock(PoolList::get().mu);
+        PoolList::get().pools.insert(this);
+    }
+    ScratchPool(const ScratchPool &) = delete;
+    ScratchPool &operator=(const ScratchPool &) = delete;
     static constexpr size_t kKeep = (size_t)2 << 30;
     static constexpr size_t kBlocks = 16;
     std::mutex mu;
@@ -126,7 +142,7 @@ struct ScratchPool {
         cudaError_t e = cudaMalloc(&p, bytes);
         if (e == cudaErrorMemoryAllocation) {
             cudaGetLastError();
-            drop();
+            hsim::release_scratch();
             e = cudaMalloc(&p, bytes);
         }
         if (e != cudaSuccess) {
@@ -165,8 +181,21 @@ struct ScratchPool {
         for (size_t i = 0; i < used; ++i) cudaFree(free[i].second);
         used = kept = 0;
     }
-    ~ScratchPool() { drop(); }
+    ~ScratchPool() {
+        {
+            std::lock_guard<std::mutex> lock(PoolList::get().mu);
+            PoolList::get().pools.erase(this);
+        }
+        drop();
+    }
 };
+
+namespace hsim {
+void release_scratch() noexcept {
+    std::lock_guard<std::mutex> lock(PoolList::get().mu);
+    for (ScratchPool *p : PoolList::get().pools) p->drop();
+}
+}  // namespace hsim
 
 struct hsim_ctx {
     int device = 0;

@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(256) k_col_sums(int n, int k, int rows, const 
 template <class F>
 void col_sums(cudaStream_t s, int n, int k, const F &f) {
     if (n <= 0 || k <= 0) return;
-    const int rows = (int64_t)n * cdiv(k, 32) >= (int64_t)256 * 8 * 152 ? 256 : 64;
+    const int rows = (int64_t)n * cdiv(k, 32) >= (int64_t)256 * 8 * sm_count() ? 256 : 64;
     k_col_sums<<<cdiv(n, rows) * cdiv(k, 32), 256, 0, s>>>(n, k, rows, f);
     HSIM_LAUNCHED();
 }

@@ -950,15 +950,25 @@ void inv_diag_blocks(cudaStream_t s, const FrontDev &fd, const int2 *blk, int nb
     HSIM_LAUNCHED();
 }
 
+// SMs of the current device (queried per call: a process may drive GPUs of
+// different sizes)
+static int device_sms() {
+    int dev = 0, c = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev);
+    return c > 0 ? c : 1;
+}
+
 template <typename T>
 void gemm_tasks(cudaStream_t s, const GemmTask *tasks, int ntasks, int tiles, const T *Ab, const T *Bb, T *Cb) {
     if (ntasks <= 0 || tiles <= 0) return;
     // FP64: a 64 x 64 tile is 16 instructions of 77 clocks per step and warp; tiles
     // of 32 or 16 rows and columns where those of 64 leave SMs idle (inversion of
     // the factor at n = 1000: 2.6 ms with 64, 0.6 with 16)
-    if (sizeof(T) == 8 && tiles <= 76)
+    const int sms = device_sms();
+    if (sizeof(T) == 8 && tiles <= sms / 2)
         k_gemm_tasks<T, sizeof(T) == 8 ? 16 : kGemmTile><<<dim3(tiles, 16), 256, 0, s>>>(tasks, ntasks, Ab, Bb, Cb);
-    else if (sizeof(T) == 8 && tiles <= 304)
+    else if (sizeof(T) == 8 && tiles <= 2 * sms)
         k_gemm_tasks<T, sizeof(T) == 8 ? 32 : kGemmTile><<<dim3(tiles, 4), 256, 0, s>>>(tasks, ntasks, Ab, Bb, Cb);
     else
         k_gemm_tasks<T, kGemmTile><<<tiles, 256, 0, s>>>(tasks, ntasks, Ab, Bb, Cb);
@@ -1002,15 +1012,6 @@ void launch_bwd_inv(cudaStream_t s, const FrontDev &fd, const int *nodes, int n_
         <<<dim3((unsigned)((int64_t)n_nodes * rt), cdiv(k, inv_cols<T>()), (unsigned)ksplit), 256, sm, s>>>(
             fd, nodes, rt, arena, dinv, k, X, Y, ldx, vec, ksplit);
     HSIM_LAUNCHED();
-}
-
-// SMs of the current device (queried per call: a process may drive GPUs of
-// different sizes)
-int device_sms() {
-    int dev = 0, c = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev);
-    return c > 0 ? c : 1;
 }
 
 // One K step per tile when every front of the height has ns <= 32 (the

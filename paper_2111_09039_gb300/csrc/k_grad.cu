@@ -14,10 +14,13 @@
 // and its part of the loss is E = sum_k t_k D_k / (2 s) - P s / 6 with the edges
 // e_0 = x_2 - x_1, e_1 = x_0 - x_2, e_2 = x_1 - x_0, t_k = -e_{k+1}.e_{k+2} (the
 // corner's u.w), s = |u x w| = 2 A, cot_k = t_k / s.  In the squared lengths l_k
-// = e_k.e_k, t_k = (l_{k+1} + l_{k+2} - l_k) / 2 and ds/dl_k = t_k / (2 s), so
-//     dE/dl_k = (D_{k+1} + D_{k+2} - D_k) / (4 s) + E_s t_k / (2 s),
-//     E_s = -sum_k t_k D_k / (2 s^2) - P / 6,
-// and with G_k = 2 dE/dl_k e_k the corners get G_1 - G_2, G_2 - G_0, G_0 - G_1.
+// = e_k.e_k, t_k = (l_{k+1} + l_{k+2} - l_k) / 2, and with the unit normal N = e_1 x
+// e_2 / s the derivative of s by corner k is N x e_k, so
+//     dE/dx_k = c_{k+1} e_{k+1} - c_{k+2} e_{k+2} + E_s N x e_k,
+//     c_k = (D_{k+1} + D_{k+2} - D_k) / (2 s),  E_s = -sum_k t_k D_k / (2 s^2) - P / 6
+// (and dE/dx_2 = -dE/dx_0 - dE/dx_1).  N x e_k is taken as a cross product: the same
+// vector as the difference (t_{k+1} e_{k+1} - t_{k+2} e_{k+2}) / s has four times the
+// rounding error in a flat obtuse triangle, where the two edges nearly cancel.
 // One thread per triangle; the nine partial derivatives go to the vertices
 // with FP64 atomics (the order of the additions, hence the last bits, vary
 // from run to run).
@@ -41,6 +44,7 @@ struct v3 {
     double x, y, z;
 };
 __device__ __forceinline__ v3 sub(v3 a, v3 b) { return {a.x - b.x, a.y - b.y, a.z - b.z}; }
+__device__ __forceinline__ v3 add(v3 a, v3 b) { return {a.x + b.x, a.y + b.y, a.z + b.z}; }
 __device__ __forceinline__ v3 mul(double s, v3 a) { return {s * a.x, s * a.y, s * a.z}; }
 __device__ __forceinline__ double dot(v3 a, v3 b) { return a.x * b.x + a.y * b.y + a.z * b.z; }
 __device__ __forceinline__ v3 cross(v3 a, v3 b) {
@@ -100,19 +104,18 @@ __global__ void __launch_bounds__(64) k_eig_grad(int m, int p, const double *__r
     }
     const v3 x0 = load(V, c[0]), x1 = load(V, c[1]), x2 = load(V, c[2]);
     const v3 e0 = sub(x2, x1), e1 = sub(x0, x2), e2 = sub(x1, x0);
-    const v3 nrm = cross(e2, e1);  // u x w with the sign left out
+    const v3 nrm = cross(e1, e2);
     const double s = sqrt(dot(nrm, nrm)), inv = 1.0 / s;
     const double t0 = -dot(e1, e2), t1 = -dot(e2, e0), t2 = -dot(e0, e1);
     const double P = Pv[c[0]] + Pv[c[1]] + Pv[c[2]];
     const double N = fma(t0, D0, fma(t1, D1, t2 * D2));
-    // 2 dE/dl_k = ((D_{k+1} + D_{k+2} - D_k) / 2 + E_s t_k) / s
-    const double Es = fma(-0.5 * N * inv, inv, P * (-1.0 / 6.0));
-    const v3 G0 = mul(inv * fma(Es, t0, 0.5 * (D1 + D2 - D0)), e0);
-    const v3 G1 = mul(inv * fma(Es, t1, 0.5 * (D2 + D0 - D1)), e1);
-    const v3 G2 = mul(inv * fma(Es, t2, 0.5 * (D0 + D1 - D2)), e2);
-    atomic_add3(g, c[0], sub(G1, G2));
-    atomic_add3(g, c[1], sub(G2, G0));
-    atomic_add3(g, c[2], sub(G0, G1));
+    const double Es = fma(-0.5 * N * inv, inv, P * (-1.0 / 6.0)), h = 0.5 * inv;
+    const v3 C0 = mul(h * (D1 + D2 - D0), e0), C1 = mul(h * (D2 + D0 - D1), e1), C2 = mul(h * (D0 + D1 - D2), e2);
+    const v3 ns = mul(Es * inv, nrm);
+    const v3 g0 = add(sub(C1, C2), cross(ns, e0)), g1 = add(sub(C2, C0), cross(ns, e1));
+    atomic_add3(g, c[0], g0);
+    atomic_add3(g, c[1], g1);
+    atomic_add3(g, c[2], {-(g0.x + g1.x), -(g0.y + g1.y), -(g0.z + g1.z)});
 }
 
 }  // namespace

@@ -190,15 +190,16 @@ void col_sums(cudaStream_t s, int n, int k, const F &f) {
     HSIM_LAUNCHED();
 }
 
-// FP32 terms (the mixed path's Rayleigh quotients and residual norms): a warp
-// takes 256 rows of 32 columns, a lane a column, its rows added in their order,
-// then one FP64 atomic per column and sum.  The order is part of the result: the
-// quotients' FP32 rounding goes into every correction step, and other partial
-// sums (eight lanes of 8 to 32 rows) moved the eigenvectors of a batch at tol 1e-5
-// by 0.4 to 1.5e-9 where two of them are 10^-5 of their eigenvalue apart, next to a
-// spread between runs of 0.3 to 2e-9.
-// What bounds it: the latency of the loads where the matrices are small (hence 16
-// rows in flight), their bandwidth where they are large.
+// FP32 terms (the mixed path's Rayleigh quotients and residual norms): 256 rows of
+// 32 columns at a time, a lane a column, the rows added in their order, then one
+// FP64 atomic per column and sum.  The order is part of the result: the quotients'
+// FP32 rounding goes into every correction step, and other partial sums (eight
+// lanes of 8 to 32 rows) moved the eigenvectors of a batch at tol 1e-5 by 0.3 to
+// 1.9e-9 where two of them are 10^-5 of their eigenvalue apart, next to a spread
+// between runs of 0.3 to 2e-9.
+// What bounds it: bandwidth where the matrices are large (a warp per block, 16 rows
+// in flight), the latency of the loads where they are small: up to four blocks per
+// SM eight warps load a block's rows, 16 at a time, and one adds them (@CSFIG).
 constexpr int kSeqRows = 256, kSeqBatch = 16;
 template <class F>
 __global__ void __launch_bounds__(128) k_col_sums_seq(int n, int k, const F f) {
@@ -214,15 +215,60 @@ __global__ void __launch_bounds__(128) k_col_sums_seq(int n, int k, const F f) {
 #pragma unroll
     for (int u = 0; u < F::N; ++u) a[u] = A(0);
     const double c = f.column(j);
+    auto add = [&](const typename F::In &in) {
+        float t[F::NP];
+        f.terms(in, c, t);
+        f.add_terms(t, a);
+    };
     int r = (int)r0;
     for (; r + kSeqBatch <= r_end; r += kSeqBatch) {
         typename F::In in[kSeqBatch];
 #pragma unroll
         for (int q = 0; q < kSeqBatch; ++q) in[q] = f.load(r + q, j);
 #pragma unroll
-        for (int q = 0; q < kSeqBatch; ++q) f.add(in[q], c, a);
+        for (int q = 0; q < kSeqBatch; ++q) add(in[q]);
     }
-    for (; r < r_end; ++r) f.add(f.load(r, j), c, a);
+    for (; r < r_end; ++r) add(f.load(r, j));
+#pragma unroll
+    for (int u = 0; u < F::N; ++u) atomicAdd(f.sum(j, u), (double)a[u]);
+}
+
+// the same block by one CTA: its terms meet in shared memory
+template <class F>
+__global__ void __launch_bounds__(256) k_col_sums_block(int n, int k, const F f) {
+    extern __shared__ float terms[];  // [row][F::NP][32]
+    using A = typename F::Acc;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int ncb = (k + 31) / 32, rb = blockIdx.x / ncb, j = (blockIdx.x - rb * ncb) * 32 + lane;
+    const int r0 = rb * kSeqRows, rows = min(kSeqRows, n - r0);
+    const bool live = j < k;
+    const double c = live ? f.column(j) : 0.0;
+    for (int q0 = wid; q0 < rows; q0 += 8 * kSeqBatch) {
+        typename F::In in[kSeqBatch];
+#pragma unroll
+        for (int q = 0; q < kSeqBatch; ++q)
+            if (live && q0 + 8 * q < rows) in[q] = f.load(r0 + q0 + 8 * q, j);
+#pragma unroll
+        for (int q = 0; q < kSeqBatch; ++q)
+            if (live && q0 + 8 * q < rows) {
+                float t[F::NP];
+                f.terms(in[q], c, t);
+#pragma unroll
+                for (int u = 0; u < F::NP; ++u) terms[((q0 + 8 * q) * F::NP + u) * 32 + lane] = t[u];
+            }
+    }
+    __syncthreads();
+    if (wid != 0 || !live) return;
+    A a[F::N];
+#pragma unroll
+    for (int u = 0; u < F::N; ++u) a[u] = A(0);
+#pragma unroll 8
+    for (int r = 0; r < rows; ++r) {
+        float t[F::NP];
+#pragma unroll
+        for (int u = 0; u < F::NP; ++u) t[u] = terms[(r * F::NP + u) * 32 + lane];
+        f.add_terms(t, a);
+    }
 #pragma unroll
     for (int u = 0; u < F::N; ++u) atomicAdd(f.sum(j, u), (double)a[u]);
 }
@@ -230,7 +276,15 @@ __global__ void __launch_bounds__(128) k_col_sums_seq(int n, int k, const F f) {
 template <class F>
 void col_sums_seq(cudaStream_t s, int n, int k, const F &f) {
     if (n <= 0 || k <= 0) return;
-    k_col_sums_seq<<<cdiv((int64_t)cdiv(n, kSeqRows) * cdiv(k, 32), 4), 128, 0, s>>>(n, k, f);
+    const int64_t blocks = (int64_t)cdiv(n, kSeqRows) * cdiv(k, 32);
+    if (blocks <= 4 * sm_count()) {
+        constexpr size_t smem = (size_t)kSeqRows * 32 * F::NP * sizeof(float);
+        HSIM_SMEM_LIMIT_ONCE(k_col_sums_block<F>, smem);
+        k_col_sums_block<<<(unsigned)blocks, 256, smem, s>>>(n, k, f);
+        HSIM_LAUNCHED();
+        return;
+    }
+    k_col_sums_seq<<<cdiv(blocks, 4), 128, 0, s>>>(n, k, f);
     HSIM_LAUNCHED();
 }
 
@@ -277,12 +331,14 @@ struct ResidualSumsMixed {
     __device__ In load(int r, int j) const {
         return {SP[(size_t)r * lds + j], MP[(size_t)r * ldm + j], dinv ? dinv[r] : 1.0};
     }
-    __device__ void add(const In &in, double l, float (&a)[3]) const {
-        const float rr = d2f_trunc(fma(-l, in.m, in.s)), sf = d2f_trunc(in.s), mf = d2f_trunc(in.m);
-        const float w = d2f_trunc(in.w);
-        a[0] = fmaf(w * rr, rr, a[0]);
-        a[1] = fmaf(w * sf, sf, a[1]);
-        a[2] = fmaf(w * mf, mf, a[2]);
+    static constexpr int NP = 4;
+    __device__ void terms(const In &in, double l, float (&t)[4]) const {
+        t[0] = d2f_trunc(fma(-l, in.m, in.s)), t[1] = d2f_trunc(in.s), t[2] = d2f_trunc(in.m), t[3] = d2f_trunc(in.w);
+    }
+    __device__ void add_terms(const float (&t)[4], float (&a)[3]) const {
+        a[0] = fmaf(t[3] * t[0], t[0], a[0]);
+        a[1] = fmaf(t[3] * t[1], t[1], a[1]);
+        a[2] = fmaf(t[3] * t[2], t[2], a[2]);
     }
 };
 
@@ -306,10 +362,13 @@ struct ColDots2Mixed {
     __device__ In load(int r, int j) const {
         return {X[(size_t)r * ldx + j], Y1[(size_t)r * ldy + j], Y2[(size_t)r * ldy + j]};
     }
-    __device__ void add(const In &in, double, float (&a)[2]) const {
-        const float x = d2f_trunc(in.x);
-        a[0] = fmaf(x, d2f_trunc(in.y1), a[0]);
-        a[1] = fmaf(x, d2f_trunc(in.y2), a[1]);
+    static constexpr int NP = 3;
+    __device__ void terms(const In &in, double, float (&t)[3]) const {
+        t[0] = d2f_trunc(in.x), t[1] = d2f_trunc(in.y1), t[2] = d2f_trunc(in.y2);
+    }
+    __device__ void add_terms(const float (&t)[3], float (&a)[2]) const {
+        a[0] = fmaf(t[0], t[1], a[0]);
+        a[1] = fmaf(t[0], t[2], a[1]);
     }
 };
 
@@ -329,10 +388,13 @@ struct ColDots2DiagMixed {
         double x, y, m;
     };
     __device__ In load(int r, int j) const { return {X[(size_t)r * ldx + j], Y1[(size_t)r * ldy + j], m[r]}; }
-    __device__ void add(const In &in, double, float (&a)[2]) const {
-        const float x = d2f_trunc(in.x);
-        a[0] = fmaf(x, d2f_trunc(in.y), a[0]);
-        a[1] = fmaf(d2f_trunc(in.m) * x, x, a[1]);
+    static constexpr int NP = 3;
+    __device__ void terms(const In &in, double, float (&t)[3]) const {
+        t[0] = d2f_trunc(in.x), t[1] = d2f_trunc(in.y), t[2] = d2f_trunc(in.m) * t[0];
+    }
+    __device__ void add_terms(const float (&t)[3], float (&a)[2]) const {
+        a[0] = fmaf(t[0], t[1], a[0]);
+        a[1] = fmaf(t[2], t[0], a[1]);
     }
 };
 

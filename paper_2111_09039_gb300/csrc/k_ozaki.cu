@@ -112,12 +112,23 @@ __device__ __forceinline__ void add_abs(unsigned h, int &ref, float &sum) {
 // per-column exponents of a row-major R x C FP64 block (ex pre-set to kNoExp);
 // SHIFT: of the block whose row r is scaled by 2^rexp[r]; SUMS: sum of |x| added per
 // column.  A CTA takes 64 columns (two per thread, 32 threads) of `rows` rows (eight
-// at a time).  Without SHIFT the upper words decide (three integer instructions an
-// entry where exp_bits takes a dozen; subnormal columns are read again).
+// at a time); blockIdx.z: one of two blocks.  Without SHIFT the upper words decide
+// (three integer instructions an entry where exp_bits takes a dozen; subnormal
+// columns are read again).
+struct ExpsArgs {
+    const double *X;
+    int C, ldx;
+    bool vec;  // rows of 16-byte pairs
+    int *ex;
+    double *sums;
+};
 template <bool SHIFT, bool SUMS>
-__global__ void __launch_bounds__(256) k_col_exps(int R, int C, const double *__restrict__ X, int ldx, int rows,
-                                                  const int *__restrict__ rexp, bool vec, int *__restrict__ ex,
-                                                  double *__restrict__ sums) {
+__global__ void __launch_bounds__(256) k_col_exps(int R, ExpsArgs p0, ExpsArgs p1, int rows, const int *__restrict__ rexp) {
+    const ExpsArgs p = blockIdx.z ? p1 : p0;
+    const double *__restrict__ X = p.X;
+    const int C = p.C, ldx = p.ldx;
+    const bool vec = p.vec;
+    if ((int)blockIdx.y * 64 >= C) return;
     __shared__ int red[8][64];
     __shared__ double reds[SUMS ? 8 : 1][64];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -128,14 +139,14 @@ __global__ void __launch_bounds__(256) k_col_exps(int R, int C, const double *__
     float s0 = 0.f, s1 = 0.f;
 #pragma unroll 4
     for (int r = ra; r < r1; r += 8) {
-        const double *p = X + (size_t)r * ldx + j;
+        const double *x = X + (size_t)r * ldx + j;
         double a = 0.0, b = 0.0;
         if (vec && j + 1 < C) {
-            const double2 v = *reinterpret_cast<const double2 *>(p);
+            const double2 v = *reinterpret_cast<const double2 *>(x);
             a = v.x, b = v.y;
         } else {
-            if (j < C) a = p[0];
-            if (j + 1 < C) b = p[1];
+            if (j < C) a = x[0];
+            if (j + 1 < C) b = x[1];
         }
         if (SHIFT) {
             int ea = exp_bits(a), eb = exp_bits(b);
@@ -177,12 +188,12 @@ __global__ void __launch_bounds__(256) k_col_exps(int R, int C, const double *__
         int m = red[0][threadIdx.x];
 #pragma unroll
         for (int q = 1; q < 8; ++q) m = max(m, red[q][threadIdx.x]);
-        if (m != kNoExp) atomicMax(&ex[blockIdx.y * 64 + threadIdx.x], m);
+        if (m != kNoExp) atomicMax(&p.ex[blockIdx.y * 64 + threadIdx.x], m);
         if (SUMS) {
             double t = reds[0][threadIdx.x];
 #pragma unroll
             for (int q = 1; q < 8; ++q) t += reds[q][threadIdx.x];
-            if (t != 0.0) atomicAdd(&sums[blockIdx.y * 64 + threadIdx.x], t);
+            if (t != 0.0) atomicAdd(&p.sums[blockIdx.y * 64 + threadIdx.x], t);
         }
     }
 }
@@ -370,12 +381,24 @@ __global__ void __launch_bounds__(256) k_split_rows(int R, int K, const double *
 // 6.1 TB/s; a tile per block through registers 0.75 ms, waiting for its loads).
 constexpr int kSplitPitch = 66;                         // doubles: 16-byte rows
 constexpr int kSplitSmem = 3 * 32 * kSplitPitch * 8;    // three tiles
+// blockIdx.z: one of two blocks.
+struct SplitArgs {
+    const double *X;
+    int C, ldx;
+    bool vec;  // rows of 16-byte pairs
+    const int *ex;
+    __nv_bfloat16 *out;
+    int rows_p, rb_log;
+};
 template <int SL>
-__global__ void __launch_bounds__(256, 4) k_split_cols(int K, int C, const double *__restrict__ X, int ldx, bool vec,
-                                                       const int *__restrict__ ex, const int *__restrict__ rexp,
-                                                       __nv_bfloat16 *__restrict__ out, int rows_p, int kp, int rb_log,
-                                                       float *__restrict__ sums, int tiles) {
+__global__ void __launch_bounds__(256, 4) k_split_cols(int K, SplitArgs p0, SplitArgs p1, const int *__restrict__ rexp,
+                                                       int kp, float *__restrict__ sums, int tiles) {
     extern __shared__ __align__(16) double tile[];
+    const SplitArgs p = blockIdx.z ? p1 : p0;
+    const double *__restrict__ X = p.X;
+    const int C = p.C, ldx = p.ldx, rows_p = p.rows_p, rb_log = p.rb_log;
+    const bool vec = p.vec;
+    if ((int)blockIdx.y * 64 >= rows_p) return;
     const int c0 = blockIdx.y * 64, t0 = blockIdx.x * tiles, t1 = min(t0 + tiles, (kp + 31) / 32);
     auto stage = [&](int t) {
         if (t < t1) {
@@ -405,7 +428,7 @@ __global__ void __launch_bounds__(256, 4) k_split_cols(int K, int C, const doubl
     };
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int lc = (lane & 15) + 16 * (wid & 3), kg = (lane >> 4) + 2 * (wid >> 2), r = c0 + lc;
-    const int er = r < C ? ex[r] : kNoExp;
+    const int er = r < C ? p.ex[r] : kNoExp;
     float ss = 0.f;
     stage(t0);
     stage(t0 + 1);
@@ -423,7 +446,7 @@ __global__ void __launch_bounds__(256, 4) k_split_cols(int K, int C, const doubl
             e[u] = er - (rexp && k + u < K ? rexp[k + u] : 0);
         }
         if (r < rows_p && k < kp)
-            split8_store<SL>(v, e, out + tiled_off<SL>(r, k, rows_p >> rb_log, rb_log), (size_t)16 << rb_log);
+            split8_store<SL>(v, e, p.out + tiled_off<SL>(r, k, rows_p >> rb_log, rb_log), (size_t)16 << rb_log);
         if (SL == 1 && sums) {
 #pragma unroll
             for (int u = 0; u < 8; ++u) ss += scaled_abs(v[u], e[u]);
@@ -1296,32 +1319,43 @@ static OzakiOperand make_operand(int rows, int kdim, void *scratch, int digits, 
 
 static int role_log(OzakiRole r) { return r == OzakiRole::X ? 7 : 6; }
 
-static void ozaki_col_exps(cudaStream_t s, int n, int cols, const double *X, int ldx, int *exps, const int *rexp,
-                           double *sums = nullptr) {
-    k_fill_int<<<cdiv(cols, 256), 256, 0, s>>>(cols, kNoExp, exps);
-    HSIM_LAUNCHED();
+// exponents (preset: kNoExp) and, where they are asked for, sums (added) of one or
+// two blocks of n rows
+static void launch_col_exps(cudaStream_t s, int n, const ExpsArgs &a, const ExpsArgs *b, const int *rexp) {
     // rows per CTA: about eight CTAs per SM, 32 to 1024 rows
-    const int64_t cb = cdiv(cols, 64), want = std::max<int64_t>(1, 8 * (int64_t)sm_count_oz() / cb);
+    const int64_t ca = cdiv(a.C, 64), cb = b ? cdiv(b->C, 64) : 0;
+    const int64_t want = std::max<int64_t>(1, 8 * (int64_t)sm_count_oz() / (ca + cb));
     const int rows = (int)std::min<int64_t>(1024, std::max<int64_t>(32, round_up((int)cdiv(n, want), 8)));
-    const dim3 g(cdiv(n, rows), (unsigned)cb);
-    auto go = [&](auto kernel) { kernel<<<g, 256, 0, s>>>(n, cols, X, ldx, rows, rexp, pair_rows(X, ldx), exps, sums); };
+    const dim3 g(cdiv(n, rows), (unsigned)std::max(ca, cb), b ? 2 : 1);
+    auto go = [&](auto kernel) { kernel<<<g, 256, 0, s>>>(n, a, b ? *b : a, rows, rexp); };
     if (rexp) go(k_col_exps<true, false>);
-    else if (sums) go(k_col_exps<false, true>);
+    else if (a.sums) go(k_col_exps<false, true>);
     else go(k_col_exps<false, false>);
     HSIM_LAUNCHED();
 }
 
+static void ozaki_col_exps(cudaStream_t s, int n, int cols, const double *X, int ldx, int *exps, const int *rexp,
+                           double *sums = nullptr) {
+    k_fill_int<<<cdiv(cols, 256), 256, 0, s>>>(cols, kNoExp, exps);
+    HSIM_LAUNCHED();
+    launch_col_exps(s, n, {X, cols, ldx, pair_rows(X, ldx), exps, sums}, nullptr, rexp);
+}
+
+// n rows of X (and of X2 into op2, of the same K and digits)
 static void split_cols_into(cudaStream_t s, const OzakiOperand &op, int n, const double *X, int ldx, const int *rexp,
-                            float *sums = nullptr) {
+                            float *sums = nullptr, const OzakiOperand *op2 = nullptr, const double *X2 = nullptr,
+                            int ldx2 = 0) {
+    auto args = [](const OzakiOperand &o, const double *x, int ld) {
+        return SplitArgs{x, o.rows, ld, pair_rows(x, ld), o.exps, o.slices, o.rows_p, role_log(o.role)};
+    };
+    const SplitArgs a = args(op, X, ldx), b = op2 ? args(*op2, X2, ldx2) : a;
     // four blocks per SM (shared memory), each with up to eight tiles
-    const int nt = cdiv(op.kp, 32), ncb = cdiv(op.rows_p, 64);
-    const int tiles = (int)std::max<int64_t>(1, std::min<int64_t>(8, (int64_t)nt * ncb / (4 * (int64_t)sm_count_oz())));
-    const dim3 g(cdiv(nt, tiles), ncb);
-    const bool vec = pair_rows(X, ldx);
-    const int rl = role_log(op.role);
+    const int nt = cdiv(op.kp, 32), ca = cdiv(a.rows_p, 64), cb = op2 ? cdiv(b.rows_p, 64) : 0;
+    const int tiles =
+        (int)std::max<int64_t>(1, std::min<int64_t>(8, (int64_t)nt * (ca + cb) / (4 * (int64_t)sm_count_oz())));
+    const dim3 g(cdiv(nt, tiles), std::max(ca, cb), op2 ? 2 : 1);
     auto go = [&](auto kernel) {
-        kernel<<<g, 256, kSplitSmem, s>>>(n, op.rows, X, ldx, vec, op.exps, rexp, op.slices, op.rows_p, op.kp, rl, sums,
-                                          tiles);
+        kernel<<<g, 256, kSplitSmem, s>>>(n, a, b, rexp, op.kp, sums, tiles);
         HSIM_LAUNCHED();
     };
     if (op.digits == 5) {
@@ -1482,8 +1516,10 @@ void ozaki_gram(cudaStream_t s, int n, int ka, int kb, const double *A, int lda,
     int *ey = ex + exps_bytes(ka) / sizeof(int);
     unsigned char *sx = reinterpret_cast<unsigned char *>(ey) + exps_bytes(kb);
     unsigned char *sy = sx + operand_bytes(ka, std::min(range, n), digits);
-    ozaki_col_exps(s, n, ka, A, lda, ex, nullptr);
-    ozaki_col_exps(s, n, kb, B, ldb, ey, nullptr);
+    k_fill_int<<<cdiv((ey - ex) + kb, 256), 256, 0, s>>>((int)(ey - ex) + kb, kNoExp, ex);
+    HSIM_LAUNCHED();
+    const ExpsArgs ea{A, ka, lda, pair_rows(A, lda), ex, nullptr}, eb{B, kb, ldb, pair_rows(B, ldb), ey, nullptr};
+    launch_col_exps(s, n, ea, &eb, nullptr);
     const bool several = n > range;
     if (several) HSIM_CUDA(cudaMemset2DAsync(G, (size_t)ldg * sizeof(double), 0, (size_t)kb * sizeof(double), ka, s));
     for (int r0 = 0; r0 < n; r0 += range) {
@@ -1491,8 +1527,7 @@ void ozaki_gram(cudaStream_t s, int n, int ka, int kb, const double *A, int lda,
         OzakiOperand X = make_operand(ka, rows, sx, digits, OzakiRole::X), Y = make_operand(kb, rows, sy, digits, OzakiRole::Y);
         X.exps = ex;
         Y.exps = ey;
-        split_cols_into(s, X, rows, A + (size_t)r0 * lda, lda, nullptr);
-        split_cols_into(s, Y, rows, B + (size_t)r0 * ldb, ldb, nullptr);
+        split_cols_into(s, X, rows, A + (size_t)r0 * lda, lda, nullptr, nullptr, &Y, B + (size_t)r0 * ldb, ldb);
         ozaki_product(s, X, Y, G, ldg, 0, err, false, several);
     }
 }
@@ -1610,7 +1645,7 @@ struct Gram64 {
     double *sx, *sy;
     float *h;
     unsigned char *dx, *dy;
-    size_t zero_bytes, bytes;  // tiles to sy; all of it
+    size_t zero_bytes, bytes;  // tiles to h; all of it
     Gram64(int n, int ka, int kb, int lda, int ldb, void *scratch) {
         Pieces q{static_cast<unsigned char *>(scratch)};
         range = std::min(gram_rows(n, ka, kb, kDigits64), n);
@@ -1620,10 +1655,10 @@ struct Gram64 {
         tiles = q.take<int>((size_t)tile_rows(ka) * tile_cols(kb));
         sx = q.take<double>(ka);
         sy = q.take<double>(kb);
+        h = q.take<float>((size_t)ka * kb);
         zero_bytes = q.used;
         ex = q.take<int>(ka);
         ey = q.take<int>(kb);
-        h = q.take<float>((size_t)ka * kb);
         dx = q.take<unsigned char>(std::max(operand_bytes(ka, range, kDigits64), operand_bytes(ka, mag_range, 1)));
         dy = q.take<unsigned char>(std::max(operand_bytes(kb, range, kDigits64), operand_bytes(kb, mag_range, 1)));
         bytes = q.used;
@@ -1666,12 +1701,13 @@ void gram64(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, con
     const int tm = tile_rows(ka), tn = tile_cols(kb);
     HSIM_CUDA(cudaMemsetAsync(g.tiles, 0, g.zero_bytes, s));
     const bool same = A == B && ka == kb && lda == ldb;
-    ozaki_col_exps(s, n, ka, A, lda, g.ex, nullptr, g.sx);
+    k_fill_int<<<cdiv((g.ey - g.ex) + kb, 256), 256, 0, s>>>((int)(g.ey - g.ex) + kb, kNoExp, g.ex);
+    HSIM_LAUNCHED();
+    const ExpsArgs ea{A, ka, lda, pair_rows(A, lda), g.ex, g.sx}, eb{B, kb, ldb, pair_rows(B, ldb), g.ey, g.sy};
+    launch_col_exps(s, n, ea, same ? nullptr : &eb, nullptr);
     if (same) {
         HSIM_CUDA(cudaMemcpyAsync(g.ey, g.ex, (size_t)ka * sizeof(int), cudaMemcpyDeviceToDevice, s));
         HSIM_CUDA(cudaMemcpyAsync(g.sy, g.sx, (size_t)ka * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    } else {
-        ozaki_col_exps(s, n, kb, B, ldb, g.ey, nullptr, g.sy);
     }
     auto operands = [&](int rows, int digits, OzakiOperand &X, OzakiOperand &Y, const double *a, int la, const double *b,
                         int lb) {
@@ -1679,12 +1715,10 @@ void gram64(cudaStream_t s, int n, int ka, int kb, const double *A, int lda, con
         Y = make_operand(kb, rows, g.dy, digits, OzakiRole::Y);
         X.exps = g.ex;
         Y.exps = g.ey;
-        split_cols_into(s, X, rows, a, la, nullptr);
-        split_cols_into(s, Y, rows, b, lb, nullptr);
+        split_cols_into(s, X, rows, a, la, nullptr, nullptr, &Y, b, lb);
     };
     OzakiOperand X, Y;
     if (held == Held::Entries) {
-        HSIM_CUDA(cudaMemsetAsync(g.h, 0, (size_t)ka * kb * sizeof(float), s));
         MagCheck chk{};
         chk.h = g.h;
         for (int r0 = 0; r0 < g.sampled; r0 += g.mag_range) {

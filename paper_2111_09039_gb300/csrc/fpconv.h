@@ -6,8 +6,8 @@
 // every input: a conversion instruction on a rare path is predicated by the
 // compiler and takes its 77 clocks of the FP64 pipe per warp whether any lane
 // needs it or not (250,000 x 720 Rayleigh quotients with three conversions per
-// entry: 1.00 ms, 0.73 ms without; residual sums of 250,000 x 500
-// 1.18 and 0.45 ms; FP32 residuals with diagonal M 1.05 and 0.69 ms).
+// entry: 1.00 ms, 0.73 ms without, in the sums' form of that time; residual sums of
+// 250,000 x 500 1.18 and 0.45 ms; FP32 residuals with diagonal M 1.05 and 0.69 ms).
 #pragma once
 
 #include <cuda_runtime.h>

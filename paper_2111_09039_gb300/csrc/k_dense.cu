@@ -197,10 +197,14 @@ void col_sums(cudaStream_t s, int n, int k, const F &f) {
 // lanes of 8 to 32 rows) moved the eigenvectors of a batch at tol 1e-5 by 0.3 to
 // 1.9e-9 where two of them are 10^-5 of their eigenvalue apart, next to a spread
 // between runs of 0.3 to 2e-9.
-// What bounds it: bandwidth where the matrices are large (a warp per block, 16 rows
-// in flight), the latency of the loads where they are small: up to four blocks per
-// SM eight warps load a block's rows, 16 at a time, and one adds them (@CSFIG).
-constexpr int kSeqRows = 256, kSeqBatch = 16;
+// What bounds it: instructions, 75 per row of a block (three conversions on the
+// bits), and with them bandwidth where the matrices are large: a warp per block,
+// eight rows in flight (residual sums of 250,000 x 500 0.40 ms, quotients of 750
+// columns 0.44; with row lanes 0.45 and 0.76).  Up to eight blocks per SM there are
+// too few warps for that, and 32 of them load and convert a block's rows and one adds
+// them: 10 us per wave of a block per SM (residual sums of 19,800 x 50 21 us, 18
+// with row lanes; of 15,811 x 500 65, 78 with a warp per block).
+constexpr int kSeqRows = 256;
 template <class F>
 __global__ void __launch_bounds__(128) k_col_sums_seq(int n, int k, const F f) {
     using A = typename F::Acc;
@@ -218,44 +222,49 @@ __global__ void __launch_bounds__(128) k_col_sums_seq(int n, int k, const F f) {
     auto add = [&](const typename F::In &in) {
         float t[F::NP];
         f.terms(in, c, t);
-        f.add_terms(t, a);
+        f.add_terms(t, f.row_term(in), a);
     };
     int r = (int)r0;
-    for (; r + kSeqBatch <= r_end; r += kSeqBatch) {
-        typename F::In in[kSeqBatch];
+    constexpr int U = 8;
+    for (; r + U <= r_end; r += U) {
+        typename F::In in[U];
 #pragma unroll
-        for (int q = 0; q < kSeqBatch; ++q) in[q] = f.load(r + q, j);
+        for (int q = 0; q < U; ++q) in[q] = f.load(r + q, j);
 #pragma unroll
-        for (int q = 0; q < kSeqBatch; ++q) add(in[q]);
+        for (int q = 0; q < U; ++q) add(in[q]);
     }
     for (; r < r_end; ++r) add(f.load(r, j));
 #pragma unroll
     for (int u = 0; u < F::N; ++u) atomicAdd(f.sum(j, u), (double)a[u]);
 }
 
-// the same block by one CTA: its terms meet in shared memory
+// the same block by one CTA of 32 warps, eight rows each: its terms meet in shared
+// memory and the first warp adds them
+constexpr int kBlockThreads = 1024, kWarpRows = kSeqRows / (kBlockThreads / 32);
 template <class F>
-__global__ void __launch_bounds__(256) k_col_sums_block(int n, int k, const F f) {
-    extern __shared__ float terms[];  // [row][F::NP][32]
+__global__ void __launch_bounds__(kBlockThreads, 1) k_col_sums_block(int n, int k, const F f) {
+    extern __shared__ float terms[];  // [row][F::NP][32], [row]
+    float *row_terms = terms + kSeqRows * F::NP * 32;
     using A = typename F::Acc;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int ncb = (k + 31) / 32, rb = blockIdx.x / ncb, j = (blockIdx.x - rb * ncb) * 32 + lane;
     const int r0 = rb * kSeqRows, rows = min(kSeqRows, n - r0);
     const bool live = j < k;
     const double c = live ? f.column(j) : 0.0;
-    for (int q0 = wid; q0 < rows; q0 += 8 * kSeqBatch) {
-        typename F::In in[kSeqBatch];
+    typename F::In in[kWarpRows];
 #pragma unroll
-        for (int q = 0; q < kSeqBatch; ++q)
-            if (live && q0 + 8 * q < rows) in[q] = f.load(r0 + q0 + 8 * q, j);
+    for (int q = 0; q < kWarpRows; ++q)
+        if (live && wid + 32 * q < rows) in[q] = f.load(r0 + wid + 32 * q, j);
 #pragma unroll
-        for (int q = 0; q < kSeqBatch; ++q)
-            if (live && q0 + 8 * q < rows) {
-                float t[F::NP];
-                f.terms(in[q], c, t);
+    for (int q = 0; q < kWarpRows; ++q) {
+        const int r = wid + 32 * q;
+        if (live && r < rows) {
+            float t[F::NP];
+            f.terms(in[q], c, t);
 #pragma unroll
-                for (int u = 0; u < F::NP; ++u) terms[((q0 + 8 * q) * F::NP + u) * 32 + lane] = t[u];
-            }
+            for (int u = 0; u < F::NP; ++u) terms[(r * F::NP + u) * 32 + lane] = t[u];
+            if (lane == 0) row_terms[r] = f.row_term(in[q]);
+        }
     }
     __syncthreads();
     if (wid != 0 || !live) return;
@@ -267,7 +276,7 @@ __global__ void __launch_bounds__(256) k_col_sums_block(int n, int k, const F f)
         float t[F::NP];
 #pragma unroll
         for (int u = 0; u < F::NP; ++u) t[u] = terms[(r * F::NP + u) * 32 + lane];
-        f.add_terms(t, a);
+        f.add_terms(t, row_terms[r], a);
     }
 #pragma unroll
     for (int u = 0; u < F::N; ++u) atomicAdd(f.sum(j, u), (double)a[u]);
@@ -277,10 +286,10 @@ template <class F>
 void col_sums_seq(cudaStream_t s, int n, int k, const F &f) {
     if (n <= 0 || k <= 0) return;
     const int64_t blocks = (int64_t)cdiv(n, kSeqRows) * cdiv(k, 32);
-    if (blocks <= 4 * sm_count()) {
-        constexpr size_t smem = (size_t)kSeqRows * 32 * F::NP * sizeof(float);
+    if (blocks <= 8 * sm_count()) {
+        constexpr size_t smem = (size_t)kSeqRows * (32 * F::NP + 1) * sizeof(float);
         HSIM_SMEM_LIMIT_ONCE(k_col_sums_block<F>, smem);
-        k_col_sums_block<<<(unsigned)blocks, 256, smem, s>>>(n, k, f);
+        k_col_sums_block<<<(unsigned)blocks, kBlockThreads, smem, s>>>(n, k, f);
         HSIM_LAUNCHED();
         return;
     }
@@ -331,14 +340,15 @@ struct ResidualSumsMixed {
     __device__ In load(int r, int j) const {
         return {SP[(size_t)r * lds + j], MP[(size_t)r * ldm + j], dinv ? dinv[r] : 1.0};
     }
-    static constexpr int NP = 4;
-    __device__ void terms(const In &in, double l, float (&t)[4]) const {
-        t[0] = d2f_trunc(fma(-l, in.m, in.s)), t[1] = d2f_trunc(in.s), t[2] = d2f_trunc(in.m), t[3] = d2f_trunc(in.w);
+    static constexpr int NP = 3;
+    __device__ void terms(const In &in, double l, float (&t)[3]) const {
+        t[0] = d2f_trunc(fma(-l, in.m, in.s)), t[1] = d2f_trunc(in.s), t[2] = d2f_trunc(in.m);
     }
-    __device__ void add_terms(const float (&t)[4], float (&a)[3]) const {
-        a[0] = fmaf(t[3] * t[0], t[0], a[0]);
-        a[1] = fmaf(t[3] * t[1], t[1], a[1]);
-        a[2] = fmaf(t[3] * t[2], t[2], a[2]);
+    __device__ float row_term(const In &in) const { return d2f_trunc(in.w); }
+    __device__ void add_terms(const float (&t)[3], float w, float (&a)[3]) const {
+        a[0] = fmaf(w * t[0], t[0], a[0]);
+        a[1] = fmaf(w * t[1], t[1], a[1]);
+        a[2] = fmaf(w * t[2], t[2], a[2]);
     }
 };
 
@@ -366,7 +376,8 @@ struct ColDots2Mixed {
     __device__ void terms(const In &in, double, float (&t)[3]) const {
         t[0] = d2f_trunc(in.x), t[1] = d2f_trunc(in.y1), t[2] = d2f_trunc(in.y2);
     }
-    __device__ void add_terms(const float (&t)[3], float (&a)[2]) const {
+    __device__ float row_term(const In &) const { return 0.f; }
+    __device__ void add_terms(const float (&t)[3], float, float (&a)[2]) const {
         a[0] = fmaf(t[0], t[1], a[0]);
         a[1] = fmaf(t[0], t[2], a[1]);
     }
@@ -392,7 +403,8 @@ struct ColDots2DiagMixed {
     __device__ void terms(const In &in, double, float (&t)[3]) const {
         t[0] = d2f_trunc(in.x), t[1] = d2f_trunc(in.y), t[2] = d2f_trunc(in.m) * t[0];
     }
-    __device__ void add_terms(const float (&t)[3], float (&a)[2]) const {
+    __device__ float row_term(const In &) const { return 0.f; }
+    __device__ void add_terms(const float (&t)[3], float, float (&a)[2]) const {
         a[0] = fmaf(t[0], t[1], a[0]);
         a[1] = fmaf(t[2], t[0], a[1]);
     }

@@ -99,6 +99,15 @@ def test_gram_outlier(hs, ctx, n):
     check(on_digits(hs, lambda: hs.gram(ctx, dev(A), dev(B))), A, B)
 
 
+@pytest.mark.parametrize("n,k", [(1024, 33), (20000, 70)])
+def test_gram_of_one_block(hs, ctx, n, k):
+    """Both operands the same buffer: exponents and sums are taken once."""
+    A = np.random.default_rng(n).standard_normal((n, k))
+    A[n // 3, k // 2] = 1e9
+    dA = dev(A)
+    check(on_digits(hs, lambda: hs.gram(ctx, dA, dA)), A, A)
+
+
 # one row, tiles of 128 and 64 and their remainders, K steps of 16, two row ranges
 # (16 k bytes of digits to a row, 1 GiB to a range)
 SHAPES = [(1, 200, 20000), (127, 170, 130), (129, 177, 129), (1024, 165, 63), (4097, 200, 65), (70003, 41, 63),

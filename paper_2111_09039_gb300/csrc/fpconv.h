@@ -1,10 +1,11 @@
 // Device helpers for the element-wise kernels on n x k blocks.
 //
-// FP64 instructions issue at a 64th of the FP32 rate on this GPU, and the
-// FP64 <-> FP32 conversion instructions are not free either, so conversions
+// FP64 instructions issue at a 64th of the FP32 rate on this GPU (a warp's takes 64
+// clocks of its sub-partition alone, 76 where all four issue FMAs back to back, 69 in
+// S X), and the FP64 <-> FP32 conversion instructions are not free either, so conversions
 // on the hot blocks are done on the bit patterns with integer operations, for
 // every input: a conversion instruction on a rare path is predicated by the
-// compiler and takes its 77 clocks of the FP64 pipe per warp whether any lane
+// compiler and takes its 64 to 76 clocks of the FP64 pipe per warp whether any lane
 // needs it or not (250,000 x 720 Rayleigh quotients with three conversions per
 // entry: 1.00 ms, 0.73 ms without, in the sums' form of that time; residual sums of
 // 250,000 x 500 1.18 and 0.45 ms; FP32 residuals with diagonal M 1.05 and 0.69 ms).

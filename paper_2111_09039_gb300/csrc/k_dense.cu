@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(256) k_gemm_nn(int n, int kk, int m, const T *
 //
 // FP64 terms: a CTA takes `rows` rows of 32 columns, warp w the rows w, w + 8, ...,
 // a lane a column; the eight partial sums meet in shared memory, then one FP64
-// atomic per column and sum (an FP64 instruction of a warp takes 77 clocks, so a
+// atomic per column and sum (an FP64 instruction of a warp takes 64 to 76 clocks, so a
 // block of rows is spread over the sub-partitions).
 template <class F>
 __global__ void __launch_bounds__(256) k_col_sums(int n, int k, int rows, const F f) {

@@ -962,7 +962,7 @@ static int device_sms() {
 template <typename T>
 void gemm_tasks(cudaStream_t s, const GemmTask *tasks, int ntasks, int tiles, const T *Ab, const T *Bb, T *Cb) {
     if (ntasks <= 0 || tiles <= 0) return;
-    // FP64: a 64 x 64 tile is 16 instructions of 77 clocks per step and warp; tiles
+    // FP64: a 64 x 64 tile is 16 instructions of 64 to 76 clocks per step and warp; tiles
     // of 32 or 16 rows and columns where those of 64 leave SMs idle (inversion of
     // the factor at n = 1000: 2.6 ms with 64, 0.6 with 16)
     const int sms = device_sms();

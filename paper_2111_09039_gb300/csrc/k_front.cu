@@ -11,7 +11,7 @@
 //            back in place; FP64 fronts keep the inverse of its unit lower
 //            factor there, which turns every triangle of the panel and of the
 //            solves into a product (a triangle of 32 is a chain of 496
-//            dependent FP64 instructions of 77 clocks, whatever the width);
+//            dependent FP64 instructions of 64 clocks and more, whatever the width);
 //   panel:   L21 = A21 L11^-T D^-1;
 //   update:  A22 -= L21 D L21^T on lower-triangular tiles;
 // and the children's update blocks are added into the parent front
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(128) k_front_panel(FrontDev fd, const int *__r
 // I] without the part above the diagonal).  Lane r of every warp holds row r,
 // warp w the columns w, w + 4, ... of the block and of the inverse, so a pivot
 // step is up to 8 + 8 FP64 instructions per warp, one warp per SM sub-partition,
-// around a chain of reciprocal, product and update.  32 pivots take 26 us;
+// around a chain of reciprocal, product and update.  32 pivots take 28 us;
 // with the block in shared memory, three barriers a pivot and a division per
 // entry they took 36.6, without the inverse.  (A correction step on the quotients
 // of l and of the panel left the solves' error as it was.)
@@ -377,7 +377,7 @@ __global__ void k_front_maxdiag(FrontDev fd, const T *__restrict__ arena, unsign
 // ---- FP64 solves (FP32 factors are solved in the inverted form, k_finv.cu) -----
 // Every diagonal block holds the inverse of its unit lower factor (k_front_diag_inv),
 // so the triangles are products; tiles are small where a height has few fronts
-// (an SM's FP64 pipes take 1.67 lanes per clock: 64 x 64 x 32 products keep one
+// (an SM's FP64 pipes take 1.7 to 1.9 lanes per clock: 64 x 64 x 32 products keep one
 // SM busy for 38 us while others idle).
 
 // Li[r][c] = the inverse block (rows and columns beyond kb: identity)

@@ -25,9 +25,9 @@
 // with FP64 atomics (the order of the additions, hence the last bits, vary
 // from run to run).
 //
-// What bounds it: FP64 instructions (1.67 lanes per clock and SM), nine per
-// triangle and eigenpair, two per vertex and eigenpair and about 90 per
-// triangle: 80,000 triangles x 50 pairs take 90 + 12 us, where fourteen (P per triangle)
+// What bounds it: FP64 instructions (1.7 to 1.9 lanes per clock and SM), nine per
+// triangle and eigenpair, two per vertex and eigenpair and about 100 per
+// triangle: 80,000 triangles x 50 pairs take 93 + 12 us, where fourteen (P per triangle)
 // and the derivatives of the three cotangents one by one took 206 us.  CTAs of 64
 // threads spread 1,250 over 152 SMs evenly; of 256 threads 313 left a third of
 // them a CTA behind.

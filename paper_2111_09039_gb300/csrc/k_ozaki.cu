@@ -40,7 +40,7 @@ constexpr int kBadExp = 1 << 20;  // the same in a block whose rows or columns a
 inline unsigned cdiv(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
 // Exponents and digits are taken from the bits of the FP64 values with integer
-// arithmetic only (the FP64 pipe of this part is ~1/60 of the FP32 pipe).
+// arithmetic only (the FP64 pipe of this part is a 64th of the FP32 pipe).
 //
 // smallest e with |x| < 2^e for a nonzero x: biased exponent - 1022 (subnormals
 // by their leading bit); kNoExp for zero
@@ -492,10 +492,15 @@ int sm_count_oz() {
 //
 // Exactness: a digit product is at most 2^14 in magnitude, and the sum for D
 // takes D + 1 pairs per K row, so after kChunk = 256 rows the sums for D <= 3
-// are below 2^24 and exact in FP32.  The sums for D >= 4 carry a weight of
-// 2^-32 and less; they pass 2^24 only when hundreds of same-signed full-size
-// digits meet, and then lose one unit of 2^-32 per chunk next to a D = 0 sum of
-// 2^22.  Every chunk is drained into FP32 expansions in registers.
+// are at most 2^24 and exact in FP32.  A sum for D >= 4 (weight 2^-32 and less)
+// can pass 2^24, and each MMA after that may round it by a unit.  For D = 4 and 5
+// that takes digits of one sign and nearly full size in all D + 1 pairs, those of the
+// leading digits among them: four pairs alone stay within 2^24.  With the leading
+// digit of the smaller factor at r of its full size, at most r / 4 of the chunk's
+// 80 (D = 4) MMAs come after, 20 r units of 2^-46 of the maxima's product next to
+// 190 r of that product in sum |x| |y|: 2^-49 of it at the worst.  From D = 6 on the
+// units weigh 2^-62 and less.  Every chunk is drained into FP32 expansions in
+// registers.
 //
 // The drain stops the tensor cores briefly: the accumulators of the highest D
 // (three of five digits' sums, two of six digits') have two sets of TMEM
@@ -517,8 +522,8 @@ int sm_count_oz() {
 // Warp roles (320 threads): warp 0 issues the loads, warp 1 owns TMEM and
 // issues the MMAs (one thread), warps 2..9 drain, one TMEM lane (output row)
 // and 32 of the 64 columns per thread, and write the item's results while the
-// MMAs of the next item run.  Every mbarrier wait gives up after 2 s, records
-// that in the caller's error word, which the host checks, and the CTA still drains its own copies
+// MMAs of the next item run.  Every mbarrier wait gives up after 2 s, records that
+// in the caller's error word, which the host checks, and the CTA still drains its own copies
 // and MMAs and frees its TMEM.
 // ------------------------------------------------------------------------------
 constexpr int TC_M = 128, TC_N = 64, TC_K = 16;
@@ -1106,7 +1111,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 // accumulators.  Either h is added to chk.h (ld N), or it is checked against the
 // sums of the rows' and columns' magnitudes and the tiles that fail are marked.
 // What bounds it: the loads.  Update of 163,842 x 300 x 300 (98 MB of magnitudes):
-// @MAGUPD us; as one-block items with a stage per K step 205.  Roles, waits and
+// 57 us; as one-block items with a stage per K step 205.  Roles, waits and
 // teardown as k_ozaki_tc's.
 constexpr int kMagSteps = 4, kMagBlocks = 4, kMagStages = 4;
 constexpr uint32_t kMagA = 2u * TC_M * TC_K, kMagB = 2u * TC_N * TC_K;  // bytes per K step and block
@@ -1564,12 +1569,19 @@ void ozaki_update(cudaStream_t s, int n, int k, int m, const double *A, int lda,
 // exactly, so that their mean magnitudes meet (means: one large entry must not move
 // the scale of the others).
 //
+// What the check costs (calls with a wait, without and with it): Gram 163,842 x 300
+// 1,407 and 1,445 us, 1,024 x 300 110 and 120; update 163,842 x 300 1,124 and 1,172,
+// 1,024 x 165 97 and 111.  Inputs that it sends to the FP64 kernel pay for it there:
+// a Gram of 16,384 x 75 530 -> 670, of 163,842 x 300 28,000 to 33,000 with every row
+// of tiles flagged, 14,900 with one column.
+//
 // Where the line lies (us, FP64 kernel / digits, calls with a wait): Gram 1,024
-// rows x 30 to 300 columns 281 / 73 to 283 / 81, 16,384 x 75 530 / 101, 163,842 x
-// 300 36,600 / 1,473; fewer rows than 1,024 are left to the FP64 kernel (its time
+// rows x 30 to 300 columns 281 / 100 to 283 / 120, 16,384 x 75 530 / 139, 163,842 x
+// 300 33,000 / 1,445; fewer rows than 1,024 are left to the FP64 kernel (its time
 // falls with them, and the rule on standing-out entries has no room).  Update
 // with k = 30 44 / 57 to 8,192 rows and 75 / 60 at 16,384, k = 50 77 / 55 from
-// 1,024 rows on, 163,842 x 300 25,700 / 1,049.  A context's first call also
+// 1,024 rows on (the solve's form, without the check), 163,842 x 300 25,700 / 1,172.
+// A context's first call also
 // allocates the scratch, about 140 us: where the scratch is not held by the caller
 // an update takes the digits only if the FP64 kernel is slower than both (about 1.5
 // us per inner term when it waits for its chain, 1.1 TFLOP/s otherwise; 15,923 x 36
@@ -1589,11 +1601,13 @@ namespace {
 // Powers of two c_k: half the gap between the mean magnitudes of column k of A (sum
 // over n rows) and row k of B (sum in units of 2^eb over m columns), less the mean
 // gap of all k (a common factor does nothing); below 1.5 left at 0, so that pairs
-// alike are not told apart by rounding.  One CTA; zeros and infinities: 0.
+// alike are not told apart by rounding.  One CTA; zeros and infinities: 0.  ey (m):
+// preset for k_col_exps.
 __global__ void __launch_bounds__(256) k_balance(int k, int n, int m, const double *__restrict__ suma,
                                                  const int *__restrict__ eb, const float *__restrict__ sumb,
-                                                 int *__restrict__ c) {
+                                                 int *__restrict__ c, int *__restrict__ ey) {
     __shared__ float red[2][8];
+    for (int j = threadIdx.x; j < m; j += 256) ey[j] = kNoExp;
     auto log2_of = [](double x, float &l) {
         const int h = __double2hiint(x), e = (h >> 20) & 0x7FF;
         l = (float)(e - 1023) + __log2f(__int_as_float(0x3F800000 | ((h & 0xFFFFF) << 3)));
@@ -1748,15 +1762,16 @@ void update64(cudaStream_t s, int n, int k, int m, const double *A, int lda, con
     const Update64 u(n, k, m, scratch);
     const int tn = tile_cols(m);
     HSIM_CUDA(cudaMemsetAsync(u.tiles, 0, u.zero_bytes, s));
-    // means over part of the rows: they only set the scale
+    // means over part of the rows: they only set the scale (the maxima beside them, in
+    // cexp, are not used)
     const int step = sample_step(n, lda), sampled = (int)cdiv(n, step);
-    ozaki_col_exps(s, sampled, k, A, lda * step, u.cexp, nullptr, u.suma);
+    launch_col_exps(s, sampled, {A, k, lda * step, pair_rows(A, lda * step), u.cexp, u.suma}, nullptr, nullptr);
     k_row_exps<<<cdiv(k, 8), 256, 0, s>>>(k, m, B, ldb, nullptr, u.bexp, u.sumb);
     HSIM_LAUNCHED();
-    k_balance<<<1, 256, 0, s>>>(k, sampled, m, u.suma, u.bexp, u.sumb, u.cexp);
-    HSIM_LAUNCHED();
     OzakiOperand Y = make_operand(m, k, u.dy, kDigits64, OzakiRole::Y), Ym = make_operand(m, k, u.my, 1, OzakiRole::Y);
-    ozaki_col_exps(s, k, m, B, ldb, Y.exps, u.cexp);
+    k_balance<<<1, 256, 0, s>>>(k, sampled, m, u.suma, u.bexp, u.sumb, u.cexp, Y.exps);
+    HSIM_LAUNCHED();
+    launch_col_exps(s, k, {B, m, ldb, pair_rows(B, ldb), Y.exps, nullptr}, nullptr, u.cexp);
     split_cols_into(s, Y, k, B, ldb, u.cexp);
     Ym.exps = Y.exps;
     const bool entries = held == Held::Entries;

@@ -144,8 +144,8 @@ constexpr int kSpmmRows = 16;  // rows (warps) per CTA of the column-block SpMM
 // Y = A X for k > 64: a CTA takes 16 consecutive rows of one 128-column block,
 // the column block the slow index: the CTA's gathered 1 KB row segments stay in
 // L1, and concurrently running CTAs share the same column block in L2.  Bound by
-// the FP64 pipe, 94 % of its rate at 10^6 rows x 750 (9.0 ms), where an
-// instruction costs a warp the same 77 clocks however many lanes it serves.
+// the FP64 pipe, 1.86 of nominally 2 lanes per clock and SM at 10^6 rows x 750 (9.0
+// ms), where an instruction costs a warp the same time however many lanes it serves.
 // Two layouts of a block on the lanes:
 // k_spmm4: four consecutive columns per lane, read as pairs (every block at
 //   least 97 columns wide: nothing to skip; 0.5 to 1 % faster than the other);

@@ -156,7 +156,7 @@ constexpr int kTrdThreads = 128;
 
 // Sum over the warp in fixed point: every value as a 57-bit integer against the
 // warp's largest exponent, three limbs added by redux, the total rounded once.
-// An FP64 add of a warp costs 77 issue clocks and 106 through a shuffle, five of
+// An FP64 add of a warp costs 64 to 76 issue clocks and 106 through a shuffle, five of
 // them 530; this takes about 200, and the values' truncation (2^-57 of the
 // largest) stays below the rounding of the FP64 tree.
 __device__ __forceinline__ double warp_sum_fixed(double v) {
@@ -315,16 +315,16 @@ __device__ __forceinline__ void rows_pass(int L, int n, double *a, const double 
 // ||A|| / ||u||^2: A is brought near 1 by a power of two where it is not within
 // 2^+-100 (as the rows are loaded; k_tri_prep takes it off T), and a column whose
 // norm is below 2^-400 is taken as reduced (its entries below the first are
-// dropped, a backward error of 2^-300 ||A|| at the most), so neither overflows.  With p = t A22 u and w = p - (t/2)(p.u) u
-// the update of row r is -(u_r w + w_r u) = -(u_r p + b_r u), b_r = p_r - t (p.u)
+// dropped, a backward error of 2^-300 ||A|| at the most), so neither overflows.
+// With p = t A22 u and w = p - (t/2)(p.u) u the update of row r is -(u_r w + w_r u) = -(u_r p + b_r u), b_r = p_r - t (p.u)
 // u_r: w is not formed.  An entry costs three FP64 instructions.
 // The second half of a block's threads only communicates: it arrives at the
 // barrier, waits and brings the entries to shared memory.
 // What bounds it: a chain per column.  Clocks at n = 75 / 750 (152 SMs): the rows
-// 1,800 / 3,800 (FP64 issue, 77 clocks per warp instruction, 2,900 of them at 750),
-// the other warps' sums 260 / 500, then the reflector 2,600 / 3,200 beside the
-// barrier and the loads 3,300 / 4,900, u^T A u 900 / 1,450, the next column 460 /
-// 980.  Per column 3.6 us at 75 and 5.7 us at 750; with the reflector before the
+// 1,800 / 3,800 (FP64 issue, 2,900 of them at 750), the other warps' sums 260 / 500,
+// then the reflector 2,600 / 3,200 (and some 300 for the square root and the division)
+// beside the barrier and the loads 3,300 / 4,900, u^T A u 900 / 1,450, the next column
+// 460 / 980.  Per column 3.5 us at 75 and 5.8 us at 750; with the reflector before the
 // product, one thread polling and loading after it, and branches between the rows
 // 4.6 and 7.4; with scaled reflectors, w formed, FP64 shuffles for the sums and
 // divisions 8.1 at 750.  Entries tagged with their column and polled for by every
@@ -764,7 +764,7 @@ __global__ void k_tri_prep(int n, double *__restrict__ d, double *__restrict__ e
 // Eigenvalues of the scaled T below x, and det(T - x I) as fm 2^fe.  The Sturm
 // sequence p_{j+1} = (d_j - x) p_j - e_j^2 p_{j-1} without divisions: three FP64
 // instructions a step, where d - x - e^2 / q takes about ten, and an FP64
-// instruction of a warp issues every 77 clocks on a sub-partition.  The count is
+// instruction of a warp issues every 64 to 76 clocks on a sub-partition.  The count is
 // the number of sign changes (an exact zero is counted with its own or the next
 // step, whatever its sign).  |d - x| <= 2, 2^-120 <= e^2 <= 1: eight steps grow
 // p by at most 2^13 and shrink it by at most 2^-480, then the pair is rescaled
@@ -859,7 +859,7 @@ __device__ __forceinline__ int group_le(bool le, int gbase, int L) {
 // quadratically (three to four FP64 rounds at n = 750, where equal sections take
 // nine); the counts still decide, and a round that does not shrink the bracket
 // fourfold, or a bracket of several eigenvalues, is followed by equal sections.
-// What bounds it: an FP64 round is n dependent steps of three instructions of 77
+// What bounds it: an FP64 round is n dependent steps of three instructions of 64 to 76
 // clocks, 84 us at n = 750 with one warp per sub-partition (G = ceil(m / (4 SMs)):
 // a second warp on a sub-partition doubles every round).
 __global__ void k_tri_bisect(int n, int m, int G, const double *__restrict__ d, const double *__restrict__ e2,
@@ -971,7 +971,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // dependent divisions a step and three solves, one lane at work (1.32 ms for 750
 // vectors); here the two sequences run without divisions, sixteen vectors to a
 // warp (forward in the lower lanes, backward in the upper: an FP64 instruction
-// of a warp takes the same 77 clocks for one lane as for 32), 0.1 ms.
+// of a warp takes the same time for one lane as for 32), 0.1 ms.
 //
 // k_tri_minors: S_t = P_t (dir 0) and B_{n-t} (dir 1), t < n, as seq[dir][t][i]
 // 2^xs[dir][t / 8][i]

@@ -108,6 +108,23 @@ def test_gram_of_one_block(hs, ctx, n, k):
     check(on_digits(hs, lambda: hs.gram(ctx, dA, dA)), A, A)
 
 
+@pytest.mark.parametrize("low", [120, 96, 1])
+@pytest.mark.parametrize("n", [1024, 4096])
+def test_gram_full_digits(hs, ctx, n, low):
+    """Every digit of both factors positive and up to its full size, 127: the digit
+    sums from D = 4 on pass 2^24 and their partial sums are odd."""
+    rng = np.random.default_rng(low)
+
+    def block(k):
+        T = np.zeros((n, k), dtype=object)
+        for s in range(7):
+            T = T * 256 + rng.integers(low, 128, (n, k)).astype(object)
+        return np.array([[float(t) for t in row] for row in T]) * 2.0 ** -55   # 53 of the 55 bits
+
+    A, B = block(40), block(33)
+    check(on_digits(hs, lambda: hs.gram(ctx, dev(A), dev(B))), A, B)
+
+
 # one row, tiles of 128 and 64 and their remainders, K steps of 16, two row ranges
 # (16 k bytes of digits to a row, 1 GiB to a range)
 SHAPES = [(1, 200, 20000), (127, 170, 130), (129, 177, 129), (1024, 165, 63), (4097, 200, 65), (70003, 41, 63),

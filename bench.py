@@ -663,8 +663,8 @@ def roofline(info, infos, hier, p, peaks, peak_src, precision, tol):
     ms_ritz = phases["ritz"]
     rflops = (4.0 / 3.0 + 2.0) * q ** 3 * calls
     jac = rflops / (ms_ritz * 1e-3) / 1e12 if ms_ritz > 0 else 0.0
-    kernels["ritz"] = {"kernel": "k_tridiag + k_tri_* (Householder tridiagonalisation, bisection, inverse "
-                                 "iteration, back transformation; FP64)", "bound": "alu",
+    kernels["ritz"] = {"kernel": "k_tridiag_rows + k_tri_* (Householder tridiagonalisation, Sturm counts, eigenvectors "
+                                 "from minors, back transformation; FP64)", "bound": "alu",
                        "achieved": jac, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": jac / FP64_PEAK_TFLOPS,
                        "peak_source": "GB300 nominal FP64 (1.25 TFLOP/s; a DFMA probe measured 1.19)",
                        "traffic": None, "flops_per_call": (4.0 / 3.0 + 2.0) * q ** 3, "calls_per_step": calls,
@@ -726,6 +726,9 @@ def roofline(info, infos, hier, p, peaks, peak_src, precision, tol):
         top["bf16_pipe"] = {"achieved": top["achieved"], "frac": top["frac"], "unit": "TFLOP/s",
                             "note": f"{gram_pairs} (Grams) and {upd_pairs} (update) BF16 digit-pair products "
                                     "per FP64 product (emulation work)"}
+        if peaks.get("bf16_tflops"):
+            # the sustained peak is taken at the power limit, below the clock of a solve
+            top["bf16_pipe"]["frac_of_burst"] = top["achieved"] / peaks["bf16_tflops"]
         top["achieved"] = fp64_eq
         top["frac"] = fp64_eq / top["peak"]
         top["work"] = ("method FLOPs: FP64 products of the Grams Psi^T [S Psi | M Psi] (n q (q+1) each, lower "
@@ -744,17 +747,17 @@ def roofline(info, infos, hier, p, peaks, peak_src, precision, tol):
 
 
 # DRAM bytes (read + write) per operand row of one k_ozaki_tc launch, from
-# one ncu capture of each product shape at 200,000 rows, q = 750
-# (profiles/ozaki_tc_traffic_n200k_q750.md): update (6 digits) 1.852 GB read +
-# 1.170 GB written; Gram with the solve's 5 digits 3.090 GB read + 3 MB written
-# for the full square product of the capture (the solve's Grams compute the
-# lower triangle: an upper bound).
-TC_TRAFFIC_PER_ROW = {"gram": (3090402816 + 3154688) / 200000, "update": (1852248576 + 1170459392) / 200000}
+# one ncu capture of each product shape, q = 750
+# (profiles/ozaki_tc_traffic_n200k_q750.md): update (6 digits) of 100,096 rows
+# 0.911 GB read + 0.566 GB written; Gram with the solve's 5 digits of 65,536 rows
+# 1.121 GB read + 9 MB written for the full square product of the capture (the
+# solve's Grams compute the lower triangle: an upper bound).
+TC_TRAFFIC_PER_ROW = {"gram": (1120637440 + 8705280) / 65536, "update": (911433984 + 565972224) / 100096}
 
 
 def tc_traffic(sizes, iters, q, gram_digits=6):
     """Per-launch DRAM traffic of k_ozaki_tc over one solve, scaled from the
-    200,000-row captures by the rows each launch processes (traffic grows in
+    captures by the rows each launch processes (traffic grows in
     proportion to the rows), against the algorithmic bytes (the BF16 digit
     slices read once: d slices x 2 bytes per operand value, d = gram_digits
     for the Grams and 6 for the update; the update's FP64 output, 8 bytes per
@@ -773,8 +776,8 @@ def tc_traffic(sizes, iters, q, gram_digits=6):
         launches += 3 * iters[t]
     return {"per_launch": tot / launches, "algorithmic_per_launch": alg / launches,
             "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one 5-digit Gram (full square, an "
-                    "upper bound for the solve's lower-triangle Grams) and one 6-digit update launch at "
-                    "200,000 x 750, scaled by rows to every launch of the solve and averaged per launch"}
+                    "upper bound for the solve's lower-triangle Grams; 65,536 x 750) and one 6-digit update launch "
+                    "(100,096 x 750), scaled by rows to every launch of the solve and averaged per launch"}
 
 
 def cpu_baseline(workload, info):

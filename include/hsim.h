@@ -309,23 +309,29 @@ hsim_status hsim_spmm(hsim_ctx *ctx, int n_rows, int n_cols, const int32_t *row_
                       int ldx, double *Y_dev, int ldy);
 /* G = A^T B (k_a x k_b, row-major, ld k_b) for tall A (n x k_a, ld lda) and
  * B (n x k_b, ld ldb): the reduced matrices Psi^T S Psi, Psi^T M Psi of Alg. 1.
- * Large products run on the BF16 tensor cores with seven digits per value (FP64
- * accuracy; columns whose largest entry stands out and non-finite input on the
- * FP64 units); their scratch is kept by the context for the next call (at most
- * 2 GiB). */
+ * Every entry is within n 2^-53 sum |a| |b| of the exact one, as FP64 arithmetic
+ * in any order is.  Large products run on the BF16 tensor cores with seven digits
+ * per value; 64 x 64 tiles of G in which an entry could miss that bound (entries
+ * that stand out in their column, graded or disjoint columns) or that meet infinities
+ * or NaN are computed on the FP64 units, and so is everything where the device has
+ * no room for the digits' scratch.  The scratch is kept by the context for the next
+ * call (at most 2 GiB) and given back when an allocation finds no room. */
 hsim_status hsim_gram(hsim_ctx *ctx, int n, int k_a, int k_b, const double *A_dev, int lda,
                       const double *B_dev, int ldb, double *G_dev);
 
 /* C = A B for A (n x k, ld lda) and small B (k x m, ld ldb), C (n x m, ld ldc):
- * the basis update Phi = Psi Phi_bar of Alg. 1.  Large products as hsim_gram's. */
+ * the basis update Phi = Psi Phi_bar of Alg. 1.  Every entry within k 2^-53
+ * sum |a| |b| of the exact one; large products as hsim_gram's. */
 hsim_status hsim_gemm_update(hsim_ctx *ctx, int n, int k, int m, const double *A_dev, int lda,
                              const double *B_dev, int ldb, double *C_dev, int ldc);
 
 /* The same two products evaluated on BF16 tensor cores with FP64 accuracy
  * (mixed-precision path): every FP64 operand is split against a power of two
  * per row or column into 6 integer digits of at most 8 bits, digit products
- * are accumulated exactly in FP32 over chunks of 256 and summed in FP32 pairs; the
- * result matches the FP64 product to about 2^-47 of the row/column maxima.
+ * are accumulated in FP32 over chunks of 256 (exactly, but for sums of weight
+ * 2^-32 and less that full-size digits of one sign carry past 2^24) and summed in
+ * FP32 pairs; the result matches the FP64 product to about 2^-47 of the row/column
+ * maxima.
  * hsim_gram_tc takes `digits` = 6 (that accuracy) or 5 (2^-39, 15 digit
  * products instead of 21; the solve's Grams at tolerances >= 1e-6).
  * Arguments as hsim_gram and hsim_gemm_update (G is ka x kb, ld kb). */

@@ -746,13 +746,11 @@ def roofline(info, infos, hier, p, peaks, peak_src, precision, tol):
     return top
 
 
-# DRAM bytes (read + write) per operand row of one k_ozaki_tc launch, from
-# one ncu capture of each product shape, q = 750
-# (profiles/ozaki_tc_traffic_n200k_q750.md): update (6 digits) of 100,096 rows
-# 0.911 GB read + 0.566 GB written; Gram with the solve's 5 digits of 65,536 rows
-# 1.121 GB read + 9 MB written for the full square product of the capture (the
-# solve's Grams compute the lower triangle: an upper bound).
-TC_TRAFFIC_PER_ROW = {"gram": (1120637440 + 8705280) / 65536, "update": (911433984 + 565972224) / 100096}
+# DRAM bytes (read + write) per operand row of one k_ozaki_tc launch, from an ncu
+# capture of the launches of a mixed solve, 250,000 rows, q = 750
+# (profiles/ozaki_tc_traffic_n250k_q750.md): Gram (5 digits, lower triangle) 4.138 GB
+# read + 25 MB written, update (6 digits) 2.293 GB read + 1.468 GB written.
+TC_TRAFFIC_PER_ROW = {"gram": (4137828608 + 25411840) / 250000, "update": (2293127680 + 1468241664) / 250000}
 
 
 def tc_traffic(sizes, iters, q, gram_digits=6):
@@ -775,9 +773,9 @@ def tc_traffic(sizes, iters, q, gram_digits=6):
         alg += iters[t] * (2 * 4.0 * gram_digits * n * qp + (12.0 * n * qp + 8.0 * n * q))
         launches += 3 * iters[t]
     return {"per_launch": tot / launches, "algorithmic_per_launch": alg / launches,
-            "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one 5-digit Gram (full square, an "
-                    "upper bound for the solve's lower-triangle Grams; 65,536 x 750) and one 6-digit update launch "
-                    "(100,096 x 750), scaled by rows to every launch of the solve and averaged per launch"}
+            "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one 5-digit Gram and one 6-digit update "
+                    "launch of a mixed solve at 250,000 x 750, scaled by rows to every launch of the solve and "
+                    "averaged per launch"}
 
 
 def cpu_baseline(workload, info):

@@ -309,7 +309,7 @@ hsim_status hsim_spmm(hsim_ctx *ctx, int n_rows, int n_cols, const int32_t *row_
                       int ldx, double *Y_dev, int ldy);
 /* G = A^T B (k_a x k_b, row-major, ld k_b) for tall A (n x k_a, ld lda) and
  * B (n x k_b, ld ldb): the reduced matrices Psi^T S Psi, Psi^T M Psi of Alg. 1.
- * Every entry is within n 2^-53 sum |a| |b| of the exact one, as FP64 arithmetic
+ * Every entry is within about n 2^-53 sum |a| |b| of the exact one, as FP64 arithmetic
  * in any order is.  Large products run on the BF16 tensor cores with seven digits
  * per value; 64 x 64 tiles of G in which an entry could miss that bound (entries
  * that stand out in their column, graded or disjoint columns) or that meet infinities
@@ -320,7 +320,7 @@ hsim_status hsim_gram(hsim_ctx *ctx, int n, int k_a, int k_b, const double *A_de
                       const double *B_dev, int ldb, double *G_dev);
 
 /* C = A B for A (n x k, ld lda) and small B (k x m, ld ldb), C (n x m, ld ldc):
- * the basis update Phi = Psi Phi_bar of Alg. 1.  Every entry within k 2^-53
+ * the basis update Phi = Psi Phi_bar of Alg. 1.  Every entry within about k 2^-53
  * sum |a| |b| of the exact one; large products as hsim_gram's. */
 hsim_status hsim_gemm_update(hsim_ctx *ctx, int n, int k, int m, const double *A_dev, int lda,
                              const double *B_dev, int ldb, double *C_dev, int ldc);

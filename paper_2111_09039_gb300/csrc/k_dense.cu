@@ -973,8 +973,6 @@ int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar,
             double *A = Wz == T ? F : T;
             tc_mm(s, k, k, Wz, k, Sbar, lds, W, k, oz, err);
             tc_mm(s, k, k, W, k, Wz, k, A, k, oz, err);
-            k_symmetrize<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, A, k);
-            HSIM_LAUNCHED();
             sym_eig(s, k, m, A, evals, V, m, ework);
             tc_mm(s, k, m, Wz, k, V, m, X, ldx, oz, err);
             if (k > kSmallMM) ozaki_check(s, err);
@@ -1014,8 +1012,6 @@ int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar,
         HSIM_LAUNCHED();
         tc_mm(s, k, k, Cr, k, Sbar, lds, W, k, oz, err);
         tc_mm(s, k, k, W, k, Cc, k, T, k, oz, err);
-        k_symmetrize<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, T, k);
-        HSIM_LAUNCHED();
         sym_eig(s, k, m, T, evals, V, m, ework);
         tc_mm(s, k, m, Cc, k, V, m, X, ldx, oz, err);
         if (k > kSmallMM) ozaki_check(s, err);
@@ -1038,9 +1034,6 @@ int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar,
     k_transpose<<<tg, tb, 0, s>>>(k, W, k, T, k);
     HSIM_LAUNCHED();
     forward(T);
-    // symmetrise against rounding: T = (T + T^T)/2
-    k_symmetrize<<<cdiv((int64_t)k * k, 256), 256, 0, s>>>(k, T, k);
-    HSIM_LAUNCHED();
     // lowest m eigenpairs of A (ascending), eigenvectors into X (k x m)
     sym_eig(s, k, m, T, evals, X, ldx, ework);
     // X = C^-T V = L^-T D^-1/2 V

@@ -132,14 +132,24 @@ __global__ void __launch_bounds__(kTriThreads) k_tridiag(int n, double *__restri
     }
 }
 
-// Largest biased exponent of the entries of A (out starts at zero).
-__global__ void __launch_bounds__(kTriThreads) k_max_exp(int64_t n, const double *__restrict__ A, int *__restrict__ out) {
+// A = (A + A^T) / 2 against the rounding of the products that gave it, and the
+// largest biased exponent of its entries (out starts at zero).
+__global__ void __launch_bounds__(kTriThreads) k_symmetrize_max(int n, double *__restrict__ A, int *__restrict__ out) {
+    const int64_t idx = (int64_t)blockIdx.x * kTriThreads + threadIdx.x;
+    const int i = (int)(idx / n), j = (int)(idx % n);
     int m = 0;
-#pragma unroll 4
-    for (int64_t i = (int64_t)blockIdx.x * kTriThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kTriThreads)
-        m = max(m, (__double2hiint(A[i]) >> 20) & 0x7FF);
+    if (i < n && j >= i) {
+        double v = A[(size_t)i * n + j];
+        if (j > i) {
+            v = 0.5 * (v + A[(size_t)j * n + i]);
+            A[(size_t)i * n + j] = v;
+            A[(size_t)j * n + i] = v;
+        }
+        m = (__double2hiint(v) >> 20) & 0x7FF;
+    }
     m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+    // most warps find it reached already
+    if ((threadIdx.x & 31) == 0 && m > *(volatile int *)out) atomicMax(out, m);
 }
 
 // Power of two that brings a matrix with that exponent near 1; 0 where it is
@@ -1354,10 +1364,9 @@ void sym_eig(cudaStream_t s, int n, int m, double *A, double *evals, double *X, 
     unsigned *counter = reinterpret_cast<unsigned *>(bounds + 5);  // arrivals of the barriers
     int *amax = reinterpret_cast<int *>(bounds + 6);               // largest exponent of A
     HSIM_CUDA(cudaMemsetAsync(err, 0, 3 * sizeof(double), s));
+    k_symmetrize_max<<<cdiv((int64_t)n * n, kTriThreads), kTriThreads, 0, s>>>(n, A, amax);
+    HSIM_LAUNCHED();
     if (G > 0) {
-        k_max_exp<<<(unsigned)std::min<int64_t>(sms, ((int64_t)n * n + 4 * kTriThreads - 1) / (4 * kTriThreads)), kTriThreads,
-                    0, s>>>((int64_t)n * n, A, amax);
-        HSIM_LAUNCHED();
         if (rmax == 4) done = launch_tridiag_rows<4>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf, counter, err, amax);
         else if (rmax == 8) done = launch_tridiag_rows<8>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf, counter, err, amax);
         else done = launch_tridiag_rows<16>(s, G, rsmem, sms, n, A, d, e, tau, Vh, pbuf, rbuf, counter, err, amax);

@@ -127,7 +127,8 @@ void residual_sums_mixed(cudaStream_t s, int n, int k, const double *SP, int lds
 int ritz(cudaStream_t s, int k, const double *Sbar, int lds, const double *Mbar, int ldm, double *evals,
          double *X, int ldx, double *work, int *sweeps, int *flag_dev, int *flag_host, int m = 0, bool tc = false);
 // ---- tridiagonal eigensolver (k_tridiag.cu) ----------------------------------
-// lowest m eigenpairs of the symmetric n x n A (row-major, ld n, destroyed):
+// lowest m eigenpairs of the symmetric part of the n x n A (row-major, ld n,
+// destroyed):
 // evals ascending (m), X (n x m, ld ldx) orthonormal eigenvectors; work of
 // sym_eig_work_size(n, m) doubles; waits for the stream in between
 size_t sym_eig_work_size(int n, int m);
